@@ -106,7 +106,7 @@ SACZT_SAMPLE_D = 2e-3
 # launches), from a one-pass ncu capture of this workload; reported only while
 # the kernel's sources hash to what was captured (null otherwise).
 KERNEL_SOURCES = {
-    "dense": ["dense.cu", "tc_ptx.cuh", "fzp_internal.cuh"],
+    "dense": ["nodes.cu", "dense.cu", "membrane.cuh", "tc_ptx.cuh", "fzp_internal.cuh"],
     "bluestein": ["bluestein.cu", "fzp_internal.cuh"],
 }
 TRAFFIC = {
@@ -237,6 +237,34 @@ def partitioned_flops(info: dict, j0: int, j1: int) -> float:
     blocks = float(np.sum(hi // S - lo // S + 1))
     fft = 5.0 * P * lgP
     return blocks * (fft + 8.0 * P) + (j1 - j0) * fft
+
+
+def node_count(info: dict, lam: float, f: float, M: int, pitch: float, deformed: bool = False) -> int:
+    """Nodes per axis that the dense form's contraction runs on (nodes.cu), for an
+    ROI centred on the focus: the positive half of n nodes for a flat plate,
+    all of them for a membrane; 0 where the ROI's band takes the general kernel."""
+    dof = (M - (1 if deformed else 0)) * pitch * 2.0 * info["R"] / (lam * f)
+    for n, most in ((64, 36.0), (128, 80.0), (256, 170.0)):
+        ns = n if deformed else n // 2
+        if ns in (64, 128) and not (deformed and ns > 64) and dof <= most:
+            return ns
+    return 0
+
+
+def node_flops(info: dict, nodes: int, j0: int, j1: int, deformed: bool = False) -> float:
+    """Tensor work that the contraction on nodes does for rows [j0, j1), all mask
+    passes: 2 real rows x nodes x 2 flops x 2 split terms (a membrane: 3, and two
+    masks) per sample inside the disc that is left after the folds: a flat plate's
+    columns +-d are one, and so are its rows +-d when both are in the range; over
+    all rows only the part up to the diagonal is contracted."""
+    c, n = info["c"], info["N"]
+    inside = disc_samples(n, c, info["s_R"], j0, j1)
+    if deformed:
+        return 24.0 * nodes * inside
+    h = min(j1 - 1 - c, c - j0)
+    both = disc_samples(n, c, info["s_R"], c - h, c + h + 1) if h >= 0 else 0
+    whole = h >= c or (h + 1) ** 2 > info["s_R"]
+    return 8.0 * nodes * info["passes"] * (both / (8.0 if whole else 4.0) + (inside - both) / 2.0)
 
 
 def membrane_forms_and_roofline(fzp, infos: list, M: int, steps: int, ms: float):
@@ -763,12 +791,18 @@ def main():
         inside = disc_samples(N, info["c"], info["s_R"], j0, j1)
         per = 12.0 if wl.get("deform") else 8.0  # a membrane pass takes 3 split products, not 2
         flops_launch = per * M * inside * info["passes"] * args.steps / launches
+        work = f"{per:g} M flops per aperture sample inside the disc and mask pass"
+        if prof["dominant_name"] == "k_nodes":
+            nodes = node_count(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], bool(wl.get("deform")))
+            flops_launch = node_flops(info, nodes, j0, j1, bool(wl.get("deform"))) * args.steps / launches
+            work = (f"{per * (2 if wl.get('deform') else 1):g} x {nodes} nodes flops per sample inside the disc left "
+                    "after the symmetry folds")
         achieved = flops_launch / (avg_ms / 1e3) / 1e12
         peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
         roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": _traffic(args.workload, "dense"), "kernel": prof["dominant_name"],
                 "peak_source": peak_kind + " bf16 sustained",
-                "work": f"{per:g} M flops per aperture sample inside the disc and mask pass",
+                "work": work,
                 "disc_samples_per_launch": inside * args.steps / launches}
     elif args.form == "saczt":
         # k_sa_rows<1>: one pass of the padded grid through HBM (P^2 complex64

@@ -120,7 +120,11 @@ typedef struct fzp_params {
                           generated mask tile through distributed shared memory,
                           each generating its share of the rows (1, 2 or 4;
                           0 -> the largest of 4, 2, 1 dividing the M/64 tile
-                          pairs; other values pad the pairs with zero tiles)      */
+                          pairs; other values pad the pairs with zero tiles).
+                          Split-BF16 plans whose ROI samples the field several
+                          times finer than its band contract onto that many
+                          interpolation nodes instead, in single CTAs (0 and 1;
+                          nodes.cu); 2 and 4 keep the clusters                    */
   int32_t levels;      /* 0 or 1: binary amplitude FZP (Fig. 2: open where the
                           paraxial zone index is odd).  L >= 2: L-level phase FZP
                           (Fig. 18 Stage 3): transmission e^{-2 pi i q/L} inside

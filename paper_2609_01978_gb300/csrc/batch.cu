@@ -268,14 +268,15 @@ fzp_status fzp_batch_plan(const fzp_params* params, int n, fzp_batch_t* out) {
     P->c1_rows = (2 * (int64_t)P->M + 511) / 512 * 512;
     FormSizes z;
     st = P->form == FZP_FORM_DENSE ? dense_layout(*P, &z) : bluestein_layout(*P, &z);
+    if (st == FZP_OK && P->nd.n > 0) st = nodes_upload(*P);
     if (st != FZP_OK) { batch_release(b); return st; }
     mx.pre = std::max(mx.pre, z.pre); mx.H = std::max(mx.H, z.H); mx.tab = std::max(mx.tab, z.tab);
     mx.Z = std::max(mx.Z, z.Z); mx.G = std::max(mx.G, z.G); mx.A = std::max(mx.A, z.A);
-    mx.sched = std::max(mx.sched, z.sched);
-    const size_t rowsC1 = (size_t)((2 * (int64_t)P->M + 511) / 512 * 512) * (size_t)P->chunk_rows;
+    mx.sched = std::max(mx.sched, z.sched); mx.X = std::max(mx.X, z.X);
+    const size_t rowsC1 = c1_elems(*P);
     if (P->precision == FZP_PREC_FP64) c1d = std::max(c1d, rowsC1 * 8);
     else c1 = std::max(c1, rowsC1 * 4);
-    uacc = std::max(uacc, (size_t)P->M * P->M * sizeof(double2));
+    uacc = std::max(uacc, std::max((size_t)P->nd.n * P->nd.ns, (size_t)P->M * P->M) * sizeof(double2));
     metr = std::max(metr, 8192 * sizeof(double) + (size_t)P->M * P->M * sizeof(double2));
   }
   auto alloc = [&](size_t bytes) -> void* {
@@ -288,9 +289,9 @@ fzp_status fzp_batch_plan(const fzp_params* params, int n, fzp_batch_t* out) {
   };
   void *pre = alloc(mx.pre), *H = alloc(mx.H), *tab = alloc(mx.tab), *Z = alloc(mx.Z), *G = alloc(mx.G),
        *A = alloc(mx.A), *sched = alloc(mx.sched), *C1 = alloc(c1), *C1d = alloc(c1d), *U = alloc(uacc), *M = alloc(metr),
-       *err = alloc(sizeof(int));
+       *err = alloc(sizeof(int)), *X = alloc(mx.X);
   if ((mx.pre && !pre) || (mx.H && !H) || (mx.tab && !tab) || (mx.Z && !Z) || (mx.G && !G) || (mx.A && !A) ||
-      (mx.sched && !sched) ||
+      (mx.sched && !sched) || (mx.X && !X) ||
       (c1 && !C1) || (c1d && !C1d) || !U || !M || !err) {
     cudaGetLastError();
     batch_release(b);
@@ -300,6 +301,7 @@ fzp_status fzp_batch_plan(const fzp_params* params, int n, fzp_batch_t* out) {
   for (fzp_plan_s* P : b->inst) {
     P->bs.d_pre = pre; P->bs.d_H = H; P->bs.d_tab = tab; P->bs.d_Z = Z; P->bs.d_G = G;
     P->dn.d_A = A;
+    P->nd.d_X = reinterpret_cast<double2*>(X);
     P->dn.d_sched = reinterpret_cast<int*>(sched);
     P->d_C1 = reinterpret_cast<float*>(C1);
     P->d_C1d = reinterpret_cast<double*>(C1d);
@@ -320,15 +322,12 @@ fzp_status fzp_batch_plan(const fzp_params* params, int n, fzp_batch_t* out) {
 static fzp_status batch_enqueue(Plan& P, void* field, cudaStream_t s) {
   fzp_status st = P.form == FZP_FORM_DENSE ? dense_fill_tables(P, s) : bluestein_fill_tables(P, s);
   if (st != FZP_OK) return st;
-  FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, (size_t)P.M * P.M * sizeof(double2), s));
   int64_t jlo, jhi;
   disc_rows(P, jlo, jhi);
-  for (int64_t j0 = jlo; j0 < jhi; j0 += P.chunk_rows) {
-    const int64_t rows = std::min(P.chunk_rows, jhi - j0);
-    st = chunk_passes(P, j0, rows, s);
-    if (st != FZP_OK) return st;
-  }
-  return epilogue(P, field, 0, s);
+  bool sym = false;
+  st = propagate_rows(P, jlo, jhi, &sym, s);
+  if (st != FZP_OK) return st;
+  return finish_field(P, field, 0, sym, s);
 }
 
 fzp_status fzp_batch_propagate(fzp_batch_t b, void* const* d_fields, void* stream) {

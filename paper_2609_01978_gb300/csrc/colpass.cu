@@ -10,6 +10,7 @@
 // B_j = dj delta (turns, dj = j - c).  A_j and B_j are reduced in FP64 once per
 // row j; for the FP32 path B_j is split as hi + lo with hi a multiple of 2^-14
 // so that n * hi is exact in FP32 for n < 1024.
+#include <algorithm>
 #include <cmath>
 
 #include "fzp_internal.cuh"
@@ -17,13 +18,18 @@
 namespace fzp {
 namespace {
 
-constexpr int TN = 64, TM = 64, TJ = 16, JC = 2048;
+constexpr int TN = 64, TM = 64, TJ = 16;
 
 struct ColArgs {
   int64_t c, j0, rows, c1_stride;
-  int M;
+  int64_t jc;     // rows per block of the grid's z
+  int kind;       // RowKind: the row's kernel K(dj), K(dj) + K(-dj) or K(-dj)
+  int slices;       // images of C1 to be summed, slice_off values apart
+  int64_t slice_off;
+  int64_t sin_off;  // > 0: C1 holds the rows of T cos(phi) and, sin_off values on, of T sin(phi)
+  int M;          // outputs per row (m)
   double kappa, delta;
-  double msh;     // ROI shift in pitches: y_n = (n - msh) p
+  double msh;     // ROI (or node) shift in pitches: y_n = (n - msh) p
   double wr, wi;  // weight of this pass's field (1, 0 for a single-pass plate)
 };
 
@@ -31,8 +37,7 @@ template <typename R> struct RowPhase;
 template <> struct RowPhase<float> { float fa, hi, lo; };
 template <> struct RowPhase<double> { double a, b; };
 
-__device__ __forceinline__ void row_phase(const ColArgs& g, int64_t j, RowPhase<float>& rp) {
-  const double dj = (double)(j - g.c);
+__device__ __forceinline__ void row_phase(const ColArgs& g, double dj, RowPhase<float>& rp) {
   const double A = dj * dj * (0.5 * g.kappa) + g.msh * dj * g.delta;
   const double fb = frac_turns(dj * g.delta);
   const double hi = rint(fb * 16384.0) / 16384.0;
@@ -40,8 +45,7 @@ __device__ __forceinline__ void row_phase(const ColArgs& g, int64_t j, RowPhase<
   rp.hi = (float)hi;
   rp.lo = (float)(fb - hi);
 }
-__device__ __forceinline__ void row_phase(const ColArgs& g, int64_t j, RowPhase<double>& rp) {
-  const double dj = (double)(j - g.c);
+__device__ __forceinline__ void row_phase(const ColArgs& g, double dj, RowPhase<double>& rp) {
   rp.a = frac_turns(dj * dj * (0.5 * g.kappa) + g.msh * dj * g.delta);
   rp.b = frac_turns(dj * g.delta);
 }
@@ -57,16 +61,16 @@ __device__ __forceinline__ double2 kern(const RowPhase<double>& rp, int n) {
   return cis_turns_d(rp.a - (double)n * rp.b);
 }
 
-// grid (M/TM, M/TN, ceil(rows/JC)); 256 threads; each thread 4 n x 4 m outputs.
+// grid (M/TM, M/TN, ceil(rows/jc)); 256 threads; each thread 4 n x 4 m outputs.
 template <typename R>
 __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
   using C = typename Cplx<R>::T;
   __shared__ C sK[TJ][TN + 1];
   __shared__ C sC[TJ][TM + 1];
-  __shared__ RowPhase<R> sP[TJ];
+  __shared__ RowPhase<R> sP[2][TJ];  // of dj (mirrored rows: -dj) and, folded, of -dj
   const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
-  const int64_t jb = (int64_t)blockIdx.z * JC;
-  const int64_t je = jb + JC < g.rows ? jb + JC : g.rows;
+  const int64_t jb = (int64_t)blockIdx.z * g.jc;
+  const int64_t je = jb + g.jc < g.rows ? jb + g.jc : g.rows;
   const int tid = threadIdx.x;
   const int tn = tid >> 4, tm = tid & 15;  // 16 x 16 threads, 4 x 4 outputs each
   C acc[4][4];
@@ -75,10 +79,11 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
 #pragma unroll
     for (int b = 0; b < 4; ++b) { acc[a][b].x = 0; acc[a][b].y = 0; }
   for (int64_t j = jb; j < je; j += TJ) {
-    if (tid < TJ) {
+    if (tid < 2 * TJ) {
+      const double dj = (double)(g.j0 + j + (tid & (TJ - 1)) - g.c);
       RowPhase<R> rp;
-      row_phase(g, g.j0 + j + tid, rp);
-      sP[tid] = rp;
+      row_phase(g, (tid >= TJ) != (g.kind == ROWS_MIRRORED) ? -dj : dj, rp);
+      sP[tid / TJ][tid & (TJ - 1)] = rp;
     }
     // C tile: TJ rows x TM columns (j contiguous in C1)
     for (int t = tid; t < TJ * TM; t += 256) {
@@ -87,8 +92,16 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
       C v;
       v.x = 0; v.y = 0;
       if (j + jj < je) {
-        v.x = C1[(int64_t)c1_row_re(m) * g.c1_stride + j + jj];
-        v.y = C1[(int64_t)c1_row_im(m) * g.c1_stride + j + jj];
+        const int64_t re = (int64_t)c1_row_re(m) * g.c1_stride + j + jj, im = (int64_t)c1_row_im(m) * g.c1_stride + j + jj;
+        for (int sl = 0; sl < g.slices; ++sl) {
+          const R* S = C1 + sl * g.slice_off;
+          v.x += S[re];
+          v.y += S[im];
+          if (g.sin_off > 0) {  // K (T cos + i T sin)
+            v.x -= S[g.sin_off + im];
+            v.y += S[g.sin_off + re];
+          }
+        }
       }
       sC[jj][mm] = v;
     }
@@ -97,7 +110,10 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
       const int jj = t / TN, nn = t % TN;
       C k;
       k.x = 0; k.y = 0;
-      if (j + jj < je) k = kern(sP[jj], n0 + nn);
+      if (j + jj < je) {
+        k = kern(sP[0][jj], n0 + nn);
+        if (g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c) k = cadd(k, kern(sP[1][jj], n0 + nn));
+      }
       sK[jj][nn] = k;
     }
     __syncthreads();
@@ -156,13 +172,31 @@ __global__ void k_intensity(int64_t count, const double2* __restrict__ U, double
 
 }  // namespace
 
-fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, cudaStream_t s) {
-  ColArgs g{P.c, j0, rows, P.chunk_rows, P.M, P.kappa, P.delta, P.msh, 1.0, 0.0};
+fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStream_t s) {
+  const bool nodes = P.nd.n > 0;
+  ColArgs g{};
+  g.c = nodes && P.nd.fold ? 0 : P.c;
+  g.j0 = j0;
+  g.rows = rows;
+  g.c1_stride = P.c1_stride;
+  g.kind = kind;
+  g.M = nodes ? P.nd.ns : P.M;
+  g.kappa = P.kappa;
+  g.delta = nodes ? P.nd.delta : P.delta;
+  g.msh = !nodes ? P.msh : P.nd.yfull ? 0.5 * (P.nd.n - 1) : P.nd.msh;
+  g.wr = 1.0;
   if (P.pass_index >= 0) {
     g.wr = P.passes[P.pass_index].wr;
     g.wi = P.passes[P.pass_index].wi;
   }
-  dim3 grid((unsigned)(P.M / TM), (unsigned)(P.M / TN), (unsigned)((rows + JC - 1) / JC));
+  g.slices = nodes ? P.nd.slices : 1;
+  g.slice_off = nodes ? P.nd.slice_elems : 0;
+  if (nodes && P.has_deform) g.sin_off = 128 * P.c1_stride;
+  // rows per block: 2048, fewer where that leaves the GPU idle (few output tiles)
+  const int ny = nodes && P.nd.yfull ? P.nd.n : g.M;
+  const int64_t tiles = (int64_t)(g.M / TM) * (ny / TN);
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(4 * TJ, (rows * tiles / 456 + TJ - 1) / TJ * TJ));
+  dim3 grid((unsigned)(g.M / TM), (unsigned)(ny / TN), (unsigned)((rows + g.jc - 1) / g.jc));
   if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
   else k_colpass<float><<<grid, 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
   P.launches += 1;

@@ -343,7 +343,7 @@ size_t colpass_tc_smem() { return 1024 + TSTAGES * (TA_BYTES + TB_BYTES) + 256; 
 
 // Usable for dense plans (the kernel-matrix images exist) with M a multiple of 128.
 bool column_pass_tc_applies(const Plan& P) {
-  return P.form == FZP_FORM_DENSE && P.dn.d_A != nullptr && (P.M % 128) == 0 && P.precision == FZP_PREC_SPLIT_BF16;
+  return P.form == FZP_FORM_DENSE && P.nd.n == 0 && P.dn.d_A != nullptr && (P.M % 128) == 0 && P.precision == FZP_PREC_SPLIT_BF16;
 }
 
 fzp_status column_pass_tc(Plan& P, int64_t j0, int64_t rows, cudaStream_t s) {

@@ -49,6 +49,7 @@
 #include <cmath>
 
 #include "fzp_internal.cuh"
+#include "membrane.cuh"
 #include "tc_ptx.cuh"
 
 namespace fzp {
@@ -528,39 +529,6 @@ __device__ __forceinline__ void expand_signed(uint32_t disc, uint32_t odd, uint3
   expand_bits(odd, sgn);
 #pragma unroll
   for (int k = 0; k < 16; ++k) w[k] = mag[k] | ((sgn[k] << 8) & 0x80008000u);
-}
-
-// Membrane pass: one row's T cos(phi) (or T sin(phi)) on 8-column chunks of a
-// 32-column block given the block's open bits, as BF16 hi and lo planes (the
-// 16-byte chunks of the 64-byte-swizzled row).  phi / 2 pi = 2 w / lambda in
-// FP32, walked along the row from the first column: the wrinkle's phasor
-// e^{2 pi i t} (t = di kx + dj ky, integer turns dropped exactly) turns by
-// e^{2 pi i kx} per column, a ridge's g = exp(-q d^2) by its ratio r, which
-// itself scales by rho = exp(-2 q nx^2); the sum is reduced to [-1/2, 1/2]
-// turns before one hardware sine or cosine (absolute error below 4e-7; the
-// walk adds ~1e-6 relative over 32 columns).  A ridge below 1e-30 at the
-// first column stays below 1e-29 in the block (its width is hundreds of
-// columns) and is left out.
-struct CxRow {
-  float fjkh, fjkl, fj2, cr[3];  // row terms: dj kyh, dj kyl, dj^2, ridge offsets
-};
-
-__device__ __forceinline__ void cx_row_init(const DeformCoef& d, int64_t dj, CxRow& r) {
-  const float fj = (float)dj;
-  r.fjkh = fj * d.kyh;
-  r.fjkl = fj * d.kyl;
-  r.fj2 = fj * fj;
-#pragma unroll
-  for (int e = 0; e < 3; ++e) r.cr[e] = (fj - d.pj[e]) * d.ny[e] - d.pi_[e] * d.nx[e];
-}
-
-// Two FP32 values -> packed BF16 hi (RN) and lo (RN of the remainder), lower
-// half from a: one cvt.rn.bf16x2 per plane (a goes to the upper half of the
-// instruction's result when given first, so b is given first).
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
-  const float ah = __uint_as_float(hi << 16), bh = __uint_as_float(hi & 0xffff0000u);
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b - bh), "f"(a - ah));
 }
 
 // Chunks [q0, q0 + nq) of the row (8 columns each); di0 = column of the block
@@ -1378,10 +1346,14 @@ fzp_status run_dense(Plan& P, DenseArgs& a, int mode, const char* name, cudaStre
 
 }  // namespace
 
-fzp_status dense_layout(Plan& P, FormSizes* out) { return layout_cols(P, P.N, out); }
+fzp_status dense_layout(Plan& P, FormSizes* out) {
+  const fzp_status st = layout_cols(P, P.N, out);
+  return st == FZP_OK && P.nd.n > 0 ? nodes_layout(P, out) : st;
+}
 
 fzp_status dense_fill_tables(Plan& P, cudaStream_t s) {
   Dense& d = P.dn;
+  if (P.nd.n > 0) return nodes_fill(P, s);
   k_build_A<<<8 * d.num_sms, 256, 0, s>>>(P.M, P.msh, P.N, d.kblocks, d.npairs, P.c, P.kappa, P.delta,
                                           reinterpret_cast<uint8_t*>(d.d_A));
   P.launches += 1;
@@ -1423,7 +1395,12 @@ fzp_status dense_build_tables(Plan& P) {
   FZP_CUDA_TRY(cudaMalloc(&P.dn.d_A, z.A));
   FZP_CUDA_TRY(cudaMalloc(&P.dn.d_sched, z.sched));
   P.device_bytes += z.A + z.sched;
-  if (P.dn.extra_ctas > 0) {
+  if (P.nd.n > 0) {
+    FZP_CUDA_TRY(cudaMalloc(&P.nd.d_X, z.X));
+    P.device_bytes += z.X;
+    st = nodes_upload(P);
+    if (st != FZP_OK) return st;
+  } else if (P.dn.extra_ctas > 0) {
     FZP_CUDA_TRY(cudaMalloc(&P.dn.d_sched2, z.sched));
     FZP_CUDA_TRY(cudaStreamCreateWithFlags(&P.dn.s2, cudaStreamNonBlocking));
     FZP_CUDA_TRY(cudaEventCreateWithFlags(&P.dn.ev_fork, cudaEventDisableTiming));
@@ -1437,6 +1414,7 @@ fzp_status dense_build_tables(Plan& P) {
 // mode for plates with passes (L >= 4, positive-centred), the block-wise
 // generator for cluster launches, the walker for single-CTA launches.
 fzp_status dense_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t s) {
+  if (P.nd.n > 0) return nodes_mask(P, j0, rows, out, s);
   const bool level = !P.passes.empty();
   const int mode = level ? (P.mg.centre_open ? EXPORT_EVEN : EXPORT_LEVELS)
                          : (P.levels == 2 ? EXPORT_SIGNED : EXPORT_BITS);

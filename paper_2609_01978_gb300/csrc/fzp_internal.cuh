@@ -207,6 +207,28 @@ struct Dense {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
+// The dense form on interpolation nodes (nodes.cu): n nodes across the ROI, of
+// which ns are evaluated (the positive half of them for an even field).
+struct NodeSet {
+  int n = 0, ns = 0;       // n = 0: the plan does not use nodes
+  int Mo = 0;              // outputs per side of the interpolation (even: M / 2 + 1)
+  bool even = false;       // flat plate, ROI centred on the focus
+  bool fold = false;       // flat plate: columns and rows +-d folded
+  int64_t kblocks = 0;     // ceil(columns / 32)
+  double half = 0, h = 0;  // ROI half width and node pitch, in ROI pitches
+  double band = 0;         // 2 R p / (lambda f): the field's band, cycles per pitch
+  double delta = 0, msh = 0;  // the nodes as a grid: x_k = (k - msh) h p, delta = h p dx / (lambda f)
+  double* d_W = nullptr;   // interpolation [ns][Mo] (owned by the plan, also in a batch)
+  double* d_Wy = nullptr;  // [n][M], behind d_W: along y when the rows are not symmetric
+  bool yfull = false;      // the call being run takes all n nodes along y
+  int slices = 1;          // images of C1 in the chunk being run, and their distance
+  int64_t slice_elems = 0;
+  double2* d_X = nullptr;  // [ns][Mo] rows interpolated
+};
+
+// What a row of the column pass stands for (flat plates: distances from the axis).
+enum RowKind { ROWS_PLAIN = 0, ROWS_FOLDED = 1, ROWS_MIRRORED = 2 };
+
 // SA-CZT (Sec. 3.6, Fig. 5): padded grid and its buffers.
 struct SaCzt {
   int64_t P = 0;           // padded grid side, a power of two >= 1.5 N
@@ -256,6 +278,8 @@ struct Plan {
   Bluestein bs;
   SaCzt sa;
   Dense dn;
+  NodeSet nd;
+  int64_t c1_stride = 0;        // row length of C1 in the chunk being run
   // tracing: kernel launches issued, and CUDA events around the dominant
   // kernel (recorded on the launching stream when profiling is enabled)
   int64_t launches = 0;
@@ -264,6 +288,14 @@ struct Plan {
   size_t prof_used = 0;
   const char* dominant = "";
 };
+
+// Elements of a plan's row intermediate: C1 of one chunk; a small membrane on
+// nodes takes eight images of its two masks' rows.
+inline size_t c1_elems(const Plan& P) {
+  const size_t all = (size_t)((2 * (int64_t)P.M + 511) / 512 * 512) * (size_t)P.chunk_rows;
+  if (P.nd.n > 0 && P.has_deform && P.N <= 8192) return all > 2048u * (size_t)P.chunk_rows ? all : 2048u * (size_t)P.chunk_rows;
+  return all;
+}
 
 // FP32 deformation coefficients of a plan with a deformation (host).
 DeformCoef deform_coef(const Plan& P);
@@ -277,6 +309,7 @@ void prof_end(Plan& P, cudaStream_t s);
 struct FormSizes {
   size_t pre = 0, H = 0, tab = 0, Z = 0, G = 0;  // Bluestein
   size_t A = 0, sched = 0;                       // dense
+  size_t X = 0;                                  // dense on nodes
 };
 fzp_status bluestein_layout(Plan& P, FormSizes* out);
 fzp_status bluestein_fill_tables(Plan& P, cudaStream_t s);  // buffers already assigned
@@ -291,11 +324,22 @@ fzp_status dense_rows(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream);
 // then row passes over a real FP32 matrix [rows][stride] loaded as the B operand.
 fzp_status dense_zoom_build(Plan& P, int64_t ncols, int64_t c, double kappa, double delta);
 fzp_status dense_zoom_rows(Plan& P, const float* src, int64_t rows, int64_t stride, cudaStream_t stream);
-fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream);
+fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStream_t stream);
 bool column_pass_tc_applies(const Plan& P);
-// Row pass and column pass of rows [j0, j0 + rows) (every mask pass of a dense
-// phase plate), accumulated into the ROI accumulator.
-fzp_status chunk_passes(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream);
+// Aperture rows [a, b) (clipped to the disc's) into the ROI accumulator (zeroed
+// first), chunk by chunk: row pass and column pass of every mask pass.  *sym:
+// the field is the accumulator plus its transpose.
+fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t stream);
+// The accumulator to the caller's field (interpolation, output chirp, prefactor).
+fzp_status finish_field(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t stream);
+// Form (b) on nodes (nodes.cu).
+void nodes_choose(Plan& P);
+fzp_status nodes_layout(Plan& P, FormSizes* out);
+fzp_status nodes_upload(Plan& P);
+fzp_status nodes_fill(Plan& P, cudaStream_t s);
+fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s);
+fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t s);
+fzp_status nodes_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t s);
 fzp_status column_pass_tc(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream);
 // The same with the pass's field weighted by (wr + i wi).
 fzp_status column_pass_tc_w(Plan& P, int64_t j0, int64_t rows, double wr, double wi, cudaStream_t stream);

@@ -1,0 +1,1151 @@
+// nodes.cu -- form (b) on interpolation nodes: the dense contraction evaluated
+// at as many focal-plane points as the aperture can distinguish.
+//
+// The field on the ROI is band limited: Eq. 2 without its output chirp is a
+// Fourier sum over the aperture disc, so along x it has about
+//   d = M p 2R / (lambda f)
+// degrees of freedom on the ROI's M samples (64 of 512 at the usual pitch
+// lambda f/# / 8).  The contraction U = K T K^T therefore runs on n uniform
+// nodes x_k across the ROI (and a margin of a quarter of it), n = 64, 128 or
+// 256 with d at most 0.56 n, 0.62 n, 0.66 n, and the ROI is read from the
+// nodes by the least-squares interpolation of functions of that band,
+//   U = W V W^T,  V = K_x T K_x^T,  W = S(x_m, x_k) S(x_k, x_l)^-1,
+// S(x, y) = sin(B (x - y)) / (B (x - y)).  W's rows have norm about 1 (it adds
+// no error to V's) and it reproduces e^{i nu x}, |nu| <= B, to 3e-8 rms (under
+// 2e-6 at the band's ends, the rim), far below the split-BF16 kernel's 2^-17.
+//
+// A flat plate is a function of di^2 + dj^2, which every step exploits:
+//   - columns +-d fold into one kernel column K(x, d) + K(x, -d) (half the
+//     contraction), rows +-d have the same row transform (half the rows), and
+//     over the whole aperture T is its own transpose: with L = T below the
+//     diagonal plus half of T on the diagonal tiles, T = L + L^T and
+//     V = F + F^T, F = K L K^T (half of the rest);
+//   - for an ROI centred on the focus K(x, d) + K(x, -d) is even in x, so the
+//     nodes x > 0 carry V (half the nodes).
+// A range of rows that is not its own mirror image keeps the column fold and the
+// evenness along x; its V takes all nodes along y.
+// Deformed membranes have no symmetry; they take all nodes, all columns, and
+// both real masks T cos(phi) and T sin(phi) in one pass (the phase is
+// evaluated once).
+//
+// k_nodes is a persistent tcgen05 kernel, one CTA per SM:
+//   unit    : a stripe of BN aperture rows x one chunk of K blocks
+//   stage   : 32 columns; A = NT node tiles of 128 kernel rows (Re and Im of 64
+//             nodes), BF16 hi and lo, pre-swizzled in HBM, one bulk copy; B =
+//             the masks of BN rows, generated into shared memory
+//   flat, NT = 1: 512 rows, two 128 x 256 accumulators (row halves) share A
+//   flat, NT = 2: 256 rows, two accumulators (node tiles)
+//   membrane    : 256 rows, accumulators T cos and T sin, hi and lo planes
+//   warps 0-7 epilogue, 8 loader, 9 MMA issuer, 10-25 mask generators
+// The mask rule in the generators: the zone index of a sample is the integer
+// part of s kappa, s = di^2 + dj^2; the 64-bit fixed-point phase s K mod 2^64
+// (its top bit the zone's parity, or its top log2 L bits the level) is carried
+// exactly from block to block, and its upper 32 bits run along a block with
+// two integer additions per sample.  Their error is below E units; a block in
+// which a phase comes within E of a zone boundary (about one in 10^4) takes
+// the exact rule with the threshold table, sample by sample.  Per sample: two
+// additions, three halves for the test, one for the BF16 value.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "fzp_internal.cuh"
+#include "membrane.cuh"
+#include "tc_ptx.cuh"
+
+namespace fzp {
+namespace {
+
+using namespace tc;
+
+constexpr int BK = 32;                   // columns per stage: one 64-byte swizzle row of BF16
+constexpr int SUB = 128 * BK * 2;        // 8 KiB: one (tile, hi | lo) operand image
+constexpr int PLANE = 256 * BK * 2;      // 16 KiB: one mask plane of 256 rows
+constexpr int EPI_WARPS = 8, LOAD_WARP = 8, MMA_WARP = 9, GEN_WARP0 = 10, GEN_WARPS = 16;
+constexpr int NUM_THREADS = (GEN_WARP0 + GEN_WARPS) * 32;
+constexpr int TMEM_COLS = 512;
+constexpr int EPI_BOX = 32;
+constexpr int EPI_BYTES = EPI_WARPS * EPI_BOX * EPI_BOX * 4;
+constexpr int ERR_BASE = 300;
+
+enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3 };
+
+// Fixed-point zone phase: phase64(s) = s K mod 2^64 (K = floor(kappa 2^63): the
+// zone's parity is the top bit; MASK_LEVELS: K = floor(kappa_L / L 2^64), the
+// level is floor(phase L / 2^64)).  The true phase lies less than s (in units
+// of 2^-64) above it; the 32-bit walk over a block adds less than 600 units of
+// 2^-32 and fl(s kappa) less than 8, so E = 640 + (s_max >> 32).
+struct PhaseRule {
+  uint64_t K;
+  uint32_t E;
+  int lmod;            // MASK_LEVELS: L
+  uint64_t pos, neg;   // MASK_LEVELS: level sets with value +1, -1
+  int open_even;       // 1: positive-centred binary plate
+};
+
+struct NodeArgs {
+  MaskGeom mg;              // c = 0 for a folded (flat) plate
+  PhaseRule ph;
+  int64_t j_begin, j_end;   // rows of this launch (folded: distances from the axis)
+  int n_stripes;
+  int octant;               // 1: columns up to the row only, diagonal tiles halved
+  int64_t kblocks;          // K blocks of the kernel image
+  const int* sched;         // off[nchunks + 1], slo[nchunks], cnt[nchunks]
+  int nchunks, group, promote;
+  int slices;               // images of C1, chunk g adds into image g slices / nchunks
+  DeformCoef df;            // membrane
+  const uint8_t* A;
+  int* err;
+};
+
+template <int NT, bool CX>
+struct Shape {
+  static constexpr int BN = (NT == 1 && !CX) ? 512 : 256;         // rows per unit
+  static constexpr int PLANES = CX ? 4 : BN / 256;                // mask planes per stage
+  static constexpr int A_BYTES = NT * 2 * SUB;
+  static constexpr int B_BYTES = PLANES * PLANE;
+  static constexpr int STAGES = CX ? 2 : (NT == 1 ? 4 : 4);
+  static constexpr int SMEM = 1024 + STAGES * (A_BYTES + B_BYTES) + EPI_BYTES + 256;
+  static_assert(!CX || NT == 1, "two node tiles of a membrane pass need more tensor memory than there is");
+};
+
+__device__ __forceinline__ uint64_t sdesc(const void* p) {
+  const uint64_t a = smem_u32(p);
+  return ((a >> 4) & 0x3FFFull) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
+}
+// kind::f16, D = F32, A = B = BF16, K-major, N = 256, M = 128
+constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+
+__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
+          dtmem),
+      "l"(ad), "l"(bd), "r"(IDESC), "r"(accumulate)
+      : "memory");
+}
+
+__device__ __forceinline__ int64_t isqrt_floor(int64_t t) {  // largest a with a^2 <= t (t >= 0)
+  int64_t a = (int64_t)sqrt((double)t);
+  while (a * a > t) --a;
+  while ((a + 1) * (a + 1) <= t) ++a;
+  return a;
+}
+
+// ------------------------------------------------------------------ work list
+// K blocks [klo, khi) of the stripe of rows [jb, je): the chord of its row
+// nearest the axis; with the octant, columns below je only.  At least one
+// block (every stripe writes its rows of C1).
+__device__ __forceinline__ void stripe_kspan(const NodeArgs& a, int64_t jb, int64_t je, int64_t& klo, int64_t& khi) {
+  const int64_t c = a.mg.c;
+  const int64_t jn = c < jb ? jb : (c >= je ? je - 1 : c);
+  const int64_t t = a.mg.sR - (jn - c) * (jn - c);
+  const int64_t b = t < 0 ? -1 : isqrt_floor(t);
+  klo = c - b > 0 ? (c - b) / BK : 0;
+  khi = (c + b) / BK + 1;
+  if (khi > a.kblocks) khi = a.kblocks;
+  if (a.octant && khi > (je + BK - 1) / BK) khi = (je + BK - 1) / BK;
+  if (klo >= a.kblocks) klo = a.kblocks - 1;
+  if (khi <= klo) khi = klo + 1;
+}
+
+template <int BN>
+__device__ __forceinline__ void span_of(const NodeArgs& a, int64_t s, int64_t& klo, int64_t& khi) {
+  const int64_t jb = a.j_begin + s * BN;
+  stripe_kspan(a, jb, jb + BN < a.j_end ? jb + BN : a.j_end, klo, khi);
+}
+
+// Zeroes C1 (all blocks but the first) and builds the work list (the first):
+// units (chunk g, stripe s) in chunk order, so that the CTAs at work at one time
+// share kernel blocks.  Every chunk's stripes are one range around the stripe
+// whose span holds the others' ends: the one nearest the axis or, with the
+// octant, where the chord takes over from the diagonal.
+template <int BN>
+__global__ void __launch_bounds__(1024) k_nodes_prep(const NodeArgs a, int* sched, float4* c1, int64_t c1_vec) {
+  if (blockIdx.x > 0) {
+    const int64_t step = (int64_t)(gridDim.x - 1) * blockDim.x;
+    for (int64_t t = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x; t < c1_vec; t += step)
+      c1[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
+  }
+  int* off = sched;
+  int* slo = sched + a.nchunks + 1;
+  int* cnt = slo + a.nchunks;
+  __shared__ int s_part[1024];
+  const int64_t ns = a.n_stripes;
+  int64_t sc = a.mg.c < a.j_begin ? 0 : (a.mg.c - a.j_begin) / BN;
+  if (sc >= ns) sc = ns - 1;
+  if (a.octant) {
+    int64_t lo = 0, hi = ns - 1;  // first stripe whose chord ends below its last row
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      const int64_t jb = a.j_begin + mid * BN, je = jb + BN < a.j_end ? jb + BN : a.j_end;
+      const int64_t t = a.mg.sR - jb * jb;
+      if (t < 0 || isqrt_floor(t) < je) hi = mid;
+      else lo = mid + 1;
+    }
+    sc = lo;
+    if (lo > 0) {
+      int64_t k0, h0, k1, h1;
+      span_of<BN>(a, lo - 1, k0, h0);
+      span_of<BN>(a, lo, k1, h1);
+      if (h0 > h1) sc = lo - 1;
+    }
+  }
+  int mine = 0;
+  const int per = (a.nchunks + (int)blockDim.x - 1) / (int)blockDim.x;  // consecutive chunks of this thread
+  const int g0 = threadIdx.x * per, g1 = min(g0 + per, a.nchunks);
+  for (int g = g0; g < g1; ++g) {
+    const int64_t c0 = (int64_t)g * a.group, c1k = c0 + a.group;
+    auto meets = [&](int64_t st) {
+      int64_t klo, khi;
+      span_of<BN>(a, st, klo, khi);
+      return klo < c1k && khi > c0;
+    };
+    int first = (int)sc, n = 0;
+    if (meets(sc)) {
+      int64_t lo = 0, hi = sc;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (meets(mid)) hi = mid;
+        else lo = mid + 1;
+      }
+      first = (int)lo;
+      lo = sc;
+      hi = ns - 1;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi + 1) >> 1;
+        if (meets(mid)) lo = mid;
+        else hi = mid - 1;
+      }
+      n = (int)lo - first + 1;
+    }
+    slo[g] = first;
+    cnt[g] = n;
+    mine += n;
+  }
+  s_part[threadIdx.x] = mine;
+  __syncthreads();
+  for (int d = 1; d < (int)blockDim.x; d <<= 1) {  // inclusive prefix sums over the threads
+    const int v = (int)threadIdx.x >= d ? s_part[threadIdx.x - d] : 0;
+    __syncthreads();
+    s_part[threadIdx.x] += v;
+    __syncthreads();
+  }
+  int acc = s_part[threadIdx.x] - mine;
+  for (int g = g0; g < g1; ++g) {
+    off[g] = acc;
+    acc += cnt[g];
+  }
+  if (threadIdx.x == blockDim.x - 1) off[a.nchunks] = s_part[threadIdx.x];
+}
+
+struct Unit {
+  int64_t jb, je, kb0, kb1;
+  int slice;
+};
+
+template <int BN>
+__device__ __forceinline__ Unit unit_at(const NodeArgs& a, int it) {
+  const int* off = a.sched;
+  const int* slo = a.sched + a.nchunks + 1;
+  int lo = 0, hi = a.nchunks - 1;  // largest g with off[g] <= it (chunks without units share an offset)
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(off + mid) <= it) lo = mid;
+    else hi = mid - 1;
+  }
+  Unit u;
+  const int64_t s = __ldg(slo + lo) + (it - __ldg(off + lo));
+  u.jb = a.j_begin + s * BN;
+  u.je = u.jb + BN < a.j_end ? u.jb + BN : a.j_end;
+  int64_t klo, khi;
+  stripe_kspan(a, u.jb, u.je, klo, khi);
+  const int64_t c0 = (int64_t)lo * a.group, c1 = c0 + a.group;
+  u.kb0 = klo > c0 ? klo : c0;
+  u.kb1 = khi < c1 ? khi : c1;
+  u.slice = lo * a.slices / a.nchunks;
+  return u;
+}
+
+// ------------------------------------------------------------------ generator
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
+
+// bits 2q, 2q + 1 of `bits` as two half-word masks
+__device__ __forceinline__ uint32_t pair_mask(uint32_t bits, int q) {
+  return (((bits >> (2 * q)) & 1u) ? 0xFFFFu : 0u) | (((bits >> (2 * q + 1)) & 1u) ? 0xFFFF0000u : 0u);
+}
+
+// Columns [di0, di0 + 32) of row dj inside the disc chord (bmax = -1: none).
+__device__ __forceinline__ uint32_t chord_bits(int64_t di0, int64_t bmax) {
+  const int64_t lo = -bmax - di0, hi = bmax - di0;
+  if (bmax < 0 || hi < 0 || lo > 31) return 0u;
+  const uint32_t a = lo <= 0 ? 0xFFFFFFFFu : (0xFFFFFFFFu << (uint32_t)lo);
+  const uint32_t b = hi >= 31 ? 0xFFFFFFFFu : (0xFFFFFFFFu >> (uint32_t)(31 - hi));
+  return a & b;
+}
+
+// The exact rule on the block's columns [di0, di0 + 32): bits with value +1 and
+// with value -1 before the chord is applied (MASK_SIGNED: every column +1 or -1).
+template <int MASK>
+__device__ __noinline__ void exact_bits(int64_t di0, int64_t dj2, const MaskGeom& g, const PhaseRule& r, uint32_t& pb,
+                                        uint32_t& nb) {
+  pb = nb = 0u;
+  for (int k = 0; k < 32; ++k) {
+    const int64_t d = di0 + k, s = dj2 + d * d;
+    const int64_t z = zone_of(s < g.sR ? s : g.sR, g);
+    if (MASK == MASK_LEVELS) {
+      const int q = (int)(z % r.lmod);
+      pb |= (uint32_t)((r.pos >> q) & 1ull) << k;
+      nb |= (uint32_t)((r.neg >> q) & 1ull) << k;
+    } else if (MASK == MASK_SIGNED) {
+      if (z & 1) nb |= 1u << k;
+      else pb |= 1u << k;
+    } else {
+      pb |= (uint32_t)((z ^ r.open_even) & 1) << k;
+    }
+  }
+}
+
+// A row's walk over its blocks: the exact 64-bit phase at the block's first
+// column and its first difference.
+struct RowWalk {
+  uint64_t phase, step;  // s K and (2 di + 1) K mod 2^64
+  int64_t di0, dj2, bmax;
+};
+
+__device__ __forceinline__ void row_start(RowWalk& w, int64_t dj, int64_t di0, bool live, const MaskGeom& g,
+                                          const PhaseRule& r) {
+  w.dj2 = dj * dj;
+  w.di0 = di0;
+  const int64_t t = g.sR - w.dj2;
+  w.bmax = (live && t >= 0) ? isqrt_floor(t) : -1;
+  w.phase = (uint64_t)(w.dj2 + di0 * di0) * r.K + (r.open_even ? (1ull << 63) : 0ull);
+  w.step = (uint64_t)(2 * di0 + 1) * r.K;
+}
+
+// On to the next 32 columns.
+__device__ __forceinline__ void row_next(RowWalk& w, const PhaseRule& r) {
+  w.phase += 32ull * w.step + 992ull * r.K;  // K ((d + 32)^2 - d^2) = 32 (2 d + 1) K + 992 K
+  w.step += 64ull * r.K;
+  w.di0 += 32;
+}
+
+// The block's mask as 16 words of two BF16 values; `one` = +-1 (or +-1/2) in
+// both halves.  Whole warp (the votes), every lane a row.
+template <int MASK>
+__device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
+                                            uint32_t (&wd)[16]) {
+  const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);  // upper 32 bits of 2 K
+  uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
+  uint32_t near = 0xFFFFFFFFu;
+  const uint32_t chord = chord_bits(w.di0, w.bmax);
+  if (MASK == MASK_LEVELS) {
+    const uint32_t el = r.E * (uint32_t)r.lmod;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      uint32_t v = 0u;
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        const uint64_t p = (uint64_t)f * (uint32_t)r.lmod;
+        near = min(near, (uint32_t)p + el);
+        const int lv = (int)(p >> 32);
+        const uint32_t pb = (uint32_t)(r.pos >> lv) & 1u, nb = (uint32_t)(r.neg >> lv) & 1u;
+        v |= ((pb | nb) * 0xFFFFu & ((nb << 15) | (one & 0x7FFFu))) << (16 * z);
+        f += d;
+        d += c2;
+      }
+      wd[q] = v;
+    }
+    near = near < 2u * el ? 1u : 0u;
+  } else {
+    const uint32_t e2 = 2u * r.E;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const uint32_t fa = f, fb = f + d;
+      f = fb + d + c2;
+      d += 2u * c2;
+      near = min(near, min((fa << 1) + e2, (fb << 1) + e2));
+      const uint32_t s = prmt(fa, fb, 0xFFBBu);  // each value's sign in its half-word
+      wd[q] = MASK == MASK_SIGNED ? ((s & 0x80008000u) | one) : (s & one);
+    }
+    near = near < 2u * e2 ? 1u : 0u;
+  }
+  if (__any_sync(0xffffffffu, near != 0u && chord != 0u)) {
+    if (near && chord) {
+      uint32_t pb, nb;
+      exact_bits<MASK>(w.di0, w.dj2, g, r, pb, nb);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) wd[q] = (pair_mask(pb | nb, q) & one) | (pair_mask(nb, q) & 0x80008000u);
+    }
+  }
+  if (__any_sync(0xffffffffu, chord != 0xFFFFFFFFu)) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) wd[q] &= pair_mask(chord, q);
+  }
+}
+
+// The block's open bits (parity rule, chord applied), for the membrane pass.
+__device__ __forceinline__ uint32_t block_open(const RowWalk& w, const MaskGeom& g, const PhaseRule& r) {
+  const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);
+  uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
+  uint32_t near = 0xFFFFFFFFu, bits = 0u;
+  const uint32_t chord = chord_bits(w.di0, w.bmax), e2 = 2u * r.E;
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    near = min(near, (f << 1) + e2);
+    bits |= (f >> 31) << k;
+    f += d;
+    d += c2;
+  }
+  if (near < 2u * e2 && chord != 0u) {
+    uint32_t nb;
+    exact_bits<MASK_PARITY>(w.di0, w.dj2, g, r, bits, nb);
+  }
+  return bits & chord;
+}
+
+// ------------------------------------------------------------------ kernel
+template <int NT, int MASK>
+__global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, const __grid_constant__ CUtensorMap tmC1) {
+  constexpr bool CX = MASK == MASK_MEMBRANE;
+  using S = Shape<NT, CX>;
+  constexpr int NST = S::STAGES, BN = S::BN;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sA = base;
+  uint8_t* sB = base + NST * S::A_BYTES;
+  uint8_t* sE = sB + NST * S::B_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sE + EPI_BYTES);
+  uint64_t* fullA = bars;
+  uint64_t* fullB = bars + NST;
+  uint64_t* empty = bars + 2 * NST;
+  uint64_t* accFull = bars + 3 * NST;
+  uint64_t* accEmpty = accFull + 1;
+  uint64_t* drain = accEmpty + 1;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(drain + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
+  volatile int* epi_ok = reinterpret_cast<volatile int*>(drain + 3);  // [2], by promotion parity
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(&fullA[s], 1);
+      mbar_init(&fullB[s], GEN_WARPS);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accFull, 1);
+    mbar_init(accEmpty, EPI_WARPS);
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == MMA_WARP) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int n_items = __ldg(a.sched + a.nchunks);
+
+  if (warp == LOAD_WARP) {
+    // ---------------- kernel images: one bulk copy per stage
+    if (lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      int last[NST];
+#pragma unroll
+      for (int s2 = 0; s2 < NST; ++s2) last[s2] = -1;
+      for (int it = blockIdx.x; it < n_items && !*abort_flag; it += gridDim.x) {
+        const Unit un = unit_at<BN>(a, it);
+        for (int64_t kb = un.kb0; kb < un.kb1; ++kb) {
+          if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 1)) break;
+          mbar_arrive_tx(&fullA[stage], S::A_BYTES);
+          bulk_g2s(sA + stage * S::A_BYTES, a.A + kb * S::A_BYTES, S::A_BYTES, &fullA[stage]);
+          last[stage] = (int)phase;
+          if (++stage == NST) { stage = 0; phase ^= 1; }
+        }
+      }
+      if (*abort_flag) {
+        // copies already issued must land before shared memory is released
+#pragma unroll
+        for (int s2 = 0; s2 < NST; ++s2) {
+          if (last[s2] < 0) continue;
+          const uint64_t t0 = gtimer();
+          while (!mbar_try(&fullA[s2], (uint32_t)last[s2]) && gtimer() - t0 < WAIT_NS) {
+          }
+        }
+      }
+    }
+  } else if (warp == MMA_WARP) {
+    // ---------------- MMA issuer
+    if (lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0, accph = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+        const Unit un = unit_at<BN>(a, it);
+        for (int64_t p0 = un.kb0; p0 < un.kb1 && ok; p0 += a.promote) {
+          const int64_t p1 = p0 + a.promote < un.kb1 ? p0 + a.promote : un.kb1;
+          if (!mbar_wait(accEmpty, accph ^ 1, abort_flag, a.err, ERR_BASE + 2)) { ok = false; break; }
+          tc_fence_after();
+          for (int64_t kb = p0; kb < p1; ++kb) {
+            if (!mbar_wait(&fullA[stage], phase, abort_flag, a.err, ERR_BASE + 3) ||
+                !mbar_wait(&fullB[stage], phase, abort_flag, a.err, ERR_BASE + 4)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t ad = sdesc(sA + stage * S::A_BYTES), bd = sdesc(sB + stage * S::B_BYTES);
+#pragma unroll
+            for (int ks = 0; ks < BK / 16; ++ks) {
+              const uint64_t o = (uint64_t)((ks * 32) >> 4);
+              const uint32_t acc = (kb > p0 || ks > 0) ? 1u : 0u;
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                // flat: accumulator q = row half q (NT = 1) or node tile q (NT = 2);
+                // membrane: q = 0 T cos, 1 T sin, planes 2q (hi) and 2q + 1 (lo)
+                const uint32_t dt = tmem + (uint32_t)(q * 256);
+                const int at = NT == 2 ? q : 0;
+                const int bp = CX ? 2 * q : (NT == 2 ? 0 : q);
+                const uint64_t a_hi = ad + (uint64_t)((at * SUB) >> 4) + o;
+                const uint64_t a_lo = ad + (uint64_t)(((NT + at) * SUB) >> 4) + o;
+                const uint64_t b0 = bd + (uint64_t)((bp * PLANE) >> 4) + o;
+                mma_bf16(dt, a_hi, b0, acc);
+                mma_bf16(dt, a_lo, b0, 1u);
+                if (CX) mma_bf16(dt, a_hi, b0 + (uint64_t)(PLANE >> 4), 1u);
+              }
+            }
+            mma_commit(&empty[stage]);
+            if (++stage == NST) { stage = 0; phase ^= 1; }
+          }
+          if (!ok) break;
+          mma_commit(accFull);
+          accph ^= 1;
+        }
+      }
+      // all issued MMAs complete before tensor memory is released
+      mma_commit(drain);
+      const uint64_t t0 = gtimer();
+      while (!mbar_try(drain, 0) && gtimer() - t0 < WAIT_NS) {
+      }
+    }
+  } else if (warp >= GEN_WARP0) {
+    // ---------------- mask generators: a lane per row.  Flat, 512 rows: warp
+    // gw takes rows 32 gw .. + 31; 256 rows: warps gw and gw + 8 take the same
+    // rows' even and odd blocks of a unit (flat) or 16-column halves (membrane)
+    const int gw = warp - GEN_WARP0;
+    const int row = (BN == 512 ? gw : gw & 7) * 32 + lane;  // row of the stripe
+    const int half = BN == 512 ? 0 : gw >> 3;
+    // 64-byte swizzle: row at (row / 8) 512 + (row % 8) 64, 16-byte part q at q ^ ((row % 8) / 2)
+    uint8_t* rowbase = sB + (row >> 8) * PLANE + ((row & 255) >> 3) * 512 + (row & 7) * 64;
+    const int sw = (row & 7) >> 1;
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+      const Unit un = unit_at<BN>(a, it);
+      const int64_t j = un.jb + row;
+      RowWalk w;
+      row_start(w, j - a.mg.c, un.kb0 * BK - a.mg.c, j < un.je, a.mg, a.ph);
+      const int64_t diag = a.octant ? un.jb / BK : INT64_MAX;  // blocks of the diagonal tile: half weight
+      if constexpr (CX) {
+        CxRow cxr;
+        cx_row_init(a.df, j - a.mg.c, cxr);
+        for (int64_t kb = un.kb0; kb < un.kb1; ++kb) {
+          const uint32_t bits = block_open(w, a.mg, a.ph);
+          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+          uint8_t* rp = rowbase + stage * S::B_BYTES;
+          cx_store2(a.df, cxr, w.di0, bits, rp, rp + PLANE, rp + 2 * PLANE, rp + 3 * PLANE, sw, 2 * half, 2);
+          row_next(w, a.ph);
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&fullB[stage]);
+          if (++stage == NST) { stage = 0; phase ^= 1; }
+        }
+      } else {
+        for (int64_t kb = un.kb0; kb < un.kb1; ++kb) {
+          const bool mine = BN == 512 || ((kb ^ half) & 1) == 0;
+          uint32_t wd[16];
+          if (mine) block_words<MASK>(w, a.mg, a.ph, kb >= diag ? 0x3F003F00u : 0x3F803F80u, wd);
+          row_next(w, a.ph);
+          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+          if (mine) {
+            uint8_t* rp = rowbase + stage * S::B_BYTES;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              *reinterpret_cast<uint4*>(rp + ((q ^ sw) << 4)) =
+                  make_uint4(wd[4 * q], wd[4 * q + 1], wd[4 * q + 2], wd[4 * q + 3]);
+            fence_proxy_async();
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&fullB[stage]);
+          if (++stage == NST) { stage = 0; phase ^= 1; }
+        }
+      }
+    }
+  } else {
+    // ---------------- epilogue: warp w drains accumulator w / 4, TMEM lanes 32 (w % 4) ..:
+    // each 32 x 32 piece goes to shared memory (128-byte swizzle) and from
+    // there by one TMA reduce-add into C1, once per promotion
+    const int q = warp >> 2;
+    uint8_t* eb = sE + warp * (EPI_BOX * EPI_BOX * 4);
+    uint32_t accph = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+      const Unit un = unit_at<BN>(a, it);
+      const int x0 = (int)(un.jb - a.j_begin) + ((NT == 1 && !CX) ? q * 256 : 0);
+      const int y0 = un.slice * (NT * 128 * (CX ? 2 : 1)) + ((NT == 2 || CX) ? q * 128 : 0) + (warp & 3) * 32;
+      const int xn = (int)min((int64_t)256, un.je - a.j_begin - x0);  // live columns (may be <= 0)
+      for (int64_t p0 = un.kb0; p0 < un.kb1; p0 += a.promote) {
+        if (threadIdx.x == 0) epi_ok[accph] = mbar_wait(accFull, accph, abort_flag, a.err, ERR_BASE + 6) ? 1 : 0;
+        named_bar_sync(1, EPI_WARPS * 32);
+        if (!epi_ok[accph]) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * 256);
+#pragma unroll 1
+        for (int col = 0; col < xn; col += EPI_BOX) {
+          float v[32];
+          tmem_ld32(taddr + col, v);
+          if (lane == 0) bulk_wait_read0();  // the previous piece has been read out of eb
+          __syncwarp();
+#pragma unroll
+          for (int c4 = 0; c4 < 8; ++c4)
+            *reinterpret_cast<float4*>(eb + lane * 128 + ((c4 ^ (lane & 7)) << 4)) =
+                make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) {
+            tma_reduce_add_2d(&tmC1, eb, x0 + col, y0);
+            bulk_commit();
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(accEmpty);
+        accph ^= 1;
+      }
+    }
+    if (lane == 0) bulk_wait0();  // C1 complete before the kernel ends
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == MMA_WARP) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ tables
+// Kernel images of the nodes: K block kb = [tile 0 hi] .. [tile NT-1 hi][tile 0 lo] ..,
+// each 128 rows x 32 BF16, 64-byte swizzle; tile t holds Re K (rows 0-63) and
+// Im K (rows 64-127) of nodes 64 t ..; folded: column d holds K(x, d) + K(x, -d).
+__global__ void k_nodes_A(int nt, int64_t ncols, int64_t kblocks, int64_t c, int fold, double kappa, double msh,
+                          double delta, uint8_t* A) {
+  const int64_t total = kblocks * 4 * (int64_t)nt * 64;  // one thread per node and 8 columns
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k8 = e % (kblocks * 4);
+    const int node = (int)(e / (kblocks * 4));
+    const int t = node >> 6, r = node & 63;
+    const double x = (double)node - msh;
+    float re[8], im[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int64_t i = 8 * k8 + u;
+      re[u] = im[u] = 0.f;
+      if (i < ncols) {
+        const double di = (double)(i - c), q = di * di * (0.5 * kappa), l = x * di * delta;
+        const float2 v = cis_turns_f(q - l);
+        re[u] = v.x;
+        im[u] = v.y;
+        if (fold && i > c) {
+          const float2 m = cis_turns_f(q + l);
+          re[u] += m.x;
+          im[u] += m.y;
+        }
+      }
+    }
+    uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      split2(re[2 * u], re[2 * u + 1], rh[u], rl[u]);
+      split2(im[2 * u], im[2 * u + 1], ih[u], il[u]);
+    }
+    const int k = (int)(k8 & 3);
+    uint8_t* blk = A + (k8 >> 2) * (int64_t)(nt * 2 * SUB);
+    auto put = [&](int plane, int rr, const uint32_t (&v)[4]) {
+      *reinterpret_cast<uint4*>(blk + plane * SUB + (rr >> 3) * 512 + (rr & 7) * 64 + ((k ^ ((rr & 7) >> 1)) << 4)) =
+          make_uint4(v[0], v[1], v[2], v[3]);
+    };
+    put(t, r, rh);
+    put(nt + t, r, rl);
+    put(t, 64 + r, ih);
+    put(nt + t, 64 + r, il);
+  }
+}
+
+// ------------------------------------------------------------------ interpolation
+// X[o, l] = sum_k Wy[o, k] (V[k, l] (+ V[l, k])), k over the ny nodes of the rows'
+// axis: one thread per (o, l).
+__global__ void k_interp_rows(int ny, int ns, int Mo, int sym, const double* __restrict__ Wy,
+                              const double2* __restrict__ V, double2* __restrict__ X) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y * blockDim.y + threadIdx.y;
+  if (l >= ns || o >= Mo) return;
+  double2 x = make_double2(0.0, 0.0);
+  for (int k = 0; k < ny; ++k) {
+    double2 v = V[k * ns + l];
+    if (sym) {
+      const double2 u = V[l * ns + k];
+      v.x += u.x;
+      v.y += u.y;
+    }
+    const double w = Wy[k * Mo + o];
+    x.x = fma(w, v.x, x.x);
+    x.y = fma(w, v.y, x.y);
+  }
+  X[l * Mo + o] = x;
+}
+
+struct InterpOut {
+  int M, ns;
+  int Moy, eveny, Mox, evenx;  // outputs of the two axes (even: M / 2 + 1)
+  double msh, p, lf, f_over_lambda, amp;
+  int accumulate;
+};
+
+// U[on, om] = sum_l X[on, l] W[om, l], the output chirp and prefactor, and the
+// stores: with an even field output o stands for the samples M/2 + o and
+// M/2 - o (o = M/2: sample 0 alone).
+constexpr int IT = 32;  // outputs per block and side
+__global__ void __launch_bounds__(256) k_interp_cols(const InterpOut a, const double* __restrict__ W,
+                                                     const double2* __restrict__ X, double2* __restrict__ out) {
+  __shared__ double2 sX[16][IT];
+  __shared__ double sW[16][IT];
+  const int n0 = blockIdx.y * IT, m0 = blockIdx.x * IT;
+  const int tm = threadIdx.x & 15, tn = threadIdx.x >> 4;  // 2 x 2 outputs each
+  double2 u[2][2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) u[i][j] = make_double2(0.0, 0.0);
+  for (int l0 = 0; l0 < a.ns; l0 += 16) {
+    for (int t = threadIdx.x; t < 16 * IT; t += 256) {
+      const int l = t / IT, o = t % IT;
+      sX[l][o] = n0 + o < a.Moy ? X[(l0 + l) * a.Moy + n0 + o] : make_double2(0.0, 0.0);
+      sW[l][o] = m0 + o < a.Mox ? W[(l0 + l) * a.Mox + m0 + o] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int l = 0; l < 16; ++l) {
+      double2 x[2];
+      double w[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) x[i] = sX[l][tn + 16 * i];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) w[j] = sW[l][tm + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          u[i][j].x = fma(w[j], x[i].x, u[i][j].x);
+          u[i][j].y = fma(w[j], x[i].y, u[i][j].y);
+        }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int on = n0 + tn + 16 * i, om = m0 + tm + 16 * j;
+      if (on >= a.Moy || om >= a.Mox) continue;
+      const int h = a.M / 2;
+      const int n = a.eveny ? (h + on) % a.M : on, m = a.evenx ? (h + om) % a.M : om;
+      const double xm = (double)m - a.msh, yn = (double)n - a.msh;
+      const double ph = frac_turns(a.f_over_lambda) - 0.25 + (xm * xm + yn * yn) * (a.p * a.p) / (2.0 * a.lf);
+      double2 w = cis_turns_d(ph);
+      w.x *= a.amp;
+      w.y *= a.amp;
+      const double2 v = make_double2(w.x * u[i][j].x - w.y * u[i][j].y, w.x * u[i][j].y + w.y * u[i][j].x);
+      auto put = [&](int nn, int mm) {
+        double2* o = out + (int64_t)nn * a.M + mm;
+        double2 z = v;
+        if (a.accumulate) {
+          z.x += o->x;
+          z.y += o->y;
+        }
+        *o = z;
+      };
+      // samples with a mirror image of their own
+      const bool fn = a.eveny && on > 0 && on < h, fm = a.evenx && om > 0 && om < h;
+      put(n, m);
+      if (fn) put(h - on, m);
+      if (fm) put(n, h - om);
+      if (fn && fm) put(h - on, h - om);
+    }
+}
+
+// ------------------------------------------------------------------ mask export
+__global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int64_t j0, int64_t rows, uint8_t* out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r0 = warp * 32; r0 < rows; r0 += nwarps * 32) {
+    const int64_t r = r0 + lane;
+    const int64_t dj = j0 + r - mg.c;
+    RowWalk w;
+    row_start(w, dj, -mg.c, r < rows, mg, ph);
+    for (int64_t i0 = 0; i0 < N; i0 += 32) {
+      const uint32_t disc = chord_bits(w.di0, w.bmax);
+      uint8_t v[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) v[k] = 0;
+      uint32_t wd[16];
+      if (mask == MASK_LEVELS) {
+        PhaseRule one = ph;
+        one.neg = 0;
+        for (int q = 0; q < ph.lmod; ++q) {
+          one.pos = 1ull << q;
+          block_words<MASK_LEVELS>(w, mg, one, 0x3F803F80u, wd);
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            if ((wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu) v[k] = (uint8_t)(1 + q);
+        }
+      } else if (mask == MASK_SIGNED) {
+        block_words<MASK_SIGNED>(w, mg, ph, 0x3F803F80u, wd);
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          v[k] = ((disc >> k) & 1u) ? (uint8_t)(1 + ((wd[k / 2] >> (16 * (k & 1) + 15)) & 1u)) : 0;
+      } else if (mask == MASK_MEMBRANE) {
+        const uint32_t bits = block_open(w, mg, ph);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = (uint8_t)((bits >> k) & 1u);
+      } else {
+        block_words<MASK_PARITY>(w, mg, ph, 0x3F803F80u, wd);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = ((wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu) ? 1 : 0;
+      }
+      if (r < rows)
+        for (int k = 0; k < 32 && i0 + k < N; ++k) out[r * N + i0 + k] = v[k];
+      row_next(w, ph);
+    }
+  }
+}
+
+fzp_status c1_map(const Plan& P, int64_t stride, int rows, CUtensorMap* tm) {
+  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  if (!encode) {
+    cudaDriverEntryPointQueryResult q;
+    void* fn = nullptr;
+    FZP_CUDA_TRY(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q));
+    if (q != cudaDriverEntryPointSuccess || !fn) return set_error(FZP_E_CUDA, "cuTensorMapEncodeTiled unavailable");
+    encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  }
+  const cuuint64_t dims[2] = {(cuuint64_t)stride, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)stride * 4};
+  const cuuint32_t box[2] = {EPI_BOX, EPI_BOX};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, P.d_C1, dims, strides, box, estr,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return set_error(FZP_E_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+  return FZP_OK;
+}
+
+PhaseRule phase_rule(const Plan& P, const MaskPass* mp) {
+  PhaseRule r{};
+  r.E = 640u + (uint32_t)(P.mg.sR >> 32);
+  if (P.levels > 2) {
+    r.K = (uint64_t)std::floor(std::ldexp(P.kappa_mask / P.levels, 64));
+    r.lmod = P.levels;
+    if (mp) {
+      r.pos = mp->pos;
+      r.neg = mp->neg;
+    }
+  } else {
+    r.K = (uint64_t)std::floor(std::ldexp(P.kappa_mask, 63));
+    r.open_even = P.mg.centre_open;
+  }
+  return r;
+}
+
+int mask_kind(const Plan& P) {
+  return P.has_deform ? MASK_MEMBRANE : P.levels > 2 ? MASK_LEVELS : P.levels == 2 ? MASK_SIGNED : MASK_PARITY;
+}
+
+// W (transposed: [node][output]) for n nodes x_k = (k - (n - 1)/2) h across +-1
+// and outputs x_o, band half-width `c` (radians per unit): the normal equations
+// of the least-squares problem over the band, S W = s, with a regularisation
+// of 1e-13 (the sinc matrix is singular to working precision), by Cholesky.
+struct Interp {
+  int n, Mo;
+  std::vector<double> dist, minus, plus;  // sinc at the node distances q h; at x_o -+ x_k, k > 0 half (or x_o - x_k, all)
+  bool half;
+
+  Interp(int n_, double h, double c, const std::vector<double>& xo, bool half_) : n(n_), Mo((int)xo.size()), half(half_) {
+    auto sinc = [&](double t) { const double z = c * t; return std::fabs(z) < 1e-9 ? 1.0 : std::sin(z) / z; };
+    const int ns = half ? n / 2 : n;
+    dist.resize(n);
+    for (int q = 0; q < n; ++q) dist[q] = sinc(q * h);
+    minus.resize((size_t)ns * Mo);
+    if (half) plus.resize((size_t)ns * Mo);
+    for (int k = 0; k < ns; ++k) {
+      const double x = ((double)(half ? k + n / 2 : k) - 0.5 * (n - 1)) * h;
+      for (int o = 0; o < Mo; ++o) {
+        minus[(size_t)k * Mo + o] = sinc(xo[o] - x);
+        if (half) plus[(size_t)k * Mo + o] = sinc(xo[o] + x);
+      }
+    }
+  }
+
+  // parity 0: all nodes; +1 / -1: of an even / odd function, over the nodes x > 0
+  std::vector<double> solve(int parity) const {
+    const int ns = half ? n / 2 : n;
+    std::vector<double> L((size_t)ns * ns), W = minus;
+    for (int k = 0; k < ns; ++k)
+      for (int l = 0; l <= k; ++l)  // x_k + x_l = (k + l + 1) h on the half grid
+        L[(size_t)k * ns + l] = dist[k - l] + (parity ? parity * dist[k + l + 1] : 0.0) + (k == l ? 1e-13 : 0.0);
+    for (int k = 0; k < ns; ++k)
+      for (int l = 0; l <= k; ++l) {
+        double s = L[(size_t)k * ns + l];
+        for (int q = 0; q < l; ++q) s -= L[(size_t)k * ns + q] * L[(size_t)l * ns + q];
+        L[(size_t)k * ns + l] = k == l ? std::sqrt(std::max(s, 1e-15)) : s / L[(size_t)l * ns + l];
+      }
+    if (parity)
+      for (size_t t = 0; t < W.size(); ++t) W[t] += parity * plus[t];
+    for (int k = 0; k < ns; ++k) {  // L y = s, all outputs at once
+      double* w = &W[(size_t)k * Mo];
+      for (int q = 0; q < k; ++q) axpy(w, &W[(size_t)q * Mo], -L[(size_t)k * ns + q]);
+      scale(w, 1.0 / L[(size_t)k * ns + k]);
+    }
+    for (int k = ns - 1; k >= 0; --k) {  // L^T w = y
+      double* w = &W[(size_t)k * Mo];
+      for (int q = k + 1; q < ns; ++q) axpy(w, &W[(size_t)q * Mo], -L[(size_t)q * ns + k]);
+      scale(w, 1.0 / L[(size_t)k * ns + k]);
+    }
+    return W;
+  }
+  void axpy(double* __restrict__ w, const double* __restrict__ v, double f) const {
+    for (int o = 0; o < Mo; ++o) w[o] += f * v[o];
+  }
+  void scale(double* w, double f) const {
+    for (int o = 0; o < Mo; ++o) w[o] *= f;
+  }
+};
+
+template <int NT, int MASK>
+fzp_status smem_attr() {
+  static std::atomic<uint64_t> done{0};
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_nodes<NT, MASK>, Shape<NT, MASK == MASK_MEMBRANE>::SMEM, done));
+  return FZP_OK;
+}
+
+template <int NT, int MASK>
+fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
+  using S = Shape<NT, MASK == MASK_MEMBRANE>;
+  constexpr bool CX = MASK == MASK_MEMBRANE;
+  fzp_status st = smem_attr<NT, MASK>();
+  if (st != FZP_OK) return st;
+  const int64_t rows = a.j_end - a.j_begin;
+  a.n_stripes = (int)((rows + S::BN - 1) / S::BN);
+  P.c1_stride = (rows + 255) / 256 * 256;
+  const int c1r = NT * 128 * (CX ? 2 : 1);
+  // A sum of two is the same in either order: up to 256 K blocks of the whole
+  // grid (N <= 8192, where the FP32 sums of whole chunks were reproducible) the
+  // chunks of a unit's stripe add by twos into separate images of C1, which
+  // the column pass sums in order.  Larger plates add into one image.
+  a.slices = 1;
+  if (P.N <= 256 * BK) {
+    const int64_t cap = std::max<int64_t>(1, (int64_t)(c1_elems(P) / ((size_t)c1r * P.c1_stride)));
+    a.group = (int)std::max<int64_t>(a.group, (a.kblocks + 2 * cap - 1) / (2 * cap));
+    a.nchunks = (int)((a.kblocks + a.group - 1) / a.group);
+    a.slices = (int)std::min<int64_t>(cap, (a.nchunks + 1) / 2);
+  }
+  P.nd.slices = a.slices;
+  P.nd.slice_elems = (int64_t)c1r * P.c1_stride;
+  CUtensorMap tm;
+  st = c1_map(P, P.c1_stride, c1r * a.slices, &tm);
+  if (st != FZP_OK) return st;
+  const int64_t vec = (int64_t)c1r * P.c1_stride * a.slices / 4;
+  const unsigned zb = (unsigned)std::min<int64_t>(2 * P.dn.num_sms, (vec + 4095) / 4096);
+  k_nodes_prep<S::BN><<<1 + zb, 1024, 0, s>>>(a, P.dn.d_sched, reinterpret_cast<float4*>(P.d_C1), vec);
+  prof_begin(P, s);
+  k_nodes<NT, MASK><<<P.dn.num_sms, NUM_THREADS, S::SMEM, s>>>(a, tm);
+  prof_end(P, s);
+  P.launches += 2;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+}  // namespace
+
+// The rule of the node form (host).  It takes split-BF16 plans whose band
+// leaves room on the nodes; a coarser pitch (or a larger ROI) than that, BF16
+// without the split and explicit clusters of 2 or 4 CTAs stay with k_dense,
+// and so do plates of 6 and more levels (L/2 passes: the plain FP32 form's
+// single pass is the faster one there) and membranes that need two node tiles
+// (four accumulators do not fit the tensor memory).
+void nodes_choose(Plan& P) {
+  NodeSet& z = P.nd;
+  z = NodeSet{};
+  if (P.form != FZP_FORM_DENSE || P.precision != FZP_PREC_SPLIT_BF16 || P.cluster_req > 1 || P.levels > 4) return;
+  const bool flat = !P.has_deform;
+  const bool centred = P.msh == (double)(P.M / 2);
+  const bool even = flat && centred;
+  const double half = even ? 0.5 * P.M : 0.5 * (P.M - 1);  // half width of the ROI, pitches
+  const double band = 2.0 * P.R / (P.lambda * P.f) * P.p;  // cycles per pitch, both signs
+  const double dof = 2.0 * half * band;
+  struct { int n; double most; } sizes[] = {{64, 36.0}, {128, 80.0}, {256, 170.0}};
+  for (auto& q : sizes) {
+    const int ns = even ? q.n / 2 : q.n;
+    if (ns < 64 || ns > 128 || (!flat && ns > 64) || dof > q.most) continue;
+    z.n = q.n;
+    z.ns = ns;
+    break;
+  }
+  if (!z.n) return;
+  z.even = even;
+  z.fold = flat;
+  z.Mo = even ? P.M / 2 + 1 : P.M;
+  z.half = half;
+  z.band = band;
+  const double h = 2.0 * half * 1.25 / z.n;  // node pitch in ROI pitches: a margin of a quarter
+  const double centre = even ? 0.0 : 0.5 * (P.M - 1) - P.msh;
+  z.h = h;
+  z.delta = P.delta * h;
+  // node k at x = (k - msh) h: the first stored node
+  const double first = centre + ((even ? z.n / 2 : 0) - 0.5 * (z.n - 1)) * h;
+  z.msh = -first / h;
+}
+
+fzp_status nodes_layout(Plan& P, FormSizes* out) {
+  NodeSet& z = P.nd;
+  const int64_t ncols = z.fold ? P.c + 1 : P.N;
+  z.kblocks = (ncols + BK - 1) / BK;
+  out->A = (size_t)z.kblocks * (size_t)(z.ns / 64) * 2 * SUB;
+  out->sched = sizeof(int) * (size_t)(3 * ((z.kblocks + 7) / 8) + 1);
+  out->X = (size_t)z.ns * P.M * sizeof(double2);
+  return FZP_OK;
+}
+
+// W: per plan, also in a batch (it depends on the plan's band).  An even field's
+// plan also gets the matrix of all n nodes, for row ranges that are not their
+// own mirror image (a batch runs whole apertures only): w(+-x_k) = (even +- odd) / 2.
+fzp_status nodes_upload(Plan& P) {
+  NodeSet& z = P.nd;
+  std::vector<double> xo(z.Mo);
+  for (int o = 0; o < z.Mo; ++o) xo[o] = (z.even ? (double)o : (double)o - 0.5 * (P.M - 1)) / z.half;
+  const Interp in(z.n, z.h / z.half, M_PI * z.band * z.half, xo, z.even);
+  std::vector<double> W = in.solve(z.even ? 1 : 0);
+  const bool full = z.even && P.owns_buffers;
+  if (full) {
+    const std::vector<double> We = W, Wo = in.solve(-1);
+    const int M = P.M, hm = M / 2;
+    W.resize(We.size() + (size_t)z.n * M);
+    double* F = W.data() + We.size();  // [node][output]
+    for (int k = 0; k < z.ns; ++k)
+      for (int o = 0; o <= hm; ++o) {
+        const double e = We[(size_t)k * z.Mo + o], d = Wo[(size_t)k * z.Mo + o];
+        const int kp = z.ns + k, km = z.ns - 1 - k;  // +x_k and -x_k
+        if (o < hm) {  // +x_o
+          F[(size_t)kp * M + hm + o] = 0.5 * (e + d);
+          F[(size_t)km * M + hm + o] = 0.5 * (e - d);
+        }
+        if (o > 0) {  // -x_o
+          F[(size_t)kp * M + hm - o] = 0.5 * (e - d);
+          F[(size_t)km * M + hm - o] = 0.5 * (e + d);
+        }
+      }
+  }
+  FZP_CUDA_TRY(cudaMalloc(&z.d_W, W.size() * sizeof(double)));
+  P.device_bytes += W.size() * sizeof(double);
+  FZP_CUDA_TRY(cudaMemcpy(z.d_W, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice));
+  z.d_Wy = full ? z.d_W + (size_t)z.ns * z.Mo : z.d_W;
+  return FZP_OK;
+}
+
+fzp_status nodes_fill(Plan& P, cudaStream_t s) {
+  const NodeSet& z = P.nd;
+  const int64_t ncols = z.fold ? P.c + 1 : P.N;
+  const int64_t threads = z.kblocks * 4 * z.ns;
+  const unsigned grid = (unsigned)std::min<int64_t>(8 * P.dn.num_sms, (threads + 255) / 256);
+  k_nodes_A<<<grid, 256, 0, s>>>(z.ns / 64, ncols, z.kblocks, z.fold ? 0 : P.c, z.fold ? 1 : 0, P.kappa, z.msh, z.delta,
+                                 reinterpret_cast<uint8_t*>(P.dn.d_A));
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s) {
+  const NodeSet& z = P.nd;
+  NodeArgs a{};
+  a.mg = P.mg;
+  if (z.fold) a.mg.c = 0;
+  a.ph = phase_rule(P, P.pass_index >= 0 ? &P.passes[P.pass_index] : nullptr);
+  a.j_begin = j0;
+  a.j_end = j0 + rows;
+  a.octant = octant ? 1 : 0;
+  a.kblocks = z.kblocks;
+  a.promote = P.dn.promote_kblocks;
+  // K blocks per unit: about three units per SM where the aperture is small
+  // (every unit ends in a promotion of 256 KiB into C1), whole promotions where
+  // it is large
+  const double R = std::sqrt((double)P.mg.sR), share = (double)rows / (z.fold ? P.c + 1 : P.N);
+  const double blocks = M_PI * R * R * (z.fold ? 0.25 : 1.0) * (octant ? 0.5 : 1.0) * share / (BK * 512.0);
+  a.group = (int)std::min<double>(std::max(8.0, std::ceil(blocks / (3.0 * P.dn.num_sms))), (double)a.promote);
+  if (a.group < 8) a.group = 8;
+  a.nchunks = (int)((z.kblocks + a.group - 1) / a.group);
+  a.sched = P.dn.d_sched;
+  a.A = reinterpret_cast<const uint8_t*>(P.dn.d_A);
+  a.err = P.d_err;
+  P.dominant = "k_nodes";
+  const int mask = mask_kind(P);
+  if (mask == MASK_MEMBRANE) {
+    a.df = deform_coef(P);
+    return launch<1, MASK_MEMBRANE>(P, a, s);
+  }
+  if (z.ns == 64)
+    return mask == MASK_PARITY   ? launch<1, MASK_PARITY>(P, a, s)
+           : mask == MASK_SIGNED ? launch<1, MASK_SIGNED>(P, a, s)
+                                 : launch<1, MASK_LEVELS>(P, a, s);
+  return mask == MASK_PARITY   ? launch<2, MASK_PARITY>(P, a, s)
+         : mask == MASK_SIGNED ? launch<2, MASK_SIGNED>(P, a, s)
+                               : launch<2, MASK_LEVELS>(P, a, s);
+}
+
+fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t s) {
+  const NodeSet& z = P.nd;
+  const bool eveny = z.even && !z.yfull;
+  const int ny = z.yfull ? z.n : z.ns, Moy = eveny ? z.Mo : P.M;
+  dim3 b1(32, 4), g1((unsigned)((z.ns + 31) / 32), (unsigned)((Moy + 3) / 4));
+  k_interp_rows<<<g1, b1, 0, s>>>(ny, z.ns, Moy, sym ? 1 : 0, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
+  const double lf = P.lambda * P.f;
+  InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf, accumulate};
+  k_interp_cols<<<dim3((unsigned)((z.Mo + IT - 1) / IT), (unsigned)((Moy + IT - 1) / IT)), 256, 0, s>>>(
+      a, z.d_W, z.d_X, reinterpret_cast<double2*>(d_field));
+  P.launches += 2;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+fzp_status nodes_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t s) {
+  const int64_t warps = (rows + 31) / 32;
+  const unsigned grid = (unsigned)std::min<int64_t>((warps + 3) / 4, 65535);
+  k_mask_nodes<<<grid, 128, 0, s>>>(P.mg, phase_rule(P, nullptr), mask_kind(P), P.N, j0, rows, out);
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+}  // namespace fzp

@@ -85,9 +85,10 @@ void release_plan(Plan* P) {
   if (P->dn.ev_fork) cudaEventDestroy(P->dn.ev_fork);
   if (P->dn.ev_join) cudaEventDestroy(P->dn.ev_join);
   if (P->dn.s2) cudaStreamDestroy(P->dn.s2);
+  if (P->nd.d_W) cudaFree(P->nd.d_W);
   if (P->owns_buffers) {
     void* ptrs[] = {P->d_C1, P->d_C1d, P->d_Uacc, P->d_err, P->d_metrics,
-                    P->bs.d_pre, P->bs.d_H, P->bs.d_Z, P->bs.d_G, P->bs.d_tab, P->dn.d_A, P->dn.d_sched,
+                    P->bs.d_pre, P->bs.d_H, P->bs.d_Z, P->bs.d_G, P->bs.d_tab, P->dn.d_A, P->dn.d_sched, P->nd.d_X,
                     P->sa.d_G, P->sa.d_T, P->sa.d_tw, P->sa.d_K, P->sa.d_RT, P->sa.d_xthr};
     for (void* q : ptrs)
       if (q) cudaFree(q);
@@ -255,6 +256,7 @@ fzp_status validate_and_derive(const fzp_params* in, Plan& P) {
   if (in->cluster != 0 && in->cluster != 1 && in->cluster != 2 && in->cluster != 4)
     return set_error(FZP_E_INVALID, "cluster must be 0, 1, 2 or 4");
   P.cluster_req = in->cluster;
+  nodes_choose(P);
   return FZP_OK;
 }
 
@@ -280,17 +282,59 @@ fzp_status build_mask_tables(Plan& P) {
   return FZP_OK;
 }
 
-fzp_status chunk_passes(Plan& P, int64_t j0, int64_t rows, cudaStream_t s) {
-  const int np = (P.form == FZP_FORM_DENSE && !P.passes.empty()) ? (int)P.passes.size() : 1;
+// Row pass and column pass of rows [j0, j0 + rows) (every mask pass of a dense
+// phase plate), accumulated into the ROI accumulator.  Folded plans: rows are
+// distances from the axis, `kind` says what each stands for.
+static fzp_status chunk_passes(Plan& P, int64_t j0, int64_t rows, RowKind kind, bool octant, cudaStream_t s) {
+  const bool nodes = P.nd.n > 0;
+  // a membrane on nodes takes both of its masks in one pass
+  const int np = (P.form == FZP_FORM_DENSE && !P.passes.empty() && !(nodes && P.has_deform)) ? (int)P.passes.size() : 1;
   fzp_status st = FZP_OK;
+  P.c1_stride = P.chunk_rows;
   for (int k = 0; k < np && st == FZP_OK; ++k) {
-    P.pass_index = np > 1 || !P.passes.empty() ? k : -1;
-    st = (P.form == FZP_FORM_DENSE) ? dense_rows(P, j0, rows, s) : bluestein_rows(P, j0, rows, s);
+    P.pass_index = P.form == FZP_FORM_DENSE && !P.passes.empty() && !(nodes && P.has_deform) ? k : -1;
+    st = nodes                          ? nodes_rows(P, j0, rows, octant, s)
+         : P.form == FZP_FORM_DENSE ? dense_rows(P, j0, rows, s)
+                                        : bluestein_rows(P, j0, rows, s);
     if (st == FZP_OK)
-      st = column_pass_tc_applies(P) ? column_pass_tc(P, j0, rows, s) : column_pass(P, j0, rows, s);
+      st = column_pass_tc_applies(P) ? column_pass_tc(P, j0, rows, s) : column_pass(P, j0, rows, kind, s);
   }
   P.pass_index = -1;
   return st;
+}
+
+fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t s) {
+  *sym = false;
+  // rows up and down from the axis
+  const int64_t c = P.c, up = b - 1 - c, dn = c - a, h = std::min(up, dn);
+  const bool nodes = P.nd.n > 0;
+  P.nd.yfull = P.nd.even && up != dn;
+  const size_t acc = nodes ? (size_t)(P.nd.yfull ? P.nd.n : P.nd.ns) * P.nd.ns : (size_t)P.M * P.M;
+  FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, acc * sizeof(double2), s));
+  if (a >= b) return FZP_OK;
+  auto run = [&](int64_t j0, int64_t j1, RowKind kind, bool octant) {
+    fzp_status st = FZP_OK;
+    for (int64_t j = j0; j < j1 && st == FZP_OK; j += P.chunk_rows)
+      st = chunk_passes(P, j, std::min(P.chunk_rows, j1 - j), kind, octant, s);
+    return st;
+  };
+  if (!(nodes && P.nd.fold)) return run(a, b, ROWS_PLAIN, false);
+  // a flat plate: the rows at distance d on either side of the axis have one
+  // row transform; h: the distances present on both sides
+  fzp_status st = FZP_OK;
+  if (h >= 0) {
+    // every row that meets the disc: the plate is its own transpose
+    *sym = up == dn && (up == P.c || (up + 1) * (up + 1) > P.mg.sR);
+    st = run(0, h + 1, ROWS_FOLDED, *sym);
+  }
+  const int64_t first = std::max<int64_t>(h, std::max(-up, -dn) - 1) + 1;  // one-sided distances
+  if (st == FZP_OK && up > h && up >= first) st = run(first, up + 1, ROWS_PLAIN, false);
+  if (st == FZP_OK && dn > h && dn >= first) st = run(first, dn + 1, ROWS_MIRRORED, false);
+  return st;
+}
+
+fzp_status finish_field(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t s) {
+  return P.nd.n > 0 ? nodes_epilogue(P, d_field, accumulate, sym, s) : epilogue(P, d_field, accumulate, s);
 }
 
 // cudaMalloc of a plan's row intermediate.  Host-side fault injection for
@@ -366,7 +410,7 @@ fzp_status fzp_plan(const fzp_params* params, fzp_plan_t* out) {
     const size_t esz = P->precision == FZP_PREC_FP64 ? sizeof(double) : sizeof(float);
     cudaError_t e = cudaSuccess;
     while (true) {
-      const size_t bytes = (size_t)(M2 * P->chunk_rows) * esz;
+      const size_t bytes = c1_elems(*P) * esz;
       void* c1 = nullptr;
       e = workspace_malloc(&c1, bytes);
       if (e == cudaSuccess) {
@@ -379,7 +423,9 @@ fzp_status fzp_plan(const fzp_params* params, fzp_plan_t* out) {
       cudaGetLastError();
       P->chunk_rows = std::max<int64_t>(256, (P->chunk_rows / 2 + 255) / 256 * 256);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&P->d_Uacc, (size_t)P->M * P->M * sizeof(double2));
+    // the nodes can outnumber a small ROI's samples
+    const size_t nacc = std::max<size_t>((size_t)P->M * P->M, (size_t)P->nd.n * P->nd.ns);
+    if (e == cudaSuccess) e = cudaMalloc(&P->d_Uacc, nacc * sizeof(double2));
     if (e == cudaSuccess) e = cudaMalloc(&P->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&P->d_metrics, 8192 * sizeof(double) + (size_t)P->M * P->M * sizeof(double2));
     if (e == cudaSuccess) e = cudaMemset(P->d_err, 0, sizeof(int));
@@ -518,11 +564,11 @@ fzp_status fzp_propagate_roi(fzp_plan_t plan, int64_t row_begin, int64_t row_end
     return set_error(FZP_E_INVALID, "row range [%lld, %lld) outside [0, %lld]", (long long)row_begin,
                      (long long)row_end, (long long)P.N);
   cudaStream_t s = (cudaStream_t)stream;
-  FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, (size_t)P.M * P.M * sizeof(double2), s));
   int64_t jlo, jhi;
   disc_rows(P, jlo, jhi);
   const int64_t a = std::max(row_begin, jlo), b = std::min(row_end, jhi);
   if (P.form == FZP_FORM_SACZT) {
+    FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, (size_t)P.M * P.M * sizeof(double2), s));
     // the whole padded plane at once (rows outside the range masked to zero)
     if (a < b) {
       const fzp_status st = saczt_propagate(P, a, b, s);
@@ -530,11 +576,10 @@ fzp_status fzp_propagate_roi(fzp_plan_t plan, int64_t row_begin, int64_t row_end
     }
     return epilogue_z(P, d_field, accumulate, P.sa.zF, s);
   }
-  for (int64_t j0 = a; j0 < b; j0 += P.chunk_rows) {
-    const fzp_status st = chunk_passes(P, j0, std::min(P.chunk_rows, b - j0), s);
-    if (st != FZP_OK) return st;
-  }
-  return epilogue(P, d_field, accumulate, s);
+  bool sym = false;
+  const fzp_status st = propagate_rows(P, a, b, &sym, s);
+  if (st != FZP_OK) return st;
+  return finish_field(P, d_field, accumulate, sym, s);
 }
 
 fzp_status fzp_aperture_mask(fzp_plan_t plan, int64_t row_begin, int64_t row_end, void* d_mask, void* stream) {
