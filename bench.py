@@ -239,6 +239,32 @@ def partitioned_flops(info: dict, j0: int, j1: int) -> float:
     return blocks * (fft + 8.0 * P) + (j1 - j0) * fft
 
 
+def folded_flops(info: dict, nodes: int, j0: int, j1: int) -> float:
+    """FP32 flops that the partitioned row pass does for rows [j0, j1) of a flat
+    plate whose ROI is centred on the focus: each distance from the axis once, a
+    row's columns from the axis to its chord -- to the diagonal when the range is
+    the whole aperture -- in blocks of S, with 2 x nodes outputs per row (0
+    nodes: the ROI's samples, all columns)."""
+    import numpy as np
+    P, fft = 4096, 5.0 * 4096 * 12
+    S = 256 * min(15, (4097 - (2 * nodes or info["M"])) // 256)
+    c, s_R = info["c"], info["s_R"]
+    h = min(j1 - 1 - c, c - j0)
+    whole = nodes > 0 and j1 - 1 - c == c - j0 and (h >= c or (h + 1) ** 2 > s_R)
+    if h >= 0:
+        d = np.concatenate([np.arange(0, h + 1), np.arange(h + 1, max(j1 - 1 - c, c - j0) + 1)])
+    else:
+        d = np.arange(max(c - j1 + 1, j0 - c), max(j1 - 1 - c, c - j0) + 1)
+    rem = s_R - d.astype(np.int64) ** 2
+    d, rem = d[rem >= 0], rem[rem >= 0]
+    b = np.minimum(np.floor(np.sqrt(rem.astype(np.float64))).astype(np.int64), c)
+    if nodes:
+        blocks = (np.minimum(b, d) if whole else b) // S + 1
+    else:
+        blocks = (c + b) // S - (c - b) // S + 1
+    return float(np.sum(blocks)) * (fft + 8.0 * P) + len(d) * fft
+
+
 def node_count(info: dict, lam: float, f: float, M: int, pitch: float, deformed: bool = False) -> int:
     """Nodes per axis that the dense form's contraction runs on (nodes.cu), for an
     ROI centred on the focus: the positive half of n nodes for a flat plate,
@@ -816,13 +842,17 @@ def main():
                 "work": "16 P^2 bytes per launch (P = padded grid side)"}
     else:
         launches = max(1, prof["dominant_launches"])
+        flat = not wl.get("deform")
+        nodes = node_count(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], not flat)
         if info["conv"] == 2:
-            flops_launch = partitioned_flops(info, j0, j1) * args.steps / launches
-            work = ("per block of S columns meeting a row's chord 5 P log2 P + 8 P, per row 5 P log2 P "
-                    "(P = 4096)")
+            flops_launch = (folded_flops(info, nodes, j0, j1) if flat else partitioned_flops(info, j0, j1)) \
+                * args.steps / launches
+            work = ("per block of S columns of a row's chord 5 P log2 P + 8 P, per row 5 P log2 P "
+                    "(P = 4096), over the rows and columns left after the symmetry folds")
         else:
-            flops_launch = bluestein_f2_flops(info, rows * args.steps / launches)
-            work = "per row L1 (10 L2 log2 L2 + 6 L2)"
+            both = max(0, min(j1 - 1 - info["c"], info["c"] - j0))  # rows whose mirror image is in the range
+            flops_launch = bluestein_f2_flops(info, (rows - (both if flat else 0)) * args.steps / launches)
+            work = "per row (mirror images once) L1 (10 L2 log2 L2 + 6 L2)"
         achieved = flops_launch / (avg_ms / 1e3) / 1e12
         peak = SM_COUNT * 128 * 2 * SM_MAX_MHZ_NOMINAL * 1e6 / 1e12  # FP32 FMA lanes x clock
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,

@@ -168,7 +168,10 @@ typedef struct fzp_params {
                           each block's 4096-point spectrum times the
                           precomputed spectrum of its chirp piece, summed over
                           the blocks that meet the row's disc chord, then one
-                          inverse 4096-point FFT per row, all on chip; FP32
+                          inverse 4096-point FFT per row, all on chip (where
+                          the ROI samples the field several times finer than
+                          its band, the row's outputs are that many
+                          interpolation nodes and M above is their count); FP32
                           only (FZP_E_UNSUPPORTED with FP64).  Other values
                           are invalid; the other forms ignore it            */
 } fzp_params;

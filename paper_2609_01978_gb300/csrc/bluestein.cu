@@ -160,6 +160,9 @@ struct RowArgs {
   const void* vin;   // input sequence for the table-building mode (length L)
   int S;             // partitioned convolution: columns per block
   int64_t nseg;      // partitioned convolution: blocks per row (spectra in H)
+  int64_t col0;      // partitioned convolution: first column of block 0
+  int half;          // even output grid: columns from the axis on, outputs m and M - 1 - m added
+  int octant;        // columns up to the row's distance from the axis only, the last one halved
 };
 
 // Aperture transmission of sample (j, i): T e^{i phi}, optional deformation.
@@ -792,7 +795,7 @@ __device__ __forceinline__ bool chunk_zones(int64_t x, int64_t dj2, const MaskGe
 }
 
 // G_s = FFT_P(g_s) for every block s (one CTA per block, grid-strided).
-__global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int S, int M, double delta, float2* G) {
+__global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int64_t col0, int S, int M, double delta, float2* G) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* b0 = reinterpret_cast<float2*>(smem_raw);
   float2* b1 = b0 + SBUF;
@@ -801,7 +804,7 @@ __global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int S, int M, 
   seg_twiddles(twA, twB);
   const int t = threadIdx.x;
   for (int64_t s = blockIdx.x; s < nseg; s += gridDim.x) {
-    const int64_t is = s * (int64_t)S;
+    const int64_t is = col0 + s * (int64_t)S;
     float2 v[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
@@ -833,8 +836,19 @@ __global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int S, int M, 
 // phase).  A block's input chirp loads are issued together before the
 // transmission is evaluated, and the spectra G_s before the last FFT pass,
 // so each waits one memory latency.
+//
+// Flat plates (FOLD; rows j >= c: each stands for itself and its mirror image):
+// `half`, for an output grid symmetric about the axis, transforms the columns
+// from the axis on and adds the outputs at x and -x (the axis column, counted
+// twice, at half weight); `octant`, for the whole aperture, stops at the
+// diagonal |di| = dj with half weight there (the field is this one plus its
+// transpose).  Half the blocks each, a quarter both, and half the rows; with the
+// outputs on nodes (nodes.cu: 128 instead of 512) the column pass shrinks too.
+// Whole propagation, ROI 512^2: D = 5 cm (N = 63,213) 17.14 -> 2.31 ms, L = 16
+// on N = 50,001 15.75 -> 2.13 ms.
 template <int MODE>
 __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
+  constexpr bool FOLD = MODE == SEG_FLAT || MODE == SEG_LEVELS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* b0 = reinterpret_cast<float2*>(smem_raw);
   float2* b1 = b0 + SBUF;
@@ -866,12 +880,13 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
 #pragma unroll
     for (int d = 0; d < 16; ++d) acc[d] = make_float2(0.0f, 0.0f);
     if (rem >= 0) {
-      const int64_t bmax = isqrt_row(rem);
+      int64_t bmax = isqrt_row(rem);
+      if (FOLD && a.octant) bmax = min(bmax, dj);
       // the row's disc chord, within the grid (a given N may cut the disc)
-      const int64_t lo = max(a.mg.c - bmax, (int64_t)0), hi = min(a.mg.c + bmax, a.N - 1);
-      const int64_t s1 = hi / S;
-      for (int64_t s = lo / S; s <= s1; ++s) {
-        const int64_t is = s * (int64_t)S;
+      const int64_t lo = FOLD && a.half ? a.mg.c : max(a.mg.c - bmax, (int64_t)0), hi = min(a.mg.c + bmax, a.N - 1);
+      const int64_t col0 = FOLD ? a.col0 : 0, s1 = (hi - col0) / S;
+      for (int64_t s = (lo - col0) / S; s <= s1; ++s) {
+        const int64_t is = col0 + s * (int64_t)S;
         float2 v[16];
         if (MODE == SEG_FLAT || MODE == SEG_MEMBRANE) {
           // the block's chord [olo, ohi] in block offsets; loads clamped into
@@ -957,6 +972,23 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
             if (q < RS && i >= lo && i <= hi) v[q] = cmul(aperture<float>(a, j, i), v[q]);
           }
         }
+        if (FOLD) {
+          // half weight of the axis column and of the diagonal's columns (few blocks hold one)
+          const int64_t oa = a.half ? a.mg.c - is : -1, od = a.octant ? a.mg.c + dj - is : -1,
+                        oe = a.octant && !a.half && dj > 0 ? a.mg.c - dj - is : -1;
+          const bool ha = oa >= 0 && oa < S, hd = od >= 0 && od < S, he = oe >= 0 && oe < S;
+          if (ha || hd || he) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+              const int o = t + 256 * q;
+              float w = ha && o == (int)oa ? 0.5f : 1.0f;
+              if (hd && o == (int)od) w *= 0.5f;
+              if (he && o == (int)oe) w *= 0.5f;
+              v[q].x *= w;
+              v[q].y *= w;
+            }
+          }
+        }
         // forward FFT (passes A and B), spectrum loads, pass C, product-sum
         dft16(v);
 #pragma unroll
@@ -997,6 +1029,20 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
     for (int d = 0; d < 16; ++d) acc[d].y = -acc[d].y;
     fft_p(acc, b0, b1, twA, twB);
     const int64_t jl = j - a.c1_j0;
+    if (FOLD && a.half) {
+      // outputs x and -x meet in the transpose buffer that the transform's last
+      // pass does not read (M <= 256 nodes: one output per thread)
+      if (t < a.M) b0[t] = cmul(make_float2(acc[0].x * scale, -acc[0].y * scale), post[t]);
+      __syncthreads();
+      const int hm = a.M / 2;
+      if (t < hm) {
+        const float2 y = cadd(b0[hm + t], b0[hm - 1 - t]);
+        C1[(int64_t)c1_row_re(t) * a.c1_stride + jl] = y.x;
+        C1[(int64_t)c1_row_im(t) * a.c1_stride + jl] = y.y;
+      }
+      __syncthreads();
+      continue;
+    }
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
       const int m = t + 256 * d;
@@ -1107,6 +1153,11 @@ static RowArgs make_args(const Plan& P) {
   a.vin = b.d_tab;
   a.S = b.S;
   a.nseg = b.nseg;
+  a.col0 = b.col0;
+  if (P.nd.n > 0) {
+    a.M = P.nd.n;
+    a.half = P.nd.even ? 1 : 0;
+  }
   return a;
 }
 
@@ -1125,20 +1176,21 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
   b.seg = (sizeof(R) == 4 && P.conv_req != 1) ? 1 : 0;
   if (b.seg) {
     // partitioned convolution: S + M - 1 <= 4096, S a multiple of 256 (at most 15 x 256)
-    b.S = 256 * std::min(15, (4097 - P.M) / 256);
-    b.nseg = (P.N + b.S - 1) / b.S;
+    const int M = P.nd.n > 0 ? P.nd.n : P.M;  // outputs per row: the nodes, or the ROI samples
+    b.S = 256 * std::min(15, (4097 - M) / 256);
+    b.col0 = P.nd.even ? P.c : 0;
+    b.nseg = (P.N - b.col0 + b.S - 1) / b.S;
     b.rows = P.chunk_rows;
     out->pre = sizeof(C) * P.N;
     out->H = sizeof(C) * (size_t)SP * (size_t)b.nseg;
-    out->tab = sizeof(C) * (b.L + (int)b.L2 + P.M + 4096);
+    out->tab = sizeof(C) * (b.L + (int)b.L2 + std::max(P.M, M) + 4096);
     out->Z = 0;
     out->G = 0;
-    static std::atomic<uint64_t> attr_seg{0}, attr_segt{0};
-    static std::atomic<uint64_t> attr_segl{0}, attr_segm{0}, attr_segg{0};
-    FZP_CUDA_TRY(smem_attr_once((const void*)k_seg<SEG_FLAT>, (int)SEG_SMEM, attr_seg));
-    FZP_CUDA_TRY(smem_attr_once((const void*)k_seg<SEG_LEVELS>, (int)SEG_SMEM, attr_segl));
-    FZP_CUDA_TRY(smem_attr_once((const void*)k_seg<SEG_MEMBRANE>, (int)SEG_SMEM, attr_segm));
-    FZP_CUDA_TRY(smem_attr_once((const void*)k_seg<SEG_GENERAL>, (int)SEG_SMEM, attr_segg));
+    out->X = (size_t)P.nd.ns * P.M * sizeof(double2);
+    static std::atomic<uint64_t> attr_segt{0}, attr_seg[4];
+    const void* kern[4] = {(const void*)k_seg<SEG_FLAT>, (const void*)k_seg<SEG_LEVELS>,
+                           (const void*)k_seg<SEG_MEMBRANE>, (const void*)k_seg<SEG_GENERAL>};
+    for (int q = 0; q < 4; ++q) FZP_CUDA_TRY(smem_attr_once(kern[q], (int)SEG_SMEM, attr_seg[q]));
     FZP_CUDA_TRY(smem_attr_once((const void*)k_seg_tables, (int)SEG_SMEM, attr_segt));
     return FZP_OK;
   }
@@ -1167,13 +1219,18 @@ fzp_status fill_tables_t(Plan& P, cudaStream_t s) {
   const int twN = (int)b.L2;
   b.d_tw = reinterpret_cast<C*>(b.d_tab) + b.L;
   b.d_post = reinterpret_cast<C*>(b.d_tw) + twN;
-  b.d_twL = reinterpret_cast<C*>(b.d_post) + P.M;
-  k_tables<R><<<1024, 256, 0, s>>>(P.N, P.M, P.msh, b.L, P.c, P.kappa, P.delta, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
+  // the outputs: the ROI's samples, or the nodes (all n of them)
+  const bool nodes = P.nd.n > 0;
+  const int M = nodes ? P.nd.n : P.M;
+  const double delta = nodes ? P.nd.delta : P.delta;
+  const double msh = nodes ? P.nd.msh + (P.nd.even ? P.nd.n / 2 : 0) : P.msh;
+  b.d_twL = reinterpret_cast<C*>(b.d_post) + M;
+  k_tables<R><<<1024, 256, 0, s>>>(P.N, M, msh, b.L, P.c, P.kappa, delta, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
                                    b.d_twL);
   FZP_CUDA_TRY(cudaGetLastError());
   if (b.seg) {
     const unsigned g = (unsigned)std::min<int64_t>(b.nseg, 1024);
-    k_seg_tables<<<g, STH, SEG_SMEM, s>>>(b.nseg, b.S, P.M, P.delta, reinterpret_cast<float2*>(b.d_H));
+    k_seg_tables<<<g, STH, SEG_SMEM, s>>>(b.nseg, b.col0, b.S, M, delta, reinterpret_cast<float2*>(b.d_H));
     FZP_CUDA_TRY(cudaGetLastError());
     P.launches += 2;
     return FZP_OK;
@@ -1203,11 +1260,17 @@ fzp_status build_tables_t(Plan& P) {
   if (z.Z) FZP_CUDA_TRY(cudaMalloc(&b.d_Z, z.Z));
   if (z.G) FZP_CUDA_TRY(cudaMalloc(&b.d_G, z.G));
   P.device_bytes += z.pre + z.H + z.tab + z.Z + z.G;
+  if (P.nd.n > 0) {
+    FZP_CUDA_TRY(cudaMalloc(&P.nd.d_X, z.X));
+    P.device_bytes += z.X;
+    st = nodes_upload(P);
+    if (st != FZP_OK) return st;
+  }
   return fill_tables_t<R>(P, 0);
 }
 
 template <typename R>
-fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, cudaStream_t s) {
+fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s) {
   using C = typename Cplx<R>::T;
   const Bluestein& b = P.bs;
   RowArgs a = make_args(P);
@@ -1218,20 +1281,18 @@ fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, cudaStream_t s) {
     FZP_CUDA_TRY(cudaGetDevice(&dev));
     FZP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int mode = P.has_deform ? (P.levels >= 2 ? SEG_GENERAL : SEG_MEMBRANE) : (P.levels >= 2 ? SEG_LEVELS : SEG_FLAT);
-    const void* kern = mode == SEG_FLAT ? (const void*)k_seg<SEG_FLAT>
-                       : mode == SEG_LEVELS ? (const void*)k_seg<SEG_LEVELS>
-                       : mode == SEG_MEMBRANE ? (const void*)k_seg<SEG_MEMBRANE>
-                                              : (const void*)k_seg<SEG_GENERAL>;
+    a.octant = octant ? 1 : 0;
+    void (*kern)(RowArgs) = mode == SEG_FLAT       ? k_seg<SEG_FLAT>
+                            : mode == SEG_LEVELS   ? k_seg<SEG_LEVELS>
+                            : mode == SEG_MEMBRANE ? k_seg<SEG_MEMBRANE>
+                                                   : k_seg<SEG_GENERAL>;
     FZP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, kern, STH, SEG_SMEM));
     if (ctas_per_sm < 1) ctas_per_sm = 1;
     a.j0 = j0;
     a.rows = rows;
     const int64_t grid = std::min<int64_t>(rows, (int64_t)ctas_per_sm * sms);
     prof_begin(P, s);
-    if (mode == SEG_FLAT) k_seg<SEG_FLAT><<<(unsigned)grid, STH, SEG_SMEM, s>>>(a);
-    else if (mode == SEG_LEVELS) k_seg<SEG_LEVELS><<<(unsigned)grid, STH, SEG_SMEM, s>>>(a);
-    else if (mode == SEG_MEMBRANE) k_seg<SEG_MEMBRANE><<<(unsigned)grid, STH, SEG_SMEM, s>>>(a);
-    else k_seg<SEG_GENERAL><<<(unsigned)grid, STH, SEG_SMEM, s>>>(a);
+    kern<<<(unsigned)grid, STH, SEG_SMEM, s>>>(a);
     prof_end(P, s);
     P.launches += 1;
     FZP_CUDA_TRY(cudaGetLastError());
@@ -1292,10 +1353,10 @@ fzp_status bluestein_fill_tables(Plan& P, cudaStream_t s) {
   return P.precision == FZP_PREC_FP64 ? fill_tables_t<double>(P, s) : fill_tables_t<float>(P, s);
 }
 
-fzp_status bluestein_rows(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream) {
+fzp_status bluestein_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t stream) {
   P.dominant = P.precision == FZP_PREC_FP64 ? "bluestein_f2<double>"
                                              : (P.bs.seg ? "k_seg (partitioned convolution)" : "bluestein_f2<float>");
-  return P.precision == FZP_PREC_FP64 ? rows_t<double>(P, j0, rows, stream) : rows_t<float>(P, j0, rows, stream);
+  return P.precision == FZP_PREC_FP64 ? rows_t<double>(P, j0, rows, false, stream) : rows_t<float>(P, j0, rows, octant, stream);
 }
 
 }  // namespace fzp

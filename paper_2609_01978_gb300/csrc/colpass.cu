@@ -175,7 +175,7 @@ __global__ void k_intensity(int64_t count, const double2* __restrict__ U, double
 fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStream_t s) {
   const bool nodes = P.nd.n > 0;
   ColArgs g{};
-  g.c = nodes && P.nd.fold ? 0 : P.c;
+  g.c = P.form == FZP_FORM_DENSE && P.fold ? 0 : P.c;
   g.j0 = j0;
   g.rows = rows;
   g.c1_stride = P.c1_stride;
@@ -189,9 +189,9 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
     g.wr = P.passes[P.pass_index].wr;
     g.wi = P.passes[P.pass_index].wi;
   }
-  g.slices = nodes ? P.nd.slices : 1;
-  g.slice_off = nodes ? P.nd.slice_elems : 0;
-  if (nodes && P.has_deform) g.sin_off = 128 * P.c1_stride;
+  g.slices = P.nd.slices;
+  g.slice_off = P.nd.slice_elems;
+  if (nodes && P.has_deform && P.form == FZP_FORM_DENSE) g.sin_off = 128 * P.c1_stride;
   // rows per block: 2048, fewer where that leaves the GPU idle (few output tiles)
   const int ny = nodes && P.nd.yfull ? P.nd.n : g.M;
   const int64_t tiles = (int64_t)(g.M / TM) * (ny / TN);

@@ -177,6 +177,7 @@ struct Bluestein {
   int seg = 0;
   int S = 0;
   int64_t nseg = 0;
+  int64_t col0 = 0;       // first column of block 0 (the axis for an even output grid)
 };
 
 // One signed-mask pass of a phase plate in the dense form: the mask is +1 on
@@ -207,13 +208,12 @@ struct Dense {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
-// The dense form on interpolation nodes (nodes.cu): n nodes across the ROI, of
-// which ns are evaluated (the positive half of them for an even field).
+// A form on interpolation nodes (nodes.cu): n nodes across the ROI, of which ns
+// are evaluated (the positive half of them for an even field).
 struct NodeSet {
   int n = 0, ns = 0;       // n = 0: the plan does not use nodes
   int Mo = 0;              // outputs per side of the interpolation (even: M / 2 + 1)
   bool even = false;       // flat plate, ROI centred on the focus
-  bool fold = false;       // flat plate: columns and rows +-d folded
   int64_t kblocks = 0;     // ceil(columns / 32)
   double half = 0, h = 0;  // ROI half width and node pitch, in ROI pitches
   double band = 0;         // 2 R p / (lambda f): the field's band, cycles per pitch
@@ -279,6 +279,7 @@ struct Plan {
   SaCzt sa;
   Dense dn;
   NodeSet nd;
+  bool fold = false;            // flat plate: the rows at distances +-d from the axis run once
   int64_t c1_stride = 0;        // row length of C1 in the chunk being run
   // tracing: kernel launches issued, and CUDA events around the dominant
   // kernel (recorded on the launching stream when profiling is enabled)
@@ -314,7 +315,7 @@ struct FormSizes {
 fzp_status bluestein_layout(Plan& P, FormSizes* out);
 fzp_status bluestein_fill_tables(Plan& P, cudaStream_t s);  // buffers already assigned
 fzp_status bluestein_build_tables(Plan& P);                 // layout + allocate + fill
-fzp_status bluestein_rows(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream);
+fzp_status bluestein_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t stream);
 fzp_status dense_layout(Plan& P, FormSizes* out);
 fzp_status dense_fill_tables(Plan& P, cudaStream_t s);
 fzp_status dense_build_tables(Plan& P);

@@ -990,8 +990,8 @@ fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-// The rule of the node form (host).  It takes split-BF16 plans whose band
-// leaves room on the nodes; a coarser pitch (or a larger ROI) than that, BF16
+// The rule of the nodes (host).  The partitioned FP32 row pass (k_seg) takes
+// them wherever the ROI's band leaves room on them; so do split-BF16 plans.  BF16
 // without the split and explicit clusters of 2 or 4 CTAs stay with k_dense,
 // and so do plates of 6 and more levels (L/2 passes: the plain FP32 form's
 // single pass is the faster one there) and membranes that need two node tiles
@@ -999,7 +999,9 @@ fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
 void nodes_choose(Plan& P) {
   NodeSet& z = P.nd;
   z = NodeSet{};
-  if (P.form != FZP_FORM_DENSE || P.precision != FZP_PREC_SPLIT_BF16 || P.cluster_req > 1 || P.levels > 4) return;
+  const bool dense = P.form == FZP_FORM_DENSE && P.precision == FZP_PREC_SPLIT_BF16 && P.cluster_req <= 1 && P.levels <= 4;
+  const bool seg = P.form == FZP_FORM_BLUESTEIN && P.precision == FZP_PREC_FP32 && P.conv_req != 1;
+  if (!dense && !seg) return;
   const bool flat = !P.has_deform;
   const bool centred = P.msh == (double)(P.M / 2);
   const bool even = flat && centred;
@@ -1009,14 +1011,13 @@ void nodes_choose(Plan& P) {
   struct { int n; double most; } sizes[] = {{64, 36.0}, {128, 80.0}, {256, 170.0}};
   for (auto& q : sizes) {
     const int ns = even ? q.n / 2 : q.n;
-    if (ns < 64 || ns > 128 || (!flat && ns > 64) || dof > q.most) continue;
+    if (ns < 64 || ns > 128 || (dense && !flat && ns > 64) || dof > q.most) continue;
     z.n = q.n;
     z.ns = ns;
     break;
   }
   if (!z.n) return;
   z.even = even;
-  z.fold = flat;
   z.Mo = even ? P.M / 2 + 1 : P.M;
   z.half = half;
   z.band = band;
@@ -1031,7 +1032,7 @@ void nodes_choose(Plan& P) {
 
 fzp_status nodes_layout(Plan& P, FormSizes* out) {
   NodeSet& z = P.nd;
-  const int64_t ncols = z.fold ? P.c + 1 : P.N;
+  const int64_t ncols = P.fold ? P.c + 1 : P.N;
   z.kblocks = (ncols + BK - 1) / BK;
   out->A = (size_t)z.kblocks * (size_t)(z.ns / 64) * 2 * SUB;
   out->sched = sizeof(int) * (size_t)(3 * ((z.kblocks + 7) / 8) + 1);
@@ -1077,10 +1078,10 @@ fzp_status nodes_upload(Plan& P) {
 
 fzp_status nodes_fill(Plan& P, cudaStream_t s) {
   const NodeSet& z = P.nd;
-  const int64_t ncols = z.fold ? P.c + 1 : P.N;
+  const int64_t ncols = P.fold ? P.c + 1 : P.N;
   const int64_t threads = z.kblocks * 4 * z.ns;
   const unsigned grid = (unsigned)std::min<int64_t>(8 * P.dn.num_sms, (threads + 255) / 256);
-  k_nodes_A<<<grid, 256, 0, s>>>(z.ns / 64, ncols, z.kblocks, z.fold ? 0 : P.c, z.fold ? 1 : 0, P.kappa, z.msh, z.delta,
+  k_nodes_A<<<grid, 256, 0, s>>>(z.ns / 64, ncols, z.kblocks, P.fold ? 0 : P.c, P.fold ? 1 : 0, P.kappa, z.msh, z.delta,
                                  reinterpret_cast<uint8_t*>(P.dn.d_A));
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
@@ -1091,7 +1092,7 @@ fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream
   const NodeSet& z = P.nd;
   NodeArgs a{};
   a.mg = P.mg;
-  if (z.fold) a.mg.c = 0;
+  if (P.fold) a.mg.c = 0;
   a.ph = phase_rule(P, P.pass_index >= 0 ? &P.passes[P.pass_index] : nullptr);
   a.j_begin = j0;
   a.j_end = j0 + rows;
@@ -1101,8 +1102,8 @@ fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream
   // K blocks per unit: about three units per SM where the aperture is small
   // (every unit ends in a promotion of 256 KiB into C1), whole promotions where
   // it is large
-  const double R = std::sqrt((double)P.mg.sR), share = (double)rows / (z.fold ? P.c + 1 : P.N);
-  const double blocks = M_PI * R * R * (z.fold ? 0.25 : 1.0) * (octant ? 0.5 : 1.0) * share / (BK * 512.0);
+  const double R = std::sqrt((double)P.mg.sR), share = (double)rows / (P.fold ? P.c + 1 : P.N);
+  const double blocks = M_PI * R * R * (P.fold ? 0.25 : 1.0) * (octant ? 0.5 : 1.0) * share / (BK * 512.0);
   a.group = (int)std::min<double>(std::max(8.0, std::ceil(blocks / (3.0 * P.dn.num_sms))), (double)a.promote);
   if (a.group < 8) a.group = 8;
   a.nchunks = (int)((z.kblocks + a.group - 1) / a.group);

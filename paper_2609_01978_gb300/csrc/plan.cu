@@ -257,6 +257,8 @@ fzp_status validate_and_derive(const fzp_params* in, Plan& P) {
     return set_error(FZP_E_INVALID, "cluster must be 0, 1, 2 or 4");
   P.cluster_req = in->cluster;
   nodes_choose(P);
+  // the general dense kernels run every row of the range
+  P.fold = !P.has_deform && (P.form == FZP_FORM_BLUESTEIN || P.nd.n > 0);
   return FZP_OK;
 }
 
@@ -291,11 +293,12 @@ static fzp_status chunk_passes(Plan& P, int64_t j0, int64_t rows, RowKind kind, 
   const int np = (P.form == FZP_FORM_DENSE && !P.passes.empty() && !(nodes && P.has_deform)) ? (int)P.passes.size() : 1;
   fzp_status st = FZP_OK;
   P.c1_stride = P.chunk_rows;
+  if (P.fold && P.form == FZP_FORM_BLUESTEIN) j0 += P.c;  // its kernels take rows of the grid
   for (int k = 0; k < np && st == FZP_OK; ++k) {
     P.pass_index = P.form == FZP_FORM_DENSE && !P.passes.empty() && !(nodes && P.has_deform) ? k : -1;
-    st = nodes                          ? nodes_rows(P, j0, rows, octant, s)
-         : P.form == FZP_FORM_DENSE ? dense_rows(P, j0, rows, s)
-                                        : bluestein_rows(P, j0, rows, s);
+    st = nodes && P.form == FZP_FORM_DENSE ? nodes_rows(P, j0, rows, octant, s)
+         : P.form == FZP_FORM_DENSE        ? dense_rows(P, j0, rows, s)
+                                           : bluestein_rows(P, j0, rows, octant, s);
     if (st == FZP_OK)
       st = column_pass_tc_applies(P) ? column_pass_tc(P, j0, rows, s) : column_pass(P, j0, rows, kind, s);
   }
@@ -318,13 +321,14 @@ fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t
       st = chunk_passes(P, j, std::min(P.chunk_rows, j1 - j), kind, octant, s);
     return st;
   };
-  if (!(nodes && P.nd.fold)) return run(a, b, ROWS_PLAIN, false);
+  if (!P.fold) return run(a, b, ROWS_PLAIN, false);
   // a flat plate: the rows at distance d on either side of the axis have one
   // row transform; h: the distances present on both sides
   fzp_status st = FZP_OK;
   if (h >= 0) {
-    // every row that meets the disc: the plate is its own transpose
-    *sym = up == dn && (up == P.c || (up + 1) * (up + 1) > P.mg.sR);
+    // every row that meets the disc: the plate is its own transpose (the row
+    // passes on nodes use that)
+    *sym = nodes && up == dn && (up == P.c || (up + 1) * (up + 1) > P.mg.sR);
     st = run(0, h + 1, ROWS_FOLDED, *sym);
   }
   const int64_t first = std::max<int64_t>(h, std::max(-up, -dn) - 1) + 1;  // one-sided distances
