@@ -297,7 +297,11 @@ fzp_status fzp_batch_plan(const fzp_params* params, int n, fzp_batch_t* out) {
     batch_release(b);
     return set_error(FZP_E_OOM, "batch workspace allocation failed");
   }
-  if (cudaMemset(err, 0, sizeof(int)) != cudaSuccess) { batch_release(b); return set_error(FZP_E_CUDA, "memset"); }
+  // the interpolation matrices are built by then, whichever stream replays the graph
+  if (cudaMemset(err, 0, sizeof(int)) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+    batch_release(b);
+    return set_error(FZP_E_CUDA, "batch tables");
+  }
   for (fzp_plan_s* P : b->inst) {
     P->bs.d_pre = pre; P->bs.d_H = H; P->bs.d_tab = tab; P->bs.d_Z = Z; P->bs.d_G = G;
     P->dn.d_A = A;

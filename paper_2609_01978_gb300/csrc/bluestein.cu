@@ -1111,6 +1111,7 @@ DeformCoef deform_coef(const Plan& P) {
   c.tq = (float)(d.taper * P.dx * P.dx / (P.R * P.R));
   c.zc = (float)std::cos(2.0 * M_PI * kx);
   c.zs = (float)std::sin(2.0 * M_PI * kx);
+  c.z4 = (float)(4.0 * std::sin(M_PI * kx) * std::sin(M_PI * kx));
   c.n = d.n_ridges;
   for (int k = 0; k < d.n_ridges && k < 3; ++k) {
     const double nx = -std::sin(d.ridge_alpha[k]), ny = std::cos(d.ridge_alpha[k]);

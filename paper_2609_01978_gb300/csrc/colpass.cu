@@ -18,7 +18,7 @@
 namespace fzp {
 namespace {
 
-constexpr int TN = 64, TM = 64, TJ = 16;
+constexpr int TN = 64, TM = 64, TJ = 16, PJ = 128;
 
 struct ColArgs {
   int64_t c, j0, rows, c1_stride;
@@ -26,7 +26,7 @@ struct ColArgs {
   int kind;       // RowKind: the row's kernel K(dj), K(dj) + K(-dj) or K(-dj)
   int slices;       // images of C1 to be summed, slice_off values apart
   int64_t slice_off;
-  int64_t sin_off;  // > 0: C1 holds the rows of T cos(phi) and, sin_off values on, of T sin(phi)
+  int64_t sin_off;  // > 0: C1 holds the rows of Re T and, sin_off values on, of Im T
   int M;          // outputs per row (m)
   double kappa, delta;
   double msh;     // ROI (or node) shift in pitches: y_n = (n - msh) p
@@ -67,7 +67,9 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
   using C = typename Cplx<R>::T;
   __shared__ C sK[TJ][TN + 1];
   __shared__ C sC[TJ][TM + 1];
-  __shared__ RowPhase<R> sP[2][TJ];  // of dj (mirrored rows: -dj) and, folded, of -dj
+  // phases of 128 rows at a time (they are FP64, at two operations per clock and
+  // SM): of dj (mirrored rows: -dj) and, folded, of -dj
+  __shared__ RowPhase<R> sP[2][PJ];
   const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
   const int64_t jb = (int64_t)blockIdx.z * g.jc;
   const int64_t je = jb + g.jc < g.rows ? jb + g.jc : g.rows;
@@ -79,11 +81,15 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
 #pragma unroll
     for (int b = 0; b < 4; ++b) { acc[a][b].x = 0; acc[a][b].y = 0; }
   for (int64_t j = jb; j < je; j += TJ) {
-    if (tid < 2 * TJ) {
-      const double dj = (double)(g.j0 + j + (tid & (TJ - 1)) - g.c);
-      RowPhase<R> rp;
-      row_phase(g, (tid >= TJ) != (g.kind == ROWS_MIRRORED) ? -dj : dj, rp);
-      sP[tid / TJ][tid & (TJ - 1)] = rp;
+    const int pj = (int)(j - jb) & (PJ - 1);
+    if (pj == 0) {
+      const int r = tid & (PJ - 1);
+      if (j + r < je && (tid < PJ || g.kind == ROWS_FOLDED)) {
+        const double dj = (double)(g.j0 + j + r - g.c);
+        RowPhase<R> rp;
+        row_phase(g, (tid >= PJ) != (g.kind == ROWS_MIRRORED) ? -dj : dj, rp);
+        sP[tid / PJ][r] = rp;
+      }
     }
     // C tile: TJ rows x TM columns (j contiguous in C1)
     for (int t = tid; t < TJ * TM; t += 256) {
@@ -97,7 +103,7 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
           const R* S = C1 + sl * g.slice_off;
           v.x += S[re];
           v.y += S[im];
-          if (g.sin_off > 0) {  // K (T cos + i T sin)
+          if (g.sin_off > 0) {  // K (Re T + i Im T)
             v.x -= S[g.sin_off + im];
             v.y += S[g.sin_off + re];
           }
@@ -111,8 +117,8 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
       C k;
       k.x = 0; k.y = 0;
       if (j + jj < je) {
-        k = kern(sP[0][jj], n0 + nn);
-        if (g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c) k = cadd(k, kern(sP[1][jj], n0 + nn));
+        k = kern(sP[0][pj + jj], n0 + nn);
+        if (g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c) k = cadd(k, kern(sP[1][pj + jj], n0 + nn));
       }
       sK[jj][nn] = k;
     }
@@ -139,9 +145,14 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int n = n0 + tn + 16 * a, m = m0 + tm + 16 * b;
-      const double ux = (double)acc[a][b].x, uy = (double)acc[a][b].y;
-      atomicAdd(&Uacc[(int64_t)n * g.M + m].x, g.wr * ux - g.wi * uy);
-      atomicAdd(&Uacc[(int64_t)n * g.M + m].y, g.wr * uy + g.wi * ux);
+      double ux = (double)acc[a][b].x, uy = (double)acc[a][b].y;
+      if (g.wi != 0.0 || g.wr != 1.0) {
+        const double t = g.wr * ux - g.wi * uy;
+        uy = g.wr * uy + g.wi * ux;
+        ux = t;
+      }
+      atomicAdd(&Uacc[(int64_t)n * g.M + m].x, ux);
+      atomicAdd(&Uacc[(int64_t)n * g.M + m].y, uy);
     }
 }
 
@@ -191,7 +202,7 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   }
   g.slices = P.nd.slices;
   g.slice_off = P.nd.slice_elems;
-  if (nodes && P.has_deform && P.form == FZP_FORM_DENSE) g.sin_off = 128 * P.c1_stride;
+  if (nodes_two_masks(P)) g.sin_off = 128 * P.c1_stride;
   // rows per block: 2048, fewer where that leaves the GPU idle (few output tiles)
   const int ny = nodes && P.nd.yfull ? P.nd.n : g.M;
   const int64_t tiles = (int64_t)(g.M / TM) * (ny / TN);

@@ -106,6 +106,7 @@ struct DeformCoef {
   // the wrinkle phasor turns by e^{2 pi i kx}; a ridge's ratio g(di+1)/g(di)
   // is multiplied by rho_k = exp(-2 q_k nx_k^2)
   float zc, zs, rho[3];
+  float z4;  // 4 sin^2(pi kx): the wrinkle's second difference per column
 };
 
 // --------------------------------------------------------------------------
@@ -335,6 +336,7 @@ fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t
 fzp_status finish_field(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t stream);
 // Form (b) on nodes (nodes.cu).
 void nodes_choose(Plan& P);
+bool nodes_two_masks(const Plan& P);  // both real masks of a complex transmission in one row pass
 fzp_status nodes_layout(Plan& P, FormSizes* out);
 fzp_status nodes_upload(Plan& P);
 fzp_status nodes_fill(Plan& P, cudaStream_t s);

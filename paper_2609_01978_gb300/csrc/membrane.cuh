@@ -41,75 +41,82 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b - bh), "f"(a - ah));
 }
 
-// Both masks of a membrane, T cos(phi) and T sin(phi), on the 8-column parts
-// [q0, q0 + nq) of a 32-column block: the walk above, one sine and one cosine
-// per sample, each split into its hi and lo plane; NR ridges.
+// Both masks of a membrane, T cos(phi) and T sin(phi), on the 16 columns from
+// di0 (bit k of `bits`: column k open), as 16-byte parts q0 and q0 + 1 of the
+// planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart).  The walk's
+// steps, per column: the scaled wrinkle amp sin by its second difference,
+// s' = s + e, e' = e - 4 sin^2(pi kx) s (one product instead of a rotation's
+// four, and no growth of the rounding at the small angles of a wrinkle), the
+// taper by its constant second difference, a ridge by its ratio; each starts
+// exactly every 16 columns.  NR ridges.
 template <int NR>
-__device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r, int64_t di0, uint32_t bits,
-                                            uint8_t* ch, uint8_t* cl, uint8_t* sh, uint8_t* sl, int sw, int q0,
-                                            int nq) {
+__device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits,
+                                            uint8_t* base, uint32_t plane, int sw, int q0) {
   constexpr float TWO_PI = 6.28318530717958648f;
-  float fi = (float)(di0 + 8 * q0);
+  const float fi = (float)di0;
   const float th = fmaf(fi, d.kxh, r.fjkh);
   float tt = (th - rintf(th)) + fmaf(fi, d.kxl, r.fjkl);
   tt -= rintf(tt);
   float ws, wc;
   __sincosf(TWO_PI * tt, &ws, &wc);
+  float s = d.amp2 * ws, e = d.amp2 * fmaf(0.5f * d.z4, ws, d.zs * wc);  // s, and s minus its left neighbour
+  float tap = fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f), dt = -d.tq * fmaf(2.0f, fi, 1.0f);
+  const float ddt = -2.0f * d.tq;
   float g[NR > 0 ? NR : 1], rr[NR > 0 ? NR : 1];
 #pragma unroll
-  for (int e = 0; e < NR; ++e) {
-    g[e] = 0.0f;
-    rr[e] = 1.0f;
-    const float d0 = fmaf(fi, d.nx[e], r.cr[e]);
-    const float ex = d.q[e] * d0 * d0;
+  for (int k = 0; k < NR; ++k) {
+    g[k] = 0.0f;
+    rr[k] = 1.0f;
+    const float d0 = fmaf(fi, d.nx[k], r.cr[k]);
+    const float ex = d.q[k] * d0 * d0;
     if (ex < 69.0f) {
-      g[e] = __expf(-ex);
-      rr[e] = __expf(-d.q[e] * d.nx[e] * fmaf(2.0f, d0, d.nx[e]));
+      g[k] = d.h2[k] * __expf(-ex);
+      rr[k] = __expf(-d.q[k] * d.nx[k] * fmaf(2.0f, d0, d.nx[k]));
     }
   }
 #pragma unroll 1
-  for (int q = q0; q < q0 + nq; ++q) {
+  for (int q = q0; q < q0 + 2; ++q, bits >>= 8) {
     uint32_t hc[4], lc[4], hs[4], ls[4];
 #pragma unroll
     for (int k = 0; k < 8; k += 2) {
       float vc[2], vs[2];
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        float wz = d.amp2 * ws * fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f);
+        float wz = s * tap;
+        e = fmaf(-d.z4, s, e);
+        s += e;
+        tap += dt;
+        dt += ddt;
 #pragma unroll
-        for (int e = 0; e < NR; ++e) {
-          wz = fmaf(d.h2[e], g[e], wz);
-          g[e] *= rr[e];
-          rr[e] *= d.rho[e];
+        for (int v = 0; v < NR; ++v) {
+          wz += g[v];
+          g[v] *= rr[v];
+          rr[v] *= d.rho[v];
         }
-        const float nws = fmaf(ws, d.zc, wc * d.zs);
-        wc = fmaf(wc, d.zc, -ws * d.zs);
-        ws = nws;
-        fi += 1.0f;
         wz -= rintf(wz);
         const float x = TWO_PI * wz;
-        const bool open = ((bits >> (8 * q + k + z)) & 1u) != 0;
-        vc[z] = open ? __cosf(x) : 0.0f;
-        vs[z] = open ? __sinf(x) : 0.0f;
+        const uint32_t open = (uint32_t)((int32_t)(bits << (31 - (k + z))) >> 31);
+        vc[z] = __uint_as_float(__float_as_uint(__cosf(x)) & open);
+        vs[z] = __uint_as_float(__float_as_uint(__sinf(x)) & open);
       }
       split2(vc[0], vc[1], hc[k / 2], lc[k / 2]);
       split2(vs[0], vs[1], hs[k / 2], ls[k / 2]);
     }
-    const int o = (q ^ sw) << 4;
-    *reinterpret_cast<uint4*>(ch + o) = make_uint4(hc[0], hc[1], hc[2], hc[3]);
-    *reinterpret_cast<uint4*>(cl + o) = make_uint4(lc[0], lc[1], lc[2], lc[3]);
-    *reinterpret_cast<uint4*>(sh + o) = make_uint4(hs[0], hs[1], hs[2], hs[3]);
-    *reinterpret_cast<uint4*>(sl + o) = make_uint4(ls[0], ls[1], ls[2], ls[3]);
+    uint8_t* o = base + ((q ^ sw) << 4);
+    *reinterpret_cast<uint4*>(o) = make_uint4(hc[0], hc[1], hc[2], hc[3]);
+    *reinterpret_cast<uint4*>(o + plane) = make_uint4(lc[0], lc[1], lc[2], lc[3]);
+    *reinterpret_cast<uint4*>(o + 2 * plane) = make_uint4(hs[0], hs[1], hs[2], hs[3]);
+    *reinterpret_cast<uint4*>(o + 3 * plane) = make_uint4(ls[0], ls[1], ls[2], ls[3]);
   }
 }
 
-__device__ __forceinline__ void cx_store2(const DeformCoef& d, const CxRow& r, int64_t di0, uint32_t bits, uint8_t* ch,
-                                          uint8_t* cl, uint8_t* sh, uint8_t* sl, int sw, int q0, int nq) {
+__device__ __forceinline__ void cx_store2(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits, uint8_t* base,
+                                          uint32_t plane, int sw, int q0) {
   switch (d.n) {
-    case 0: cx_store2_n<0>(d, r, di0, bits, ch, cl, sh, sl, sw, q0, nq); break;
-    case 1: cx_store2_n<1>(d, r, di0, bits, ch, cl, sh, sl, sw, q0, nq); break;
-    case 2: cx_store2_n<2>(d, r, di0, bits, ch, cl, sh, sl, sw, q0, nq); break;
-    default: cx_store2_n<3>(d, r, di0, bits, ch, cl, sh, sl, sw, q0, nq); break;
+    case 0: cx_store2_n<0>(d, r, di0, bits, base, plane, sw, q0); break;
+    case 1: cx_store2_n<1>(d, r, di0, bits, base, plane, sw, q0); break;
+    case 2: cx_store2_n<2>(d, r, di0, bits, base, plane, sw, q0); break;
+    default: cx_store2_n<3>(d, r, di0, bits, base, plane, sw, q0); break;
   }
 }
 

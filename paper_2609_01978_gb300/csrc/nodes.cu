@@ -35,6 +35,7 @@
 //             the masks of BN rows, generated into shared memory
 //   flat, NT = 1: 512 rows, two 128 x 256 accumulators (row halves) share A
 //   flat, NT = 2: 256 rows, two accumulators (node tiles)
+//   four levels : 256 rows, accumulators Re T and Im T, a plane each
 //   membrane    : 256 rows, accumulators T cos and T sin, hi and lo planes
 //   warps 0-7 epilogue, 8 loader, 9 MMA issuer, 10-25 mask generators
 // The mask rule in the generators: the zone index of a sample is the integer
@@ -72,7 +73,7 @@ constexpr int EPI_BOX = 32;
 constexpr int EPI_BYTES = EPI_WARPS * EPI_BOX * EPI_BOX * 4;
 constexpr int ERR_BASE = 300;
 
-enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3 };
+enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4 };
 
 // Fixed-point zone phase: phase64(s) = s K mod 2^64 (K = floor(kappa 2^63): the
 // zone's parity is the top bit; MASK_LEVELS: K = floor(kappa_L / L 2^64), the
@@ -102,15 +103,18 @@ struct NodeArgs {
   int* err;
 };
 
-template <int NT, bool CX>
+template <int NT, int MASK>
 struct Shape {
-  static constexpr int BN = (NT == 1 && !CX) ? 512 : 256;         // rows per unit
-  static constexpr int PLANES = CX ? 4 : BN / 256;                // mask planes per stage
+  static constexpr bool CX = MASK == MASK_MEMBRANE;
+  static constexpr bool TWO = CX || MASK == MASK_QUAD;            // two masks: one accumulator each
+  static constexpr int BN = (NT == 1 && !TWO) ? 512 : 256;        // rows per unit
+  static constexpr int PLANES = CX ? 4 : TWO ? 2 : BN / 256;      // mask planes per stage
   static constexpr int A_BYTES = NT * 2 * SUB;
   static constexpr int B_BYTES = PLANES * PLANE;
-  static constexpr int STAGES = CX ? 2 : (NT == 1 ? 4 : 4);
+  static constexpr int STAGES = CX ? 2 : 4;
+  static constexpr int C1_ROWS = NT * 128 * (TWO ? 2 : 1);
   static constexpr int SMEM = 1024 + STAGES * (A_BYTES + B_BYTES) + EPI_BYTES + 256;
-  static_assert(!CX || NT == 1, "two node tiles of a membrane pass need more tensor memory than there is");
+  static_assert(!TWO || NT == 1, "two node tiles of two masks need more tensor memory than there is");
 };
 
 __device__ __forceinline__ uint64_t sdesc(const void* p) {
@@ -314,39 +318,56 @@ __device__ __noinline__ void exact_bits(int64_t di0, int64_t dj2, const MaskGeom
   }
 }
 
+// The same for four levels: bits of the level's parity and of its upper half.
+__device__ __noinline__ void exact_quad(int64_t di0, int64_t dj2, const MaskGeom& g, uint32_t& odd, uint32_t& high) {
+  odd = high = 0u;
+  for (int k = 0; k < 32; ++k) {
+    const int64_t d = di0 + k, s = dj2 + d * d;
+    const uint32_t z = (uint32_t)zone_of(s < g.sR ? s : g.sR, g);
+    odd |= (z & 1u) << k;
+    high |= ((z >> 1) & 1u) << k;
+  }
+}
+
 // A row's walk over its blocks: the exact 64-bit phase at the block's first
 // column and its first difference.
 struct RowWalk {
   uint64_t phase, step;  // s K and (2 di + 1) K mod 2^64
-  int64_t di0, dj2, bmax;
+  int32_t di0, dj, bmax;  // |di|, |dj| < 2^24
 };
 
 __device__ __forceinline__ void row_start(RowWalk& w, int64_t dj, int64_t di0, bool live, const MaskGeom& g,
                                           const PhaseRule& r) {
-  w.dj2 = dj * dj;
-  w.di0 = di0;
-  const int64_t t = g.sR - w.dj2;
-  w.bmax = (live && t >= 0) ? isqrt_floor(t) : -1;
-  w.phase = (uint64_t)(w.dj2 + di0 * di0) * r.K + (r.open_even ? (1ull << 63) : 0ull);
+  const int64_t t = g.sR - dj * dj;
+  w.dj = (int32_t)dj;
+  w.di0 = (int32_t)di0;
+  w.bmax = (live && t >= 0) ? (int32_t)isqrt_floor(t) : -1;
+  w.phase = (uint64_t)(dj * dj + di0 * di0) * r.K + (r.open_even ? (1ull << 63) : 0ull);
   w.step = (uint64_t)(2 * di0 + 1) * r.K;
 }
 
-// On to the next 32 columns.
+// On by `n` columns: K ((d + n)^2 - d^2) = n (2 d + 1) K + n (n - 1) K.
+template <int n>
 __device__ __forceinline__ void row_next(RowWalk& w, const PhaseRule& r) {
-  w.phase += 32ull * w.step + 992ull * r.K;  // K ((d + 32)^2 - d^2) = 32 (2 d + 1) K + 992 K
-  w.step += 64ull * r.K;
-  w.di0 += 32;
+  w.phase += (uint64_t)n * w.step + (uint64_t)(n * (n - 1)) * r.K;
+  w.step += (uint64_t)(2 * n) * r.K;
+  w.di0 += n;
+}
+
+// The block's columns inside the disc chord, for a walk from the axis on.
+__device__ __forceinline__ uint32_t chord_up(const RowWalk& w) {
+  const int n = w.bmax + 1 - w.di0;
+  return n >= 32 ? 0xFFFFFFFFu : n <= 0 ? 0u : (1u << n) - 1u;
 }
 
 // The block's mask as 16 words of two BF16 values; `one` = +-1 (or +-1/2) in
 // both halves.  Whole warp (the votes), every lane a row.
 template <int MASK>
 __device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
-                                            uint32_t (&wd)[16]) {
+                                            uint32_t chord, uint32_t (&wd)[16]) {
   const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);  // upper 32 bits of 2 K
   uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
   uint32_t near = 0xFFFFFFFFu;
-  const uint32_t chord = chord_bits(w.di0, w.bmax);
   if (MASK == MASK_LEVELS) {
     const uint32_t el = r.E * (uint32_t)r.lmod;
 #pragma unroll
@@ -381,7 +402,7 @@ __device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g,
   if (__any_sync(0xffffffffu, near != 0u && chord != 0u)) {
     if (near && chord) {
       uint32_t pb, nb;
-      exact_bits<MASK>(w.di0, w.dj2, g, r, pb, nb);
+      exact_bits<MASK>(w.di0, (int64_t)w.dj * w.dj, g, r, pb, nb);
 #pragma unroll
       for (int q = 0; q < 16; ++q) wd[q] = (pair_mask(pb | nb, q) & one) | (pair_mask(nb, q) & 0x80008000u);
     }
@@ -392,22 +413,66 @@ __device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g,
   }
 }
 
-// The block's open bits (parity rule, chord applied), for the membrane pass.
-__device__ __forceinline__ uint32_t block_open(const RowWalk& w, const MaskGeom& g, const PhaseRule& r) {
+// Four levels (T = e^{-2 pi i q / 4} = 1, -i, -1, i, q the phase's top two bits):
+// the block's Re T and Im T, 16 words each.
+__device__ __forceinline__ void block_quad(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
+                                           uint32_t chord, uint32_t (&re)[16], uint32_t (&im)[16]) {
+  const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);  // upper 32 bits of 2 K
+  uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
+  uint32_t near = 0xFFFFFFFFu;
+  const uint32_t e4 = 4u * r.E;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const uint32_t fa = f, fb = f + d;
+    f = fb + d + c2;
+    d += 2u * c2;
+    near = min(near, min((fa << 2) + e4, (fb << 2) + e4));
+    const uint32_t s = prmt(fa, fb, 0xFFBBu) & 0x80008000u;      // q >= 2
+    const uint32_t t = prmt(fa << 1, fb << 1, 0xFFBBu);          // q odd
+    re[q] = ~t & (one | s);
+    im[q] = t & (one | (s ^ 0x80008000u));
+  }
+  const bool redo = near < 2u * e4 && chord != 0u;
+  if (__any_sync(0xffffffffu, redo)) {
+    if (redo) {
+      uint32_t odd = 0u, high = 0u;
+      exact_quad(w.di0, (int64_t)w.dj * w.dj, g, odd, high);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const uint32_t t = pair_mask(odd, q), s = pair_mask(high, q) & 0x80008000u;
+        re[q] = ~t & (one | s);
+        im[q] = t & (one | (s ^ 0x80008000u));
+      }
+    }
+  }
+  if (__any_sync(0xffffffffu, chord != 0xFFFFFFFFu)) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const uint32_t m = pair_mask(chord, q);
+      re[q] &= m;
+      im[q] &= m;
+    }
+  }
+}
+
+// Open bits of the 16 columns from the walk's (parity rule, chord applied), for
+// the membrane pass.
+__device__ __forceinline__ uint32_t open16(const RowWalk& w, const MaskGeom& g, const PhaseRule& r) {
   const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);
   uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
   uint32_t near = 0xFFFFFFFFu, bits = 0u;
-  const uint32_t chord = chord_bits(w.di0, w.bmax), e2 = 2u * r.E;
+  const uint32_t chord = chord_bits(w.di0, w.bmax) & 0xFFFFu, e2 = 2u * r.E;
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
+  for (int k = 0; k < 16; ++k) {
     near = min(near, (f << 1) + e2);
-    bits |= (f >> 31) << k;
+    bits = __funnelshift_l(f, bits, 1);  // the sign shifts in: column k at bit 15 - k
     f += d;
     d += c2;
   }
+  bits = __brev(bits) >> 16;
   if (near < 2u * e2 && chord != 0u) {
     uint32_t nb;
-    exact_bits<MASK_PARITY>(w.di0, w.dj2, g, r, bits, nb);
+    exact_bits<MASK_PARITY>(w.di0, (int64_t)w.dj * w.dj, g, r, bits, nb);
   }
   return bits & chord;
 }
@@ -415,8 +480,8 @@ __device__ __forceinline__ uint32_t block_open(const RowWalk& w, const MaskGeom&
 // ------------------------------------------------------------------ kernel
 template <int NT, int MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, const __grid_constant__ CUtensorMap tmC1) {
-  constexpr bool CX = MASK == MASK_MEMBRANE;
-  using S = Shape<NT, CX>;
+  using S = Shape<NT, MASK>;
+  constexpr bool CX = S::CX, TWO = S::TWO;
   constexpr int NST = S::STAGES, BN = S::BN;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -438,7 +503,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(&fullA[s], 1);
-      mbar_init(&fullB[s], GEN_WARPS);
+      mbar_init(&fullB[s], CX ? GEN_WARPS : GEN_WARPS / 2);
       mbar_init(&empty[s], 1);
     }
     mbar_init(accFull, 1);
@@ -515,7 +580,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
 #pragma unroll
               for (int q = 0; q < 2; ++q) {
                 // flat: accumulator q = row half q (NT = 1) or node tile q (NT = 2);
-                // membrane: q = 0 T cos, 1 T sin, planes 2q (hi) and 2q + 1 (lo)
+                // two masks: q = 0, 1; membrane planes 2q (hi) and 2q + 1 (lo)
                 const uint32_t dt = tmem + (uint32_t)(q * 256);
                 const int at = NT == 2 ? q : 0;
                 const int bp = CX ? 2 * q : (NT == 2 ? 0 : q);
@@ -542,57 +607,93 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
       }
     }
   } else if (warp >= GEN_WARP0) {
-    // ---------------- mask generators: a lane per row.  Flat, 512 rows: warp
-    // gw takes rows 32 gw .. + 31; 256 rows: warps gw and gw + 8 take the same
-    // rows' even and odd blocks of a unit (flat) or 16-column halves (membrane)
-    const int gw = warp - GEN_WARP0;
-    const int row = (BN == 512 ? gw : gw & 7) * 32 + lane;  // row of the stripe
-    const int half = BN == 512 ? 0 : gw >> 3;
+    // ---------------- mask generators.  Membrane: warps gw and gw + 8 take the
+    // same 32 rows' 16-column halves of every block.  Otherwise two groups of
+    // eight warps take every other block of the CTA's sequence (with an even
+    // number of stages a stage has one group), a lane per row, or per two rows
+    // 256 apart where the unit has 512
+    static_assert(CX || NST % 2 == 0, "a stage must keep its generator group");
+    const int gw = warp - GEN_WARP0, grp = gw >> 3;
+    const int row = (gw & 7) * 32 + lane;  // row of the stripe (and row + 256)
     // 64-byte swizzle: row at (row / 8) 512 + (row % 8) 64, 16-byte part q at q ^ ((row % 8) / 2)
-    uint8_t* rowbase = sB + (row >> 8) * PLANE + ((row & 255) >> 3) * 512 + (row & 7) * 64;
+    uint8_t* rowbase = sB + (row >> 3) * 512 + (row & 7) * 64;
     const int sw = (row & 7) >> 1;
-    int stage = 0;
-    uint32_t phase = 0;
     bool ok = true;
-    for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
-      const Unit un = unit_at<BN>(a, it);
-      const int64_t j = un.jb + row;
-      RowWalk w;
-      row_start(w, j - a.mg.c, un.kb0 * BK - a.mg.c, j < un.je, a.mg, a.ph);
-      const int64_t diag = a.octant ? un.jb / BK : INT64_MAX;  // blocks of the diagonal tile: half weight
-      if constexpr (CX) {
+    if constexpr (CX) {
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+        const Unit un = unit_at<BN>(a, it);
+        const int64_t j = un.jb + row;
+        RowWalk w;
+        row_start(w, j - a.mg.c, un.kb0 * BK - a.mg.c + 16 * grp, j < un.je, a.mg, a.ph);
         CxRow cxr;
         cx_row_init(a.df, j - a.mg.c, cxr);
-        for (int64_t kb = un.kb0; kb < un.kb1; ++kb) {
-          const uint32_t bits = block_open(w, a.mg, a.ph);
+        for (int kb = (int)un.kb0; kb < (int)un.kb1; ++kb) {
+          const uint32_t bits = open16(w, a.mg, a.ph);
           if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
           uint8_t* rp = rowbase + stage * S::B_BYTES;
-          cx_store2(a.df, cxr, w.di0, bits, rp, rp + PLANE, rp + 2 * PLANE, rp + 3 * PLANE, sw, 2 * half, 2);
-          row_next(w, a.ph);
+          cx_store2(a.df, cxr, w.di0, bits, rp, PLANE, sw, 2 * grp);
+          row_next<BK>(w, a.ph);
           fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive(&fullB[stage]);
           if (++stage == NST) { stage = 0; phase ^= 1; }
         }
-      } else {
-        for (int64_t kb = un.kb0; kb < un.kb1; ++kb) {
-          const bool mine = BN == 512 || ((kb ^ half) & 1) == 0;
-          uint32_t wd[16];
-          if (mine) block_words<MASK>(w, a.mg, a.ph, kb >= diag ? 0x3F003F00u : 0x3F803F80u, wd);
-          row_next(w, a.ph);
-          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
-          if (mine) {
-            uint8_t* rp = rowbase + stage * S::B_BYTES;
+      }
+    } else {
+      constexpr int RPL = BN / 256;  // rows per lane
+      int stage = grp;
+      uint32_t phase = 0;
+      int skip = grp;  // blocks before this group's next one
+      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
+        const Unit un = unit_at<BN>(a, it);
+        const int nkb = (int)(un.kb1 - un.kb0);
+        RowWalk w[RPL];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+        for (int h = 0; h < RPL; ++h) {
+          const int64_t j = un.jb + row + 256 * h;
+          row_start(w[h], j, (un.kb0 + skip) * BK, j < un.je, a.mg, a.ph);
+        }
+        // blocks of the diagonal tile: half weight
+        const int diag = a.octant ? (int)(un.jb / BK - un.kb0) : nkb;
+        int b = skip;
+        for (; b < nkb; b += 2) {
+          const uint32_t one = b >= diag ? 0x3F003F00u : 0x3F803F80u;
+          uint8_t* rp = rowbase + stage * S::B_BYTES;
+          if constexpr (MASK == MASK_QUAD) {
+            uint32_t re[16], im[16];
+            block_quad(w[0], a.mg, a.ph, one, chord_up(w[0]), re, im);
+            if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
               *reinterpret_cast<uint4*>(rp + ((q ^ sw) << 4)) =
-                  make_uint4(wd[4 * q], wd[4 * q + 1], wd[4 * q + 2], wd[4 * q + 3]);
-            fence_proxy_async();
+                  make_uint4(re[4 * q], re[4 * q + 1], re[4 * q + 2], re[4 * q + 3]);
+              *reinterpret_cast<uint4*>(rp + PLANE + ((q ^ sw) << 4)) =
+                  make_uint4(im[4 * q], im[4 * q + 1], im[4 * q + 2], im[4 * q + 3]);
+            }
+          } else {
+#pragma unroll
+            for (int h = 0; h < RPL; ++h) {
+              uint32_t wd[16];
+              block_words<MASK>(w[h], a.mg, a.ph, one, chord_up(w[h]), wd);
+              if (h == 0 && !warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<uint4*>(rp + h * PLANE + ((q ^ sw) << 4)) =
+                    make_uint4(wd[4 * q], wd[4 * q + 1], wd[4 * q + 2], wd[4 * q + 3]);
+            }
+            if (!ok) break;
           }
+#pragma unroll
+          for (int h = 0; h < RPL; ++h) row_next<2 * BK>(w[h], a.ph);
+          fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive(&fullB[stage]);
-          if (++stage == NST) { stage = 0; phase ^= 1; }
+          stage += 2;
+          if (stage >= NST) { stage -= NST; phase ^= 1; }
         }
+        skip = b - nkb;
       }
     }
   } else {
@@ -605,8 +706,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
     bool ok = true;
     for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
       const Unit un = unit_at<BN>(a, it);
-      const int x0 = (int)(un.jb - a.j_begin) + ((NT == 1 && !CX) ? q * 256 : 0);
-      const int y0 = un.slice * (NT * 128 * (CX ? 2 : 1)) + ((NT == 2 || CX) ? q * 128 : 0) + (warp & 3) * 32;
+      const int x0 = (int)(un.jb - a.j_begin) + (BN == 512 ? q * 256 : 0);
+      const int y0 = un.slice * S::C1_ROWS + (BN == 512 ? 0 : q * 128) + (warp & 3) * 32;
       const int xn = (int)min((int64_t)256, un.je - a.j_begin - x0);  // live columns (may be <= 0)
       for (int64_t p0 = un.kb0; p0 < un.kb1; p0 += a.promote) {
         if (threadIdx.x == 0) epi_ok[accph] = mbar_wait(accFull, accph, abort_flag, a.err, ERR_BASE + 6) ? 1 : 0;
@@ -696,20 +797,73 @@ __global__ void k_nodes_A(int nt, int64_t ncols, int64_t kblocks, int64_t c, int
 }
 
 // ------------------------------------------------------------------ interpolation
-// X[o, l] = sum_k Wy[o, k] (V[k, l] (+ V[l, k])), k over the ny nodes of the rows'
-// axis: one thread per (o, l).
-__global__ void k_interp_rows(int ny, int ns, int Mo, int sym, const double* __restrict__ Wy,
-                              const double2* __restrict__ V, double2* __restrict__ X) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y * blockDim.y + threadIdx.y;
-  if (l >= ns || o >= Mo) return;
-  double2 x = make_double2(0.0, 0.0);
-  for (int k = 0; k < ny; ++k) {
-    double2 v = V[k * ns + l];
-    if (sym) {
-      const double2 u = V[l * ns + k];
-      v.x += u.x;
-      v.y += u.y;
+// FP64 runs at two multiply-adds per clock and SM here, so the outputs are cut
+// into small blocks over the whole GPU and the chirp is applied per axis.
+__device__ __forceinline__ double sinc_d(double z) { return fabs(z) < 1e-9 ? 1.0 : sin(z) / z; }
+
+// W from the Cholesky factors of the node matrix (host): a block per four
+// outputs, a thread per (output, node), both triangular solves with the
+// unknowns in registers.  F: per parity the factor by columns, then by rows
+// (ns x ns each), reciprocals on the diagonal.
+struct InterpSpec {
+  int n, ns, M, Mo, even;
+  double h, c, half;  // node pitch and band (radians) per ROI half width; half width in pitches
+};
+
+__global__ void __launch_bounds__(512) k_interp_W(const InterpSpec a, const double* __restrict__ F, double* __restrict__ W,
+                                                  double* __restrict__ Wy) {
+  __shared__ double pivot[2][4];
+  const int ns = a.ns, r = threadIdx.x % ns, q = threadIdx.x / ns, o = blockIdx.x * 4 + q;
+  const double xo = (a.even ? (double)o : (double)o - 0.5 * (a.M - 1)) / a.half;
+  const double x = ((double)(a.even ? r + ns : r) - 0.5 * (a.n - 1)) * a.h;
+  const double sm = sinc_d(a.c * (xo - x)), sp = a.even ? sinc_d(a.c * (xo + x)) : 0.0;
+  double w[2] = {0.0, 0.0};
+  for (int side = 0; side < (a.even && Wy ? 2 : 1); ++side) {
+    const double* C = F + (size_t)side * 2 * ns * ns;  // by columns, behind it by rows
+    const double* R = C + (size_t)ns * ns;
+    const double inv = C[r * ns + r];
+    double v = side ? sm - sp : sm + sp;
+    for (int k = 0; k < ns; ++k) {
+      if (r == k) pivot[k & 1][q] = v = v * inv;
+      __syncthreads();
+      if (r > k) v = fma(-C[k * ns + r], pivot[k & 1][q], v);
     }
+    __syncthreads();
+    for (int k = ns - 1; k >= 0; --k) {
+      if (r == k) pivot[k & 1][q] = v = v * inv;
+      __syncthreads();
+      if (r < k) v = fma(-R[k * ns + r], pivot[k & 1][q], v);
+    }
+    __syncthreads();
+    w[side] = v;
+  }
+  if (o >= a.Mo) return;
+  W[(size_t)r * a.Mo + o] = w[0];
+  if (a.even && Wy) {
+    // the matrix of all nodes: w(+-x_k) = (even +- odd) / 2, at x_o and mirrored at -x_o
+    const int hm = a.M / 2, kp = ns + r, km = ns - 1 - r;
+    const double same = 0.5 * (w[0] + w[1]), other = 0.5 * (w[0] - w[1]);
+    if (o < hm) {
+      Wy[(size_t)kp * a.M + hm + o] = same;
+      Wy[(size_t)km * a.M + hm + o] = other;
+    }
+    if (o > 0) {
+      Wy[(size_t)kp * a.M + hm - o] = other;
+      Wy[(size_t)km * a.M + hm - o] = same;
+    }
+  }
+}
+
+// X[l][o] = sum_k Wy[k][o] V[k][l], k over the ny nodes of the rows' axis: a
+// block per 4 outputs and 32 nodes.
+__global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, const double* __restrict__ Wy,
+                                                     const double2* __restrict__ V, double2* __restrict__ X) {
+  const int l = blockIdx.x * 32 + (threadIdx.x & 31), o = blockIdx.y * 4 + (threadIdx.x >> 5);
+  if (o >= Mo) return;
+  double2 x = make_double2(0.0, 0.0);
+#pragma unroll 8
+  for (int k = 0; k < ny; ++k) {
+    const double2 v = V[k * ns + l];
     const double w = Wy[k * Mo + o];
     x.x = fma(w, v.x, x.x);
     x.y = fma(w, v.y, x.y);
@@ -720,80 +874,77 @@ __global__ void k_interp_rows(int ny, int ns, int Mo, int sym, const double* __r
 struct InterpOut {
   int M, ns;
   int Moy, eveny, Mox, evenx;  // outputs of the two axes (even: M / 2 + 1)
+  int sym;                     // the field is this one plus its transpose
   double msh, p, lf, f_over_lambda, amp;
   int accumulate;
 };
 
-// U[on, om] = sum_l X[on, l] W[om, l], the output chirp and prefactor, and the
-// stores: with an even field output o stands for the samples M/2 + o and
-// M/2 - o (o = M/2: sample 0 alone).
-constexpr int IT = 32;  // outputs per block and side
-__global__ void __launch_bounds__(256) k_interp_cols(const InterpOut a, const double* __restrict__ W,
-                                                     const double2* __restrict__ X, double2* __restrict__ out) {
-  __shared__ double2 sX[16][IT];
-  __shared__ double sW[16][IT];
+// U[on, om] = sum_l X[l][on] W[l][om] (sym: plus the same with on and om
+// exchanged; only blocks on and below the diagonal run and both are stored),
+// the output chirp and prefactor, and the stores: with an even field output o
+// stands for the samples M/2 + o and M/2 - o (o = M/2: sample 0 alone).
+// Block: 8 x 8 outputs, one per thread.
+constexpr int IT = 8;
+__global__ void __launch_bounds__(IT * IT) k_interp_cols(const InterpOut a, const double* __restrict__ W,
+                                                         const double2* __restrict__ X, double2* __restrict__ out) {
+  if (a.sym && blockIdx.x > blockIdx.y) return;
+  __shared__ double2 chy[IT], chx[IT];
   const int n0 = blockIdx.y * IT, m0 = blockIdx.x * IT;
-  const int tm = threadIdx.x & 15, tn = threadIdx.x >> 4;  // 2 x 2 outputs each
-  double2 u[2][2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) u[i][j] = make_double2(0.0, 0.0);
-  for (int l0 = 0; l0 < a.ns; l0 += 16) {
-    for (int t = threadIdx.x; t < 16 * IT; t += 256) {
-      const int l = t / IT, o = t % IT;
-      sX[l][o] = n0 + o < a.Moy ? X[(l0 + l) * a.Moy + n0 + o] : make_double2(0.0, 0.0);
-      sW[l][o] = m0 + o < a.Mox ? W[(l0 + l) * a.Mox + m0 + o] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int l = 0; l < 16; ++l) {
-      double2 x[2];
-      double w[2];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) x[i] = sX[l][tn + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) w[j] = sW[l][tm + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          u[i][j].x = fma(w[j], x[i].x, u[i][j].x);
-          u[i][j].y = fma(w[j], x[i].y, u[i][j].y);
-        }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int on = n0 + tn + 16 * i, om = m0 + tm + 16 * j;
-      if (on >= a.Moy || om >= a.Mox) continue;
-      const int h = a.M / 2;
-      const int n = a.eveny ? (h + on) % a.M : on, m = a.evenx ? (h + om) % a.M : om;
-      const double xm = (double)m - a.msh, yn = (double)n - a.msh;
-      const double ph = frac_turns(a.f_over_lambda) - 0.25 + (xm * xm + yn * yn) * (a.p * a.p) / (2.0 * a.lf);
-      double2 w = cis_turns_d(ph);
+  const int tm = threadIdx.x % IT, tn = threadIdx.x / IT;
+  const int h = a.M / 2;
+  if (threadIdx.x < 2 * IT) {  // e^{i pi x^2 / (lambda f)} of the block's outputs, the prefactor with the rows'
+    const bool rowaxis = threadIdx.x < IT;
+    const int o = (rowaxis ? n0 : m0) + threadIdx.x % IT;
+    const int i = (rowaxis ? a.eveny : a.evenx) ? (h + o) % a.M : o;
+    const double x = ((double)i - a.msh) * a.p;
+    double2 w = cis_turns_d(x * x / (2.0 * a.lf) + (rowaxis ? frac_turns(a.f_over_lambda) - 0.25 : 0.0));
+    if (rowaxis) {
       w.x *= a.amp;
       w.y *= a.amp;
-      const double2 v = make_double2(w.x * u[i][j].x - w.y * u[i][j].y, w.x * u[i][j].y + w.y * u[i][j].x);
-      auto put = [&](int nn, int mm) {
-        double2* o = out + (int64_t)nn * a.M + mm;
-        double2 z = v;
-        if (a.accumulate) {
-          z.x += o->x;
-          z.y += o->y;
-        }
-        *o = z;
-      };
-      // samples with a mirror image of their own
-      const bool fn = a.eveny && on > 0 && on < h, fm = a.evenx && om > 0 && om < h;
-      put(n, m);
-      if (fn) put(h - on, m);
-      if (fm) put(n, h - om);
-      if (fn && fm) put(h - on, h - om);
+      chy[threadIdx.x] = w;
+    } else {
+      chx[threadIdx.x - IT] = w;
     }
+  }
+  const int on = n0 + tn, om = m0 + tm;
+  const int cn = min(on, a.Moy - 1), cm = min(om, a.Mox - 1);
+  double2 u = make_double2(0.0, 0.0), t = u;
+#pragma unroll 8
+  for (int l = 0; l < a.ns; ++l) {
+    const double2 x = __ldg(X + l * a.Moy + cn);
+    const double w = __ldg(W + l * a.Mox + cm);
+    u.x = fma(w, x.x, u.x);
+    u.y = fma(w, x.y, u.y);
+    if (a.sym) {
+      const double2 y = __ldg(X + l * a.Moy + cm);
+      const double v = __ldg(W + l * a.Mox + cn);
+      t.x = fma(v, y.x, t.x);
+      t.y = fma(v, y.y, t.y);
+    }
+  }
+  __syncthreads();
+  if (on >= a.Moy || om >= a.Mox || (a.sym && om > on)) return;
+  const double2 v = cmul(cmul(make_double2(u.x + t.x, u.y + t.y), chx[tm]), chy[tn]);
+  const int n = a.eveny ? (h + on) % a.M : on, m = a.evenx ? (h + om) % a.M : om;
+  auto put = [&](int nn, int mm) {
+    double2* o = out + (int64_t)nn * a.M + mm;
+    double2 z = v;
+    if (a.accumulate) {
+      z.x += o->x;
+      z.y += o->y;
+    }
+    *o = z;
+  };
+  // samples with a mirror image of their own
+  const bool fn = a.eveny && on > 0 && on < h, fm = a.evenx && om > 0 && om < h;
+  auto put4 = [&](int nn, int mm, bool f1, bool f2) {
+    put(nn, mm);
+    if (f1) put(a.M - nn, mm);
+    if (f2) put(nn, a.M - mm);
+    if (f1 && f2) put(a.M - nn, a.M - mm);
+  };
+  put4(n, m, fn, fm);
+  if (a.sym && on != om) put4(m, n, fm, fn);
 }
 
 // ------------------------------------------------------------------ mask export
@@ -812,33 +963,43 @@ __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int
 #pragma unroll
       for (int k = 0; k < 32; ++k) v[k] = 0;
       uint32_t wd[16];
-      if (mask == MASK_LEVELS) {
+      if (mask == MASK_QUAD) {
+        uint32_t wi[16];
+        block_quad(w, mg, ph, 0x3F803F80u, disc, wd, wi);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          const uint32_t x = (wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu, y = (wi[k / 2] >> (16 * (k & 1))) & 0xFFFFu;
+          v[k] = (uint8_t)(x ? 1 + (x >> 15) * 2 : y ? 4 - (y >> 15) * 2 : 0);
+        }
+      } else if (mask == MASK_LEVELS) {
         PhaseRule one = ph;
         one.neg = 0;
         for (int q = 0; q < ph.lmod; ++q) {
           one.pos = 1ull << q;
-          block_words<MASK_LEVELS>(w, mg, one, 0x3F803F80u, wd);
+          block_words<MASK_LEVELS>(w, mg, one, 0x3F803F80u, disc, wd);
 #pragma unroll
           for (int k = 0; k < 32; ++k)
             if ((wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu) v[k] = (uint8_t)(1 + q);
         }
       } else if (mask == MASK_SIGNED) {
-        block_words<MASK_SIGNED>(w, mg, ph, 0x3F803F80u, wd);
+        block_words<MASK_SIGNED>(w, mg, ph, 0x3F803F80u, disc, wd);
 #pragma unroll
         for (int k = 0; k < 32; ++k)
           v[k] = ((disc >> k) & 1u) ? (uint8_t)(1 + ((wd[k / 2] >> (16 * (k & 1) + 15)) & 1u)) : 0;
       } else if (mask == MASK_MEMBRANE) {
-        const uint32_t bits = block_open(w, mg, ph);
+        RowWalk w2 = w;
+        row_next<16>(w2, ph);
+        const uint32_t bits = open16(w, mg, ph) | (open16(w2, mg, ph) << 16);
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = (uint8_t)((bits >> k) & 1u);
       } else {
-        block_words<MASK_PARITY>(w, mg, ph, 0x3F803F80u, wd);
+        block_words<MASK_PARITY>(w, mg, ph, 0x3F803F80u, disc, wd);
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = ((wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu) ? 1 : 0;
       }
       if (r < rows)
         for (int k = 0; k < 32 && i0 + k < N; ++k) out[r * N + i0 + k] = v[k];
-      row_next(w, ph);
+      row_next<BK>(w, ph);
     }
   }
 }
@@ -881,86 +1042,55 @@ PhaseRule phase_rule(const Plan& P, const MaskPass* mp) {
 }
 
 int mask_kind(const Plan& P) {
-  return P.has_deform ? MASK_MEMBRANE : P.levels > 2 ? MASK_LEVELS : P.levels == 2 ? MASK_SIGNED : MASK_PARITY;
+  return P.has_deform ? MASK_MEMBRANE : P.levels > 2 ? (P.nd.ns == 64 ? MASK_QUAD : MASK_LEVELS) : P.levels == 2 ? MASK_SIGNED : MASK_PARITY;
 }
 
-// W (transposed: [node][output]) for n nodes x_k = (k - (n - 1)/2) h across +-1
-// and outputs x_o, band half-width `c` (radians per unit): the normal equations
-// of the least-squares problem over the band, S W = s, with a regularisation
-// of 1e-13 (the sinc matrix is singular to working precision), by Cholesky.
-struct Interp {
-  int n, Mo;
-  std::vector<double> dist, minus, plus;  // sinc at the node distances q h; at x_o -+ x_k, k > 0 half (or x_o - x_k, all)
-  bool half;
-
-  Interp(int n_, double h, double c, const std::vector<double>& xo, bool half_) : n(n_), Mo((int)xo.size()), half(half_) {
-    auto sinc = [&](double t) { const double z = c * t; return std::fabs(z) < 1e-9 ? 1.0 : std::sin(z) / z; };
-    const int ns = half ? n / 2 : n;
-    dist.resize(n);
-    for (int q = 0; q < n; ++q) dist[q] = sinc(q * h);
-    minus.resize((size_t)ns * Mo);
-    if (half) plus.resize((size_t)ns * Mo);
-    for (int k = 0; k < ns; ++k) {
-      const double x = ((double)(half ? k + n / 2 : k) - 0.5 * (n - 1)) * h;
-      for (int o = 0; o < Mo; ++o) {
-        minus[(size_t)k * Mo + o] = sinc(xo[o] - x);
-        if (half) plus[(size_t)k * Mo + o] = sinc(xo[o] + x);
-      }
+// Cholesky factor (by columns, then by rows; reciprocals on the diagonal) of the node
+// matrix S(x_k, x_l) + 1e-13 (the sinc matrix is singular to working
+// precision) for nodes x_k = (k - (n - 1)/2) h and the band half-width c
+// (radians): the normal equations of the least-squares interpolation.
+// parity +1 / -1: of even / odd functions, over the nodes x > 0.
+void node_factor(int n, int ns, int parity, double h, double c, double* T) {
+  std::vector<double> dist(n);
+  for (int q = 0; q < n; ++q) {
+    const double z = c * q * h;
+    dist[q] = q ? std::sin(z) / z : 1.0;
+  }
+  for (int l = 0; l < ns; ++l)
+    for (int k = l; k < ns; ++k)  // x_k + x_l = (k + l + 1) h on the half grid
+      T[(size_t)l * ns + k] = dist[k - l] + (parity ? parity * dist[k + l + 1] : 0.0) + (k == l ? 1e-13 : 0.0);
+  for (int l = 0; l < ns; ++l) {
+    double* __restrict__ cl = &T[(size_t)l * ns];
+    const double r = 1.0 / std::sqrt(std::max(cl[l], 1e-15));
+    for (int k = l + 1; k < ns; ++k) cl[k] *= r;
+    for (int q = l + 1; q < ns; ++q) {
+      double* __restrict__ cq = &T[(size_t)q * ns];
+      const double f = cl[q];
+      for (int k = q; k < ns; ++k) cq[k] -= f * cl[k];
     }
+    cl[l] = r;
   }
-
-  // parity 0: all nodes; +1 / -1: of an even / odd function, over the nodes x > 0
-  std::vector<double> solve(int parity) const {
-    const int ns = half ? n / 2 : n;
-    std::vector<double> L((size_t)ns * ns), W = minus;
-    for (int k = 0; k < ns; ++k)
-      for (int l = 0; l <= k; ++l)  // x_k + x_l = (k + l + 1) h on the half grid
-        L[(size_t)k * ns + l] = dist[k - l] + (parity ? parity * dist[k + l + 1] : 0.0) + (k == l ? 1e-13 : 0.0);
-    for (int k = 0; k < ns; ++k)
-      for (int l = 0; l <= k; ++l) {
-        double s = L[(size_t)k * ns + l];
-        for (int q = 0; q < l; ++q) s -= L[(size_t)k * ns + q] * L[(size_t)l * ns + q];
-        L[(size_t)k * ns + l] = k == l ? std::sqrt(std::max(s, 1e-15)) : s / L[(size_t)l * ns + l];
-      }
-    if (parity)
-      for (size_t t = 0; t < W.size(); ++t) W[t] += parity * plus[t];
-    for (int k = 0; k < ns; ++k) {  // L y = s, all outputs at once
-      double* w = &W[(size_t)k * Mo];
-      for (int q = 0; q < k; ++q) axpy(w, &W[(size_t)q * Mo], -L[(size_t)k * ns + q]);
-      scale(w, 1.0 / L[(size_t)k * ns + k]);
-    }
-    for (int k = ns - 1; k >= 0; --k) {  // L^T w = y
-      double* w = &W[(size_t)k * Mo];
-      for (int q = k + 1; q < ns; ++q) axpy(w, &W[(size_t)q * Mo], -L[(size_t)q * ns + k]);
-      scale(w, 1.0 / L[(size_t)k * ns + k]);
-    }
-    return W;
-  }
-  void axpy(double* __restrict__ w, const double* __restrict__ v, double f) const {
-    for (int o = 0; o < Mo; ++o) w[o] += f * v[o];
-  }
-  void scale(double* w, double f) const {
-    for (int o = 0; o < Mo; ++o) w[o] *= f;
-  }
-};
+  double* L = T + (size_t)ns * ns;
+  for (int k = 0; k < ns; ++k)
+    for (int l = 0; l <= k; ++l) L[(size_t)k * ns + l] = T[(size_t)l * ns + k];
+}
 
 template <int NT, int MASK>
 fzp_status smem_attr() {
   static std::atomic<uint64_t> done{0};
-  FZP_CUDA_TRY(smem_attr_once((const void*)k_nodes<NT, MASK>, Shape<NT, MASK == MASK_MEMBRANE>::SMEM, done));
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_nodes<NT, MASK>, Shape<NT, MASK>::SMEM, done));
   return FZP_OK;
 }
 
 template <int NT, int MASK>
 fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
-  using S = Shape<NT, MASK == MASK_MEMBRANE>;
-  constexpr bool CX = MASK == MASK_MEMBRANE;
+  using S = Shape<NT, MASK>;
   fzp_status st = smem_attr<NT, MASK>();
   if (st != FZP_OK) return st;
   const int64_t rows = a.j_end - a.j_begin;
   a.n_stripes = (int)((rows + S::BN - 1) / S::BN);
   P.c1_stride = (rows + 255) / 256 * 256;
-  const int c1r = NT * 128 * (CX ? 2 : 1);
+  const int c1r = S::C1_ROWS;
   // A sum of two is the same in either order: up to 256 K blocks of the whole
   // grid (N <= 8192, where the FP32 sums of whole chunks were reproducible) the
   // chunks of a unit's stripe add by twos into separate images of C1, which
@@ -1030,6 +1160,12 @@ void nodes_choose(Plan& P) {
   z.msh = -first / h;
 }
 
+bool nodes_two_masks(const Plan& P) {
+  if (P.nd.n == 0 || P.form != FZP_FORM_DENSE) return false;
+  const int m = mask_kind(P);
+  return m == MASK_MEMBRANE || m == MASK_QUAD;
+}
+
 fzp_status nodes_layout(Plan& P, FormSizes* out) {
   NodeSet& z = P.nd;
   const int64_t ncols = P.fold ? P.c + 1 : P.N;
@@ -1042,37 +1178,26 @@ fzp_status nodes_layout(Plan& P, FormSizes* out) {
 
 // W: per plan, also in a batch (it depends on the plan's band).  An even field's
 // plan also gets the matrix of all n nodes, for row ranges that are not their
-// own mirror image (a batch runs whole apertures only): w(+-x_k) = (even +- odd) / 2.
+// own mirror image (a batch runs whole apertures only).  Factors on the host
+// (ns^3 / 6 multiply-adds), solves for all outputs on the GPU (on the host the
+// two matrices of a 512^2 ROI took 0.8 ms of a plan).
 fzp_status nodes_upload(Plan& P) {
   NodeSet& z = P.nd;
-  std::vector<double> xo(z.Mo);
-  for (int o = 0; o < z.Mo; ++o) xo[o] = (z.even ? (double)o : (double)o - 0.5 * (P.M - 1)) / z.half;
-  const Interp in(z.n, z.h / z.half, M_PI * z.band * z.half, xo, z.even);
-  std::vector<double> W = in.solve(z.even ? 1 : 0);
   const bool full = z.even && P.owns_buffers;
-  if (full) {
-    const std::vector<double> We = W, Wo = in.solve(-1);
-    const int M = P.M, hm = M / 2;
-    W.resize(We.size() + (size_t)z.n * M);
-    double* F = W.data() + We.size();  // [node][output]
-    for (int k = 0; k < z.ns; ++k)
-      for (int o = 0; o <= hm; ++o) {
-        const double e = We[(size_t)k * z.Mo + o], d = Wo[(size_t)k * z.Mo + o];
-        const int kp = z.ns + k, km = z.ns - 1 - k;  // +x_k and -x_k
-        if (o < hm) {  // +x_o
-          F[(size_t)kp * M + hm + o] = 0.5 * (e + d);
-          F[(size_t)km * M + hm + o] = 0.5 * (e - d);
-        }
-        if (o > 0) {  // -x_o
-          F[(size_t)kp * M + hm - o] = 0.5 * (e - d);
-          F[(size_t)km * M + hm - o] = 0.5 * (e + d);
-        }
-      }
-  }
-  FZP_CUDA_TRY(cudaMalloc(&z.d_W, W.size() * sizeof(double)));
-  P.device_bytes += W.size() * sizeof(double);
-  FZP_CUDA_TRY(cudaMemcpy(z.d_W, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice));
-  z.d_Wy = full ? z.d_W + (size_t)z.ns * z.Mo : z.d_W;
+  const size_t nw = (size_t)z.ns * z.Mo, nf = (size_t)z.ns * z.ns * (full ? 4 : 2);
+  const size_t total = nw + (full ? (size_t)z.n * P.M : 0) + nf;
+  FZP_CUDA_TRY(cudaMalloc(&z.d_W, total * sizeof(double)));
+  P.device_bytes += total * sizeof(double);
+  z.d_Wy = full ? z.d_W + nw : z.d_W;
+  double* dL = z.d_W + (total - nf);
+  std::vector<double> L(nf);
+  InterpSpec a{z.n, z.ns, P.M, z.Mo, z.even ? 1 : 0, z.h / z.half, M_PI * z.band * z.half, z.half};
+  node_factor(z.n, z.ns, z.even ? 1 : 0, a.h, a.c, L.data());
+  if (full) node_factor(z.n, z.ns, -1, a.h, a.c, L.data() + (size_t)2 * z.ns * z.ns);
+  FZP_CUDA_TRY(cudaMemcpy(dL, L.data(), nf * sizeof(double), cudaMemcpyHostToDevice));
+  k_interp_W<<<(unsigned)((z.Mo + 3) / 4), 4 * z.ns>>>(a, dL, z.d_W, full ? z.d_Wy : nullptr);
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
 }
 
@@ -1116,10 +1241,8 @@ fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream
     a.df = deform_coef(P);
     return launch<1, MASK_MEMBRANE>(P, a, s);
   }
-  if (z.ns == 64)
-    return mask == MASK_PARITY   ? launch<1, MASK_PARITY>(P, a, s)
-           : mask == MASK_SIGNED ? launch<1, MASK_SIGNED>(P, a, s)
-                                 : launch<1, MASK_LEVELS>(P, a, s);
+  if (mask == MASK_QUAD) return launch<1, MASK_QUAD>(P, a, s);
+  if (z.ns == 64) return mask == MASK_PARITY ? launch<1, MASK_PARITY>(P, a, s) : launch<1, MASK_SIGNED>(P, a, s);
   return mask == MASK_PARITY   ? launch<2, MASK_PARITY>(P, a, s)
          : mask == MASK_SIGNED ? launch<2, MASK_SIGNED>(P, a, s)
                                : launch<2, MASK_LEVELS>(P, a, s);
@@ -1129,11 +1252,12 @@ fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cuda
   const NodeSet& z = P.nd;
   const bool eveny = z.even && !z.yfull;
   const int ny = z.yfull ? z.n : z.ns, Moy = eveny ? z.Mo : P.M;
-  dim3 b1(32, 4), g1((unsigned)((z.ns + 31) / 32), (unsigned)((Moy + 3) / 4));
-  k_interp_rows<<<g1, b1, 0, s>>>(ny, z.ns, Moy, sym ? 1 : 0, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
+  k_interp_rows<<<dim3((unsigned)(z.ns / 32), (unsigned)((Moy + 3) / 4)), 128, 0, s>>>(
+      ny, z.ns, Moy, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
   const double lf = P.lambda * P.f;
-  InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf, accumulate};
-  k_interp_cols<<<dim3((unsigned)((z.Mo + IT - 1) / IT), (unsigned)((Moy + IT - 1) / IT)), 256, 0, s>>>(
+  InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, sym ? 1 : 0, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf,
+              accumulate};
+  k_interp_cols<<<dim3((unsigned)((z.Mo + IT - 1) / IT), (unsigned)((Moy + IT - 1) / IT)), IT * IT, 0, s>>>(
       a, z.d_W, z.d_X, reinterpret_cast<double2*>(d_field));
   P.launches += 2;
   FZP_CUDA_TRY(cudaGetLastError());

@@ -289,13 +289,13 @@ fzp_status build_mask_tables(Plan& P) {
 // distances from the axis, `kind` says what each stands for.
 static fzp_status chunk_passes(Plan& P, int64_t j0, int64_t rows, RowKind kind, bool octant, cudaStream_t s) {
   const bool nodes = P.nd.n > 0;
-  // a membrane on nodes takes both of its masks in one pass
-  const int np = (P.form == FZP_FORM_DENSE && !P.passes.empty() && !(nodes && P.has_deform)) ? (int)P.passes.size() : 1;
+  const bool passes = P.form == FZP_FORM_DENSE && !P.passes.empty() && !nodes_two_masks(P);
+  const int np = passes ? (int)P.passes.size() : 1;
   fzp_status st = FZP_OK;
   P.c1_stride = P.chunk_rows;
   if (P.fold && P.form == FZP_FORM_BLUESTEIN) j0 += P.c;  // its kernels take rows of the grid
   for (int k = 0; k < np && st == FZP_OK; ++k) {
-    P.pass_index = P.form == FZP_FORM_DENSE && !P.passes.empty() && !(nodes && P.has_deform) ? k : -1;
+    P.pass_index = passes ? k : -1;
     st = nodes && P.form == FZP_FORM_DENSE ? nodes_rows(P, j0, rows, octant, s)
          : P.form == FZP_FORM_DENSE        ? dense_rows(P, j0, rows, s)
                                            : bluestein_rows(P, j0, rows, octant, s);
