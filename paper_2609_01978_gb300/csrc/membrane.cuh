@@ -41,17 +41,17 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b - bh), "f"(a - ah));
 }
 
-// Both masks of a membrane, T cos(phi) and T sin(phi), on the 16 columns from
-// di0 (bit k of `bits`: column k open), as 16-byte parts q0 and q0 + 1 of the
+// Both masks of a membrane, T cos(phi) and T sin(phi), on the 32 columns from
+// di0 (bit k of `bits`: column k open), as the row's four 16-byte parts in the
 // planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart).  The walk's
 // steps, per column: the scaled wrinkle amp sin by its second difference,
 // s' = s + e, e' = e - 4 sin^2(pi kx) s (one product instead of a rotation's
 // four, and no growth of the rounding at the small angles of a wrinkle), the
 // taper by its constant second difference, a ridge by its ratio; each starts
-// exactly every 16 columns.  NR ridges.
+// exactly every 32 columns.  NR ridges.
 template <int NR>
 __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits,
-                                            uint8_t* base, uint32_t plane, int sw, int q0) {
+                                            uint8_t* base, uint32_t plane, int sw) {
   constexpr float TWO_PI = 6.28318530717958648f;
   const float fi = (float)di0;
   const float th = fmaf(fi, d.kxh, r.fjkh);
@@ -75,7 +75,7 @@ __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r,
     }
   }
 #pragma unroll 1
-  for (int q = q0; q < q0 + 2; ++q, bits >>= 8) {
+  for (int q = 0; q < 4; ++q, bits >>= 8) {
     uint32_t hc[4], lc[4], hs[4], ls[4];
 #pragma unroll
     for (int k = 0; k < 8; k += 2) {
@@ -111,12 +111,12 @@ __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r,
 }
 
 __device__ __forceinline__ void cx_store2(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits, uint8_t* base,
-                                          uint32_t plane, int sw, int q0) {
+                                          uint32_t plane, int sw) {
   switch (d.n) {
-    case 0: cx_store2_n<0>(d, r, di0, bits, base, plane, sw, q0); break;
-    case 1: cx_store2_n<1>(d, r, di0, bits, base, plane, sw, q0); break;
-    case 2: cx_store2_n<2>(d, r, di0, bits, base, plane, sw, q0); break;
-    default: cx_store2_n<3>(d, r, di0, bits, base, plane, sw, q0); break;
+    case 0: cx_store2_n<0>(d, r, di0, bits, base, plane, sw); break;
+    case 1: cx_store2_n<1>(d, r, di0, bits, base, plane, sw); break;
+    case 2: cx_store2_n<2>(d, r, di0, bits, base, plane, sw); break;
+    default: cx_store2_n<3>(d, r, di0, bits, base, plane, sw); break;
   }
 }
 

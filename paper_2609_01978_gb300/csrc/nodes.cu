@@ -37,7 +37,7 @@
 //   flat, NT = 2: 256 rows, two accumulators (node tiles)
 //   four levels : 256 rows, accumulators Re T and Im T, a plane each
 //   membrane    : 256 rows, accumulators T cos and T sin, hi and lo planes
-//   warps 0-7 epilogue, 8 loader, 9 MMA issuer, 10-25 mask generators
+//   warps 0-3 epilogue, 4 loader, 5 MMA issuer, 6-21 mask generators
 // The mask rule in the generators: the zone index of a sample is the integer
 // part of s kappa, s = di^2 + dj^2; the 64-bit fixed-point phase s K mod 2^64
 // (its top bit the zone's parity, or its top log2 L bits the level) is carried
@@ -66,11 +66,11 @@ using namespace tc;
 constexpr int BK = 32;                   // columns per stage: one 64-byte swizzle row of BF16
 constexpr int SUB = 128 * BK * 2;        // 8 KiB: one (tile, hi | lo) operand image
 constexpr int PLANE = 256 * BK * 2;      // 16 KiB: one mask plane of 256 rows
-constexpr int EPI_WARPS = 8, LOAD_WARP = 8, MMA_WARP = 9, GEN_WARP0 = 10, GEN_WARPS = 16;
+constexpr int EPI_WARPS = 4, LOAD_WARP = 4, MMA_WARP = 5, GEN_WARP0 = 6, GEN_WARPS = 16;
 constexpr int NUM_THREADS = (GEN_WARP0 + GEN_WARPS) * 32;
 constexpr int TMEM_COLS = 512;
 constexpr int EPI_BOX = 32;
-constexpr int EPI_BYTES = EPI_WARPS * EPI_BOX * EPI_BOX * 4;
+constexpr int EPI_BYTES = EPI_WARPS * 2 * EPI_BOX * EPI_BOX * 4;  // two boxes per warp
 constexpr int ERR_BASE = 300;
 
 enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4 };
@@ -387,27 +387,26 @@ __device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g,
     }
     near = near < 2u * el ? 1u : 0u;
   } else {
-    const uint32_t e2 = 2u * r.E;
+    const uint32_t e2 = 2u * r.E, c4 = 2u * c2;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const uint32_t fa = f, fb = f + d;
       f = fb + d + c2;
-      d += 2u * c2;
+      d += c4;
       near = min(near, min((fa << 1) + e2, (fb << 1) + e2));
       const uint32_t s = prmt(fa, fb, 0xFFBBu);  // each value's sign in its half-word
       wd[q] = MASK == MASK_SIGNED ? ((s & 0x80008000u) | one) : (s & one);
     }
     near = near < 2u * e2 ? 1u : 0u;
   }
-  if (__any_sync(0xffffffffu, near != 0u && chord != 0u)) {
+  // rare: a phase near a zone boundary, columns beyond the chord
+  if (__any_sync(0xffffffffu, near != 0u || chord != 0xFFFFFFFFu)) {
     if (near && chord) {
       uint32_t pb, nb;
       exact_bits<MASK>(w.di0, (int64_t)w.dj * w.dj, g, r, pb, nb);
 #pragma unroll
       for (int q = 0; q < 16; ++q) wd[q] = (pair_mask(pb | nb, q) & one) | (pair_mask(nb, q) & 0x80008000u);
     }
-  }
-  if (__any_sync(0xffffffffu, chord != 0xFFFFFFFFu)) {
 #pragma unroll
     for (int q = 0; q < 16; ++q) wd[q] &= pair_mask(chord, q);
   }
@@ -426,14 +425,15 @@ __device__ __forceinline__ void block_quad(const RowWalk& w, const MaskGeom& g, 
     const uint32_t fa = f, fb = f + d;
     f = fb + d + c2;
     d += 2u * c2;
-    near = min(near, min((fa << 2) + e4, (fb << 2) + e4));
+    const uint32_t ga = fa << 1, gb = fb << 1;
+    near = min(near, min((ga << 1) + e4, (gb << 1) + e4));
     const uint32_t s = prmt(fa, fb, 0xFFBBu) & 0x80008000u;      // q >= 2
-    const uint32_t t = prmt(fa << 1, fb << 1, 0xFFBBu);          // q odd
+    const uint32_t t = prmt(ga, gb, 0xFFBBu);                    // q odd
     re[q] = ~t & (one | s);
     im[q] = t & (one | (s ^ 0x80008000u));
   }
   const bool redo = near < 2u * e4 && chord != 0u;
-  if (__any_sync(0xffffffffu, redo)) {
+  if (__any_sync(0xffffffffu, redo || chord != 0xFFFFFFFFu)) {
     if (redo) {
       uint32_t odd = 0u, high = 0u;
       exact_quad(w.di0, (int64_t)w.dj * w.dj, g, odd, high);
@@ -444,8 +444,6 @@ __device__ __forceinline__ void block_quad(const RowWalk& w, const MaskGeom& g, 
         im[q] = t & (one | (s ^ 0x80008000u));
       }
     }
-  }
-  if (__any_sync(0xffffffffu, chord != 0xFFFFFFFFu)) {
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const uint32_t m = pair_mask(chord, q);
@@ -455,26 +453,30 @@ __device__ __forceinline__ void block_quad(const RowWalk& w, const MaskGeom& g, 
   }
 }
 
-// Open bits of the 16 columns from the walk's (parity rule, chord applied), for
-// the membrane pass.
-__device__ __forceinline__ uint32_t open16(const RowWalk& w, const MaskGeom& g, const PhaseRule& r) {
+// The block's open bits (parity rule, chord applied), for the membrane pass.
+__device__ __forceinline__ uint32_t block_open(const RowWalk& w, const MaskGeom& g, const PhaseRule& r) {
   const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);
   uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
   uint32_t near = 0xFFFFFFFFu, bits = 0u;
-  const uint32_t chord = chord_bits(w.di0, w.bmax) & 0xFFFFu, e2 = 2u * r.E;
+  const uint32_t chord = chord_bits(w.di0, w.bmax), e2 = 2u * r.E;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
+  for (int k = 0; k < 32; ++k) {
     near = min(near, (f << 1) + e2);
-    bits = __funnelshift_l(f, bits, 1);  // the sign shifts in: column k at bit 15 - k
+    bits = __funnelshift_l(f, bits, 1);  // the sign shifts in: column k at bit 31 - k
     f += d;
     d += c2;
   }
-  bits = __brev(bits) >> 16;
+  bits = __brev(bits);
   if (near < 2u * e2 && chord != 0u) {
     uint32_t nb;
     exact_bits<MASK_PARITY>(w.di0, (int64_t)w.dj * w.dj, g, r, bits, nb);
   }
   return bits & chord;
+}
+
+// Whole-warp wait: usually the stage is free and one test passes.
+__device__ __forceinline__ bool stage_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
+  return __all_sync(0xffffffffu, mbar_try(bar, parity)) || warp_wait(bar, parity, abort_flag, err, code);
 }
 
 // ------------------------------------------------------------------ kernel
@@ -503,7 +505,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(&fullA[s], 1);
-      mbar_init(&fullB[s], CX ? GEN_WARPS : GEN_WARPS / 2);
+      mbar_init(&fullB[s], GEN_WARPS / 2);
       mbar_init(&empty[s], 1);
     }
     mbar_init(accFull, 1);
@@ -607,41 +609,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
       }
     }
   } else if (warp >= GEN_WARP0) {
-    // ---------------- mask generators.  Membrane: warps gw and gw + 8 take the
-    // same 32 rows' 16-column halves of every block.  Otherwise two groups of
-    // eight warps take every other block of the CTA's sequence (with an even
-    // number of stages a stage has one group), a lane per row, or per two rows
-    // 256 apart where the unit has 512
-    static_assert(CX || NST % 2 == 0, "a stage must keep its generator group");
+    // ---------------- mask generators: two groups of eight warps take every
+    // other block of the CTA's sequence (with an even number of stages a stage
+    // has one group), a lane per row, or per two rows 256 apart where the unit
+    // has 512
+    static_assert(NST % 2 == 0, "a stage must keep its generator group");
     const int gw = warp - GEN_WARP0, grp = gw >> 3;
     const int row = (gw & 7) * 32 + lane;  // row of the stripe (and row + 256)
     // 64-byte swizzle: row at (row / 8) 512 + (row % 8) 64, 16-byte part q at q ^ ((row % 8) / 2)
     uint8_t* rowbase = sB + (row >> 3) * 512 + (row & 7) * 64;
     const int sw = (row & 7) >> 1;
     bool ok = true;
-    if constexpr (CX) {
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
-        const Unit un = unit_at<BN>(a, it);
-        const int64_t j = un.jb + row;
-        RowWalk w;
-        row_start(w, j - a.mg.c, un.kb0 * BK - a.mg.c + 16 * grp, j < un.je, a.mg, a.ph);
-        CxRow cxr;
-        cx_row_init(a.df, j - a.mg.c, cxr);
-        for (int kb = (int)un.kb0; kb < (int)un.kb1; ++kb) {
-          const uint32_t bits = open16(w, a.mg, a.ph);
-          if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
-          uint8_t* rp = rowbase + stage * S::B_BYTES;
-          cx_store2(a.df, cxr, w.di0, bits, rp, PLANE, sw, 2 * grp);
-          row_next<BK>(w, a.ph);
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&fullB[stage]);
-          if (++stage == NST) { stage = 0; phase ^= 1; }
-        }
-      }
-    } else {
+    {
       constexpr int RPL = BN / 256;  // rows per lane
       int stage = grp;
       uint32_t phase = 0;
@@ -653,18 +632,24 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
 #pragma unroll
         for (int h = 0; h < RPL; ++h) {
           const int64_t j = un.jb + row + 256 * h;
-          row_start(w[h], j, (un.kb0 + skip) * BK, j < un.je, a.mg, a.ph);
+          row_start(w[h], j - a.mg.c, (un.kb0 + skip) * BK - a.mg.c, j < un.je, a.mg, a.ph);
         }
+        CxRow cxr;
+        if constexpr (CX) cx_row_init(a.df, un.jb + row - a.mg.c, cxr);
         // blocks of the diagonal tile: half weight
         const int diag = a.octant ? (int)(un.jb / BK - un.kb0) : nkb;
         int b = skip;
         for (; b < nkb; b += 2) {
           const uint32_t one = b >= diag ? 0x3F003F00u : 0x3F803F80u;
           uint8_t* rp = rowbase + stage * S::B_BYTES;
-          if constexpr (MASK == MASK_QUAD) {
+          if constexpr (CX) {
+            const uint32_t bits = block_open(w[0], a.mg, a.ph);
+            if (!stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+            cx_store2(a.df, cxr, w[0].di0, bits, rp, PLANE, sw);
+          } else if constexpr (MASK == MASK_QUAD) {
             uint32_t re[16], im[16];
             block_quad(w[0], a.mg, a.ph, one, chord_up(w[0]), re, im);
-            if (!warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+            if (!stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               *reinterpret_cast<uint4*>(rp + ((q ^ sw) << 4)) =
@@ -677,7 +662,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
             for (int h = 0; h < RPL; ++h) {
               uint32_t wd[16];
               block_words<MASK>(w[h], a.mg, a.ph, one, chord_up(w[h]), wd);
-              if (h == 0 && !warp_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+              if (h == 0 && !stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
 #pragma unroll
               for (int q = 0; q < 4; ++q)
                 *reinterpret_cast<uint4*>(rp + h * PLANE + ((q ^ sw) << 4)) =
@@ -697,39 +682,45 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
       }
     }
   } else {
-    // ---------------- epilogue: warp w drains accumulator w / 4, TMEM lanes 32 (w % 4) ..:
-    // each 32 x 32 piece goes to shared memory (128-byte swizzle) and from
-    // there by one TMA reduce-add into C1, once per promotion
-    const int q = warp >> 2;
-    uint8_t* eb = sE + warp * (EPI_BOX * EPI_BOX * 4);
-    uint32_t accph = 0;
+    // ---------------- epilogue: warp w drains TMEM lanes 32 w .. of both
+    // accumulators: each 32 x 32 piece goes to shared memory (128-byte swizzle,
+    // two boxes in turn) and from there by one TMA reduce-add into C1, once per
+    // promotion
+    uint8_t* eb = sE + warp * (2 * EPI_BOX * EPI_BOX * 4);
+    uint32_t accph = 0, box = 0;
     bool ok = true;
     for (int it = blockIdx.x; it < n_items && ok; it += gridDim.x) {
       const Unit un = unit_at<BN>(a, it);
-      const int x0 = (int)(un.jb - a.j_begin) + (BN == 512 ? q * 256 : 0);
-      const int y0 = un.slice * S::C1_ROWS + (BN == 512 ? 0 : q * 128) + (warp & 3) * 32;
-      const int xn = (int)min((int64_t)256, un.je - a.j_begin - x0);  // live columns (may be <= 0)
+      const int rows = (int)(un.je - un.jb);
       for (int64_t p0 = un.kb0; p0 < un.kb1; p0 += a.promote) {
         if (threadIdx.x == 0) epi_ok[accph] = mbar_wait(accFull, accph, abort_flag, a.err, ERR_BASE + 6) ? 1 : 0;
         named_bar_sync(1, EPI_WARPS * 32);
         if (!epi_ok[accph]) { ok = false; break; }
         tc_fence_after();
-        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * 256);
 #pragma unroll 1
-        for (int col = 0; col < xn; col += EPI_BOX) {
-          float v[32];
-          tmem_ld32(taddr + col, v);
-          if (lane == 0) bulk_wait_read0();  // the previous piece has been read out of eb
-          __syncwarp();
+        for (int q = 0; q < 2; ++q) {
+          const int xs = BN == 512 ? q * 256 : 0, x0 = (int)(un.jb - a.j_begin) + xs;
+          const int y0 = un.slice * S::C1_ROWS + (BN == 512 ? 0 : q * 128) + warp * 32;
+          const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(q * 256);
+          const int xn = min(256, rows - xs);  // live columns (may be <= 0)
+#pragma unroll 1
+          for (int col = 0; col < xn; col += EPI_BOX) {
+            float v[32];
+            tmem_ld32(taddr + col, v);
+            uint8_t* bx = eb + box * (EPI_BOX * EPI_BOX * 4);
+            box ^= 1u;
+            if (lane == 0) bulk_wait_read1();  // the piece before the last has been read out
+            __syncwarp();
 #pragma unroll
-          for (int c4 = 0; c4 < 8; ++c4)
-            *reinterpret_cast<float4*>(eb + lane * 128 + ((c4 ^ (lane & 7)) << 4)) =
-                make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) {
-            tma_reduce_add_2d(&tmC1, eb, x0 + col, y0);
-            bulk_commit();
+            for (int c4 = 0; c4 < 8; ++c4)
+              *reinterpret_cast<float4*>(bx + lane * 128 + ((c4 ^ (lane & 7)) << 4)) =
+                  make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+              tma_reduce_add_2d(&tmC1, bx, x0 + col, y0);
+              bulk_commit();
+            }
           }
         }
         tc_fence_before();
@@ -987,9 +978,7 @@ __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int
         for (int k = 0; k < 32; ++k)
           v[k] = ((disc >> k) & 1u) ? (uint8_t)(1 + ((wd[k / 2] >> (16 * (k & 1) + 15)) & 1u)) : 0;
       } else if (mask == MASK_MEMBRANE) {
-        RowWalk w2 = w;
-        row_next<16>(w2, ph);
-        const uint32_t bits = open16(w, mg, ph) | (open16(w2, mg, ph) << 16);
+        const uint32_t bits = block_open(w, mg, ph);
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = (uint8_t)((bits >> k) & 1u);
       } else {
