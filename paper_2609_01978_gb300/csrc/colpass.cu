@@ -206,7 +206,7 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   // rows per block: 2048, fewer where that leaves the GPU idle (few output tiles)
   const int ny = nodes && P.nd.yfull ? P.nd.n : g.M;
   const int64_t tiles = (int64_t)(g.M / TM) * (ny / TN);
-  g.jc = std::min<int64_t>(2048, std::max<int64_t>(4 * TJ, (rows * tiles / 456 + TJ - 1) / TJ * TJ));
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / 304 + TJ - 1) / TJ * TJ));
   dim3 grid((unsigned)(g.M / TM), (unsigned)(ny / TN), (unsigned)((rows + g.jc - 1) / g.jc));
   if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
   else k_colpass<float><<<grid, 256, 0, s>>>(g, P.d_C1, P.d_Uacc);

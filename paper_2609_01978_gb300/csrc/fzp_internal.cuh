@@ -224,7 +224,8 @@ struct NodeSet {
   bool yfull = false;      // the call being run takes all n nodes along y
   int slices = 1;          // images of C1 in the chunk being run, and their distance
   int64_t slice_elems = 0;
-  double2* d_X = nullptr;  // [ns][Mo] rows interpolated
+  double2* d_chirp = nullptr;  // [M] output chirp of the ROI samples, behind d_W
+  double2* d_X = nullptr;  // [ns][M] rows interpolated
 };
 
 // What a row of the column pass stands for (flat plates: distances from the axis).

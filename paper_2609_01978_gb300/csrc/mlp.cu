@@ -13,8 +13,18 @@
 //   forward  z_l   = h_{l-1} . W_l^T          (A = h, B = W)
 //   backward dh    = g . W_l                  (A = g, B = W^T  kept transposed)
 //            dW_l  = g^T . h_{l-1}            (A = g^T, B = h^T: transposed copies)
+// At this network's sizes (batch 256, 512 hidden, 4114 outputs: 6.7 GFLOP of a
+// training step, 3.5 us of the tensor rate) a step is bound by launches and by
+// the length of each product's chain, so the products take 128 x 64 tiles with
+// an eight-deep ring of loads, what follows a product (bias, SiLU and its
+// derivative, the loss gradient, BF16 copies in both orders, column sums) is
+// its epilogue, and a layer's two backward products share a launch.  Every
+// product keeps one accumulation in K order: a split of the longest (dh of the
+// output layer, K = 4160) was no slower to write but moves g in its last FP32
+// bits, and with them the BF16 rounding of 3 % of g's values.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <new>
 #include <vector>
@@ -27,9 +37,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int GM = 128, GN = 128, GK = 64;  // GEMM tile; K step = one 128-byte swizzle row
-constexpr int GEMM_THREADS = 128;
-constexpr int GEMM_SMEM = 1024 + 2 * GM * GK * 2 + 64 + 16384;  // extra slack caps residency at 4 CTAs/SM
+constexpr int GM = 128, GN = 64, GK = 64;  // GEMM tile; K step = one 128-byte swizzle row
+constexpr int GEMM_THREADS = 256;  // warps 0-3: columns 0-31 of the tile in the epilogue, 4-7: 32-63
+constexpr int RING = 8, AHEAD = RING - 2;  // K steps loaded ahead (a slot rests one step, its MMAs in flight)
+constexpr int STAGE_BYTES = (GM + GN) * GK * 2;
+constexpr int GEMM_SMEM = 1024 + RING * STAGE_BYTES + 128;  // the epilogue's tile of g reuses the ring
 
 __host__ __device__ inline int64_t pad64(int64_t x) { return (x + 63) / 64 * 64; }
 
@@ -48,34 +60,85 @@ __device__ __forceinline__ void mma_g(uint32_t dtmem, uint64_t ad, uint64_t bd, 
       : "memory");
 }
 
-// Load a 128-row x 64-column BF16 tile (rows r0.., columns k0..) into the
-// 128-byte-swizzled K-major layout; out-of-range elements are zero.
-__device__ __forceinline__ void load_tile(uint8_t* s, const __nv_bfloat16* g, int64_t ld, int64_t rows, int64_t K,
-                                          int64_t r0, int64_t k0) {
-  for (int t = threadIdx.x; t < GM * 8; t += GEMM_THREADS) {
-    const int r = t >> 3, ch = t & 7;
-    const int64_t gr = r0 + r, gk = k0 + ch * 8;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (gr < rows && gk < K) v = *reinterpret_cast<const uint4*>(g + gr * ld + gk);  // K, ld multiples of 8
-    *reinterpret_cast<uint4*>(s + (r >> 3) * 1024 + (r & 7) * 128 + ((ch ^ (r & 7)) << 4)) = v;
+// 16 bytes global -> shared, or zeros (the address is not read then).
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool live) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(live ? 16 : 0)
+               : "memory");
+}
+
+__device__ __forceinline__ float sigm(float z) { return 1.f / (1.f + expf(-z)); }
+
+// What follows a product.
+enum Epi {
+  EPI_HIDDEN = 0,  // z = acc + bias -> Z; h = silu(z) -> Hb (and, training, HTb)
+  EPI_Y = 1,       // y = acc + bias -> C
+  EPI_LOSS = 2,    // g = 2 (acc + bias - y) / (B n) -> Gb, GTb, column sums; loss
+  EPI_DW = 3,      // C = acc (a layer's gradient, packed); the first tile column also adds the bias gradient up
+  EPI_DH = 4       // g = acc silu'(z) -> Gb, GTb, column sums
+};
+
+struct Gemm {
+  const __nv_bfloat16 *A, *B;
+  int64_t lda, ldb;
+  int M, N, K;         // K a multiple of 8
+  int tiles_n, tiles;  // tiles along N, and all
+  int epi;
+  const float* bias;
+  float* C;            // EPI_Y, EPI_DW
+  int64_t ldc;
+  float* Z;            // EPI_HIDDEN (written), EPI_DH (read)
+  int64_t ldz;
+  __nv_bfloat16 *rows, *cols;  // Hb / Gb and HTb / GTb (cols may be null)
+  int64_t ldr, ldt;
+  const float* y;      // EPI_LOSS
+  double* lpart;       // EPI_LOSS: squared errors of each tile; EPI_DW of the first layer: to be totalled
+  int nlpart;
+  float* loss;         // EPI_DW of the first layer (may be null): the mean of the squared errors
+  double loss_scale;
+  float* sums;         // column sums per 128-row tile [tile][ld_sums]
+  int64_t ld_sums;
+  const float* bsums;  // EPI_DW: the column sums whose total is the bias gradient
+  float* db;
+  int nsums;
+};
+
+// Columns [c0, c0 + 32) of a row of g or h in BF16, row-major (64 bytes a
+// thread) and transposed (a warp's 32 rows per column).  Columns from n on and
+// rows from m on are zero in `v` / not stored.
+__device__ __forceinline__ void store_bf16(const Gemm& p, const float (&v)[32], int r, int c0, bool row_live) {
+  if (!row_live) return;
+  uint32_t w[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+    w[q] = *reinterpret_cast<const uint32_t*>(&t);
+  }
+  if (c0 < p.ldr) {
+    uint4* o = reinterpret_cast<uint4*>(p.rows + (int64_t)r * p.ldr + c0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+  }
+  if (p.cols) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q)
+      if (c0 + q < p.N) p.cols[(int64_t)(c0 + q) * p.ldt + r] = __float2bfloat16_rn(v[q]);
   }
 }
 
-// C[M x N] (FP32, ldc) = A[M x K] . B[N x K]^T (+ bias[N]).  K must be a multiple of 8.
-__global__ void __launch_bounds__(GEMM_THREADS) k_gemm_tn(int64_t M, int64_t N, int64_t K, const __nv_bfloat16* A,
-                                                          int64_t lda, const __nv_bfloat16* B, int64_t ldb, float* C,
-                                                          int64_t ldc, const float* bias, int* err) {
+// One tile of one of up to two products per CTA.
+__global__ void __launch_bounds__(GEMM_THREADS) k_gemm(const Gemm g0, const Gemm g1, int n0_blocks, int* err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sA = base;
-  uint8_t* sB = base + GM * GK * 2;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sB + GN * GK * 2);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 1);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + 2);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t m0 = (int64_t)blockIdx.y * GM, n0 = (int64_t)blockIdx.x * GN;
-  if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(base + RING * STAGE_BYTES);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + RING);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + RING + 1);
+  const bool first = (int)blockIdx.x < n0_blocks;
+  const Gemm& p = first ? g0 : g1;
+  const int tile = first ? blockIdx.x : blockIdx.x - n0_blocks;
+  const int m0 = tile / p.tiles_n * GM, n0 = tile % p.tiles_n * GN;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int q = 0; q < RING; ++q) mbar_init(&bar[q], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -89,40 +152,148 @@ __global__ void __launch_bounds__(GEMM_THREADS) k_gemm_tn(int64_t M, int64_t N, 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int64_t nk = (K + GK - 1) / GK;
+  const int nk = (p.K + GK - 1) / GK;
+  // K step kb into its ring slot: 128 + 64 rows of 128 bytes, swizzled
+  auto load = [&](int kb) {
+    uint8_t* s = base + kb % RING * STAGE_BYTES;
+    const int ch = tid & 7, gk = kb * GK + ch * 8;
+#pragma unroll
+    for (int q = 0; q < (GM + GN) / 32; ++q) {
+      const int r = q * 32 + (tid >> 3);
+      const bool isA = q < GM / 32;
+      const int gr = isA ? m0 + r : n0 + r - GM;
+      const bool live = gk < p.K && gr < (isA ? p.M : p.N);
+      const __nv_bfloat16* src = isA ? p.A + (int64_t)gr * p.lda + gk : p.B + (int64_t)gr * p.ldb + gk;
+      cp16(s + (r >> 3) * 1024 + (r & 7) * 128 + ((ch ^ (r & 7)) << 4), live ? src : (isA ? p.A : p.B), live);
+    }
+  };
+#pragma unroll
+  for (int q = 0; q < AHEAD; ++q) {
+    if (q < nk) load(q);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
   bool ok = true;
-  for (int64_t kb = 0; kb < nk && ok; ++kb) {
-    load_tile(sA, A, lda, M, K, m0, kb * GK);
-    load_tile(sB, B, ldb, N, K, n0, kb * GK);
+  for (int kb = 0; kb < nk; ++kb) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
     fence_proxy_async();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       tc_fence_after();
-      const uint64_t ad = sdesc128(sA), bd = sdesc128(sB);
+      uint8_t* s = base + kb % RING * STAGE_BYTES;
+      const uint64_t ad = sdesc128(s), bd = sdesc128(s + GM * GK * 2);
 #pragma unroll
       for (int kk = 0; kk < GK / 16; ++kk)
         mma_g(tmem, ad + (uint64_t)((kk * 32) >> 4), bd + (uint64_t)((kk * 32) >> 4), (kb > 0 || kk > 0) ? 1u : 0u);
-      mma_commit(bar);
+      mma_commit(&bar[kb % RING]);
     }
-    // every thread waits for the MMAs of this step: the tile buffers are reused
-    ok = mbar_wait(bar, (uint32_t)(kb & 1), abort_flag, err, 200);
-    tc_fence_after();
-    __syncthreads();
-    ok = !*abort_flag;
+    // the slot of step kb - 2 is free once its MMAs are done
+    if (kb + AHEAD < nk) {
+      if (kb > 1) ok = mbar_wait(&bar[(kb - 2) % RING], (uint32_t)((kb - 2) / RING & 1), abort_flag, err, 200) && ok;
+      load(kb + AHEAD);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  const int last = nk - 1;
+  ok = mbar_wait(&bar[last % RING], (uint32_t)(last / RING & 1), abort_flag, err, 201) && ok;
+  tc_fence_after();
+  __syncthreads();  // every wait above has ended in all threads
+  ok = ok && !*abort_flag;
   if (ok) {
-    const int64_t r = m0 + warp * 32 + lane;
-#pragma unroll 1
-    for (int c0 = 0; c0 < GN; c0 += 32) {
+    const int tr = tid & (GM - 1), r = m0 + tr;
+    const bool row_live = r < p.M;
+    float* tile_g = reinterpret_cast<float*>(base);  // [128][65] of g, for the column sums
+    float lsum = 0.f;
+    const float scale = 2.f / ((float)p.M * (float)p.N);
+    {
+      const int cc = (warp >> 2) * 32, c0 = n0 + cc;
       float v[32];
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-      if (r < M) {
+      tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cc, v);
+      if (p.epi == EPI_HIDDEN) {
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-          const int64_t n = n0 + c0 + q;
-          if (n < N) C[r * ldc + n] = v[q] + (bias ? bias[n] : 0.f);
+        for (int q = 0; q < 32; ++q) v[q] = c0 + q < p.N ? v[q] + p.bias[c0 + q] : 0.f;
+        if (row_live && p.Z) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)  // the padding columns too (zeros)
+            if (c0 + 4 * q < p.ldz)
+              *reinterpret_cast<float4*>(p.Z + (int64_t)r * p.ldz + c0 + 4 * q) =
+                  make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = v[q] * sigm(v[q]);
+        store_bf16(p, v, r, c0, row_live);
+      } else if (p.epi == EPI_LOSS || p.epi == EPI_DH) {
+        if (p.epi == EPI_LOSS) {
+#pragma unroll
+          for (int q = 0; q < 32; ++q) {
+            float d = 0.f;
+            if (row_live && c0 + q < p.N) d = v[q] + p.bias[c0 + q] - p.y[(int64_t)r * p.N + c0 + q];
+            lsum += d * d;
+            v[q] = scale * d;
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < 32; ++q) {
+            float d = 0.f;
+            if (row_live && c0 + q < p.N) {
+              const float zz = p.Z[(int64_t)r * p.ldz + c0 + q], sg = sigm(zz);
+              d = v[q] * (sg * (1.f + zz * (1.f - sg)));
+            }
+            v[q] = d;
+          }
+        }
+        store_bf16(p, v, r, c0, row_live);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) tile_g[tr * 65 + cc + q] = v[q];
+      } else {
+        if (row_live) {
+#pragma unroll
+          for (int q = 0; q < 32; ++q)
+            if (c0 + q < p.N) v[q] += p.epi == EPI_Y ? p.bias[c0 + q] : 0.f;
+          float* C = p.C + (int64_t)r * p.ldc + c0;
+          if ((p.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(p.C) & 15) == 0 && c0 + 32 <= p.N) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              *reinterpret_cast<float4*>(C + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+              if (c0 + q < p.N) C[q] = v[q];
+          }
         }
       }
+    }
+    if (p.epi == EPI_LOSS || p.epi == EPI_DH) {
+      __syncthreads();
+      if (tid < GN && n0 + tid < p.N) {
+        float s = 0.f;
+        for (int q = 0; q < GM; ++q) s += tile_g[q * 65 + tid];
+        p.sums[(int64_t)(m0 / GM) * p.ld_sums + n0 + tid] = s;
+      }
+      if (p.epi == EPI_LOSS) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        float* part = tile_g + GM * 65;
+        if (lane == 0) part[warp] = lsum;
+        __syncthreads();
+        if (tid == 0) {
+          double t = 0.0;
+          for (int q = 0; q < GEMM_THREADS / 32; ++q) t += (double)part[q];
+          p.lpart[tile] = t;
+        }
+      }
+    }
+    if (p.epi == EPI_DW && p.loss && tile == 0 && warp == 7) {
+      double t = 0.0;
+      for (int q = lane; q < p.nlpart; q += 32) t += p.lpart[q];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) *p.loss = (float)(t * p.loss_scale);
+    }
+    if (p.epi == EPI_DW && n0 == 0 && row_live && tid < GM) {
+      float s = 0.f;
+      for (int q = 0; q < p.nsums; ++q) s += p.bsums[(int64_t)q * p.ld_sums + r];
+      p.db[r] = s;
     }
   }
   tc_fence_before();
@@ -133,96 +304,38 @@ __global__ void __launch_bounds__(GEMM_THREADS) k_gemm_tn(int64_t M, int64_t N, 
   }
 }
 
-__device__ __forceinline__ float sigm(float z) { return 1.f / (1.f + expf(-z)); }
-
-// dst[r][c] = bf16(act ? silu(src) : src) for r < R, c < Cn (ld in elements).
-__global__ void k_to_bf16(int64_t R, int64_t Cn, const float* src, int64_t lds, __nv_bfloat16* dst, int64_t ldd,
-                          int act) {
+// The batch's inputs in BF16, row-major (zero padded) and, training, transposed.
+__global__ void k_inputs(int64_t R, int64_t Cn, const float* x, __nv_bfloat16* rows, int64_t ldr, __nv_bfloat16* cols,
+                         int64_t ldt) {
   const int64_t total = R * Cn;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = t / Cn, c = t % Cn;
-    float v = src[r * lds + c];
-    if (act) v = v * sigm(v);
-    dst[r * ldd + c] = __float2bfloat16_rn(v);
+    const __nv_bfloat16 v = __float2bfloat16_rn(x[t]);
+    rows[r * ldr + c] = v;
+    if (cols) cols[c * ldt + r] = v;
   }
 }
 
-// dst[c][r] = bf16(act ? silu(src[r][c]) : src[r][c])  (transposed copy).
-__global__ void k_to_bf16_t(int64_t R, int64_t Cn, const float* src, int64_t lds, __nv_bfloat16* dst, int64_t ldd,
-                            int act) {
-  __shared__ float tile[32][33];
-  const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int64_t r = r0 + k, c = c0 + threadIdx.x;
-    float v = 0.f;
-    if (r < R && c < Cn) {
-      v = src[r * lds + c];
-      if (act) v = v * sigm(v);
-    }
-    tile[k][threadIdx.x] = v;
-  }
-  __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int64_t c = c0 + k, r = r0 + threadIdx.x;
-    if (r < R && c < Cn) dst[c * ldd + r] = __float2bfloat16_rn(tile[threadIdx.x][k]);
-  }
-}
-
-// g = dh * silu'(z)
-__global__ void k_silu_back(int64_t R, int64_t Cn, const float* dh, const float* z, int64_t ld, float* g) {
-  const int64_t total = R * Cn;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = t / Cn, c = t % Cn;
-    const float zz = z[r * ld + c], s = sigm(zz);
-    g[r * ld + c] = dh[r * ld + c] * (s * (1.f + zz * (1.f - s)));
-  }
-}
-
-// g = 2 (yhat - y) / (B n); loss += mean((yhat - y)^2)
-__global__ void k_mse(int64_t B, int64_t n, const float* yhat, int64_t ldy, const float* y, float* g, float* loss) {
-  __shared__ float sh[256];
-  float acc = 0.f;
-  const float scale = 2.f / (float)(B * n);
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < B * n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = t / n, c = t % n;
-    const float d = yhat[r * ldy + c] - y[r * n + c];
-    g[r * ldy + c] = scale * d;
-    acc += d * d;
-  }
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && loss) atomicAdd(loss, sh[0] / (float)(B * n));
-}
-
-// db[c] = sum_r g[r][c]
-__global__ void k_colsum(int64_t R, int64_t Cn, const float* g, int64_t ld, float* db) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= Cn) return;
-  float s = 0.f;
-  for (int64_t r = 0; r < R; ++r) s += g[r * ld + c];
-  db[c] = s;
-}
-
-// copy dW (FP32, [n_out][ld]) into the flat gradient vector
-__global__ void k_pack(int64_t R, int64_t Cn, const float* src, int64_t ld, float* dst) {
-  const int64_t total = R * Cn;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x)
-    dst[t] = src[(t / Cn) * ld + t % Cn];
-}
-
-__global__ void k_adamw(int64_t n, float* p, const float* g, float* m, float* v, float lr, float wd, float b1, float b2,
-                        float eps, float c1, float c2) {
+// AdamW on one layer's weights and biases (decay on the weights only), and the
+// weights' BF16 copies: Wb [n_out][ld_in], WTb [n_in][ld_out].
+__global__ void k_adamw(int64_t n_out, int64_t n_in, float* p, const float* g, float* m, float* v, float lr, float wd,
+                        float b1, float b2, float eps, float c1, float c2, __nv_bfloat16* Wb, int64_t ld_in,
+                        __nv_bfloat16* WTb, int64_t ld_out) {
+  const int64_t nw = n_out * n_in, n = nw + n_out;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const float gg = g[t];
     const float mm = b1 * m[t] + (1.f - b1) * gg;
     const float vv = b2 * v[t] + (1.f - b2) * gg * gg;
     m[t] = mm;
     v[t] = vv;
-    p[t] -= lr * ((mm / c1) / (sqrtf(vv / c2) + eps) + wd * p[t]);
+    const float w = p[t], pw = w - lr * ((mm / c1) / (sqrtf(vv / c2) + eps) + (t < nw ? wd : 0.f) * w);
+    p[t] = pw;
+    if (t < nw) {
+      const int64_t o = t / n_in, i = t % n_in;
+      const __nv_bfloat16 b = __float2bfloat16_rn(pw);
+      Wb[o * ld_in + i] = b;
+      WTb[i * ld_out + o] = b;
+    }
   }
 }
 
@@ -268,8 +381,9 @@ struct fzp_surrogate_s {
   std::vector<float*> Z;             // pre-activations per layer [B][ld_out] FP32
   std::vector<__nv_bfloat16*> Hb;    // layer inputs, BF16 [B][ld_in]
   std::vector<__nv_bfloat16*> HTb;   // layer inputs transposed [ld_in... n_in][ldB]
-  float *G = nullptr, *dH = nullptr, *dW = nullptr;
-  __nv_bfloat16 *Gb = nullptr, *GTb = nullptr;
+  __nv_bfloat16 *Gb[2] = {}, *GTb[2] = {};  // g of a layer and of the one below it
+  float* sums[2] = {};               // its column sums per 128 rows [tile][maxw]
+  double* lpart = nullptr;           // squared errors of the output layer's tiles
   int64_t ldB = 0, maxw = 0;
   int* err = nullptr;
   std::vector<void*> allocs;
@@ -277,73 +391,102 @@ struct fzp_surrogate_s {
 
 namespace {
 
-fzp_status gemm(fzp_surrogate_s& S, int64_t M, int64_t N, int64_t K, const __nv_bfloat16* A, int64_t lda,
-                const __nv_bfloat16* B, int64_t ldb, float* C, int64_t ldc, const float* bias, cudaStream_t s) {
-  dim3 grid((unsigned)((N + GN - 1) / GN), (unsigned)((M + GM - 1) / GM));
-  k_gemm_tn<<<grid, GEMM_THREADS, GEMM_SMEM, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, S.err);
-  FZP_CUDA_TRY(cudaGetLastError());
-  return FZP_OK;
-}
-
 unsigned blocks(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, 4096); }
 
-// Forward pass for a batch of B rows (x: FP32 [B][n_in0], contiguous).
-fzp_status forward(fzp_surrogate_s& S, const float* x, int64_t B, cudaStream_t s) {
+Gemm product(int64_t M, int64_t N, int64_t K, const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb,
+             int epi) {
+  Gemm p{};
+  p.A = A; p.B = B; p.lda = lda; p.ldb = ldb;
+  p.M = (int)M; p.N = (int)N; p.K = (int)K;
+  p.tiles_n = (int)((N + GN - 1) / GN);
+  p.tiles = p.tiles_n * (int)((M + GM - 1) / GM);
+  p.epi = epi;
+  return p;
+}
+
+fzp_status run_gemm(fzp_surrogate_s& S, const Gemm& a, const Gemm* b, cudaStream_t s) {
+  const int na = a.tiles, nb = b ? b->tiles : 0;
+  k_gemm<<<(unsigned)(na + nb), GEMM_THREADS, GEMM_SMEM, s>>>(a, b ? *b : a, na, S.err);
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+// Forward pass for a batch of B rows (x: FP32 [B][n_in0], contiguous).  y null:
+// inference, the output to `out` (FP32 [B][n_out]).  Otherwise the tiles' squared
+// errors, the output layer's g, and what the backward pass needs.
+fzp_status forward(fzp_surrogate_s& S, const float* x, int64_t B, const float* y, float* out, cudaStream_t s) {
   const Layer& l0 = S.L[0];
-  k_to_bf16<<<blocks(B * l0.n_in), 256, 0, s>>>(B, l0.n_in, x, l0.n_in, S.Hb[0], l0.ld_in, 0);
+  const bool train = y != nullptr;
+  k_inputs<<<blocks(B * l0.n_in), 256, 0, s>>>(B, l0.n_in, x, S.Hb[0], l0.ld_in, train ? S.HTb[0] : nullptr, S.ldB);
   for (size_t l = 0; l < S.L.size(); ++l) {
     const Layer& ly = S.L[l];
-    fzp_status st = gemm(S, B, ly.n_out, ly.ld_in, S.Hb[l], ly.ld_in, ly.Wb, ly.ld_in, S.Z[l], ly.ld_out,
-                         S.params + ly.off_b, s);
+    const bool top = l + 1 == S.L.size();
+    Gemm p = product(B, ly.n_out, ly.ld_in, S.Hb[l], ly.ld_in, ly.Wb, ly.ld_in, !top ? EPI_HIDDEN : train ? EPI_LOSS : EPI_Y);
+    p.bias = S.params + ly.off_b;
+    if (!top) {
+      p.Z = train ? S.Z[l] : nullptr;
+      p.ldz = ly.ld_out;
+      p.rows = S.Hb[l + 1];
+      p.ldr = S.L[l + 1].ld_in;
+      p.cols = train ? S.HTb[l + 1] : nullptr;
+      p.ldt = S.ldB;
+    } else if (train) {
+      p.y = y;
+      p.lpart = S.lpart;
+      p.rows = S.Gb[0];
+      p.ldr = S.maxw;
+      p.cols = S.GTb[0];
+      p.ldt = S.ldB;
+      p.sums = S.sums[0];
+      p.ld_sums = S.maxw;
+    } else {
+      p.C = out;
+      p.ldc = ly.n_out;
+    }
+    const fzp_status st = run_gemm(S, p, nullptr, s);
     if (st != FZP_OK) return st;
-    if (l + 1 < S.L.size())
-      k_to_bf16<<<blocks(B * ly.n_out), 256, 0, s>>>(B, ly.n_out, S.Z[l], ly.ld_out, S.Hb[l + 1], S.L[l + 1].ld_in, 1);
   }
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
 }
 
-// Loss and gradients into S.grads (flat, same layout as params).
-// Requires forward() and transposed_inputs() for the same batch.
-fzp_status backward(fzp_surrogate_s& S, const float* y, int64_t B, float* d_loss, cudaStream_t s) {
-  fzp_status st = FZP_OK;
+// Gradients into `grads` (flat, same layout as params) and the loss (if d_loss),
+// after forward() on the same batch.  A layer's dW and dh run in one launch; g alternates between two
+// buffers, as dh's epilogue writes the next one while dW still reads this one.
+fzp_status backward(fzp_surrogate_s& S, int64_t B, float* grads, float* d_loss, cudaStream_t s) {
   const int nl = (int)S.L.size();
-  const Layer& lo = S.L[nl - 1];
-  if (d_loss) FZP_CUDA_TRY(cudaMemsetAsync(d_loss, 0, sizeof(float), s));
-  k_mse<<<256, 256, 0, s>>>(B, lo.n_out, S.Z[nl - 1], lo.ld_out, y, S.G, d_loss);
-  for (int l = nl - 1; l >= 0; --l) {
+  for (int l = nl - 1, cur = 0; l >= 0; --l, cur ^= 1) {
     const Layer& ly = S.L[l];
-    // db = sum over batch of g; g in BF16 (row-major and transposed)
-    k_colsum<<<(unsigned)((ly.n_out + 255) / 256), 256, 0, s>>>(B, ly.n_out, S.G, ly.ld_out, S.grads + ly.off_b);
-    k_to_bf16<<<blocks(B * ly.n_out), 256, 0, s>>>(B, ly.n_out, S.G, ly.ld_out, S.Gb, S.maxw, 0);
-    dim3 tg((unsigned)((ly.n_out + 31) / 32), (unsigned)((B + 31) / 32));
-    k_to_bf16_t<<<tg, dim3(32, 8), 0, s>>>(B, ly.n_out, S.G, ly.ld_out, S.GTb, S.ldB, 0);
     // dW = g^T h  (M = n_out, N = n_in, K = B; B is a multiple of 8, so the
     // 8-element loads never reach columns a larger earlier batch left behind)
-    st = gemm(S, ly.n_out, ly.n_in, B, S.GTb, S.ldB, S.HTb[l], S.ldB, S.dW, ly.ld_in, nullptr, s);
-    if (st != FZP_OK) return st;
-    k_pack<<<blocks(ly.n_out * ly.n_in), 256, 0, s>>>(ly.n_out, ly.n_in, S.dW, ly.ld_in, S.grads + ly.off_w);
-    if (l > 0) {
-      // dh = g W  (M = B, N = n_in, K = n_out), then g = dh silu'(z_{l-1})
-      st = gemm(S, B, ly.n_in, ly.ld_out, S.Gb, S.maxw, ly.WTb, ly.ld_out, S.dH, S.L[l - 1].ld_out, nullptr, s);
-      if (st != FZP_OK) return st;
-      k_silu_back<<<blocks(B * ly.n_in), 256, 0, s>>>(B, ly.n_in, S.dH, S.Z[l - 1], S.L[l - 1].ld_out, S.G);
+    Gemm w = product(ly.n_out, ly.n_in, B, S.GTb[cur], S.ldB, S.HTb[l], S.ldB, EPI_DW);
+    w.C = grads + ly.off_w;
+    w.ldc = ly.n_in;
+    w.bsums = S.sums[cur];
+    w.ld_sums = S.maxw;
+    w.nsums = (int)((B + GM - 1) / GM);
+    w.db = grads + ly.off_b;
+    if (l == 0) {
+      const Layer& lo = S.L[nl - 1];
+      w.loss = d_loss;
+      w.lpart = S.lpart;
+      w.nlpart = (int)(((B + GM - 1) / GM) * ((lo.n_out + GN - 1) / GN));
+      w.loss_scale = 1.0 / ((double)B * (double)lo.n_out);
+      return run_gemm(S, w, nullptr, s);
     }
+    // dh = g W  (M = B, N = n_in, K = n_out), then g = dh silu'(z_{l-1})
+    Gemm h = product(B, ly.n_in, ly.ld_out, S.Gb[cur], S.maxw, ly.WTb, ly.ld_out, EPI_DH);
+    h.Z = S.Z[l - 1];
+    h.ldz = S.L[l - 1].ld_out;
+    h.rows = S.Gb[cur ^ 1];
+    h.ldr = S.maxw;
+    h.cols = S.GTb[cur ^ 1];
+    h.ldt = S.ldB;
+    h.sums = S.sums[cur ^ 1];
+    h.ld_sums = S.maxw;
+    const fzp_status st = run_gemm(S, h, &w, s);
+    if (st != FZP_OK) return st;
   }
-  FZP_CUDA_TRY(cudaGetLastError());
-  return FZP_OK;
-}
-
-// h^T copies are needed by the weight gradient: refresh them from Hb after forward.
-fzp_status transposed_inputs(fzp_surrogate_s& S, const float* x, int64_t B, cudaStream_t s) {
-  for (size_t l = 0; l < S.L.size(); ++l) {
-    const Layer& ly = S.L[l];
-    const float* src = l == 0 ? x : S.Z[l - 1];
-    const int64_t lds = l == 0 ? ly.n_in : S.L[l - 1].ld_out;
-    dim3 tg((unsigned)((ly.n_in + 31) / 32), (unsigned)((B + 31) / 32));
-    k_to_bf16_t<<<tg, dim3(32, 8), 0, s>>>(B, ly.n_in, src, lds, S.HTb[l], S.ldB, l == 0 ? 0 : 1);
-  }
-  FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
 }
 
@@ -355,11 +498,10 @@ fzp_status refresh_weights(fzp_surrogate_s& S, cudaStream_t s) {
   return FZP_OK;
 }
 
-fzp_status grad_all(fzp_surrogate_s& S, const float* x, const float* y, int64_t B, float* d_loss, cudaStream_t s) {
-  fzp_status st = forward(S, x, B, s);
-  if (st == FZP_OK) st = transposed_inputs(S, x, B, s);
-  if (st == FZP_OK) st = backward(S, y, B, d_loss, s);
-  return st;
+fzp_status grad_all(fzp_surrogate_s& S, const float* x, const float* y, int64_t B, float* grads, float* d_loss,
+                    cudaStream_t s) {
+  const fzp_status st = forward(S, x, B, y, nullptr, s);
+  return st == FZP_OK ? backward(S, B, grads, d_loss, s) : st;
 }
 
 void surrogate_release(fzp_surrogate_s* S) {
@@ -430,20 +572,21 @@ fzp_status fzp_surrogate_create(int n_in, int hidden, int n_hidden_layers, int n
     S->Hb.push_back((__nv_bfloat16*)A(sizeof(__nv_bfloat16) * max_batch * ly.ld_in));
     S->HTb.push_back((__nv_bfloat16*)A(sizeof(__nv_bfloat16) * ly.ld_in * S->ldB));
   }
-  S->G = (float*)A(sizeof(float) * max_batch * maxw);
-  S->dH = (float*)A(sizeof(float) * max_batch * maxw);
-  S->dW = (float*)A(sizeof(float) * maxw * maxw);
-  S->Gb = (__nv_bfloat16*)A(sizeof(__nv_bfloat16) * max_batch * maxw);
-  S->GTb = (__nv_bfloat16*)A(sizeof(__nv_bfloat16) * maxw * S->ldB);
+  for (int q = 0; q < 2; ++q) {
+    S->Gb[q] = (__nv_bfloat16*)A(sizeof(__nv_bfloat16) * max_batch * maxw);
+    S->GTb[q] = (__nv_bfloat16*)A(sizeof(__nv_bfloat16) * maxw * S->ldB);
+    S->sums[q] = (float*)A(sizeof(float) * (size_t)((max_batch + GM - 1) / GM) * maxw);
+  }
+  S->lpart = (double*)A(sizeof(double) * (size_t)(((max_batch + GM - 1) / GM) * ((S->L.back().n_out + GN - 1) / GN)));
   if (!ok) {
     cudaGetLastError();
     surrogate_release(S);
     return set_error(FZP_E_OOM, "surrogate allocation failed");
   }
   static std::atomic<uint64_t> attr{0};
-  if (smem_attr_once((const void*)k_gemm_tn, GEMM_SMEM, attr) != cudaSuccess) {
+  if (smem_attr_once((const void*)k_gemm, GEMM_SMEM, attr) != cudaSuccess) {
     surrogate_release(S);
-    return set_error(FZP_E_CUDA, "cudaFuncSetAttribute(k_gemm_tn)");
+    return set_error(FZP_E_CUDA, "cudaFuncSetAttribute(k_gemm)");
   }
   // weights ~ U(-1/sqrt(fan_in), 1/sqrt(fan_in)); biases zero
   for (const Layer& ly : S->L)
@@ -477,12 +620,7 @@ fzp_status fzp_surrogate_params(fzp_surrogate_t S, float* h_buf, size_t count, i
 fzp_status fzp_surrogate_infer(fzp_surrogate_t S, const float* d_x, int batch, float* d_y, void* stream) {
   if (!S || !d_x || !d_y || batch < 1 || batch > S->max_batch) return set_error(FZP_E_INVALID, "bad infer arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  fzp_status st = forward(*S, d_x, batch, s);
-  if (st != FZP_OK) return st;
-  const Layer& lo = S->L.back();
-  FZP_CUDA_TRY(cudaMemcpy2DAsync(d_y, lo.n_out * sizeof(float), S->Z.back(), lo.ld_out * sizeof(float),
-                                 lo.n_out * sizeof(float), batch, cudaMemcpyDeviceToDevice, s));
-  return FZP_OK;
+  return forward(*S, d_x, batch, nullptr, d_y, s);
 }
 
 fzp_status fzp_surrogate_grad(fzp_surrogate_t S, const float* d_x, const float* d_y, int batch, float* d_grad,
@@ -490,10 +628,7 @@ fzp_status fzp_surrogate_grad(fzp_surrogate_t S, const float* d_x, const float* 
   if (!S || !d_x || !d_y || batch < 8 || batch > S->max_batch || (batch % 8) != 0)
     return set_error(FZP_E_INVALID, "bad grad arguments (batch must be a multiple of 8)");
   cudaStream_t s = (cudaStream_t)stream;
-  fzp_status st = grad_all(*S, d_x, d_y, batch, d_loss, s);
-  if (st != FZP_OK) return st;
-  if (d_grad) FZP_CUDA_TRY(cudaMemcpyAsync(d_grad, S->grads, S->n_params * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  return FZP_OK;
+  return grad_all(*S, d_x, d_y, batch, d_grad ? d_grad : S->grads, d_loss, s);
 }
 
 fzp_status fzp_surrogate_train_step(fzp_surrogate_t S, const float* d_x, const float* d_y, int batch, float lr,
@@ -501,20 +636,17 @@ fzp_status fzp_surrogate_train_step(fzp_surrogate_t S, const float* d_x, const f
   if (!S || !d_x || !d_y || batch < 8 || batch > S->max_batch || (batch % 8) != 0 || !(lr > 0))
     return set_error(FZP_E_INVALID, "bad train arguments (batch must be a multiple of 8, lr > 0)");
   cudaStream_t s = (cudaStream_t)stream;
-  fzp_status st = grad_all(*S, d_x, d_y, batch, d_loss, s);
+  fzp_status st = grad_all(*S, d_x, d_y, batch, S->grads, d_loss, s);
   if (st != FZP_OK) return st;
   S->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)S->step), c2 = 1.f - powf(b2, (float)S->step);
-  for (const Layer& ly : S->L) {
-    k_adamw<<<blocks(ly.n_in * ly.n_out), 256, 0, s>>>(ly.n_in * ly.n_out, S->params + ly.off_w,
-                                                       S->grads + ly.off_w, S->m + ly.off_w, S->v + ly.off_w, lr,
-                                                       weight_decay, b1, b2, 1e-8f, c1, c2);
-    k_adamw<<<blocks(ly.n_out), 256, 0, s>>>(ly.n_out, S->params + ly.off_b, S->grads + ly.off_b, S->m + ly.off_b,
-                                             S->v + ly.off_b, lr, 0.f, b1, b2, 1e-8f, c1, c2);
-  }
+  for (const Layer& ly : S->L)  // off_b follows the layer's weights
+    k_adamw<<<blocks((ly.n_in + 1) * ly.n_out), 256, 0, s>>>(ly.n_out, ly.n_in, S->params + ly.off_w, S->grads + ly.off_w,
+                                                             S->m + ly.off_w, S->v + ly.off_w, lr, weight_decay, b1, b2,
+                                                             1e-8f, c1, c2, ly.Wb, ly.ld_in, ly.WTb, ly.ld_out);
   FZP_CUDA_TRY(cudaGetLastError());
-  return refresh_weights(*S, s);
+  return FZP_OK;
 }
 
 fzp_status fzp_surrogate_destroy(fzp_surrogate_t S) {

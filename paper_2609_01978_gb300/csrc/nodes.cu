@@ -132,8 +132,10 @@ __device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t ad, uint64_t b
       : "memory");
 }
 
-__device__ __forceinline__ int64_t isqrt_floor(int64_t t) {  // largest a with a^2 <= t (t >= 0)
-  int64_t a = (int64_t)sqrt((double)t);
+// Largest a with a^2 <= t, 0 <= t < 2^46: the FP32 root is within 2 of it (an
+// FP64 root costs thousands of clocks at two FP64 lanes per SM).
+__device__ __forceinline__ int64_t isqrt_floor(int64_t t) {
+  int64_t a = (int64_t)sqrtf((float)t);
   while (a * a > t) --a;
   while ((a + 1) * (a + 1) <= t) ++a;
   return a;
@@ -799,10 +801,15 @@ __device__ __forceinline__ double sinc_d(double z) { return fabs(z) < 1e-9 ? 1.0
 struct InterpSpec {
   int n, ns, M, Mo, even;
   double h, c, half;  // node pitch and band (radians) per ROI half width; half width in pitches
+  double msh, chirp;  // ROI shift; p^2 / (2 lambda f)
 };
 
 __global__ void __launch_bounds__(512) k_interp_W(const InterpSpec a, const double* __restrict__ F, double* __restrict__ W,
-                                                  double* __restrict__ Wy) {
+                                                  double* __restrict__ Wy, double2* __restrict__ chirp) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.M; i += gridDim.x * blockDim.x) {
+    const double t = (double)i - a.msh;
+    chirp[i] = cis_turns_d(t * t * a.chirp);
+  }
   __shared__ double pivot[2][4];
   const int ns = a.ns, r = threadIdx.x % ns, q = threadIdx.x / ns, o = blockIdx.x * 4 + q;
   const double xo = (a.even ? (double)o : (double)o - 0.5 * (a.M - 1)) / a.half;
@@ -851,22 +858,26 @@ __global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, con
                                                      const double2* __restrict__ V, double2* __restrict__ X) {
   const int l = blockIdx.x * 32 + (threadIdx.x & 31), o = blockIdx.y * 4 + (threadIdx.x >> 5);
   if (o >= Mo) return;
-  double2 x = make_double2(0.0, 0.0);
-#pragma unroll 8
-  for (int k = 0; k < ny; ++k) {
-    const double2 v = V[k * ns + l];
-    const double w = Wy[k * Mo + o];
-    x.x = fma(w, v.x, x.x);
-    x.y = fma(w, v.y, x.y);
-  }
-  X[l * Mo + o] = x;
+  double2 x[4];  // four chains: an FP64 multiply-add's latency is long
+#pragma unroll
+  for (int q = 0; q < 4; ++q) x[q] = make_double2(0.0, 0.0);
+#pragma unroll 2
+  for (int k = 0; k < ny; k += 4)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double2 v = V[(k + q) * ns + l];
+      const double w = Wy[(k + q) * Mo + o];
+      x[q].x = fma(w, v.x, x[q].x);
+      x[q].y = fma(w, v.y, x[q].y);
+    }
+  X[l * Mo + o] = make_double2((x[0].x + x[1].x) + (x[2].x + x[3].x), (x[0].y + x[1].y) + (x[2].y + x[3].y));
 }
 
 struct InterpOut {
   int M, ns;
   int Moy, eveny, Mox, evenx;  // outputs of the two axes (even: M / 2 + 1)
   int sym;                     // the field is this one plus its transpose
-  double msh, p, lf, f_over_lambda, amp;
+  double2 pre;                 // e^{ikf} dx^2 / (i lambda f)
   int accumulate;
 };
 
@@ -874,49 +885,40 @@ struct InterpOut {
 // exchanged; only blocks on and below the diagonal run and both are stored),
 // the output chirp and prefactor, and the stores: with an even field output o
 // stands for the samples M/2 + o and M/2 - o (o = M/2: sample 0 alone).
-// Block: 8 x 8 outputs, one per thread.
-constexpr int IT = 8;
-__global__ void __launch_bounds__(IT * IT) k_interp_cols(const InterpOut a, const double* __restrict__ W,
-                                                         const double2* __restrict__ X, double2* __restrict__ out) {
-  if (a.sym && blockIdx.x > blockIdx.y) return;
-  __shared__ double2 chy[IT], chx[IT];
-  const int n0 = blockIdx.y * IT, m0 = blockIdx.x * IT;
-  const int tm = threadIdx.x % IT, tn = threadIdx.x / IT;
+// Block: 8 x 4 outputs (columns x rows), one per thread.  chirp[i] = e^{i pi
+// x_i^2 / (lambda f)} of the ROI samples, as k_interp_W left it.
+constexpr int ITX = 8, ITY = 4;
+__global__ void __launch_bounds__(ITX * ITY) k_interp_cols(const InterpOut a, const double* __restrict__ W,
+                                                           const double2* __restrict__ X,
+                                                           const double2* __restrict__ chirp, double2* __restrict__ out) {
+  const int n0 = blockIdx.y * ITY, m0 = blockIdx.x * ITX;
+  if (a.sym && m0 >= n0 + ITY) return;
   const int h = a.M / 2;
-  if (threadIdx.x < 2 * IT) {  // e^{i pi x^2 / (lambda f)} of the block's outputs, the prefactor with the rows'
-    const bool rowaxis = threadIdx.x < IT;
-    const int o = (rowaxis ? n0 : m0) + threadIdx.x % IT;
-    const int i = (rowaxis ? a.eveny : a.evenx) ? (h + o) % a.M : o;
-    const double x = ((double)i - a.msh) * a.p;
-    double2 w = cis_turns_d(x * x / (2.0 * a.lf) + (rowaxis ? frac_turns(a.f_over_lambda) - 0.25 : 0.0));
-    if (rowaxis) {
-      w.x *= a.amp;
-      w.y *= a.amp;
-      chy[threadIdx.x] = w;
-    } else {
-      chx[threadIdx.x - IT] = w;
-    }
-  }
-  const int on = n0 + tn, om = m0 + tm;
+  const int on = n0 + (int)threadIdx.x / ITX, om = m0 + (int)threadIdx.x % ITX;
   const int cn = min(on, a.Moy - 1), cm = min(om, a.Mox - 1);
-  double2 u = make_double2(0.0, 0.0), t = u;
-#pragma unroll 8
-  for (int l = 0; l < a.ns; ++l) {
-    const double2 x = __ldg(X + l * a.Moy + cn);
-    const double w = __ldg(W + l * a.Mox + cm);
-    u.x = fma(w, x.x, u.x);
-    u.y = fma(w, x.y, u.y);
-    if (a.sym) {
-      const double2 y = __ldg(X + l * a.Moy + cm);
-      const double v = __ldg(W + l * a.Mox + cn);
-      t.x = fma(v, y.x, t.x);
-      t.y = fma(v, y.y, t.y);
+  double2 u[2], t[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) u[q] = t[q] = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int l = 0; l < a.ns; l += 2)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double2 x = __ldg(X + (l + q) * a.Moy + cn);
+      const double w = __ldg(W + (l + q) * a.Mox + cm);
+      u[q].x = fma(w, x.x, u[q].x);
+      u[q].y = fma(w, x.y, u[q].y);
+      if (a.sym) {
+        const double2 y = __ldg(X + (l + q) * a.Moy + cm);
+        const double v = __ldg(W + (l + q) * a.Mox + cn);
+        t[q].x = fma(v, y.x, t[q].x);
+        t[q].y = fma(v, y.y, t[q].y);
+      }
     }
-  }
-  __syncthreads();
   if (on >= a.Moy || om >= a.Mox || (a.sym && om > on)) return;
-  const double2 v = cmul(cmul(make_double2(u.x + t.x, u.y + t.y), chx[tm]), chy[tn]);
-  const int n = a.eveny ? (h + on) % a.M : on, m = a.evenx ? (h + om) % a.M : om;
+  const int n = a.eveny ? (on < h ? h + on : 0) : on, m = a.evenx ? (om < h ? h + om : 0) : om;
+  const double2 v = cmul(cmul(make_double2((u[0].x + u[1].x) + (t[0].x + t[1].x), (u[0].y + u[1].y) + (t[0].y + t[1].y)),
+                              cmul(chirp[n], chirp[m])),
+                         a.pre);
   auto put = [&](int nn, int mm) {
     double2* o = out + (int64_t)nn * a.M + mm;
     double2 z = v;
@@ -1174,17 +1176,18 @@ fzp_status nodes_upload(Plan& P) {
   NodeSet& z = P.nd;
   const bool full = z.even && P.owns_buffers;
   const size_t nw = (size_t)z.ns * z.Mo, nf = (size_t)z.ns * z.ns * (full ? 4 : 2);
-  const size_t total = nw + (full ? (size_t)z.n * P.M : 0) + nf;
+  const size_t total = nw + (full ? (size_t)z.n * P.M : 0) + nf + 2 * (size_t)P.M;
   FZP_CUDA_TRY(cudaMalloc(&z.d_W, total * sizeof(double)));
   P.device_bytes += total * sizeof(double);
   z.d_Wy = full ? z.d_W + nw : z.d_W;
   double* dL = z.d_W + (total - nf);
+  z.d_chirp = reinterpret_cast<double2*>(dL - 2 * (size_t)P.M);  // 16-byte aligned: even counts throughout
   std::vector<double> L(nf);
-  InterpSpec a{z.n, z.ns, P.M, z.Mo, z.even ? 1 : 0, z.h / z.half, M_PI * z.band * z.half, z.half};
+  InterpSpec a{z.n, z.ns, P.M, z.Mo, z.even ? 1 : 0, z.h / z.half, M_PI * z.band * z.half, z.half, P.msh, P.p * P.p / (2.0 * P.lambda * P.f)};
   node_factor(z.n, z.ns, z.even ? 1 : 0, a.h, a.c, L.data());
   if (full) node_factor(z.n, z.ns, -1, a.h, a.c, L.data() + (size_t)2 * z.ns * z.ns);
   FZP_CUDA_TRY(cudaMemcpy(dL, L.data(), nf * sizeof(double), cudaMemcpyHostToDevice));
-  k_interp_W<<<(unsigned)((z.Mo + 3) / 4), 4 * z.ns>>>(a, dL, z.d_W, full ? z.d_Wy : nullptr);
+  k_interp_W<<<(unsigned)((z.Mo + 3) / 4), 4 * z.ns>>>(a, dL, z.d_W, full ? z.d_Wy : nullptr, z.d_chirp);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
@@ -1243,11 +1246,12 @@ fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cuda
   const int ny = z.yfull ? z.n : z.ns, Moy = eveny ? z.Mo : P.M;
   k_interp_rows<<<dim3((unsigned)(z.ns / 32), (unsigned)((Moy + 3) / 4)), 128, 0, s>>>(
       ny, z.ns, Moy, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
-  const double lf = P.lambda * P.f;
-  InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, sym ? 1 : 0, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf,
-              accumulate};
-  k_interp_cols<<<dim3((unsigned)((z.Mo + IT - 1) / IT), (unsigned)((Moy + IT - 1) / IT)), IT * IT, 0, s>>>(
-      a, z.d_W, z.d_X, reinterpret_cast<double2*>(d_field));
+  // e^{ikf} / i: f / lambda - 1/4 turns
+  const double turns = std::fmod(P.f / P.lambda, 1.0) - 0.25, amp = P.dx2 / (P.lambda * P.f);
+  InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, sym ? 1 : 0,
+              make_double2(amp * std::cos(2.0 * M_PI * turns), amp * std::sin(2.0 * M_PI * turns)), accumulate};
+  k_interp_cols<<<dim3((unsigned)((z.Mo + ITX - 1) / ITX), (unsigned)((Moy + ITY - 1) / ITY)), ITX * ITY, 0, s>>>(
+      a, z.d_W, z.d_X, z.d_chirp, reinterpret_cast<double2*>(d_field));
   P.launches += 2;
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
