@@ -831,15 +831,18 @@ def main():
                 "work": work,
                 "disc_samples_per_launch": inside * args.steps / launches}
     elif args.form == "saczt":
-        # k_sa_rows<1>: one pass of the padded grid through HBM (P^2 complex64
-        # read and written) with two transforms and the residual phase between
+        # k_sa_half<2>: the quadrant's half spectra read (FP32, N / 2 values for
+        # each of the P / 2 + 1 frequencies), the lower triangle of the spectrum
+        # written as two real planes, two transforms' length and the phase between
         Pg = info["fft_length"]
-        bytes_launch = 2.0 * 8.0 * Pg * Pg
+        bytes_launch = 4.0 * (Pg / 2 + 1) * (info["c"] + 1) + 8.0 * (Pg / 2 + 1) ** 2 / 2
+        if not prof["dominant_name"].startswith("k_sa_half"):
+            bytes_launch = 2.0 * 8.0 * Pg * Pg  # k_sa_rows<1>: the padded grid read and written
         achieved = bytes_launch / (avg_ms / 1e3) / 1e9
         peak = peaks["hbm_gbs"]
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": None, "kernel": prof["dominant_name"], "peak_source": peak_kind + " HBM copy",
-                "work": "16 P^2 bytes per launch (P = padded grid side)"}
+                "work": "bytes of the dominant pass over the spectrum"}
     else:
         launches = max(1, prof["dominant_launches"])
         flat = not wl.get("deform")

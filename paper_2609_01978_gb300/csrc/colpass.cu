@@ -27,6 +27,8 @@ struct ColArgs {
   int slices;       // images of C1 to be summed, slice_off values apart
   int64_t slice_off;
   int64_t sin_off;  // > 0: C1 holds the rows of Re T and, sin_off values on, of Im T
+  const float2* E;
+  int64_t estride;
   int M;          // outputs per row (m)
   double kappa, delta;
   double msh;     // ROI (or node) shift in pitches: y_n = (n - msh) p
@@ -62,7 +64,8 @@ __device__ __forceinline__ double2 kern(const RowPhase<double>& rp, int n) {
 }
 
 // grid (M/TM, M/TN, ceil(rows/jc)); 256 threads; each thread 4 n x 4 m outputs.
-template <typename R>
+// TAB: the kernel's columns from a table E [n][estride] instead of their phase.
+template <typename R, bool TAB = false>
 __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
   using C = typename Cplx<R>::T;
   __shared__ C sK[TJ][TN + 1];
@@ -82,7 +85,7 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     for (int b = 0; b < 4; ++b) { acc[a][b].x = 0; acc[a][b].y = 0; }
   for (int64_t j = jb; j < je; j += TJ) {
     const int pj = (int)(j - jb) & (PJ - 1);
-    if (pj == 0) {
+    if (!TAB && pj == 0) {
       const int r = tid & (PJ - 1);
       if (j + r < je && (tid < PJ || g.kind == ROWS_FOLDED)) {
         const double dj = (double)(g.j0 + j + r - g.c);
@@ -113,10 +116,14 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     }
     __syncthreads();
     for (int t = tid; t < TJ * TN; t += 256) {
-      const int jj = t / TN, nn = t % TN;
+      const int jj = TAB ? t % TJ : t / TN, nn = TAB ? t / TJ : t % TN;
       C k;
       k.x = 0; k.y = 0;
-      if (j + jj < je) {
+      if (TAB && j + jj < je) {
+        const float2 e = __ldg(g.E + (int64_t)(n0 + nn) * g.estride + j + jj);
+        k.x = e.x;
+        k.y = e.y;
+      } else if (j + jj < je) {
         k = kern(sP[0][pj + jj], n0 + nn);
         if (g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c) k = cadd(k, kern(sP[1][pj + jj], n0 + nn));
       }
@@ -210,6 +217,45 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   dim3 grid((unsigned)(g.M / TM), (unsigned)(ny / TN), (unsigned)((rows + g.jc - 1) / g.jc));
   if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
   else k_colpass<float><<<grid, 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+fzp_status column_pass_table(Plan& P, const void* E, int64_t rows, int64_t estride, cudaStream_t s) {
+  ColArgs g{};
+  g.rows = rows;
+  g.c1_stride = P.c1_stride;
+  g.M = P.nd.ns;
+  g.wr = 1.0;
+  g.slices = 1;
+  g.sin_off = 2 * P.nd.ns * P.c1_stride;
+  g.E = reinterpret_cast<const float2*>(E);
+  g.estride = estride;
+  const int t = g.M / TM;
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * t * t / 304 + TJ - 1) / TJ * TJ));
+  k_colpass<float, true><<<dim3((unsigned)t, (unsigned)t, (unsigned)((rows + g.jc - 1) / g.jc)), 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+fzp_status column_pass_zoom(Plan& P, int64_t rows, double lz, cudaStream_t s) {
+  const NodeSet& z = P.nd;
+  ColArgs g{};
+  g.c = rows / 2;
+  g.rows = rows;
+  g.c1_stride = P.c1_stride;
+  g.M = z.ns;
+  g.kappa = P.dx2 / lz;
+  g.delta = z.h * P.p * P.dx / lz;
+  g.msh = z.yfull ? 0.5 * (z.n - 1) : z.msh;
+  g.wr = 1.0;
+  g.slices = 1;
+  g.sin_off = 2 * z.ns * P.c1_stride;
+  const int tx = g.M / TM, ty = (z.yfull ? z.n : z.ns) / TN;
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tx * ty / 304 + TJ - 1) / TJ * TJ));
+  k_colpass<float><<<dim3((unsigned)tx, (unsigned)ty, (unsigned)((rows + g.jc - 1) / g.jc)), 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;

@@ -219,6 +219,7 @@ struct NodeSet {
   double half = 0, h = 0;  // ROI half width and node pitch, in ROI pitches
   double band = 0;         // 2 R p / (lambda f): the field's band, cycles per pitch
   double delta = 0, msh = 0;  // the nodes as a grid: x_k = (k - msh) h p, delta = h p dx / (lambda f)
+  double dist = 0;         // distance of the output chirp (f, or the SA-CZT's z_F)
   double* d_W = nullptr;   // interpolation [ns][Mo] (owned by the plan, also in a batch)
   double* d_Wy = nullptr;  // [n][M], behind d_W: along y when the rows are not symmetric
   bool yfull = false;      // the call being run takes all n nodes along y
@@ -245,6 +246,13 @@ struct SaCzt {
   void* d_RT = nullptr;    // M x P complex64: row pass, transposed
   int64_t* d_xthr = nullptr;  // exact radii: first s of every zone m = 1 .. nx
   int64_t nx = 0;
+  // whole apertures on nodes: the zoom kernel's transform E, its operand
+  // images and the work list of the contraction
+  void* d_E = nullptr;     // [nodes][E stride] complex64
+  void* d_EA = nullptr;
+  void* d_ZA = nullptr;    // images of K itself over the padded columns (a part of the rows)
+  int* d_esched = nullptr;
+  int64_t estride = 0;     // P / 2 + 32: the frequencies 0 .. P / 2 and padding
 };
 
 struct Plan {
@@ -344,6 +352,17 @@ fzp_status nodes_fill(Plan& P, cudaStream_t s);
 fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s);
 fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t s);
 fzp_status nodes_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t s);
+// Contraction of a real FP32 matrix [rows][stride] (lower: a symmetric one, its
+// lower triangle) of kblocks x 32 columns with node columns: row pass into the
+// rows part * 2 ns .. of C1.  Images from a table, or of the SA-CZT's zoom kernel.
+fzp_status nodes_table_images(Plan& P, const void* E, int64_t ncols, int64_t stride, int64_t kblocks, void* A);
+fzp_status nodes_loaded_rows(Plan& P, const float* src, int64_t rows, int64_t stride, int64_t kblocks, const void* A,
+                             int* sched, int part, bool lower, cudaStream_t s);
+fzp_status nodes_zoom_images(Plan& P, int64_t ncols, int64_t kblocks, void* A);
+// The column pass of that contraction: both parts, kernel columns from E, or of
+// the zoom kernel of the distance z (lz = lambda z) over `rows` padded rows.
+fzp_status column_pass_zoom(Plan& P, int64_t rows, double lz, cudaStream_t s);
+fzp_status column_pass_table(Plan& P, const void* E, int64_t rows, int64_t estride, cudaStream_t s);
 fzp_status column_pass_tc(Plan& P, int64_t j0, int64_t rows, cudaStream_t stream);
 // The same with the pass's field weighted by (wr + i wi).
 fzp_status column_pass_tc_w(Plan& P, int64_t j0, int64_t rows, double wr, double wi, cudaStream_t stream);
@@ -354,6 +373,7 @@ fzp_status epilogue_z(Plan& P, void* d_field, int accumulate, double z, cudaStre
 fzp_status saczt_layout(Plan& P);                      // P, fit, z_F (host)
 fzp_status saczt_build(Plan& P);                       // allocate and fill its tables
 fzp_status saczt_propagate(Plan& P, int64_t j0, int64_t j1, cudaStream_t stream);  // into d_Uacc
+bool saczt_folds(const Plan& P, int64_t j0, int64_t j1);  // the range is the whole aperture and the plan has nodes
 fzp_status saczt_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t stream);
 fzp_status intensity(Plan& P, const void* d_field, void* d_I, cudaStream_t stream);
 fzp_status metrics(Plan& P, const void* d_field, cudaStream_t stream, fzp_metrics_t* out);

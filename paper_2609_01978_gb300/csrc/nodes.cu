@@ -73,7 +73,7 @@ constexpr int EPI_BOX = 32;
 constexpr int EPI_BYTES = EPI_WARPS * 2 * EPI_BOX * EPI_BOX * 4;  // two boxes per warp
 constexpr int ERR_BASE = 300;
 
-enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4 };
+enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4, MASK_LOADED = 5 };
 
 // Fixed-point zone phase: phase64(s) = s K mod 2^64 (K = floor(kappa 2^63): the
 // zone's parity is the top bit; MASK_LEVELS: K = floor(kappa_L / L 2^64), the
@@ -99,6 +99,9 @@ struct NodeArgs {
   int nchunks, group, promote;
   int slices;               // images of C1, chunk g adds into image g slices / nchunks
   DeformCoef df;            // membrane
+  const float* ld_src;      // loaded operand: row j at ld_src + j ld_stride
+  int64_t ld_stride;
+  int y_off;                // first row of C1
   const uint8_t* A;
   int* err;
 };
@@ -106,12 +109,14 @@ struct NodeArgs {
 template <int NT, int MASK>
 struct Shape {
   static constexpr bool CX = MASK == MASK_MEMBRANE;
+  static constexpr bool LD = MASK == MASK_LOADED;                 // a real FP32 matrix in place of the masks
   static constexpr bool TWO = CX || MASK == MASK_QUAD;            // two masks: one accumulator each
-  static constexpr int BN = (NT == 1 && !TWO) ? 512 : 256;        // rows per unit
-  static constexpr int PLANES = CX ? 4 : TWO ? 2 : BN / 256;      // mask planes per stage
+  static constexpr int BN = (NT == 1 && !TWO && !LD) ? 512 : 256; // rows per unit
+  static constexpr int PLANES = CX ? 4 : (TWO || LD) ? 2 : BN / 256;  // mask planes per stage
+  static constexpr int ACCS = LD && NT == 1 ? 1 : 2;              // accumulators
   static constexpr int A_BYTES = NT * 2 * SUB;
   static constexpr int B_BYTES = PLANES * PLANE;
-  static constexpr int STAGES = CX ? 2 : 4;
+  static constexpr int STAGES = CX || (LD && NT == 2) ? 2 : 4;
   static constexpr int C1_ROWS = NT * 128 * (TWO ? 2 : 1);
   static constexpr int SMEM = 1024 + STAGES * (A_BYTES + B_BYTES) + EPI_BYTES + 256;
   static_assert(!TWO || NT == 1, "two node tiles of two masks need more tensor memory than there is");
@@ -146,6 +151,11 @@ __device__ __forceinline__ int64_t isqrt_floor(int64_t t) {
 // nearest the axis; with the octant, columns below je only.  At least one
 // block (every stripe writes its rows of C1).
 __device__ __forceinline__ void stripe_kspan(const NodeArgs& a, int64_t jb, int64_t je, int64_t& klo, int64_t& khi) {
+  if (a.ld_src) {  // dense: no chord
+    klo = 0;
+    khi = a.octant && (je + BK - 1) / BK < a.kblocks ? (je + BK - 1) / BK : a.kblocks;
+    return;
+  }
   const int64_t c = a.mg.c;
   const int64_t jn = c < jb ? jb : (c >= je ? je - 1 : c);
   const int64_t t = a.mg.sR - (jn - c) * (jn - c);
@@ -184,7 +194,9 @@ __global__ void __launch_bounds__(1024) k_nodes_prep(const NodeArgs a, int* sche
   const int64_t ns = a.n_stripes;
   int64_t sc = a.mg.c < a.j_begin ? 0 : (a.mg.c - a.j_begin) / BN;
   if (sc >= ns) sc = ns - 1;
-  if (a.octant) {
+  if (a.ld_src) {
+    sc = ns - 1;  // the last stripe's span holds the others'
+  } else if (a.octant) {
     int64_t lo = 0, hi = ns - 1;  // first stripe whose chord ends below its last row
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
@@ -485,7 +497,7 @@ __device__ __forceinline__ bool stage_wait(uint64_t* bar, uint32_t parity, volat
 template <int NT, int MASK>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, const __grid_constant__ CUtensorMap tmC1) {
   using S = Shape<NT, MASK>;
-  constexpr bool CX = S::CX, TWO = S::TWO;
+  constexpr bool CX = S::CX, LD = S::LD;
   constexpr int NST = S::STAGES, BN = S::BN;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -582,18 +594,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
               const uint64_t o = (uint64_t)((ks * 32) >> 4);
               const uint32_t acc = (kb > p0 || ks > 0) ? 1u : 0u;
 #pragma unroll
-              for (int q = 0; q < 2; ++q) {
+              for (int q = 0; q < S::ACCS; ++q) {
                 // flat: accumulator q = row half q (NT = 1) or node tile q (NT = 2);
                 // two masks: q = 0, 1; membrane planes 2q (hi) and 2q + 1 (lo)
                 const uint32_t dt = tmem + (uint32_t)(q * 256);
                 const int at = NT == 2 ? q : 0;
-                const int bp = CX ? 2 * q : (NT == 2 ? 0 : q);
+                const int bp = CX ? 2 * q : (NT == 2 || LD ? 0 : q);
                 const uint64_t a_hi = ad + (uint64_t)((at * SUB) >> 4) + o;
                 const uint64_t a_lo = ad + (uint64_t)(((NT + at) * SUB) >> 4) + o;
                 const uint64_t b0 = bd + (uint64_t)((bp * PLANE) >> 4) + o;
                 mma_bf16(dt, a_hi, b0, acc);
                 mma_bf16(dt, a_lo, b0, 1u);
-                if (CX) mma_bf16(dt, a_hi, b0 + (uint64_t)(PLANE >> 4), 1u);
+                if (CX || LD) mma_bf16(dt, a_hi, b0 + (uint64_t)(PLANE >> 4), 1u);
               }
             }
             mma_commit(&empty[stage]);
@@ -644,7 +656,29 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
         for (; b < nkb; b += 2) {
           const uint32_t one = b >= diag ? 0x3F003F00u : 0x3F803F80u;
           uint8_t* rp = rowbase + stage * S::B_BYTES;
-          if constexpr (CX) {
+          if constexpr (LD) {
+            const int64_t j = un.jb + row;
+            const float h = b >= diag ? 0.5f : 1.0f;
+            float4 v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j < un.je) {
+              const float4* src = reinterpret_cast<const float4*>(a.ld_src + j * a.ld_stride + (un.kb0 + b) * BK);
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[q] = __ldg(src + q);
+            }
+            if (!stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              uint32_t hi[4], lo[4];
+              split2(h * v[2 * q].x, h * v[2 * q].y, hi[0], lo[0]);
+              split2(h * v[2 * q].z, h * v[2 * q].w, hi[1], lo[1]);
+              split2(h * v[2 * q + 1].x, h * v[2 * q + 1].y, hi[2], lo[2]);
+              split2(h * v[2 * q + 1].z, h * v[2 * q + 1].w, hi[3], lo[3]);
+              *reinterpret_cast<uint4*>(rp + ((q ^ sw) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+              *reinterpret_cast<uint4*>(rp + PLANE + ((q ^ sw) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            }
+          } else if constexpr (CX) {
             const uint32_t bits = block_open(w[0], a.mg, a.ph);
             if (!stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
             cx_store2(a.df, cxr, w[0].di0, bits, rp, PLANE, sw);
@@ -700,9 +734,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
         if (!epi_ok[accph]) { ok = false; break; }
         tc_fence_after();
 #pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < S::ACCS; ++q) {
           const int xs = BN == 512 ? q * 256 : 0, x0 = (int)(un.jb - a.j_begin) + xs;
-          const int y0 = un.slice * S::C1_ROWS + (BN == 512 ? 0 : q * 128) + warp * 32;
+          const int y0 = a.y_off + un.slice * S::C1_ROWS + (BN == 512 ? 0 : q * 128) + warp * 32;
           const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(q * 256);
           const int xn = min(256, rows - xs);  // live columns (may be <= 0)
 #pragma unroll 1
@@ -775,6 +809,35 @@ __global__ void k_nodes_A(int nt, int64_t ncols, int64_t kblocks, int64_t c, int
     for (int u = 0; u < 4; ++u) {
       split2(re[2 * u], re[2 * u + 1], rh[u], rl[u]);
       split2(im[2 * u], im[2 * u + 1], ih[u], il[u]);
+    }
+    const int k = (int)(k8 & 3);
+    uint8_t* blk = A + (k8 >> 2) * (int64_t)(nt * 2 * SUB);
+    auto put = [&](int plane, int rr, const uint32_t (&v)[4]) {
+      *reinterpret_cast<uint4*>(blk + plane * SUB + (rr >> 3) * 512 + (rr & 7) * 64 + ((k ^ ((rr & 7) >> 1)) << 4)) =
+          make_uint4(v[0], v[1], v[2], v[3]);
+    };
+    put(t, r, rh);
+    put(nt + t, r, rl);
+    put(t, 64 + r, ih);
+    put(nt + t, 64 + r, il);
+  }
+}
+
+// The same images from a table E [node][stride] of complex columns.
+__global__ void k_nodes_table(int nt, int64_t ncols, int64_t kblocks, const float2* __restrict__ E, int64_t stride,
+                              uint8_t* A) {
+  const int64_t total = kblocks * 4 * (int64_t)nt * 64;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k8 = e % (kblocks * 4);
+    const int node = (int)(e / (kblocks * 4)), t = node >> 6, r = node & 63;
+    uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = 8 * k8 + 2 * u;
+      const float2 a = i < ncols ? E[(int64_t)node * stride + i] : make_float2(0.f, 0.f);
+      const float2 b = i + 1 < ncols ? E[(int64_t)node * stride + i + 1] : make_float2(0.f, 0.f);
+      split2(a.x, b.x, rh[u], rl[u]);
+      split2(a.y, b.y, ih[u], il[u]);
     }
     const int k = (int)(k8 & 3);
     uint8_t* blk = A + (k8 >> 2) * (int64_t)(nt * 2 * SUB);
@@ -1087,7 +1150,7 @@ fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
   // chunks of a unit's stripe add by twos into separate images of C1, which
   // the column pass sums in order.  Larger plates add into one image.
   a.slices = 1;
-  if (P.N <= 256 * BK) {
+  if (P.N <= 256 * BK && !S::LD) {
     const int64_t cap = std::max<int64_t>(1, (int64_t)(c1_elems(P) / ((size_t)c1r * P.c1_stride)));
     a.group = (int)std::max<int64_t>(a.group, (a.kblocks + 2 * cap - 1) / (2 * cap));
     a.nchunks = (int)((a.kblocks + a.group - 1) / a.group);
@@ -1096,14 +1159,15 @@ fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
   P.nd.slices = a.slices;
   P.nd.slice_elems = (int64_t)c1r * P.c1_stride;
   CUtensorMap tm;
-  st = c1_map(P, P.c1_stride, c1r * a.slices, &tm);
+  st = c1_map(P, P.c1_stride, a.y_off + c1r * a.slices, &tm);
   if (st != FZP_OK) return st;
   const int64_t vec = (int64_t)c1r * P.c1_stride * a.slices / 4;
   const unsigned zb = (unsigned)std::min<int64_t>(2 * P.dn.num_sms, (vec + 4095) / 4096);
-  k_nodes_prep<S::BN><<<1 + zb, 1024, 0, s>>>(a, P.dn.d_sched, reinterpret_cast<float4*>(P.d_C1), vec);
-  prof_begin(P, s);
+  k_nodes_prep<S::BN><<<1 + zb, 1024, 0, s>>>(a, const_cast<int*>(a.sched),
+                                             reinterpret_cast<float4*>(P.d_C1 + (size_t)a.y_off * P.c1_stride), vec);
+  if (!S::LD) prof_begin(P, s);  // (the SA-CZT's dominant kernel is another)
   k_nodes<NT, MASK><<<P.dn.num_sms, NUM_THREADS, S::SMEM, s>>>(a, tm);
-  prof_end(P, s);
+  if (!S::LD) prof_end(P, s);
   P.launches += 2;
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
@@ -1117,22 +1181,15 @@ fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
 // and so do plates of 6 and more levels (L/2 passes: the plain FP32 form's
 // single pass is the faster one there) and membranes that need two node tiles
 // (four accumulators do not fit the tensor memory).
-void nodes_choose(Plan& P) {
+// Sets the nodes for a field of `band` cycles per ROI pitch (both signs), if
+// some count of at most `hi` stored nodes holds it.
+static void place_nodes(Plan& P, bool even, double band, int hi) {
   NodeSet& z = P.nd;
-  z = NodeSet{};
-  const bool dense = P.form == FZP_FORM_DENSE && P.precision == FZP_PREC_SPLIT_BF16 && P.cluster_req <= 1 && P.levels <= 4;
-  const bool seg = P.form == FZP_FORM_BLUESTEIN && P.precision == FZP_PREC_FP32 && P.conv_req != 1;
-  if (!dense && !seg) return;
-  const bool flat = !P.has_deform;
-  const bool centred = P.msh == (double)(P.M / 2);
-  const bool even = flat && centred;
-  const double half = even ? 0.5 * P.M : 0.5 * (P.M - 1);  // half width of the ROI, pitches
-  const double band = 2.0 * P.R / (P.lambda * P.f) * P.p;  // cycles per pitch, both signs
-  const double dof = 2.0 * half * band;
-  struct { int n; double most; } sizes[] = {{64, 36.0}, {128, 80.0}, {256, 170.0}};
-  for (auto& q : sizes) {
+  const double half = even ? 0.5 * P.M : 0.5 * (P.M - 1);
+  const struct { int n; double most; } sizes[] = {{64, 36.0}, {128, 80.0}, {256, 170.0}};
+  for (const auto& q : sizes) {
     const int ns = even ? q.n / 2 : q.n;
-    if (ns < 64 || ns > 128 || (dense && !flat && ns > 64) || dof > q.most) continue;
+    if (ns < 64 || ns > hi || 2.0 * half * band > q.most) continue;
     z.n = q.n;
     z.ns = ns;
     break;
@@ -1142,13 +1199,29 @@ void nodes_choose(Plan& P) {
   z.Mo = even ? P.M / 2 + 1 : P.M;
   z.half = half;
   z.band = band;
-  const double h = 2.0 * half * 1.25 / z.n;  // node pitch in ROI pitches: a margin of a quarter
+  z.h = 2.0 * half * 1.25 / z.n;  // node pitch in ROI pitches: a margin of a quarter
   const double centre = even ? 0.0 : 0.5 * (P.M - 1) - P.msh;
-  z.h = h;
-  z.delta = P.delta * h;
+  z.delta = P.delta * z.h;
   // node k at x = (k - msh) h: the first stored node
-  const double first = centre + ((even ? z.n / 2 : 0) - 0.5 * (z.n - 1)) * h;
-  z.msh = -first / h;
+  const double first = centre + ((even ? z.n / 2 : 0) - 0.5 * (z.n - 1)) * z.h;
+  z.msh = -first / z.h;
+}
+
+void nodes_choose(Plan& P) {
+  P.nd = NodeSet{};
+  const bool centred = P.msh == (double)(P.M / 2);
+  if (P.form == FZP_FORM_SACZT) {
+    // the propagated plane fills the padded grid, P dx wide, at the distance z_F
+    if (saczt_layout(P) == FZP_OK) place_nodes(P, centred, (double)P.sa.P * P.dx * P.p / (P.lambda * P.sa.zF), 128);
+    P.nd.dist = P.sa.zF;
+    return;
+  }
+  P.nd.dist = P.f;
+  const bool dense = P.form == FZP_FORM_DENSE && P.precision == FZP_PREC_SPLIT_BF16 && P.cluster_req <= 1 && P.levels <= 4;
+  const bool seg = P.form == FZP_FORM_BLUESTEIN && P.precision == FZP_PREC_FP32 && P.conv_req != 1;
+  if (!dense && !seg) return;
+  const bool flat = !P.has_deform;
+  place_nodes(P, flat && centred, 2.0 * P.R / (P.lambda * P.f) * P.p, dense && !flat ? 64 : 128);
 }
 
 bool nodes_two_masks(const Plan& P) {
@@ -1183,7 +1256,7 @@ fzp_status nodes_upload(Plan& P) {
   double* dL = z.d_W + (total - nf);
   z.d_chirp = reinterpret_cast<double2*>(dL - 2 * (size_t)P.M);  // 16-byte aligned: even counts throughout
   std::vector<double> L(nf);
-  InterpSpec a{z.n, z.ns, P.M, z.Mo, z.even ? 1 : 0, z.h / z.half, M_PI * z.band * z.half, z.half, P.msh, P.p * P.p / (2.0 * P.lambda * P.f)};
+  InterpSpec a{z.n, z.ns, P.M, z.Mo, z.even ? 1 : 0, z.h / z.half, M_PI * z.band * z.half, z.half, P.msh, P.p * P.p / (2.0 * P.lambda * z.dist)};
   node_factor(z.n, z.ns, z.even ? 1 : 0, a.h, a.c, L.data());
   if (full) node_factor(z.n, z.ns, -1, a.h, a.c, L.data() + (size_t)2 * z.ns * z.ns);
   FZP_CUDA_TRY(cudaMemcpy(dL, L.data(), nf * sizeof(double), cudaMemcpyHostToDevice));
@@ -1240,6 +1313,44 @@ fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream
                                : launch<2, MASK_LEVELS>(P, a, s);
 }
 
+fzp_status nodes_table_images(Plan& P, const void* E, int64_t ncols, int64_t stride, int64_t kblocks, void* A) {
+  const int64_t threads = kblocks * 4 * P.nd.ns;
+  k_nodes_table<<<(unsigned)std::min<int64_t>(8 * P.dn.num_sms, (threads + 255) / 256), 256>>>(
+      P.nd.ns / 64, ncols, kblocks, reinterpret_cast<const float2*>(E), stride, reinterpret_cast<uint8_t*>(A));
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+fzp_status nodes_zoom_images(Plan& P, int64_t ncols, int64_t kblocks, void* A) {
+  const NodeSet& z = P.nd;
+  const double lz = P.lambda * z.dist;
+  const int64_t threads = kblocks * 4 * z.ns;
+  k_nodes_A<<<(unsigned)std::min<int64_t>(8 * P.dn.num_sms, (threads + 255) / 256), 256>>>(
+      z.ns / 64, ncols, kblocks, ncols / 2, 0, P.dx2 / lz, z.msh, z.h * P.p * P.dx / lz, reinterpret_cast<uint8_t*>(A));
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  return FZP_OK;
+}
+
+fzp_status nodes_loaded_rows(Plan& P, const float* src, int64_t rows, int64_t stride, int64_t kblocks, const void* A,
+                             int* sched, int part, bool lower, cudaStream_t s) {
+  NodeArgs a{};
+  a.j_end = rows;
+  a.octant = lower ? 1 : 0;
+  a.kblocks = kblocks;
+  a.promote = 128;
+  a.group = (int)std::min<int64_t>(64, std::max<int64_t>(8, rows / 256 * kblocks / (lower ? 2 : 1) / (3 * P.dn.num_sms)));
+  a.nchunks = (int)((kblocks + a.group - 1) / a.group);
+  a.sched = sched;
+  a.ld_src = src;
+  a.ld_stride = stride;
+  a.A = reinterpret_cast<const uint8_t*>(A);
+  a.err = P.d_err;
+  a.y_off = part * P.nd.ns * 2;
+  return P.nd.ns == 64 ? launch<1, MASK_LOADED>(P, a, s) : launch<2, MASK_LOADED>(P, a, s);
+}
+
 fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cudaStream_t s) {
   const NodeSet& z = P.nd;
   const bool eveny = z.even && !z.yfull;
@@ -1247,7 +1358,7 @@ fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cuda
   k_interp_rows<<<dim3((unsigned)(z.ns / 32), (unsigned)((Moy + 3) / 4)), 128, 0, s>>>(
       ny, z.ns, Moy, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
   // e^{ikf} / i: f / lambda - 1/4 turns
-  const double turns = std::fmod(P.f / P.lambda, 1.0) - 0.25, amp = P.dx2 / (P.lambda * P.f);
+  const double turns = std::fmod(P.f / P.lambda, 1.0) - 0.25, amp = P.dx2 / (P.lambda * z.dist);
   InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, sym ? 1 : 0,
               make_double2(amp * std::cos(2.0 * M_PI * turns), amp * std::sin(2.0 * M_PI * turns)), accumulate};
   k_interp_cols<<<dim3((unsigned)((z.Mo + ITX - 1) / ITX), (unsigned)((Moy + ITY - 1) / ITY)), ITX * ITY, 0, s>>>(

@@ -88,7 +88,7 @@ void release_plan(Plan* P) {
   if (P->nd.d_W) cudaFree(P->nd.d_W);
   if (P->owns_buffers) {
     void* ptrs[] = {P->d_C1, P->d_C1d, P->d_Uacc, P->d_err, P->d_metrics,
-                    P->bs.d_pre, P->bs.d_H, P->bs.d_Z, P->bs.d_G, P->bs.d_tab, P->dn.d_A, P->dn.d_sched, P->nd.d_X,
+                    P->bs.d_pre, P->bs.d_H, P->bs.d_Z, P->bs.d_G, P->bs.d_tab, P->dn.d_A, P->dn.d_sched, P->nd.d_X, P->sa.d_E, P->sa.d_EA, P->sa.d_ZA, P->sa.d_esched,
                     P->sa.d_G, P->sa.d_T, P->sa.d_tw, P->sa.d_K, P->sa.d_RT, P->sa.d_xthr};
     for (void* q : ptrs)
       if (q) cudaFree(q);
@@ -572,13 +572,16 @@ fzp_status fzp_propagate_roi(fzp_plan_t plan, int64_t row_begin, int64_t row_end
   disc_rows(P, jlo, jhi);
   const int64_t a = std::max(row_begin, jlo), b = std::min(row_end, jhi);
   if (P.form == FZP_FORM_SACZT) {
-    FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, (size_t)P.M * P.M * sizeof(double2), s));
+    const bool fold = saczt_folds(P, a, b), nodes = P.nd.n > 0;
+    P.nd.yfull = P.nd.even && !fold;
+    const size_t acc = nodes ? (size_t)(P.nd.yfull ? P.nd.n : P.nd.ns) * P.nd.ns : (size_t)P.M * P.M;
+    FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, acc * sizeof(double2), s));
     // the whole padded plane at once (rows outside the range masked to zero)
     if (a < b) {
       const fzp_status st = saczt_propagate(P, a, b, s);
       if (st != FZP_OK) return st;
     }
-    return epilogue_z(P, d_field, accumulate, P.sa.zF, s);
+    return nodes ? nodes_epilogue(P, d_field, accumulate, fold, s) : epilogue_z(P, d_field, accumulate, P.sa.zF, s);
   }
   bool sym = false;
   const fzp_status st = propagate_rows(P, a, b, &sym, s);

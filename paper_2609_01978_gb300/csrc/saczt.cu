@@ -397,6 +397,144 @@ __global__ void __launch_bounds__(512, 1) k_sa_rows(const SaRowArgs a) {
   }
 }
 
+// ---------------------------------------------------------------- whole apertures
+// The whole plate is a function of di^2 + dj^2 and so is the residual phase, so
+// with the grid's origin on the axis the spectrum A is real, even in both
+// frequencies and its own transpose, and the field needs neither the inverse
+// transforms nor three quarters of the rest:
+//   U[n, m] = sum_{fy, fx} E[n, fy] (H A)[fy, fx] E[m, fx],
+//   E[x, f] = sum_q K(x, q) e^{2 pi i f q / P}   (the zoom kernel's transform),
+// over the frequencies 0 .. P / 2 with E[x, f] + E[x, -f] in E's place.  Two
+// real rows share a complex transform (both spectra are real: one comes out as
+// the real part, the other as the imaginary part).  Frequencies stay in
+// bit-reversed order: with 2^13 of them position s of the half spectrum holds
+// frequency brev(2 s) and position P / 2 the Nyquist frequency P / 2, on both
+// axes, E's columns alike.  Only the lower triangle of H A (by positions, in
+// 256-row tiles) is formed; it is contracted on the tensor cores onto the
+// interpolation nodes (nodes.cu).
+// D = 8 mm (P = 16,384), ROI 512^2: 15.66 -> 1.79 ms a propagation (the row
+// transforms 11.1 -> 1.34 ms), error against 64 bits 1.6e-5 -> 1.1e-6.
+struct SaHalfArgs {
+  int64_t P;
+  int logP;
+  const float2* tw;
+  SaMaskArgs m;
+  SaPhase ph;
+  int64_t nd;        // distances from the axis: rows (columns) 0 .. nd - 1 of the quadrant
+  int64_t rs;        // row stride of the half spectra: P / 2 + 32
+  const float* in;   // step 2: [position][nd32] half spectra of the rows, transposed
+  int64_t is;        // its stride
+  float* out;        // step 1: [distance][rs]; step 2: two planes [position][rs]
+  int64_t plane;
+  int M;             // table: nodes as a grid (x = (k - msh) h)
+  double msh, h, lzF, dx;
+  float2* E;         // table: [node][rs]
+};
+
+// Frequency index (0 .. P / 2) at position s of a half spectrum.
+__device__ __forceinline__ int half_freq(int s, int P, int logP) { return s < P / 2 ? sa_brev(2 * s, logP) : P / 2; }
+
+// STEP 1: rows 2 b and 2 b + 1 of the quadrant (distances from the axis) as
+// real and imaginary part, transformed; STEP 2: positions 2 b and 2 b + 1 of the
+// transposed half spectra likewise, times the residual phase; STEP 3: node b's
+// kernel row K(x, q) + K(x, -q), transformed with the other sign.
+template <int STEP>
+__global__ void __launch_bounds__(512, 1) k_sa_half(const SaHalfArgs a) {
+  extern __shared__ float2 x[];
+  const int P = (int)a.P, logP = a.logP, H = P / 2;
+  float2* tws = x + (P + P / 32);
+  tw_load(tws, a.tw, P);
+  const int r0 = STEP == 3 ? blockIdx.x : 2 * blockIdx.x;
+  // element q and its mirror image P - q
+  for (int q = threadIdx.x; q <= H; q += blockDim.x) {
+    float2 v = make_float2(0.0f, 0.0f);
+    if (STEP == 1) {
+      if (q < a.nd) {
+        v.x = sa_open(a.m, r0, q) ? 1.0f : 0.0f;
+        v.y = r0 + 1 < a.nd && sa_open(a.m, r0 + 1, q) ? 1.0f : 0.0f;
+      }
+    } else if (STEP == 2) {
+      if (q < a.nd) {
+        v.x = __ldg(a.in + (int64_t)r0 * a.is + q);
+        if (r0 + 1 <= H) v.y = __ldg(a.in + (int64_t)(r0 + 1) * a.is + q);
+      }
+    } else {
+      const double u = (double)q * a.dx, xk = ((double)r0 - a.msh) * a.h, c = 0.5 * u * u;
+      const float2 k0 = cis_turns_f((c - xk * u) / a.lzF), k1 = cis_turns_f((c + xk * u) / a.lzF);
+      // K(x, q) + K(x, -q); the grid's last sample q = -P/2 has no mirror image
+      v = q < H ? cadd(k0, k1) : make_float2(2.0f * k1.x, 2.0f * k1.y);
+      v.y = -v.y;  // the transform of the conjugate is the conjugate of the other sign's
+    }
+    x[spad(q)] = v;
+    if (q > 0 && q < H) x[spad(P - q)] = v;
+  }
+  __syncthreads();
+  row_fft_fwd(x, P, logP, tws);
+  if (STEP == 1) {
+    float* o0 = a.out + (int64_t)r0 * a.rs;
+    const bool two = r0 + 1 < a.nd;
+    for (int s = threadIdx.x; s <= H; s += blockDim.x) {
+      const float2 v = x[spad(s < H ? 2 * s : 1)];
+      o0[s] = v.x;
+      if (two) o0[a.rs + s] = v.y;
+    }
+  } else if (STEP == 2) {
+    // the tile of 256 positions that holds r0 ends the row; padding reads as zero
+    const int end = min((r0 / 256 + 1) * 256, (int)a.rs);
+    const int64_t fx0 = half_freq(r0, P, logP), fx1 = r0 + 1 <= H ? half_freq(r0 + 1, P, logP) : 0;
+    float* re = a.out + (int64_t)r0 * a.rs;
+    float* im = re + a.plane;
+    for (int s = threadIdx.x; s < end; s += blockDim.x) {
+      float2 h0 = make_float2(0.0f, 0.0f), h1 = h0;
+      if (s <= H) {
+        const float2 v = x[spad(s < H ? 2 * s : 1)];
+        const int64_t fy = half_freq(s, P, logP), fy2 = fy * fy;
+        const int64_t s0 = fx0 * fx0 + fy2, s1 = fx1 * fx1 + fy2;
+        if (s0 < a.ph.s_ev) {
+          float sn, cs;
+          sincospif(2.0f * sa_turns(a.ph, s0), &sn, &cs);
+          h0 = make_float2(a.ph.scale * v.x * cs, a.ph.scale * v.x * sn);
+        }
+        if (s1 < a.ph.s_ev) {
+          float sn, cs;
+          sincospif(2.0f * sa_turns(a.ph, s1), &sn, &cs);
+          h1 = make_float2(a.ph.scale * v.y * cs, a.ph.scale * v.y * sn);
+        }
+      }
+      re[s] = h0.x;
+      im[s] = h0.y;
+      if (r0 + 1 <= H) {
+        re[a.rs + s] = h1.x;
+        im[a.rs + s] = h1.y;
+      }
+    }
+  } else {
+    float2* e = a.E + (int64_t)r0 * a.rs;
+    for (int s = threadIdx.x; s < (int)a.rs; s += blockDim.x) {
+      float2 v = make_float2(0.0f, 0.0f);
+      if (s <= H) {
+        v = x[spad(s < H ? 2 * s : 1)];
+        // frequencies 0 and P / 2 are their own mirror images
+        const float w = s == 0 || s == H ? 0.5f : 1.0f;
+        v = make_float2(w * v.x, -w * v.y);
+      }
+      e[s] = v;
+    }
+  }
+}
+
+// out[x][y] = in[y][x], ny x nx floats (32 x 32 tiles, block 32 x 8).
+__global__ void k_sa_transpose_r(const float* __restrict__ in, int64_t is, int64_t ny, int64_t nx, float* __restrict__ out,
+                                 int64_t os) {
+  __shared__ float tile[32][33];
+  const int64_t x0 = (int64_t)blockIdx.x * 32, y0 = (int64_t)blockIdx.y * 32;
+  for (int r = threadIdx.y; r < 32; r += 8)
+    tile[r][threadIdx.x] = y0 + r < ny && x0 + threadIdx.x < nx ? in[(y0 + r) * is + x0 + threadIdx.x] : 0.0f;
+  __syncthreads();
+  for (int r = threadIdx.y; r < 32; r += 8)
+    if (x0 + r < nx && y0 + threadIdx.x < ny) out[(x0 + r) * os + y0 + threadIdx.x] = tile[threadIdx.x][r];
+}
+
 // K[m][q] = e^{i k0 u_q^2 / (2 z_F) - i k0 x_m u_q / z_F}, u_q = (q - P/2) dx,
 // x_m = (m - msh) p; the phase in turns reduced in FP64.
 __global__ void k_sa_kernel(int M, int64_t P, double msh, double p, double dx, double lzF, float2* __restrict__ K) {
@@ -553,8 +691,64 @@ fzp_status saczt_layout(Plan& P) {
   return FZP_OK;
 }
 
-// The zoom runs on the tensor cores when the column pass's 128-row tiles fit M.
+// Without nodes (a band too wide for them) the zoom runs on the tensor cores
+// when the column pass's 128-row tiles fit M.
 static bool saczt_zoom_tc(const Plan& P) { return P.M % 128 == 0; }
+
+// Rows of the half spectra, padded to whole K blocks and 16 bytes.
+static int64_t half_stride(const SaCzt& s) { return s.P / 2 + 32; }
+
+static SaHalfArgs half_args(const Plan& P) {
+  SaHalfArgs a{};
+  a.P = P.sa.P;
+  a.logP = P.sa.logP;
+  a.tw = reinterpret_cast<const float2*>(P.sa.d_tw);
+  a.nd = P.c + 1;
+  a.rs = half_stride(P.sa);
+  return a;
+}
+
+// The whole-aperture path's tables: E on the nodes, its images, interpolation.
+static fzp_status saczt_nodes_build(Plan& P) {
+  SaCzt& s = P.sa;
+  NodeSet& z = P.nd;
+  int dev = 0;
+  FZP_CUDA_TRY(cudaGetDevice(&dev));
+  FZP_CUDA_TRY(cudaDeviceGetAttribute(&P.dn.num_sms, cudaDevAttrMultiProcessorCount, dev));
+  s.estride = half_stride(s);
+  const int64_t kb = s.estride / 32;
+  const int64_t zkb = s.P / 32;  // the zoom of a part of the rows: K over the padded columns
+  const size_t eb = (size_t)z.ns * s.estride * sizeof(float2), ab = (size_t)kb * (z.ns / 64) * 16384,
+               zb = (size_t)zkb * (z.ns / 64) * 16384, xb = (size_t)z.ns * P.M * sizeof(double2),
+               sb = sizeof(int) * (size_t)(3 * ((std::max(kb, zkb) + 7) / 8) + 1);
+  FZP_CUDA_TRY(cudaMalloc(&s.d_E, eb));
+  FZP_CUDA_TRY(cudaMalloc(&s.d_EA, ab));
+  FZP_CUDA_TRY(cudaMalloc(&s.d_ZA, zb));
+  FZP_CUDA_TRY(cudaMalloc(&z.d_X, xb));
+  FZP_CUDA_TRY(cudaMalloc(&s.d_esched, sb));
+  P.device_bytes += eb + ab + zb + xb + sb;
+  static std::atomic<uint64_t> a1{0}, a2{0}, a3{0};
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_sa_half<1>, (int)rows_smem(SA_PMAX), a1));
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_sa_half<2>, (int)rows_smem(SA_PMAX), a2));
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_sa_half<3>, (int)rows_smem(SA_PMAX), a3));
+  SaHalfArgs a = half_args(P);
+  a.msh = z.msh;
+  a.h = z.h * P.p;
+  a.lzF = P.lambda * s.zF;
+  a.dx = P.dx;
+  a.E = reinterpret_cast<float2*>(s.d_E);
+  k_sa_half<3><<<(unsigned)z.ns, rows_threads(s.P), rows_smem(s.P)>>>(a);
+  P.launches += 1;
+  FZP_CUDA_TRY(cudaGetLastError());
+  fzp_status st = nodes_table_images(P, s.d_E, s.P / 2 + 1, s.estride, kb, s.d_EA);
+  if (st == FZP_OK) st = nodes_zoom_images(P, s.P, zkb, s.d_ZA);
+  return st == FZP_OK ? nodes_upload(P) : st;
+}
+
+bool saczt_folds(const Plan& P, int64_t j0, int64_t j1) {
+  const int64_t up = j1 - 1 - P.c, dn = P.c - j0;
+  return P.nd.n > 0 && up == dn && (up == P.c || (up + 1) * (up + 1) > P.mg.sR);
+}
 
 fzp_status saczt_build(Plan& P) {
   SaCzt& s = P.sa;
@@ -581,6 +775,9 @@ fzp_status saczt_build(Plan& P) {
   k_sa_twiddles<<<grid_for(s.P / 2), 256>>>(s.P, reinterpret_cast<float2*>(s.d_tw));
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
+  if (P.nd.n > 0) {
+    return saczt_nodes_build(P);
+  }
   if (saczt_zoom_tc(P)) {
     // kernel images of K over the P padded columns: u = (q - P/2) dx, so the
     // phase is di^2 kappa / 2 - (m - msh) di delta turns with z_F for f
@@ -597,13 +794,50 @@ fzp_status saczt_build(Plan& P) {
   return FZP_OK;
 }
 
+// The whole aperture through the half spectra (k_sa_half), the contraction on
+// the nodes, into the node accumulator.
+static fzp_status saczt_whole(Plan& P, cudaStream_t st) {
+  const SaCzt& s = P.sa;
+  SaHalfArgs a = half_args(P);
+  a.m = mask_args(P, 0, P.N);
+  a.m.mg.c = 0;  // rows and columns are distances
+  a.ph = sa_phase_consts(P);
+  const int64_t np = s.P / 2 + 1, ds = (a.nd + 31) / 32 * 32;  // positions; stride of the transposed half spectra
+  float* R1 = reinterpret_cast<float*>(s.d_T);                 // [distance][rs]
+  float* T1 = R1 + a.nd * a.rs;                                // [position][ds]
+  float* S2 = reinterpret_cast<float*>(s.d_G);                 // two planes [position][rs]
+  const unsigned nt = rows_threads(s.P);
+  const size_t smem = rows_smem(s.P);
+  a.out = R1;
+  k_sa_half<1><<<(unsigned)((a.nd + 1) / 2), nt, smem, st>>>(a);
+  k_sa_transpose_r<<<dim3((unsigned)((np + 31) / 32), (unsigned)((a.nd + 31) / 32)), dim3(32, 8), 0, st>>>(
+      R1, a.rs, a.nd, np, T1, ds);
+  a.in = T1;
+  a.is = ds;
+  a.out = S2;
+  a.plane = np * a.rs;
+  P.dominant = "k_sa_half<2> (forward transforms, residual phase)";
+  prof_begin(P, st);
+  k_sa_half<2><<<(unsigned)((np + 1) / 2), nt, smem, st>>>(a);
+  prof_end(P, st);
+  P.launches += 3;
+  FZP_CUDA_TRY(cudaGetLastError());
+  P.nd.yfull = false;
+  for (int part = 0; part < 2; ++part) {
+    const fzp_status e = nodes_loaded_rows(P, S2 + part * a.plane, np, a.rs, a.rs / 32, s.d_EA, s.d_esched, part, true, st);
+    if (e != FZP_OK) return e;
+  }
+  return column_pass_table(P, s.d_E, np, s.estride, st);
+}
+
 fzp_status saczt_propagate(Plan& P, int64_t j0, int64_t j1, cudaStream_t st) {
+  if (saczt_folds(P, j0, j1)) return saczt_whole(P, st);
   const SaCzt& s = P.sa;
   float2* G = reinterpret_cast<float2*>(s.d_G);
   float2* T = reinterpret_cast<float2*>(s.d_T);
   const float2* tw = reinterpret_cast<const float2*>(s.d_tw);
   const dim3 tgrid((unsigned)(s.P / 32), (unsigned)(s.P / 32)), tblock(32, 8);
-  const bool tc = saczt_zoom_tc(P);
+  const bool nodes = P.nd.n > 0, tc = nodes || saczt_zoom_tc(P);
   SaRowArgs ra{};
   ra.P = s.P;
   ra.logP = s.logP;
@@ -633,6 +867,15 @@ fzp_status saczt_propagate(Plan& P, int64_t j0, int64_t j1, cudaStream_t st) {
   FZP_CUDA_TRY(cudaGetLastError());
   // the Fresnel part on the ROI: C1[m][v] = sum_u K[m][u] U1[v][u], then
   // U[n][m] += sum_v K[n][v] C1[m][v] into the FP64 accumulator
+  if (nodes) {  // a part of the rows: the field is even along x only, all nodes along y
+    P.nd.yfull = P.nd.even;
+    for (int part = 0; part < 2; ++part) {
+      const fzp_status e = nodes_loaded_rows(P, reinterpret_cast<const float*>(T) + (size_t)part * s.P * s.P, s.P, s.P,
+                                             s.P / 32, s.d_ZA, s.d_esched, part, false, st);
+      if (e != FZP_OK) return e;
+    }
+    return column_pass_zoom(P, s.P, P.lambda * s.zF, st);
+  }
   if (tc) {
     const float* re = reinterpret_cast<const float*>(T);
     for (int part = 0; part < 2; ++part) {
