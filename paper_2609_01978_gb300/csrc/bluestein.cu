@@ -32,6 +32,8 @@
 #include <cmath>
 
 #include "fzp_internal.cuh"
+#include "membrane.cuh"
+#include "zone_phase.cuh"
 
 namespace fzp {
 namespace {
@@ -161,6 +163,7 @@ struct RowArgs {
   int S;             // partitioned convolution: columns per block
   int64_t nseg;      // partitioned convolution: blocks per row (spectra in H)
   int64_t col0;      // partitioned convolution: first column of block 0
+  PhaseRule ph;      // partitioned convolution: the zone phase of the mask walk
   int half;          // even output grid: columns from the axis on, outputs m and M - 1 - m added
   int octant;        // columns up to the row's distance from the axis only, the last one halved
 };
@@ -565,37 +568,24 @@ constexpr int STH = 256;          // threads per block
 constexpr int SB0 = 256 * 17;     // transpose buffer A->B: [t][k0], row pitch 17
 constexpr int SB1 = 16 * 273;     // transpose buffer B->C: [k0][c][a], pitches 273 and 17
 constexpr int SBUF = SB1 > SB0 ? SB1 : SB0;
-constexpr size_t SEG_SMEM = sizeof(float2) * (2 * SBUF + 15 * 256 + 256 + 64) + sizeof(uint32_t) * 512;
+constexpr int NO_LEVEL = 64;      // level byte of a column outside the disc: phasor 0
+constexpr size_t SEG_SMEM = sizeof(float2) * (2 * SBUF + 15 * 256 + 256 + NO_LEVEL + 2) + SP;
 // row kernels: binary plate (chunk bits), phase plate (chunk zone steps),
 // deformed binary plate (chunk bits and the membrane phasor), general
 // transmission (a deformed phase plate)
 enum { SEG_FLAT = 0, SEG_LEVELS = 1, SEG_MEMBRANE = 2, SEG_GENERAL = 3 };
 
-// Membrane phasor e^{i phi} of the sample at (fi, fj) = (i - c, j - c) for the
-// FP32 partitioned pass: phi / 2 pi = 2 w / lambda from the FP32 coefficients
-// (the wrinkle's turns as in the transmission function: di kxh exact, its
-// integer part dropped exactly), the wrinkle's turns and the total reduced to
-// [-1/2, 1/2] before the hardware sine and cosine (absolute error below 4e-7
-// each).  Row terms: fjkh = fj kyh, fjkl = fj kyl, fj2 = fj^2, cr[e] = (fj -
-// pj_e) ny_e - pi_e nx_e, so a ridge's distance is fi nx_e + cr[e].
-__device__ __forceinline__ float2 membrane_phasor(const DeformCoef& d, float fi, float fjkh, float fjkl, float fj2,
-                                                  const float (&cr)[3]) {
-  constexpr float TWO_PI = 6.28318530717958648f;
-  const float th = fmaf(fi, d.kxh, fjkh);
-  float tt = (th - rintf(th)) + fmaf(fi, d.kxl, fjkl);
-  tt -= rintf(tt);
-  float wz = d.amp2 * __sinf(TWO_PI * tt) * fmaf(-d.tq, fmaf(fi, fi, fj2), 1.0f);
+// A membrane's phase (turns, 2 w / lambda) on the 16 columns from di0, CLOSED
+// where the plate is (bits: open columns), to shared memory at a pitch of one.
+constexpr float CLOSED = 1e30f;
+template <int NR>
+__device__ __forceinline__ void membrane_chunk(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits, float* o) {
+  MembraneWalk<NR> walk(d, r, di0);
 #pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    if (e < d.n) {
-      const float dd = fmaf(fi, d.nx[e], cr[e]);
-      wz = fmaf(d.h2[e], __expf(-d.q[e] * dd * dd), wz);
-    }
+  for (int k = 0; k < 16; ++k) {
+    const float w = walk.next();
+    o[k] = ((bits >> k) & 1u) ? w : CLOSED;
   }
-  wz -= rintf(wz);
-  float sn, cs;
-  __sincosf(TWO_PI * wz, &sn, &cs);
-  return make_float2(cs, sn);
 }
 
 // v e^{-2 pi i K / 16}
@@ -699,8 +689,10 @@ __device__ __forceinline__ void seg_twiddles(float2* twA, float2* twB) {
   __syncthreads();
 }
 
+// Largest b with b^2 <= t, 0 <= t < 2^46, from the FP32 root (every thread of a
+// row takes it, and FP64 has two lanes per SM).
 __device__ __forceinline__ int64_t isqrt_row(int64_t t) {
-  int64_t b = (int64_t)sqrt((double)t);
+  int64_t b = (int64_t)sqrtf((float)t);
   while (b > 0 && b * b > t) --b;
   while ((b + 1) * (b + 1) <= t) ++b;
   return b;
@@ -747,51 +739,41 @@ __device__ __forceinline__ uint32_t chunk_bits(int64_t x, int64_t dj2, const Mas
   return bits;
 }
 
-// Zone steps of the 16 columns [x, x + 16) of a row of the phase plate:
-// *z0 the zone at column x, *ud the columns at which the zone steps up
-// (bits 0-15) or down (bits 16-31), so that z(x + p) = z0 + popc(up & m_p) -
-// popc(down & m_p), m_p = bits 0..p.  Away from the axis the steps are the
-// boundaries between the chunk's ends, placed by the window search of
-// chunk_bits (all up right of the axis, all down left of it); within 128
-// columns of it the zone rule runs column by column.  Returns false when two
-// boundaries share a column (possible only at a sampling finer than one
-// sample per level step); the caller then evaluates the zone rule per
-// element.  Columns outside the disc come out arbitrary.
-__device__ __forceinline__ bool chunk_zones(int64_t x, int64_t dj2, const MaskGeom& g, uint32_t* z0, uint32_t* ud) {
-  const int64_t dr = x - g.c, dl = g.c - (x + 15);
-  if (dr < 128 && dl < 128) {
-    int64_t zp = zone_of(min(dj2 + dr * dr, g.sR), g);
-    *z0 = (uint32_t)zp;
-    uint32_t up = 0u, dn = 0u;
-    for (int p = 1; p < 16; ++p) {
-      const int64_t di = dr + p, z = zone_of(min(dj2 + di * di, g.sR), g);
-      if (z == zp + 1) up |= 1u << p;
-      else if (z == zp - 1) dn |= 1u << p;
-      else if (z != zp) return false;
-      zp = z;
+// The zone rule on four columns, a level byte each.
+__device__ __noinline__ uint32_t exact_levels4(int64_t di0, int64_t dj2, const MaskGeom& g) {
+  uint32_t v = 0u;
+  for (int z = 0; z < 4; ++z) {
+    const int64_t di = di0 + z;
+    v |= ((uint32_t)zone_of(min(dj2 + di * di, g.sR), g) % (uint32_t)g.levels) << (8 * z);
+  }
+  return v;
+}
+
+// Levels of the 16 columns from di0 of a row of the phase plate, a byte each in
+// the four words of `lv`: the phase's integer part over L, or, where a phase
+// comes within E of a step, the zone rule column by column.
+__device__ __forceinline__ void chunk_levels(int64_t di0, int64_t dj2, const MaskGeom& g, const PhaseRule& r,
+                                             uint32_t (&lv)[4]) {
+  Walk16 w = walk16(di0, dj2, r);
+  const uint32_t L = (uint32_t)g.levels, el = r.E * L;
+  uint32_t near = 0xFFFFFFFFu;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    uint32_t v = 0u;
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+      const uint64_t p = (uint64_t)w.f * L;
+      near = min(near, (uint32_t)p + el);
+      v |= (uint32_t)(p >> 32) << (8 * z);
+      w.f += w.d;
+      w.d += w.c2;
     }
-    *ud = up | (dn << 16);
-    return true;
+    lv[k] = v;
   }
-  const bool right = dr >= 128;
-  const int64_t d = right ? dr : dl;
-  const int64_t sn = dj2 + d * d, sf = dj2 + (d + 15) * (d + 15);
-  const int64_t zn = zone_of(min(sn, g.sR), g), zf = zone_of(min(sf, g.sR), g);
-  const float inv2d = 0.5f / (float)d;
-  const int32_t td = (int32_t)(2 * d);
-  uint32_t ev = 0u;
-  for (int64_t m = zn + 1; m <= zf; ++m) {
-    const int32_t D = (int32_t)(__ldg(g.thr + (m - 1)) - sn);
-    int32_t k = __float2int_ru((float)D * inv2d);
-    k += (k * (k + td) < D) ? 1 : 0;
-    k -= (k > 0 && (k - 1) * (k - 1 + td) >= D) ? 1 : 0;
-    k -= (k > 0 && (k - 1) * (k - 1 + td) >= D) ? 1 : 0;
-    ev |= 1u << (right ? k : 16 - k);
+  if (near < 2u * el) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) lv[k] = exact_levels4(di0 + 4 * k, dj2, g);
   }
-  if ((int64_t)__popc(ev) != zf - zn) return false;
-  *z0 = (uint32_t)(right ? zn : zf);
-  *ud = right ? ev : (ev << 16);
-  return true;
 }
 
 // G_s = FFT_P(g_s) for every block s (one CTA per block, grid-strided).
@@ -854,15 +836,14 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
   float2* b1 = b0 + SBUF;
   float2* twA = b1 + SBUF;
   float2* twB = twA + 15 * 256;
-  float2* phs = twB + 256;                             // SEG_LEVELS: e^{-2 pi i q / L}, q < L <= 64
-  uint32_t* mk = reinterpret_cast<uint32_t*>(phs + 64);  // per chunk: open bits, or zone at its first column
-  uint32_t* mk2 = mk + 256;                             // per chunk: zone steps up | down << 16
+  float2* phs = twB + 256;                              // SEG_LEVELS: e^{-2 pi i q / L}, q < L <= 64; 0 at NO_LEVEL
+  uint32_t* mk = reinterpret_cast<uint32_t*>(phs + NO_LEVEL + 2);  // SEG_FLAT: open bits per chunk of 16 columns
+  uint8_t* lev = reinterpret_cast<uint8_t*>(mk);        // SEG_LEVELS: level per column
   const uint32_t nlev = (uint32_t)max(a.mg.levels, 1);
-  const uint32_t lmagic = 0xFFFFFFFFu / nlev + 1u;     // z / L = umulhi(z, ceil(2^32 / L)) for z < 2^24
-  if (MODE == SEG_LEVELS && threadIdx.x < nlev) {
+  if (MODE == SEG_LEVELS && threadIdx.x <= NO_LEVEL) {
     float sn, cs;
     sincospif(-2.0f * (float)threadIdx.x / (float)nlev, &sn, &cs);
-    phs[threadIdx.x] = make_float2(cs, sn);
+    phs[threadIdx.x] = threadIdx.x == NO_LEVEL ? make_float2(0.0f, 0.0f) : make_float2(cs, sn);
   }
   seg_twiddles(twA, twB);
   const int t = threadIdx.x;
@@ -879,6 +860,8 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
     float2 acc[16];
 #pragma unroll
     for (int d = 0; d < 16; ++d) acc[d] = make_float2(0.0f, 0.0f);
+    CxRow cxr;
+    if (MODE == SEG_MEMBRANE) cx_row_init(a.df, dj, cxr);
     if (rem >= 0) {
       int64_t bmax = isqrt_row(rem);
       if (FOLD && a.octant) bmax = min(bmax, dj);
@@ -888,78 +871,83 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
       for (int64_t s = (lo - col0) / S; s <= s1; ++s) {
         const int64_t is = col0 + s * (int64_t)S;
         float2 v[16];
-        if (MODE == SEG_FLAT || MODE == SEG_MEMBRANE) {
-          // the block's chord [olo, ohi] in block offsets; loads clamped into
-          // the grid, every element's value decided by its bit alone
-          const int olo = (int)max(lo - is, (int64_t)0), ohi = (int)min(hi - is, (int64_t)(S - 1));
+        // the block's chord [olo, ohi] in block offsets; thread t makes the 16
+        // columns from offset 16 t (element (t, q) is offset t + 256 q)
+        const int olo = (int)max(lo - is, (int64_t)0), ohi = (int)min(hi - is, (int64_t)(S - 1)), xo = 16 * t;
+        const bool meets = t < S / 16 && xo + 15 >= olo && xo <= ohi;
+        const uint32_t inside = meets ? (0xFFFFu >> (15 - min(ohi - xo, 15) + max(olo - xo, 0))) << max(olo - xo, 0) : 0u;
+        if (MODE == SEG_FLAT || MODE == SEG_LEVELS) {
+          // loads clamped into the grid, every element's value decided by its bit or level
           const int lim = (int)min(a.N - 1 - is, (int64_t)(SP - 1));
           const float2* pb = pre + is;
 #pragma unroll
           for (int q = 0; q < 16; ++q) v[q] = __ldg(pb + min(t + 256 * q, lim));
-          // thread t < S/16 makes the bits of block offsets 16 t ... 16 t + 15
-          // (zero outside the chord and beyond S); element (t, q) is offset
-          // 256 q + t: word 16 q + t/16, bit t % 16
-          {
-            const int xo = 16 * t;
-            uint32_t w = 0u;
-            if (t < S / 16 && xo + 15 >= olo && xo <= ohi) {
-              w = chunk_bits(is + xo, dj * dj, a.mg);
-              const int p0 = max(olo - xo, 0), p1 = min(ohi - xo, 15);  // chord within the chunk
-              w &= (0xFFFFu >> (15 - p1 + p0)) << p0;
-            }
-            mk[t] = w;
-          }
+        }
+        if (MODE == SEG_FLAT) {
+          uint32_t w = 0u;
+          if (meets && !walk_bits16(walk16(is + xo - a.mg.c, dj * dj, a.ph), a.ph, w)) w = chunk_bits(is + xo, dj * dj, a.mg);
+          mk[t] = w & inside;
           __syncthreads();
 #pragma unroll
           for (int q = 0; q < 16; ++q)
             if (((mk[16 * q + (t >> 4)] >> (t & 15)) & 1u) == 0) v[q] = make_float2(0.0f, 0.0f);
-          if (MODE == SEG_MEMBRANE) {
-            const float fj = (float)dj;
-            const float fjkh = fj * a.df.kyh, fjkl = fj * a.df.kyl, fj2 = fj * fj;
-            float cr[3];
-#pragma unroll
-            for (int e = 0; e < 3; ++e) cr[e] = (fj - a.df.pj[e]) * a.df.ny[e] - a.df.pi_[e] * a.df.nx[e];
-            const float fi0 = (float)(is + t - a.mg.c);
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-              if (v[q].x != 0.0f || v[q].y != 0.0f)
-                v[q] = cmul(v[q], membrane_phasor(a.df, fi0 + 256.0f * q, fjkh, fjkl, fj2, cr));
-          }
-        } else if (MODE == SEG_LEVELS) {
-          const int olo = (int)max(lo - is, (int64_t)0), ohi = (int)min(hi - is, (int64_t)(S - 1));
+        } else if (MODE == SEG_MEMBRANE) {
+          uint32_t w = 0u;
+          if (meets && !walk_bits16(walk16(is + xo - a.mg.c, dj * dj, a.ph), a.ph, w)) w = chunk_bits(is + xo, dj * dj, a.mg);
+          w &= inside;
+          // phases by chunk through the first transpose buffer (its last readers
+          // are two barriers back; pitch 17 a chunk), the chirp's turns added and
+          // one hardware sine and cosine of the sum reduced to [-1/2, 1/2] turns
+          // (absolute error below 4e-7 each) by element
+          float* wz = reinterpret_cast<float*>(b0);
+          float* o = wz + 17 * t;
+          const float* pt = reinterpret_cast<const float*>(a.pre) + is;
           const int lim = (int)min(a.N - 1 - is, (int64_t)(SP - 1));
-          const float2* pb = pre + is;
+          float tc[16];
 #pragma unroll
-          for (int q = 0; q < 16; ++q) v[q] = __ldg(pb + min(t + 256 * q, lim));
-          // chunk t: zone at its first column (bit 31: evaluate per element) and its steps
-          {
-            const int xo = 16 * t;
-            uint32_t z0 = 0u, ud = 0u;
-            if (t < S / 16 && xo + 15 >= olo && xo <= ohi)
-              if (!chunk_zones(is + xo, dj * dj, a.mg, &z0, &ud)) z0 = 0x80000000u;
-            mk[t] = z0;
-            mk2[t] = ud;
+          for (int q = 0; q < 16; ++q) tc[q] = __ldg(pt + min(t + 256 * q, lim));
+          if (w != 0u) {
+            const int32_t di0 = (int32_t)(is + xo - a.mg.c);
+            switch (a.df.n) {
+              case 0: membrane_chunk<0>(a.df, cxr, di0, w, o); break;
+              case 1: membrane_chunk<1>(a.df, cxr, di0, w, o); break;
+              case 2: membrane_chunk<2>(a.df, cxr, di0, w, o); break;
+              default: membrane_chunk<3>(a.df, cxr, di0, w, o); break;
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) o[k] = CLOSED;
           }
           __syncthreads();
-          const uint32_t mp = (2u << (t & 15)) - 1u;  // steps at or before this thread's column of a chunk
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
-            const int o = t + 256 * q;
-            if ((unsigned)(o - olo) > (unsigned)(ohi - olo)) {
-              v[q] = make_float2(0.0f, 0.0f);  // outside the chord (and beyond S)
-              continue;
-            }
-            const uint32_t z0 = mk[16 * q + (t >> 4)], ud = mk2[16 * q + (t >> 4)];
-            uint32_t z;
-            if (z0 & 0x80000000u) {
-              const int64_t di = is + o - a.mg.c;
-              z = (uint32_t)zone_of(min(dj * dj + di * di, a.mg.sR), a.mg);
-            } else {
-              z = z0 + __popc(ud & mp) - __popc((ud >> 16) & mp);
-            }
-            const uint32_t lv = z - nlev * __umulhi(z, lmagic);
-            v[q] = cmul(v[q], phs[lv]);
+            constexpr float TWO_PI = 6.28318530717958648f;
+            const float wv = wz[t + 256 * q + ((t + 256 * q) >> 4)];
+            float x = wv + tc[q];
+            x -= rintf(x);
+            x *= TWO_PI;
+            const bool open = wv < 0.5f * CLOSED;
+            v[q] = make_float2(open ? __cosf(x) : 0.0f, open ? __sinf(x) : 0.0f);
           }
+          __syncthreads();  // pass A writes this buffer
+        } else if (MODE == SEG_LEVELS) {
+          uint32_t lv[4] = {0x40404040u, 0x40404040u, 0x40404040u, 0x40404040u};
+          if (meets) {
+            chunk_levels(is + xo - a.mg.c, dj * dj, a.mg, a.ph, lv);
+            if (inside != 0xFFFFu) {
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                uint32_t m = 0u;
+#pragma unroll
+                for (int z = 0; z < 4; ++z) m |= ((inside >> (4 * k + z)) & 1u) ? 0xFFu << (8 * z) : 0u;
+                lv[k] = (lv[k] & m) | (0x40404040u & ~m);
+              }
+            }
+          }
+          *reinterpret_cast<uint4*>(lev + 16 * t) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
+          __syncthreads();
+#pragma unroll
+          for (int q = 0; q < 16; ++q) v[q] = cmul(v[q], phs[lev[t + 256 * q]]);
         } else {
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
@@ -1057,7 +1045,7 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
 
 // Tables: pre(i), post(m)/L, convolution chirp v (length L), twiddles.
 template <typename R>
-__global__ void k_tables(int64_t N, int M, double msh, int64_t L, int64_t c, double kappa, double delta, void* pre,
+__global__ void k_tables(int64_t N, int M, double msh, int64_t L, int64_t c, double kappa, double delta, int turns, void* pre,
                          void* post,
                          void* v, void* tw, int twN, void* twL) {
   using C = typename Cplx<R>::T;
@@ -1066,7 +1054,8 @@ __global__ void k_tables(int64_t N, int M, double msh, int64_t L, int64_t c, dou
     if (t < N) {
       const double di = (double)(t - c), ti = (double)t;
       const double ph = di * di * (0.5 * kappa) - (0.5 * delta) * (ti * ti) + delta * msh * ti;
-      reinterpret_cast<C*>(pre)[t] = cis_turns<R>(ph);
+      if (turns) reinterpret_cast<R*>(pre)[t] = (R)frac_turns(ph);  // the membrane walk adds its phase to them
+      else reinterpret_cast<C*>(pre)[t] = cis_turns<R>(ph);
     }
     if (t < M) {
       const double tm = (double)t;
@@ -1152,6 +1141,7 @@ static RowArgs make_args(const Plan& P) {
   a.c1_stride = P.chunk_rows;
   a.C1 = P.precision == FZP_PREC_FP64 ? (void*)P.d_C1d : (void*)P.d_C1;
   a.vin = b.d_tab;
+  if (b.seg) a.ph = phase_rule(P, nullptr);
   a.S = b.S;
   a.nseg = b.nseg;
   a.col0 = b.col0;
@@ -1226,7 +1216,7 @@ fzp_status fill_tables_t(Plan& P, cudaStream_t s) {
   const double delta = nodes ? P.nd.delta : P.delta;
   const double msh = nodes ? P.nd.msh + (P.nd.even ? P.nd.n / 2 : 0) : P.msh;
   b.d_twL = reinterpret_cast<C*>(b.d_post) + M;
-  k_tables<R><<<1024, 256, 0, s>>>(P.N, M, msh, b.L, P.c, P.kappa, delta, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
+  k_tables<R><<<1024, 256, 0, s>>>(P.N, M, msh, b.L, P.c, P.kappa, delta, b.seg && P.has_deform && P.levels < 2 ? 1 : 0, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
                                    b.d_twL);
   FZP_CUDA_TRY(cudaGetLastError());
   if (b.seg) {

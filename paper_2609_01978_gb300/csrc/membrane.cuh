@@ -41,39 +41,69 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(b - bh), "f"(a - ah));
 }
 
+// The membrane's phase (turns, 2 w / lambda) walked along a row from column di0:
+// the scaled wrinkle amp sin by its second difference, s' = s + e, e' = e - 4
+// sin^2(pi kx) s (one product instead of a rotation's four, and no growth of the
+// rounding at the small angles of a wrinkle), the taper by its constant second
+// difference, a ridge by its ratio.  Started exactly every 16 (k_seg) or 32
+// columns (k_nodes).  NR ridges.
+template <int NR>
+struct MembraneWalk {
+  float s, e, tap, dt, ddt, z4;
+  float g[NR > 0 ? NR : 1], rr[NR > 0 ? NR : 1], rho[NR > 0 ? NR : 1];
+
+  __device__ __forceinline__ MembraneWalk(const DeformCoef& d, const CxRow& r, int32_t di0) {
+    constexpr float TWO_PI = 6.28318530717958648f;
+    const float fi = (float)di0;
+    const float th = fmaf(fi, d.kxh, r.fjkh);
+    float tt = (th - rintf(th)) + fmaf(fi, d.kxl, r.fjkl);
+    tt -= rintf(tt);
+    float ws, wc;
+    __sincosf(TWO_PI * tt, &ws, &wc);
+    z4 = d.z4;
+    s = d.amp2 * ws;
+    e = d.amp2 * fmaf(0.5f * d.z4, ws, d.zs * wc);  // s minus its left neighbour
+    tap = fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f);
+    dt = -d.tq * fmaf(2.0f, fi, 1.0f);
+    ddt = -2.0f * d.tq;
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      g[k] = 0.0f;
+      rr[k] = 1.0f;
+      rho[k] = d.rho[k];
+      const float d0 = fmaf(fi, d.nx[k], r.cr[k]);
+      const float ex = d.q[k] * d0 * d0;
+      if (ex < 69.0f) {
+        g[k] = d.h2[k] * __expf(-ex);
+        rr[k] = __expf(-d.q[k] * d.nx[k] * fmaf(2.0f, d0, d.nx[k]));
+      }
+    }
+  }
+  // the phase at the column, then one column on
+  __device__ __forceinline__ float next() {
+    float wz = s * tap;
+    e = fmaf(-z4, s, e);
+    s += e;
+    tap += dt;
+    dt += ddt;
+#pragma unroll
+    for (int v = 0; v < NR; ++v) {
+      wz += g[v];
+      g[v] *= rr[v];
+      rr[v] *= rho[v];
+    }
+    return wz;
+  }
+};
+
 // Both masks of a membrane, T cos(phi) and T sin(phi), on the 32 columns from
 // di0 (bit k of `bits`: column k open), as the row's four 16-byte parts in the
-// planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart).  The walk's
-// steps, per column: the scaled wrinkle amp sin by its second difference,
-// s' = s + e, e' = e - 4 sin^2(pi kx) s (one product instead of a rotation's
-// four, and no growth of the rounding at the small angles of a wrinkle), the
-// taper by its constant second difference, a ridge by its ratio; each starts
-// exactly every 32 columns.  NR ridges.
+// planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart).  NR ridges.
 template <int NR>
 __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits,
                                             uint8_t* base, uint32_t plane, int sw) {
   constexpr float TWO_PI = 6.28318530717958648f;
-  const float fi = (float)di0;
-  const float th = fmaf(fi, d.kxh, r.fjkh);
-  float tt = (th - rintf(th)) + fmaf(fi, d.kxl, r.fjkl);
-  tt -= rintf(tt);
-  float ws, wc;
-  __sincosf(TWO_PI * tt, &ws, &wc);
-  float s = d.amp2 * ws, e = d.amp2 * fmaf(0.5f * d.z4, ws, d.zs * wc);  // s, and s minus its left neighbour
-  float tap = fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f), dt = -d.tq * fmaf(2.0f, fi, 1.0f);
-  const float ddt = -2.0f * d.tq;
-  float g[NR > 0 ? NR : 1], rr[NR > 0 ? NR : 1];
-#pragma unroll
-  for (int k = 0; k < NR; ++k) {
-    g[k] = 0.0f;
-    rr[k] = 1.0f;
-    const float d0 = fmaf(fi, d.nx[k], r.cr[k]);
-    const float ex = d.q[k] * d0 * d0;
-    if (ex < 69.0f) {
-      g[k] = d.h2[k] * __expf(-ex);
-      rr[k] = __expf(-d.q[k] * d.nx[k] * fmaf(2.0f, d0, d.nx[k]));
-    }
-  }
+  MembraneWalk<NR> walk(d, r, di0);
 #pragma unroll 1
   for (int q = 0; q < 4; ++q, bits >>= 8) {
     uint32_t hc[4], lc[4], hs[4], ls[4];
@@ -82,17 +112,7 @@ __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r,
       float vc[2], vs[2];
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        float wz = s * tap;
-        e = fmaf(-d.z4, s, e);
-        s += e;
-        tap += dt;
-        dt += ddt;
-#pragma unroll
-        for (int v = 0; v < NR; ++v) {
-          wz += g[v];
-          g[v] *= rr[v];
-          rr[v] *= d.rho[v];
-        }
+        float wz = walk.next();
         wz -= rintf(wz);
         const float x = TWO_PI * wz;
         const uint32_t open = (uint32_t)((int32_t)(bits << (31 - (k + z))) >> 31);

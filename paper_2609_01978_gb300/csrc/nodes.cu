@@ -57,6 +57,7 @@
 #include "fzp_internal.cuh"
 #include "membrane.cuh"
 #include "tc_ptx.cuh"
+#include "zone_phase.cuh"
 
 namespace fzp {
 namespace {
@@ -74,19 +75,6 @@ constexpr int EPI_BYTES = EPI_WARPS * 2 * EPI_BOX * EPI_BOX * 4;  // two boxes p
 constexpr int ERR_BASE = 300;
 
 enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4, MASK_LOADED = 5 };
-
-// Fixed-point zone phase: phase64(s) = s K mod 2^64 (K = floor(kappa 2^63): the
-// zone's parity is the top bit; MASK_LEVELS: K = floor(kappa_L / L 2^64), the
-// level is floor(phase L / 2^64)).  The true phase lies less than s (in units
-// of 2^-64) above it; the 32-bit walk over a block adds less than 600 units of
-// 2^-32 and fl(s kappa) less than 8, so E = 640 + (s_max >> 32).
-struct PhaseRule {
-  uint64_t K;
-  uint32_t E;
-  int lmod;            // MASK_LEVELS: L
-  uint64_t pos, neg;   // MASK_LEVELS: level sets with value +1, -1
-  int open_even;       // 1: positive-centred binary plate
-};
 
 struct NodeArgs {
   MaskGeom mg;              // c = 0 for a folded (flat) plate
@@ -1076,23 +1064,6 @@ fzp_status c1_map(const Plan& P, int64_t stride, int rows, CUtensorMap* tm) {
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return set_error(FZP_E_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return FZP_OK;
-}
-
-PhaseRule phase_rule(const Plan& P, const MaskPass* mp) {
-  PhaseRule r{};
-  r.E = 640u + (uint32_t)(P.mg.sR >> 32);
-  if (P.levels > 2) {
-    r.K = (uint64_t)std::floor(std::ldexp(P.kappa_mask / P.levels, 64));
-    r.lmod = P.levels;
-    if (mp) {
-      r.pos = mp->pos;
-      r.neg = mp->neg;
-    }
-  } else {
-    r.K = (uint64_t)std::floor(std::ldexp(P.kappa_mask, 63));
-    r.open_even = P.mg.centre_open;
-  }
-  return r;
 }
 
 int mask_kind(const Plan& P) {
