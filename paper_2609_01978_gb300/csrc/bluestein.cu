@@ -162,9 +162,9 @@ struct RowArgs {
   const void* vin;   // input sequence for the table-building mode (length L)
   int S;             // partitioned convolution: columns per block
   int64_t nseg;      // partitioned convolution: blocks per row (spectra in H)
-  int64_t col0;      // partitioned convolution: first column of block 0
+  int64_t col0;      // first column of the transforms' input (the axis when `half`)
   PhaseRule ph;      // partitioned convolution: the zone phase of the mask walk
-  int half;          // even output grid: columns from the axis on, outputs m and M - 1 - m added
+  int half;          // even output grid: columns from the axis on, outputs x and -x added
   int octant;        // columns up to the row's distance from the axis only, the last one halved
 };
 
@@ -232,6 +232,21 @@ __device__ __forceinline__ typename Cplx<R>::T aperture(const RowArgs& a, int64_
   return cmul(v, cis_turns<R>(2.0 * wz * a.inv_lambda));  // phi / (2 pi) = 2 w / lambda
 }
 
+// Input n of a row's convolution: the transmission of column col0 + n times the
+// chirp; with the columns from the axis on, the axis itself (which the two
+// added outputs both count) at half weight.
+template <typename R>
+__device__ __forceinline__ typename Cplx<R>::T row_input(const RowArgs& a, int64_t j, int64_t n,
+                                                         const typename Cplx<R>::T* pre) {
+  typename Cplx<R>::T x = aperture<R>(a, j, n + a.col0);
+  if (x.x != 0 || x.y != 0) x = cmul(x, pre[n]);
+  if (a.half && n == 0) {
+    x.x *= (R)0.5;
+    x.y *= (R)0.5;
+  }
+  return x;
+}
+
 // e^{sign 2 pi i t / L} for 0 <= t < L = L1 * L2 from two tables:
 // t = th * 4096 + tl, W_L^t = W_{L1}^{th} W_L^{tl}, W_{L1}^{th} = tw[th * (twN / L1)].
 template <typename R>
@@ -271,12 +286,8 @@ __global__ void __launch_bounds__(256) k_f1(RowArgs a, int mode) {
     const int n1 = t >> a.logB, b = t & (B - 1);
     const int64_t n = (int64_t)n1 * a.L2 + n2_0 + b;
     C x;
-    if (mode == 0) {
-      x = aperture<R>(a, j, n);
-      if (x.x != 0 || x.y != 0) x = cmul(x, pre[n]);
-    } else {
-      x = vin[n];
-    }
+    if (mode == 0) x = row_input<R>(a, j, n, pre);
+    else x = vin[n];
     sm[b * (L1 + 1) + brev(n1, a.logL1)] = x;  // odd column stride: no bank conflicts across columns
   }
   __syncthreads();
@@ -306,12 +317,8 @@ __global__ void __launch_bounds__(512) k_f2(RowArgs a, int mode) {
     const C* vin = reinterpret_cast<const C*>(a.vin);
     for (int n = threadIdx.x; n < L2; n += blockDim.x) {
       C x;
-      if (mode == 0) {
-        x = aperture<R>(a, j, n);
-        if (x.x != 0 || x.y != 0) x = cmul(x, pre[n]);
-      } else {
-        x = vin[n];
-      }
+      if (mode == 0) x = row_input<R>(a, j, n, pre);
+      else x = vin[n];
       sm[brev(n, a.logL2)] = x;
     }
   } else {
@@ -334,8 +341,11 @@ __global__ void __launch_bounds__(512) k_f2(RowArgs a, int mode) {
     const C* post = reinterpret_cast<const C*>(a.post);
     R* C1 = reinterpret_cast<R*>(a.C1);
     const int64_t jl = j - a.c1_j0;
-    for (int m = threadIdx.x; m < a.M; m += blockDim.x) {
-      const C v = cmul(sm[brev(m, a.logL2)], post[m]);
+    const int hm = (a.M - 1) / 2;
+    for (int m = threadIdx.x; m < (a.half ? hm + 1 : a.M); m += blockDim.x) {
+      const int mp = a.half ? hm + m : m;
+      C v = cmul(sm[brev(mp, a.logL2)], post[mp]);
+      if (a.half) v = cadd(v, cmul(sm[brev(hm - m, a.logL2)], post[hm - m]));
       C1[(int64_t)c1_row_re(m) * a.c1_stride + jl] = v.x;
       C1[(int64_t)c1_row_im(m) * a.c1_stride + jl] = v.y;
     }
@@ -512,29 +522,35 @@ __global__ void __launch_bounds__(R8T, 2) k_f2_r8(RowArgs a, int mode) {
   }
 }
 
-// Sum over k1; tile of 32 rows x 32 m; writes C1 coalesced along rows.
+// Sum over k1; tile of 32 rows x 32 outputs; writes C1 coalesced along rows.
 template <typename R>
 __global__ void __launch_bounds__(256) k_f3(RowArgs a) {
   using C = typename Cplx<R>::T;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 warps
   const int m0 = blockIdx.x * 32;
   const int64_t r0 = (int64_t)blockIdx.y * 32;
+  const int hm = (a.M - 1) / 2, nout = a.half ? hm + 1 : a.M;
   __shared__ C tile[32][33];
   const C* G = reinterpret_cast<const C*>(a.G);
-  for (int rr = ty; rr < 32; rr += 8) {
-    const int64_t r = r0 + rr;
+  const C* post = reinterpret_cast<const C*>(a.post);
+  auto out = [&](int64_t r, int m) {
     C acc;
     acc.x = 0; acc.y = 0;
-    if (r < a.rows)
-      for (int64_t k1 = 0; k1 < a.L1; ++k1) acc = cadd(acc, G[(r * a.L1 + k1) * a.M + m0 + tx]);
-    tile[rr][tx] = cmul(acc, reinterpret_cast<const C*>(a.post)[m0 + tx]);
+    for (int64_t k1 = 0; k1 < a.L1; ++k1) acc = cadd(acc, G[(r * a.L1 + k1) * a.M + m]);
+    return cmul(acc, post[m]);
+  };
+  for (int rr = ty; rr < 32; rr += 8) {
+    const int64_t r = r0 + rr;
+    const int m = m0 + tx;
+    if (r >= a.rows || m >= nout) continue;
+    tile[rr][tx] = a.half ? cadd(out(r, hm + m), out(r, hm - m)) : out(r, m);
   }
   __syncthreads();
   R* C1 = reinterpret_cast<R*>(a.C1);
   for (int mm = ty; mm < 32; mm += 8) {
     const int64_t r = r0 + tx;
-    if (r >= a.rows) continue;
     const int m = m0 + mm;
+    if (r >= a.rows || m >= nout) continue;
     const int64_t jl = a.j0 + r - a.c1_j0;
     const C v = tile[tx][mm];
     C1[(int64_t)c1_row_re(m) * a.c1_stride + jl] = v.x;
@@ -589,36 +605,47 @@ __device__ __forceinline__ void membrane_chunk(const DeformCoef& d, const CxRow&
 }
 
 // v e^{-2 pi i K / 16}
-template <int K>
-__device__ __forceinline__ float2 w16mul(float2 v) {
-  constexpr float C1 = 0.923879532511286756f, S1 = 0.382683432365089772f, R2 = 0.707106781186547524f;
+template <int K, typename C>
+__device__ __forceinline__ C w16mul(C v) {
+  using R = decltype(C::x);
+  constexpr R C1 = (R)0.92387953251128675613, S1 = (R)0.38268343236508977173, R2 = (R)0.70710678118654752440;
+  C r;
   if constexpr (K == 0) {
-    return v;
+    r = v;
   } else if constexpr (K == 4) {
-    return make_float2(v.y, -v.x);
+    r.x = v.y;
+    r.y = -v.x;
   } else if constexpr (K == 2) {
-    return make_float2(R2 * (v.x + v.y), R2 * (v.y - v.x));
+    r.x = R2 * (v.x + v.y);
+    r.y = R2 * (v.y - v.x);
   } else if constexpr (K == 6) {
-    return make_float2(R2 * (v.y - v.x), -R2 * (v.x + v.y));
+    r.x = R2 * (v.y - v.x);
+    r.y = -R2 * (v.x + v.y);
   } else {
-    constexpr float wr = K == 1 ? C1 : (K == 3 ? S1 : -C1);  // K = 1, 3, 9
-    constexpr float wi = K == 1 ? -S1 : (K == 3 ? -C1 : S1);
-    return make_float2(v.x * wr - v.y * wi, v.x * wi + v.y * wr);
+    constexpr R wr = K == 1 ? C1 : (K == 3 ? S1 : -C1);  // K = 1, 3, 9
+    constexpr R wi = K == 1 ? -S1 : (K == 3 ? -C1 : S1);
+    r.x = v.x * wr - v.y * wi;
+    r.y = v.x * wi + v.y * wr;
   }
+  return r;
 }
 
 // Forward 4-point DFT in place.
-__device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2& a3) {
-  const float2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
+template <typename C>
+__device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3) {
+  const C t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
   a0 = cadd(t0, t2);
   a2 = csub(t0, t2);
-  a1 = make_float2(t1.x + t3.y, t1.y - t3.x);
-  a3 = make_float2(t1.x - t3.y, t1.y + t3.x);
+  a1.x = t1.x + t3.y;
+  a1.y = t1.y - t3.x;
+  a3.x = t1.x - t3.y;
+  a3.y = t1.y + t3.x;
 }
 
 // x[k] <- sum_n x[n] e^{-2 pi i n k / 16}: n = q + 4 n1, k = p + 4 k1; 4-point
 // DFTs over n1, twiddles e^{-2 pi i q p / 16}, 4-point DFTs over q.
-__device__ __forceinline__ void dft16(float2 (&x)[16]) {
+template <typename C>
+__device__ __forceinline__ void dft16(C (&x)[16]) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) dft4(x[q], x[q + 4], x[q + 8], x[q + 12]);  // (q, p) at q + 4 p
   x[5] = w16mul<1>(x[5]);
@@ -632,7 +659,7 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
   x[15] = w16mul<9>(x[15]);
 #pragma unroll
   for (int p = 0; p < 4; ++p) dft4(x[4 * p], x[4 * p + 1], x[4 * p + 2], x[4 * p + 3]);  // (p, k1) at 4 p + k1
-  float2 y[16];
+  C y[16];
 #pragma unroll
   for (int p = 0; p < 4; ++p)
 #pragma unroll
@@ -641,12 +668,29 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
   for (int k = 0; k < 16; ++k) x[k] = y[k];
 }
 
+// The outputs k = 0 and 1 of the same, in x[0] and x[1].
+template <typename C>
+__device__ __forceinline__ void dft16_two(C (&x)[16]) {
+  C e[4], o[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const C s02 = cadd(x[q], x[q + 8]), d02 = csub(x[q], x[q + 8]), s13 = cadd(x[q + 4], x[q + 12]),
+            d13 = csub(x[q + 4], x[q + 12]);
+    e[q] = cadd(s02, s13);
+    o[q].x = d02.x + d13.y;
+    o[q].y = d02.y - d13.x;
+  }
+  x[0] = cadd(cadd(e[0], e[1]), cadd(e[2], e[3]));
+  x[1] = cadd(cadd(o[0], w16mul<1>(o[1])), cadd(w16mul<2>(o[2]), w16mul<3>(o[3])));
+}
+
 // Forward P-point DFT of the block distributed as v[r] = x[t + 256 r];
 // on return v[d] = X[t + 256 d].  Two barriers; b0 and b1 alternate, so
 // back-to-back calls need no further barrier.  twA[(k0 - 1) 256 + t] =
 // e^{-2 pi i t k0 / P}, twB[c 16 + a] = e^{-2 pi i a c / 256}.
-__device__ __forceinline__ void fft_p(float2 (&v)[16], float2* b0, float2* b1, const float2* twA,
-                                      const float2* twB) {
+// TWO: only v[0] and v[1] are wanted.
+template <bool TWO = false, typename C>
+__device__ __forceinline__ void fft_p(C (&v)[16], C* b0, C* b1, const C* twA, const C* twB) {
   const int t = threadIdx.x;
   dft16(v);
 #pragma unroll
@@ -669,7 +713,8 @@ __device__ __forceinline__ void fft_p(float2 (&v)[16], float2* b0, float2* b1, c
     const int k0 = t & 15, c = t >> 4;
 #pragma unroll
     for (int a = 0; a < 16; ++a) v[a] = b1[k0 * 273 + c * 17 + a];
-    dft16(v);
+    if (TWO) dft16_two(v);
+    else dft16(v);
   }
 }
 
@@ -773,6 +818,92 @@ __device__ __forceinline__ void chunk_levels(int64_t di0, int64_t dj2, const Mas
   if (near < 2u * el) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) lv[k] = exact_levels4(di0 + 4 * k, dj2, g);
+  }
+}
+
+// The inner pass of the single convolution in FP64 (L2 = 4096; what k_f2 does for
+// the other lengths): the 4096-point transforms above, in registers, resident
+// CTAs over the (row, k1) pairs.  FP64 has two lanes per SM here (GB300: 1.25
+// TFLOP/s), so operations are what counts: radix 16 takes 3.6 per point and
+// stage instead of radix 2's 4, the inverse's last pass forms only the outputs
+// that are kept, and a flat plate's columns from the axis on fit half the
+// length.  4 mm plate (N = 5,057, L 8192 -> 4096), ROI 256^2: 6.2 -> 1.6 ms for
+// the row transforms, 22.2 -> 2.6 ms for a propagation with its metrics (rows
+// folded 8.2).
+constexpr size_t D16_SMEM = sizeof(double2) * (2 * SBUF + 15 * 256 + 256);
+__global__ void __launch_bounds__(STH, 1) k_f2_d16(RowArgs a, int mode) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* b0 = reinterpret_cast<double2*>(smem_raw);
+  double2* b1 = b0 + SBUF;
+  double2* twA = b1 + SBUF;
+  double2* twB = twA + 15 * 256;
+  const int t = threadIdx.x;
+  const double2* tw = reinterpret_cast<const double2*>(a.tw);  // e^{-2 pi i t / 4096}
+  for (int e = t; e < 15 * 256; e += STH) twA[e] = tw[(e / 256 + 1) * (e % 256)];
+  twB[t] = tw[16 * (t >> 4) * (t & 15)];
+  __syncthreads();
+  const double2* pre = reinterpret_cast<const double2*>(a.pre);
+  const double2* vin = reinterpret_cast<const double2*>(a.vin);
+  const double2* post = reinterpret_cast<const double2*>(a.post);
+  for (int64_t w = blockIdx.x; w < a.rows * a.L1; w += gridDim.x) {
+    const int64_t r = w / a.L1, k1 = w % a.L1, j = a.j0 + r;
+    double2 v[16];
+    double2* Z = reinterpret_cast<double2*>(a.Z) + r * a.L + k1 * SP;
+    if (a.L1 == 1) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) v[q] = mode == 0 ? row_input<double>(a, j, t + 256 * q, pre) : vin[t + 256 * q];
+    } else {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) v[q] = Z[t + 256 * q];
+    }
+    fft_p(v, b0, b1, twA, twB);
+    if (mode == 1) {
+#pragma unroll
+      for (int d = 0; d < 16; ++d) Z[t + 256 * d] = v[d];
+      continue;
+    }
+    const double2* H = reinterpret_cast<const double2*>(a.H) + k1 * SP + t;
+#pragma unroll
+    for (int d = 0; d < 16; ++d) {
+      v[d] = cmul(v[d], H[256 * d]);
+      v[d].y = -v[d].y;  // the inverse transform as conj(FFT(conj(.)))
+    }
+    if (a.M <= 512) fft_p<true>(v, b0, b1, twA, twB);
+    else fft_p(v, b0, b1, twA, twB);
+    const int64_t jl = j - a.c1_j0;
+    double* C1 = reinterpret_cast<double*>(a.C1);
+    if (a.L1 == 1 && a.half) {
+      // outputs x and -x meet in the buffer that the last pass does not read
+#pragma unroll
+      for (int d = 0; d < 5; ++d) {
+        const int m = t + 256 * d;
+        if (m < a.M) b0[m] = cmul(make_double2(v[d].x, -v[d].y), post[m]);
+      }
+      __syncthreads();
+      const int hm = (a.M - 1) / 2;
+      for (int m = t; m <= hm; m += STH) {
+        const double2 y = cadd(b0[hm + m], b0[hm - m]);
+        C1[(int64_t)c1_row_re(m) * a.c1_stride + jl] = y.x;
+        C1[(int64_t)c1_row_im(m) * a.c1_stride + jl] = y.y;
+      }
+      __syncthreads();
+      continue;
+    }
+#pragma unroll
+    for (int d = 0; d < 5; ++d) {
+      const int m = t + 256 * d;
+      if (m >= a.M) continue;
+      const double2 y = make_double2(v[d].x, -v[d].y);
+      if (a.L1 == 1) {
+        const double2 z = cmul(y, post[m]);
+        C1[(int64_t)c1_row_re(m) * a.c1_stride + jl] = z.x;
+        C1[(int64_t)c1_row_im(m) * a.c1_stride + jl] = z.y;
+      } else {
+        reinterpret_cast<double2*>(a.G)[(r * a.L1 + k1) * a.M + m] =
+            cmul(y, twiddle_L<double>(a, (k1 * m) & (a.L - 1), true));
+      }
+    }
+    __syncthreads();  // the next row's first pass writes b0
   }
 }
 
@@ -1145,10 +1276,9 @@ static RowArgs make_args(const Plan& P) {
   a.S = b.S;
   a.nseg = b.nseg;
   a.col0 = b.col0;
-  if (P.nd.n > 0) {
-    a.M = P.nd.n;
-    a.half = P.nd.even ? 1 : 0;
-  }
+  a.half = b.half ? 1 : 0;
+  if (P.nd.n > 0) a.M = P.nd.n;
+  else if (b.half) a.M = P.M + 1;
   return a;
 }
 
@@ -1156,20 +1286,26 @@ template <typename R>
 fzp_status layout_t(Plan& P, FormSizes* out) {
   using C = typename Cplx<R>::T;
   Bluestein& b = P.bs;
+  b.seg = (sizeof(R) == 4 && P.conv_req != 1) ? 1 : 0;
+  // columns from the axis on: flat plates whose outputs are symmetric about it
+  // (nodes, or in FP64 the ROI's samples and x = +(M / 2) p besides)
+  b.half = b.seg ? P.nd.even : sizeof(R) == 8 && bluestein_even(P);
+  b.col0 = b.half ? P.c : 0;
   b.L = 1;
   while (b.L < P.N + P.M - 1) b.L <<= 1;
+  b.L_full = b.L;
+  if (!b.seg && b.half)
+    for (b.L = 1; b.L < P.c + 1 + P.M;) b.L <<= 1;
   b.L2 = b.L < Traits<R>::L2MAX ? b.L : Traits<R>::L2MAX;
   b.L1 = b.L / b.L2;
   if (P.M > b.L2) return set_error(FZP_E_UNSUPPORTED, "M larger than the inner FFT length");
   // the F1 twiddles are read from the L2-entry table with stride L2 / L1
   if (b.L1 > b.L2) return set_error(FZP_E_UNSUPPORTED, "FFT length %lld above %lld", (long long)b.L,
                                     (long long)b.L2 * b.L2);
-  b.seg = (sizeof(R) == 4 && P.conv_req != 1) ? 1 : 0;
   if (b.seg) {
     // partitioned convolution: S + M - 1 <= 4096, S a multiple of 256 (at most 15 x 256)
     const int M = P.nd.n > 0 ? P.nd.n : P.M;  // outputs per row: the nodes, or the ROI samples
     b.S = 256 * std::min(15, (4097 - M) / 256);
-    b.col0 = P.nd.even ? P.c : 0;
     b.nseg = (P.N - b.col0 + b.S - 1) / b.S;
     b.rows = P.chunk_rows;
     out->pre = sizeof(C) * P.N;
@@ -1186,20 +1322,22 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
     return FZP_OK;
   }
   // rows per pass: requested, else a transform workspace of about 1 GiB
-  const int64_t zbytes = (int64_t)sizeof(C) * b.L;
+  const int64_t zbytes = (int64_t)sizeof(C) * b.L_full;  // (of the length that the plan reports)
   int64_t rows = P.row_batch_req > 0 ? P.row_batch_req : (1ll << 30) / zbytes;
-  if (b.L1 == 1) rows = P.row_batch_req > 0 ? P.row_batch_req : P.chunk_rows;
+  if (b.L_full <= Traits<R>::L2MAX) rows = P.row_batch_req > 0 ? P.row_batch_req : P.chunk_rows;
   b.rows = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(rows, P.chunk_rows), 65535));
-  const int twN = (int)b.L2;
+  const int twN = (int)b.L2, Mo = P.M + (b.half ? 1 : 0);
   out->pre = sizeof(C) * P.N;
   out->H = sizeof(C) * b.L;
-  out->tab = sizeof(C) * (b.L + twN + P.M + 4096);
+  out->tab = sizeof(C) * (b.L + twN + Mo + 4096);
   out->Z = sizeof(C) * b.L * (b.L1 > 1 ? b.rows : 1);  // row 0 also serves the table build
-  out->G = b.L1 > 1 ? sizeof(C) * b.L1 * P.M * b.rows : 0;
+  out->G = b.L1 > 1 ? sizeof(C) * b.L1 * Mo * b.rows : 0;
   // 64 KiB covers every FP32 case; FP64 at L1 = 4096 needs ~96 KiB
   static std::atomic<uint64_t> attr_f1{0}, attr_f2{0};
   FZP_CUDA_TRY(smem_attr_once((const void*)k_f1<R>, 200 * 1024, attr_f1));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_f2<R>, (int)(sizeof(C) * Traits<R>::L2MAX), attr_f2));
+  static std::atomic<uint64_t> attr_d16{0};
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_f2_d16, (int)D16_SMEM, attr_d16));
   return FZP_OK;
 }
 
@@ -1211,12 +1349,12 @@ fzp_status fill_tables_t(Plan& P, cudaStream_t s) {
   b.d_tw = reinterpret_cast<C*>(b.d_tab) + b.L;
   b.d_post = reinterpret_cast<C*>(b.d_tw) + twN;
   // the outputs: the ROI's samples, or the nodes (all n of them)
-  const bool nodes = P.nd.n > 0;
-  const int M = nodes ? P.nd.n : P.M;
+  const bool nodes = P.nd.n > 0, half = b.half && !nodes;
+  const int M = nodes ? P.nd.n : P.M + (half ? 1 : 0);
   const double delta = nodes ? P.nd.delta : P.delta;
   const double msh = nodes ? P.nd.msh + (P.nd.even ? P.nd.n / 2 : 0) : P.msh;
   b.d_twL = reinterpret_cast<C*>(b.d_post) + M;
-  k_tables<R><<<1024, 256, 0, s>>>(P.N, M, msh, b.L, P.c, P.kappa, delta, b.seg && P.has_deform && P.levels < 2 ? 1 : 0, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
+  k_tables<R><<<1024, 256, 0, s>>>(half ? P.c + 1 : P.N, M, msh, b.L, half ? 0 : P.c, P.kappa, delta, b.seg && P.has_deform && P.levels < 2 ? 1 : 0, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
                                    b.d_twL);
   FZP_CUDA_TRY(cudaGetLastError());
   if (b.seg) {
@@ -1232,6 +1370,7 @@ fzp_status fill_tables_t(Plan& P, cudaStream_t s) {
   a.rows = 1;
   if (b.L1 > 1) k_f1<R><<<dim3((unsigned)(b.L2 / a.B), 1), 256, f1_smem<R>(a), s>>>(a, 1);
   if (sizeof(R) == 4 && b.L2 == RL) k_f2_r8<<<dim3((unsigned)b.L1, 1), R8T, 0, s>>>(a, 1);
+  else if (sizeof(R) == 8 && b.L2 == SP) k_f2_d16<<<(unsigned)b.L1, STH, D16_SMEM, s>>>(a, 1);
   else k_f2<R><<<dim3((unsigned)b.L1, 1), 512, sizeof(C) * b.L2, s>>>(a, 1);
   FZP_CUDA_TRY(cudaGetLastError());
   FZP_CUDA_TRY(cudaMemcpyAsync(b.d_H, b.d_Z, sizeof(C) * b.L, cudaMemcpyDeviceToDevice, s));
@@ -1266,11 +1405,12 @@ fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s
   const Bluestein& b = P.bs;
   RowArgs a = make_args(P);
   a.c1_j0 = j0;
+  int sms = 0, dev = 0;
+  FZP_CUDA_TRY(cudaGetDevice(&dev));
+  FZP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (b.seg) {
     // resident CTAs only: each takes every gridDim.x-th row of the range
-    int ctas_per_sm = 0, sms = 0, dev = 0;
-    FZP_CUDA_TRY(cudaGetDevice(&dev));
-    FZP_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int ctas_per_sm = 0;
     const int mode = P.has_deform ? (P.levels >= 2 ? SEG_GENERAL : SEG_MEMBRANE) : (P.levels >= 2 ? SEG_LEVELS : SEG_FLAT);
     a.octant = octant ? 1 : 0;
     void (*kern)(RowArgs) = mode == SEG_FLAT       ? k_seg<SEG_FLAT>
@@ -1293,17 +1433,20 @@ fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s
     const int64_t rb = std::min<int64_t>(b.rows, rows - r0);
     a.j0 = j0 + r0;
     a.rows = rb;
+    const unsigned d16_grid = (unsigned)std::min<int64_t>(rb * b.L1, sms);
     if (b.L1 > 1) {
       k_f1<R><<<dim3((unsigned)(b.L2 / a.B), (unsigned)rb), 256, f1_smem<R>(a), s>>>(a, 0);
       prof_begin(P, s);
       if (sizeof(R) == 4 && b.L2 == RL) k_f2_r8<<<dim3((unsigned)b.L1, (unsigned)rb), R8T, 0, s>>>(a, 0);
+      else if (sizeof(R) == 8 && b.L2 == SP) k_f2_d16<<<d16_grid, STH, D16_SMEM, s>>>(a, 0);
       else k_f2<R><<<dim3((unsigned)b.L1, (unsigned)rb), 512, sizeof(C) * b.L2, s>>>(a, 0);
       prof_end(P, s);
-      k_f3<R><<<dim3((unsigned)(P.M / 32), (unsigned)((rb + 31) / 32)), 256, 0, s>>>(a);
+      k_f3<R><<<dim3((unsigned)((a.M + 31) / 32), (unsigned)((rb + 31) / 32)), 256, 0, s>>>(a);
       P.launches += 3;
     } else {
       prof_begin(P, s);
       if (sizeof(R) == 4 && b.L2 == RL) k_f2_r8<<<dim3(1, (unsigned)rb), R8T, 0, s>>>(a, 0);
+      else if (sizeof(R) == 8 && b.L2 == SP) k_f2_d16<<<d16_grid, STH, D16_SMEM, s>>>(a, 0);
       else k_f2<R><<<dim3(1, (unsigned)rb), 512, sizeof(C) * b.L2, s>>>(a, 0);
       prof_end(P, s);
       P.launches += 1;

@@ -29,7 +29,7 @@ struct ColArgs {
   int64_t sin_off;  // > 0: C1 holds the rows of Re T and, sin_off values on, of Im T
   const float2* E;
   int64_t estride;
-  int M;          // outputs per row (m)
+  int M, ny;      // outputs per row (m) and of the column pass (n)
   double kappa, delta;
   double msh;     // ROI (or node) shift in pitches: y_n = (n - msh) p
   double wr, wi;  // weight of this pass's field (1, 0 for a single-pass plate)
@@ -78,6 +78,8 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
   const int64_t je = jb + g.jc < g.rows ? jb + g.jc : g.rows;
   const int tid = threadIdx.x;
   const int tn = tid >> 4, tm = tid & 15;  // 16 x 16 threads, 4 x 4 outputs each
+  // outputs of this warp's rows and of the tile's columns (uniform per warp)
+  const int na = min(4, max(0, (g.ny - n0 - (tn & ~1) + 15) / 16)), nb = min(4, (g.M - m0 + 15) / 16);
   C acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
       const int m = m0 + mm;
       C v;
       v.x = 0; v.y = 0;
-      if (j + jj < je) {
+      if (j + jj < je && m < g.M) {
         const int64_t re = (int64_t)c1_row_re(m) * g.c1_stride + j + jj, im = (int64_t)c1_row_im(m) * g.c1_stride + j + jj;
         for (int sl = 0; sl < g.slices; ++sl) {
           const R* S = C1 + sl * g.slice_off;
@@ -130,6 +132,20 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
       sK[jj][nn] = k;
     }
     __syncthreads();
+    if (na == 0) {
+    } else if (na < 4 || nb < 4) {  // an edge tile: the outputs it has
+#pragma unroll 1
+      for (int jj = 0; jj < TJ; ++jj)
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            if (a < na && b < nb) {
+              const C kv = sK[jj][tn + 16 * a], cv = sC[jj][tm + 16 * b];
+              acc[a][b].x = fma(kv.x, cv.x, fma(-kv.y, cv.y, acc[a][b].x));
+              acc[a][b].y = fma(kv.x, cv.y, fma(kv.y, cv.x, acc[a][b].y));
+            }
+    } else
 #pragma unroll 4
     for (int jj = 0; jj < TJ; ++jj) {
       C kv[4], cv[4];
@@ -152,6 +168,7 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int n = n0 + tn + 16 * a, m = m0 + tm + 16 * b;
+      if (n >= g.ny || m >= g.M) continue;
       double ux = (double)acc[a][b].x, uy = (double)acc[a][b].y;
       if (g.wi != 0.0 || g.wr != 1.0) {
         const double t = g.wr * ux - g.wi * uy;
@@ -164,7 +181,8 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
 }
 
 __global__ void k_epilogue(int M, double msh, double p, double lf, double f_over_lambda, double amp,
-                           const double2* __restrict__ Uacc, double2* __restrict__ out, int accumulate) {
+                           int evenx, int eveny, const double2* __restrict__ Uacc, double2* __restrict__ out,
+                           int accumulate) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= M * M) return;
   const int n = t / M, m = t % M;
@@ -174,7 +192,9 @@ __global__ void k_epilogue(int M, double msh, double p, double lf, double f_over
   double2 w = cis_turns_d(ph);
   w.x *= amp;
   w.y *= amp;
-  const double2 u = Uacc[t];
+  // even: the accumulator holds the samples x >= 0, |m - M/2| of them from the axis
+  const int h = M / 2;
+  const double2 u = Uacc[(int64_t)(eveny ? abs(n - h) : n) * (evenx ? h + 1 : M) + (evenx ? abs(m - h) : m)];
   double2 v = make_double2(w.x * u.x - w.y * u.y, w.x * u.y + w.y * u.x);
   if (accumulate) {
     v.x += out[t].x;
@@ -198,10 +218,13 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   g.rows = rows;
   g.c1_stride = P.c1_stride;
   g.kind = kind;
-  g.M = nodes ? P.nd.ns : P.M;
+  // FP64 on the samples x >= 0: a grid from the axis on
+  const bool even = !nodes && bluestein_even(P);
+  g.M = nodes ? P.nd.ns : even ? P.M / 2 + 1 : P.M;
+  g.ny = nodes ? (P.nd.yfull ? P.nd.n : P.nd.ns) : P.nd.yfull ? P.M : g.M;
   g.kappa = P.kappa;
   g.delta = nodes ? P.nd.delta : P.delta;
-  g.msh = !nodes ? P.msh : P.nd.yfull ? 0.5 * (P.nd.n - 1) : P.nd.msh;
+  g.msh = !nodes ? (even && !P.nd.yfull ? 0.0 : P.msh) : P.nd.yfull ? 0.5 * (P.nd.n - 1) : P.nd.msh;
   g.wr = 1.0;
   if (P.pass_index >= 0) {
     g.wr = P.passes[P.pass_index].wr;
@@ -211,10 +234,10 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   g.slice_off = P.nd.slice_elems;
   if (nodes_two_masks(P)) g.sin_off = 128 * P.c1_stride;
   // rows per block: 2048, fewer where that leaves the GPU idle (few output tiles)
-  const int ny = nodes && P.nd.yfull ? P.nd.n : g.M;
-  const int64_t tiles = (int64_t)(g.M / TM) * (ny / TN);
+  const int tx = (g.M + TM - 1) / TM, ty = (g.ny + TN - 1) / TN;
+  const int64_t tiles = (int64_t)tx * ty;
   g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / 304 + TJ - 1) / TJ * TJ));
-  dim3 grid((unsigned)(g.M / TM), (unsigned)(ny / TN), (unsigned)((rows + g.jc - 1) / g.jc));
+  dim3 grid((unsigned)tx, (unsigned)ty, (unsigned)((rows + g.jc - 1) / g.jc));
   if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
   else k_colpass<float><<<grid, 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
   P.launches += 1;
@@ -232,6 +255,7 @@ fzp_status column_pass_table(Plan& P, const void* E, int64_t rows, int64_t estri
   g.sin_off = 2 * P.nd.ns * P.c1_stride;
   g.E = reinterpret_cast<const float2*>(E);
   g.estride = estride;
+  g.ny = g.M;
   const int t = g.M / TM;
   g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * t * t / 304 + TJ - 1) / TJ * TJ));
   k_colpass<float, true><<<dim3((unsigned)t, (unsigned)t, (unsigned)((rows + g.jc - 1) / g.jc)), 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
@@ -253,7 +277,8 @@ fzp_status column_pass_zoom(Plan& P, int64_t rows, double lz, cudaStream_t s) {
   g.wr = 1.0;
   g.slices = 1;
   g.sin_off = 2 * z.ns * P.c1_stride;
-  const int tx = g.M / TM, ty = (z.yfull ? z.n : z.ns) / TN;
+  g.ny = z.yfull ? z.n : z.ns;
+  const int tx = g.M / TM, ty = g.ny / TN;
   g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tx * ty / 304 + TJ - 1) / TJ * TJ));
   k_colpass<float><<<dim3((unsigned)tx, (unsigned)ty, (unsigned)((rows + g.jc - 1) / g.jc)), 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
   P.launches += 1;
@@ -264,7 +289,9 @@ fzp_status column_pass_zoom(Plan& P, int64_t rows, double lz, cudaStream_t s) {
 fzp_status epilogue(Plan& P, void* d_field, int accumulate, cudaStream_t s) {
   const double lf = P.lambda * P.f;
   const int count = P.M * P.M;
-  k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf, P.d_Uacc,
+  const bool even = bluestein_even(P);
+  k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf, even ? 1 : 0,
+                                                 even && !P.nd.yfull ? 1 : 0, P.d_Uacc,
                                                  reinterpret_cast<double2*>(d_field), accumulate);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
@@ -274,7 +301,7 @@ fzp_status epilogue(Plan& P, void* d_field, int accumulate, cudaStream_t s) {
 fzp_status epilogue_z(Plan& P, void* d_field, int accumulate, double z, cudaStream_t s) {
   const double lz = P.lambda * z;
   const int count = P.M * P.M;
-  k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lz, P.f / P.lambda, P.dx2 / lz, P.d_Uacc,
+  k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lz, P.f / P.lambda, P.dx2 / lz, 0, 0, P.d_Uacc,
                                                  reinterpret_cast<double2*>(d_field), accumulate);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());

@@ -193,7 +193,9 @@ struct Bluestein {
   int seg = 0;
   int S = 0;
   int64_t nseg = 0;
-  int64_t col0 = 0;       // first column of block 0 (the axis for an even output grid)
+  int64_t col0 = 0;       // first input column (the axis when `half`)
+  bool half = false;      // columns from the axis on, outputs x and -x added
+  int64_t L_full = 0;     // power of two >= N + M - 1 (what the plan reports)
 };
 
 // One signed-mask pass of a phase plate in the dense form: the mask is +1 on
@@ -337,6 +339,12 @@ struct FormSizes {
   size_t A = 0, sched = 0;                       // dense
   size_t X = 0;                                  // dense on nodes
 };
+// FP64 row passes of a flat plate whose ROI is centred on the focus: only the
+// samples x >= 0 (and x = (M / 2) p, the mirror image of the first) are
+// evaluated, M / 2 + 1 per axis, unless the row range is not symmetric.
+inline bool bluestein_even(const Plan& P) {
+  return P.form == FZP_FORM_BLUESTEIN && P.precision == FZP_PREC_FP64 && !P.has_deform && P.msh == (double)(P.M / 2);
+}
 fzp_status bluestein_layout(Plan& P, FormSizes* out);
 fzp_status bluestein_fill_tables(Plan& P, cudaStream_t s);  // buffers already assigned
 fzp_status bluestein_build_tables(Plan& P);                 // layout + allocate + fill

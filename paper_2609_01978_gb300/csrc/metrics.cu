@@ -29,7 +29,7 @@ constexpr double AIRY_NULL = 3.8317059702075125 / 3.14159265358979323846;
 
 __device__ __forceinline__ int64_t isqrt64(int64_t v) {
   if (v <= 0) return 0;
-  int64_t r = (int64_t)sqrt((double)v);
+  int64_t r = (int64_t)sqrtf((float)v);  // within 2 of the root below 2^46
   while (r * r > v) --r;
   while ((r + 1) * (r + 1) <= v) ++r;
   return r;
@@ -63,25 +63,42 @@ __global__ void k_sums(int M, double p, double rnull2, const double2* __restrict
 
 __global__ void k_count(int64_t N, int64_t c, int64_t sR, double* scratch) {
   unsigned long long acc = 0;
+  __shared__ unsigned long long part[8];
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
     const int64_t dj = j - c;
     if (dj * dj <= sR) acc += (unsigned long long)(2 * isqrt64(sR - dj * dj) + 1);
   }
-  atomicAdd(reinterpret_cast<unsigned long long*>(&scratch[S_COUNT]), acc);
+  // one atomic per block: a thread's each, 65,536 on one word, took 46 us
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) acc += part[q];
+    if (acc) atomicAdd(reinterpret_cast<unsigned long long*>(&scratch[S_COUNT]), acc);
+  }
 }
 
-// In-place radix-2 DIT on SMEM (bit-reversed input), FP64, twiddles computed here.
+// In-place radix-2 DIT on SMEM (bit-reversed input), FP64; the twiddles
+// e^{-2 pi i k / n}, k < n / 2, once per block behind the row (FP64 sines are
+// slow here: one per butterfly took most of the transform's time).
 __device__ void dit64(double2* x, int logn) {
   const int n = 1 << logn;
+  double2* tw = x + n;
+  for (int k = threadIdx.x; k < n / 2; k += blockDim.x) {
+    double sn, cs;
+    sincospi(-(double)k / (double)(n / 2), &sn, &cs);
+    tw[k] = make_double2(cs, sn);
+  }
+  __syncthreads();
   for (int s = 1; s <= logn; ++s) {
     const int half = 1 << (s - 1);
     for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
       const int k = b & (half - 1);
       const int i0 = ((b >> (s - 1)) << s) + k, i1 = i0 + half;
-      double sn, cs;
-      sincospi(-(double)k / (double)half, &sn, &cs);
+      const double2 w = tw[k << (logn - s)];
       const double2 a = x[i0], v = x[i1];
-      const double2 t = make_double2(v.x * cs - v.y * sn, v.x * sn + v.y * cs);
+      const double2 t = make_double2(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x);
       x[i0] = make_double2(a.x + t.x, a.y + t.y);
       x[i1] = make_double2(a.x - t.x, a.y - t.y);
     }
@@ -170,31 +187,83 @@ __device__ double crossing(const double* y, const double* s, int i, double half)
   return (double)i + 0.5 * (lo + hi);
 }
 
-// One thread: FWHM along the centre row (axis 0) or column (axis 1).
+// Spline slope at an interior point i far from both ends, by a warp: the system
+// s_{i-1} + 4 s_i + s_{i+1} = 3 (y_{i+1} - y_{i-1}) has the Green's function
+// (-q)^|k| / (2 sqrt 3), q = 2 - sqrt 3 (1e-17 at 30 points), so the ends'
+// conditions do not reach i.  g: the lane's weight (k = lane).
+__device__ double slope_at(const double* y, int i, double g) {
+  const int lane = threadIdx.x & 31;
+  double s = g * 3.0 * (y[i + lane + 1] - y[i + lane - 1]);
+  if (lane > 0) s += g * 3.0 * (y[i - lane + 1] - y[i - lane - 1]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// Root of the Hermite piece i at `half` by a warp: 32 points at a time, the
+// interval of the sign change kept (13 rounds: 2^-65).
+__device__ double crossing_warp(const double* y, const double* s, double half) {
+  const int lane = threadIdx.x & 31;
+  double lo = 0.0, w = 1.0;
+  const bool neg = y[0] - half < 0;
+  for (int it = 0; it < 13; ++it) {
+    const double t = lo + w * (double)(lane + 1) * (1.0 / 32.0);
+    const unsigned same = __ballot_sync(0xffffffffu, (hermite(y, s, 0, t) - half < 0) == neg);
+    const int k = min(31, __popc(same & ~(same + 1u)));  // points before the first change
+    lo += w * (double)k * (1.0 / 32.0);
+    w *= 1.0 / 32.0;
+  }
+  return lo + 0.5 * w;
+}
+
+// One warp: FWHM along the centre row (axis 0) or column (axis 1).  A crossing
+// within 33 points of an end takes the whole tridiagonal system, in one lane.
 __global__ void k_fwhm(int M, double p, const double2* __restrict__ U, double* work, double* scratch) {
-  if (threadIdx.x != 0) return;
-  const int axis = blockIdx.x;
+  const int axis = blockIdx.x, lane = threadIdx.x;
   double* y = work + (size_t)axis * 3 * M;
   double* s = y + M;
   double* cp = s + M;
   const int k = M / 2;
-  for (int i = 0; i < M; ++i) {
+  for (int i = lane; i < M; i += 32) {
     const double2 u = axis == 0 ? U[(int64_t)k * M + i] : U[(int64_t)i * M + k];
     y[i] = u.x * u.x + u.y * u.y;
   }
+  __syncwarp();
   const double ym = y[k - 1], y0 = y[k], yp = y[k + 1];
   const double den = ym - 2.0 * y0 + yp;
   const double peak = den != 0.0 ? y0 - 0.125 * (yp - ym) * (yp - ym) / den : y0;
   const double half = 0.5 * peak;
-  spline_slopes(y, M, s, cp);
-  int m = k;
-  while (m > 0 && y[m] >= half) --m;
-  const double xl = crossing(y, s, m, half);
-  m = k;
-  while (m < M - 1 && y[m] >= half) ++m;
-  const double xr = crossing(y, s, m - 1, half);
-  scratch[S_OUT + axis] = (xr - xl) * p;
-  if (axis == 0) scratch[S_OUT + 2] = y0;
+  // first point below half on either side (the ends if there is none)
+  int ml = k, mr = k;
+  while (ml > 0) {
+    const int i = ml - lane;
+    const unsigned stop = __ballot_sync(0xffffffffu, i <= 0 || !(y[max(i, 0)] >= half));
+    if (stop) { ml = max(ml - (__ffs(stop) - 1), 0); break; }
+    ml -= 32;
+  }
+  while (mr < M - 1) {
+    const int i = mr + lane;
+    const unsigned stop = __ballot_sync(0xffffffffu, i >= M - 1 || !(y[min(i, M - 1)] >= half));
+    if (stop) { mr = min(mr + (__ffs(stop) - 1), M - 1); break; }
+    mr += 32;
+  }
+  double xl, xr;
+  if (ml >= 33 && mr + 33 < M && mr > k) {
+    double g = 0.28867513459481288;  // 1 / (2 sqrt 3)
+    for (int q = 0; q < lane; ++q) g *= -0.26794919243112271;
+    const double sl[2] = {slope_at(y, ml, g), slope_at(y, ml + 1, g)}, sr[2] = {slope_at(y, mr - 1, g), slope_at(y, mr, g)};
+    xl = (double)ml + crossing_warp(y + ml, sl, half);
+    xr = (double)(mr - 1) + crossing_warp(y + mr - 1, sr, half);
+  } else {
+    if (lane != 0) return;
+    spline_slopes(y, M, s, cp);
+    xl = crossing(y, s, ml, half);
+    xr = crossing(y, s, mr - 1, half);
+  }
+  if (lane == 0) {
+    scratch[S_OUT + axis] = (xr - xl) * p;
+    if (axis == 0) scratch[S_OUT + 2] = y0;
+  }
 }
 
 }  // namespace
@@ -209,8 +278,8 @@ static fzp_status extract_enqueue(int M, double p, double rnull, int64_t N, int6
   FZP_CUDA_TRY(cudaMemsetAsync(scr, 0, S_FFT * sizeof(double), s));
   k_sums<<<256, 256, 0, s>>>(M, p, rnull * rnull, U, scr);
   k_count<<<256, 256, 0, s>>>(N, c, sR, scr);
-  k_fft_rows<<<M, 256, M * sizeof(double2), s>>>(M, logM, U, F);
-  k_fft_cols<<<M, 256, M * sizeof(double2), s>>>(M, logM, F, scr);
+  k_fft_rows<<<M, 256, (M + M / 2) * sizeof(double2), s>>>(M, logM, U, F);
+  k_fft_cols<<<M, 256, (M + M / 2) * sizeof(double2), s>>>(M, logM, F, scr);
   k_fwhm<<<2, 32, 0, s>>>(M, p, U, scr + S_FFT, scr);
   FZP_CUDA_TRY(cudaGetLastError());
   FZP_CUDA_TRY(cudaMemcpyAsync(h, scr, S_FFT * sizeof(double), cudaMemcpyDeviceToHost, s));

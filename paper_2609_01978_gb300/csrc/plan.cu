@@ -311,7 +311,7 @@ fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t
   // rows up and down from the axis
   const int64_t c = P.c, up = b - 1 - c, dn = c - a, h = std::min(up, dn);
   const bool nodes = P.nd.n > 0;
-  P.nd.yfull = P.nd.even && up != dn;
+  P.nd.yfull = (P.nd.even || bluestein_even(P)) && up != dn;
   const size_t acc = nodes ? (size_t)(P.nd.yfull ? P.nd.n : P.nd.ns) * P.nd.ns : (size_t)P.M * P.M;
   FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, acc * sizeof(double2), s));
   if (a >= b) return FZP_OK;
@@ -537,12 +537,12 @@ fzp_status fzp_plan_info_get(fzp_plan_t plan, fzp_plan_info* out) {
   out->dx = P.dx; out->R = P.R; out->kappa = P.kappa; out->x0 = P.x0;
   out->M = P.M; out->form = P.form; out->precision = P.precision;
   out->stripe_rows = P.stripe_rows;
-  out->fft_length = P.form == FZP_FORM_SACZT ? P.sa.P : P.bs.L;
+  out->fft_length = P.form == FZP_FORM_SACZT ? P.sa.P : P.bs.L_full;
   out->promote = P.form == FZP_FORM_DENSE ? P.dn.promote_kblocks : 0;
   out->row_batch = P.form == FZP_FORM_BLUESTEIN ? (int32_t)P.bs.rows : 0;
   out->chunk_rows = P.chunk_rows;
   out->cluster = P.form == FZP_FORM_DENSE ? P.dn.cluster : 0;
-  out->fft_inner = P.form == FZP_FORM_BLUESTEIN ? (P.bs.seg ? 4096 : (int32_t)P.bs.L2) : 0;
+  out->fft_inner = P.form == FZP_FORM_BLUESTEIN ? (P.bs.seg ? 4096 : (int32_t)std::min<int64_t>(P.bs.L_full, 4096)) : 0;
   out->conv = P.form == FZP_FORM_BLUESTEIN ? (P.bs.seg ? 2 : 1) : 0;
   out->ctas = P.form == FZP_FORM_DENSE ? P.dn.max_ctas : 0;
   out->levels = P.levels;
