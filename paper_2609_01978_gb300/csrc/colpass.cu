@@ -18,7 +18,7 @@
 namespace fzp {
 namespace {
 
-constexpr int TN = 64, TM = 64, TJ = 16, PJ = 128;
+constexpr int TN = 64, TM = 64, TJ = 16, PJ = 128;  // output tiles of 64 (48: NA = 3 outputs per thread and side)
 
 struct ColArgs {
   int64_t c, j0, rows, c1_stride;
@@ -63,28 +63,44 @@ __device__ __forceinline__ double2 kern(const RowPhase<double>& rp, int n) {
   return cis_turns_d(rp.a - (double)n * rp.b);
 }
 
+// Factors of a row's kernel values in an output tile from n0: q < 8: e^{-2 pi i
+// (n0 + 8 q) B}; q < 16: e^{-2 pi i (q - 8) B}; 16, 17: e^{2 pi i A} at dj and, of
+// a folded row, at -dj (where B changes sign: the conjugate product).
+__device__ __forceinline__ double2 factor(int q, int n0, const RowPhase<double>& r0, const RowPhase<double>& r1, bool folded) {
+  if (q == 17 && !folded) return make_double2(0.0, 0.0);
+  return cis_turns_d(q < 8 ? -(double)(n0 + 8 * q) * r0.b : q < 16 ? -(double)(q - 8) * r0.b : q == 16 ? r0.a : r1.a);
+}
+__device__ __forceinline__ float2 factor(int, int, const RowPhase<float>&, const RowPhase<float>&, bool) {
+  return make_float2(0.f, 0.f);  // (FP32 evaluates its sines)
+}
+
 // grid (M/TM, M/TN, ceil(rows/jc)); 256 threads; each thread 4 n x 4 m outputs.
 // TAB: the kernel's columns from a table E [n][estride] instead of their phase.
-template <typename R, bool TAB = false>
+template <typename R, bool TAB = false, int NA = 4>
 __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
   using C = typename Cplx<R>::T;
+  constexpr int TN = 16 * NA, TM = 16 * NA;
   __shared__ C sK[TJ][TN + 1];
   __shared__ C sC[TJ][TM + 1];
   // phases of 128 rows at a time (they are FP64, at two operations per clock and
   // SM): of dj (mirrored rows: -dj) and, folded, of -dj
   __shared__ RowPhase<R> sP[2][PJ];
+  // FP64: e^{-2 pi i n B} as products of 8 + 8 phasors per row (an FP64 sine per
+  // element took as long as the products), and the rows' e^{2 pi i A}, A at dj and -dj
+  constexpr bool FACT = sizeof(R) == 8 && !TAB;
+  __shared__ C sF[FACT ? TJ : 1][18];
   const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
   const int64_t jb = (int64_t)blockIdx.z * g.jc;
   const int64_t je = jb + g.jc < g.rows ? jb + g.jc : g.rows;
   const int tid = threadIdx.x;
   const int tn = tid >> 4, tm = tid & 15;  // 16 x 16 threads, 4 x 4 outputs each
   // outputs of this warp's rows and of the tile's columns (uniform per warp)
-  const int na = min(4, max(0, (g.ny - n0 - (tn & ~1) + 15) / 16)), nb = min(4, (g.M - m0 + 15) / 16);
-  C acc[4][4];
+  const int na = min(NA, max(0, (g.ny - n0 - (tn & ~1) + 15) / 16)), nb = min(NA, (g.M - m0 + 15) / 16);
+  C acc[NA][NA];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < NA; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) { acc[a][b].x = 0; acc[a][b].y = 0; }
+    for (int b = 0; b < NA; ++b) { acc[a][b].x = 0; acc[a][b].y = 0; }
   for (int64_t j = jb; j < je; j += TJ) {
     const int pj = (int)(j - jb) & (PJ - 1);
     if (!TAB && pj == 0) {
@@ -117,6 +133,14 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
       sC[jj][mm] = v;
     }
     __syncthreads();
+    if (FACT) {
+      for (int t = tid; t < TJ * 18; t += 256) {
+        const int jj = t / 18, q = t % 18;
+        const RowPhase<R> r0 = sP[0][pj + jj], r1 = sP[1][pj + jj];
+        if (j + jj < je) sF[jj][q] = factor(q, n0, r0, r1, g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c);
+      }
+      __syncthreads();
+    }
     for (int t = tid; t < TJ * TN; t += 256) {
       const int jj = TAB ? t % TJ : t / TN, nn = TAB ? t / TJ : t % TN;
       C k;
@@ -125,6 +149,11 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
         const float2 e = __ldg(g.E + (int64_t)(n0 + nn) * g.estride + j + jj);
         k.x = e.x;
         k.y = e.y;
+      } else if (FACT && j + jj < je) {
+        C e = cmul(sF[jj][nn >> 3], sF[jj][8 + (nn & 7)]);
+        k = cmul(sF[jj][16], e);
+        e.y = -e.y;
+        k = cadd(k, cmul(sF[jj][17], e));
       } else if (j + jj < je) {
         k = kern(sP[0][pj + jj], n0 + nn);
         if (g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c) k = cadd(k, kern(sP[1][pj + jj], n0 + nn));
@@ -133,13 +162,13 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     }
     __syncthreads();
     if (na == 0) {
-    } else if (na < 4 || nb < 4) {  // an edge tile: the outputs it has
+    } else if (na < NA || nb < NA) {  // an edge tile: the outputs it has
 #pragma unroll 1
       for (int jj = 0; jj < TJ; ++jj)
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < NA; ++a)
 #pragma unroll
-          for (int b = 0; b < 4; ++b)
+          for (int b = 0; b < NA; ++b)
             if (a < na && b < nb) {
               const C kv = sK[jj][tn + 16 * a], cv = sC[jj][tm + 16 * b];
               acc[a][b].x = fma(kv.x, cv.x, fma(-kv.y, cv.y, acc[a][b].x));
@@ -148,15 +177,15 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     } else
 #pragma unroll 4
     for (int jj = 0; jj < TJ; ++jj) {
-      C kv[4], cv[4];
+      C kv[NA], cv[NA];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) kv[a] = sK[jj][tn + 16 * a];
+      for (int a = 0; a < NA; ++a) kv[a] = sK[jj][tn + 16 * a];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) cv[b] = sC[jj][tm + 16 * b];
+      for (int b = 0; b < NA; ++b) cv[b] = sC[jj][tm + 16 * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < NA; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < NA; ++b) {
           acc[a][b].x = fma(kv[a].x, cv[b].x, fma(-kv[a].y, cv[b].y, acc[a][b].x));
           acc[a][b].y = fma(kv[a].x, cv[b].y, fma(kv[a].y, cv[b].x, acc[a][b].y));
         }
@@ -164,9 +193,9 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < NA; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
+    for (int b = 0; b < NA; ++b) {
       const int n = n0 + tn + 16 * a, m = m0 + tm + 16 * b;
       if (n >= g.ny || m >= g.M) continue;
       double ux = (double)acc[a][b].x, uy = (double)acc[a][b].y;
@@ -234,11 +263,15 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   g.slice_off = P.nd.slice_elems;
   if (nodes_two_masks(P)) g.sin_off = 128 * P.c1_stride;
   // rows per block: 2048, fewer where that leaves the GPU idle (few output tiles)
-  const int tx = (g.M + TM - 1) / TM, ty = (g.ny + TN - 1) / TN;
+  // FP64 on M / 2 + 1 outputs: tiles of 48 (129 = 3 x 43: nine equal tiles, where
+  // tiles of 64 are four full ones and five slivers that share SMs with them)
+  const int T = even ? 48 : TM;
+  const int tx = (g.M + T - 1) / T, ty = (g.ny + T - 1) / T;
   const int64_t tiles = (int64_t)tx * ty;
   g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / 304 + TJ - 1) / TJ * TJ));
   dim3 grid((unsigned)tx, (unsigned)ty, (unsigned)((rows + g.jc - 1) / g.jc));
-  if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
+  if (even) k_colpass<double, false, 3><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
+  else if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
   else k_colpass<float><<<grid, 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());

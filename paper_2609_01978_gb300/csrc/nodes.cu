@@ -162,17 +162,21 @@ __device__ __forceinline__ void span_of(const NodeArgs& a, int64_t s, int64_t& k
   stripe_kspan(a, jb, jb + BN < a.j_end ? jb + BN : a.j_end, klo, khi);
 }
 
-// Zeroes C1 (all blocks but the first) and builds the work list (the first):
+// Zeroes C1 and, at a propagation's start, the accumulator (all blocks but the
+// first) and builds the work list (the first):
 // units (chunk g, stripe s) in chunk order, so that the CTAs at work at one time
 // share kernel blocks.  Every chunk's stripes are one range around the stripe
 // whose span holds the others' ends: the one nearest the axis or, with the
 // octant, where the chord takes over from the diagonal.
 template <int BN>
-__global__ void __launch_bounds__(1024) k_nodes_prep(const NodeArgs a, int* sched, float4* c1, int64_t c1_vec) {
+__global__ void __launch_bounds__(1024) k_nodes_prep(const NodeArgs a, int* sched, float4* c1, int64_t c1_vec, float4* uacc,
+                                                      int64_t uacc_vec) {
   if (blockIdx.x > 0) {
     const int64_t step = (int64_t)(gridDim.x - 1) * blockDim.x;
     for (int64_t t = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x; t < c1_vec; t += step)
       c1[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t t = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x; t < uacc_vec; t += step)
+      uacc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
     return;
   }
   int* off = sched;
@@ -904,24 +908,28 @@ __global__ void __launch_bounds__(512) k_interp_W(const InterpSpec a, const doub
 }
 
 // X[l][o] = sum_k Wy[k][o] V[k][l], k over the ny nodes of the rows' axis: a
-// block per 4 outputs and 32 nodes.
+// block per output and 32 nodes, its four warps a quarter of the sum each.
 __global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, const double* __restrict__ Wy,
                                                      const double2* __restrict__ V, double2* __restrict__ X) {
-  const int l = blockIdx.x * 32 + (threadIdx.x & 31), o = blockIdx.y * 4 + (threadIdx.x >> 5);
-  if (o >= Mo) return;
-  double2 x[4];  // four chains: an FP64 multiply-add's latency is long
-#pragma unroll
-  for (int q = 0; q < 4; ++q) x[q] = make_double2(0.0, 0.0);
-#pragma unroll 2
-  for (int k = 0; k < ny; k += 4)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const double2 v = V[(k + q) * ns + l];
-      const double w = Wy[(k + q) * Mo + o];
-      x[q].x = fma(w, v.x, x[q].x);
-      x[q].y = fma(w, v.y, x[q].y);
-    }
-  X[l * Mo + o] = make_double2((x[0].x + x[1].x) + (x[2].x + x[3].x), (x[0].y + x[1].y) + (x[2].y + x[3].y));
+  __shared__ double2 part[4][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, l = blockIdx.x * 32 + lane, o = blockIdx.y;
+  const int n4 = ny / 4;
+  const double2* v = V + (size_t)w * n4 * ns + l;
+  const double* c = Wy + (size_t)w * n4 * Mo + o;
+  double2 x[2];
+  x[0] = x[1] = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k = 0; k < n4; k += 2, v += 2 * ns, c += 2 * Mo) {
+    const double2 v0 = v[0], v1 = v[ns];
+    const double c0 = c[0], c1 = c[Mo];
+    x[0].x = fma(c0, v0.x, x[0].x);
+    x[0].y = fma(c0, v0.y, x[0].y);
+    x[1].x = fma(c1, v1.x, x[1].x);
+    x[1].y = fma(c1, v1.y, x[1].y);
+  }
+  part[w][lane] = cadd(x[0], x[1]);
+  __syncthreads();
+  if (w == 0) X[l * Mo + o] = cadd(cadd(part[0][lane], part[1][lane]), cadd(part[2][lane], part[3][lane]));
 }
 
 struct InterpOut {
@@ -936,40 +944,59 @@ struct InterpOut {
 // exchanged; only blocks on and below the diagonal run and both are stored),
 // the output chirp and prefactor, and the stores: with an even field output o
 // stands for the samples M/2 + o and M/2 - o (o = M/2: sample 0 alone).
-// Block: 8 x 4 outputs (columns x rows), one per thread.  chirp[i] = e^{i pi
-// x_i^2 / (lambda f)} of the ROI samples, as k_interp_W left it.
+// Block: 8 x 4 outputs (columns x rows), two threads per output with half of
+// the sum each, operands through shared memory.  chirp[i] = e^{i pi x_i^2 /
+// (lambda f)} of the ROI samples, as k_interp_W left it.
 constexpr int ITX = 8, ITY = 4;
-__global__ void __launch_bounds__(ITX * ITY) k_interp_cols(const InterpOut a, const double* __restrict__ W,
-                                                           const double2* __restrict__ X,
-                                                           const double2* __restrict__ chirp, double2* __restrict__ out) {
+__global__ void __launch_bounds__(2 * ITX * ITY) k_interp_cols(const InterpOut a, const double* __restrict__ W,
+                                                               const double2* __restrict__ X,
+                                                               const double2* __restrict__ chirp,
+                                                               double2* __restrict__ out) {
   const int n0 = blockIdx.y * ITY, m0 = blockIdx.x * ITX;
   if (a.sym && m0 >= n0 + ITY) return;
-  const int h = a.M / 2;
-  const int on = n0 + (int)threadIdx.x / ITX, om = m0 + (int)threadIdx.x % ITX;
-  const int cn = min(on, a.Moy - 1), cm = min(om, a.Mox - 1);
-  double2 u[2], t[2];
-#pragma unroll
-  for (int q = 0; q < 2; ++q) u[q] = t[q] = make_double2(0.0, 0.0);
-#pragma unroll 4
-  for (int l = 0; l < a.ns; l += 2)
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const double2 x = __ldg(X + (l + q) * a.Moy + cn);
-      const double w = __ldg(W + (l + q) * a.Mox + cm);
-      u[q].x = fma(w, x.x, u[q].x);
-      u[q].y = fma(w, x.y, u[q].y);
+  __shared__ double2 sXn[64][ITY], sXm[64][ITX];
+  __shared__ double sWm[64][ITX], sWn[64][ITY];
+  __shared__ double2 half[ITX * ITY];
+  const int h = a.M / 2, tid = threadIdx.x;
+  const int side = tid / (ITX * ITY), q = tid % (ITX * ITY), qn = q / ITX, qm = q % ITX;
+  const int on = n0 + qn, om = m0 + qm;
+  double2 u = make_double2(0.0, 0.0), t = u;
+  for (int l0 = 0; l0 < a.ns; l0 += 64) {  // ns is 64 or 128
+    if (l0 > 0) __syncthreads();
+    for (int e = tid; e < 64 * ITY; e += 2 * ITX * ITY) {
+      const int l = e / ITY, c = min(n0 + e % ITY, a.Moy - 1);
+      sXn[l][e % ITY] = __ldg(X + (l0 + l) * a.Moy + c);
+      if (a.sym) sWn[l][e % ITY] = __ldg(W + (l0 + l) * a.Mox + c);
+    }
+    for (int e = tid; e < 64 * ITX; e += 2 * ITX * ITY) {
+      const int l = e / ITX, c = min(m0 + e % ITX, a.Mox - 1);
+      sWm[l][e % ITX] = __ldg(W + (l0 + l) * a.Mox + c);
+      if (a.sym) sXm[l][e % ITX] = __ldg(X + (l0 + l) * a.Moy + c);
+    }
+    __syncthreads();
+    const int lb = 32 * side;
+#pragma unroll 8
+    for (int l = lb; l < lb + 32; ++l) {
+      const double2 x = sXn[l][qn];
+      const double w = sWm[l][qm];
+      u.x = fma(w, x.x, u.x);
+      u.y = fma(w, x.y, u.y);
       if (a.sym) {
-        const double2 y = __ldg(X + (l + q) * a.Moy + cm);
-        const double v = __ldg(W + (l + q) * a.Mox + cn);
-        t[q].x = fma(v, y.x, t[q].x);
-        t[q].y = fma(v, y.y, t[q].y);
+        const double2 y = sXm[l][qm];
+        const double v = sWn[l][qn];
+        t.x = fma(v, y.x, t.x);
+        t.y = fma(v, y.y, t.y);
       }
     }
+  }
+  u = cadd(u, t);
+  if (side) half[q] = u;
+  __syncthreads();
+  if (side) return;
+  u = cadd(u, half[q]);
   if (on >= a.Moy || om >= a.Mox || (a.sym && om > on)) return;
   const int n = a.eveny ? (on < h ? h + on : 0) : on, m = a.evenx ? (om < h ? h + om : 0) : om;
-  const double2 v = cmul(cmul(make_double2((u[0].x + u[1].x) + (t[0].x + t[1].x), (u[0].y + u[1].y) + (t[0].y + t[1].y)),
-                              cmul(chirp[n], chirp[m])),
-                         a.pre);
+  const double2 v = cmul(cmul(u, cmul(chirp[n], chirp[m])), a.pre);
   auto put = [&](int nn, int mm) {
     double2* o = out + (int64_t)nn * a.M + mm;
     double2 z = v;
@@ -1135,7 +1162,9 @@ fzp_status launch(Plan& P, NodeArgs& a, cudaStream_t s) {
   const int64_t vec = (int64_t)c1r * P.c1_stride * a.slices / 4;
   const unsigned zb = (unsigned)std::min<int64_t>(2 * P.dn.num_sms, (vec + 4095) / 4096);
   k_nodes_prep<S::BN><<<1 + zb, 1024, 0, s>>>(a, const_cast<int*>(a.sched),
-                                             reinterpret_cast<float4*>(P.d_C1 + (size_t)a.y_off * P.c1_stride), vec);
+                                             reinterpret_cast<float4*>(P.d_C1 + (size_t)a.y_off * P.c1_stride), vec,
+                                             reinterpret_cast<float4*>(P.d_Uacc), P.nd.zero_acc);
+  P.nd.zero_acc = 0;
   if (!S::LD) prof_begin(P, s);  // (the SA-CZT's dominant kernel is another)
   k_nodes<NT, MASK><<<P.dn.num_sms, NUM_THREADS, S::SMEM, s>>>(a, tm);
   if (!S::LD) prof_end(P, s);
@@ -1326,13 +1355,13 @@ fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cuda
   const NodeSet& z = P.nd;
   const bool eveny = z.even && !z.yfull;
   const int ny = z.yfull ? z.n : z.ns, Moy = eveny ? z.Mo : P.M;
-  k_interp_rows<<<dim3((unsigned)(z.ns / 32), (unsigned)((Moy + 3) / 4)), 128, 0, s>>>(
+  k_interp_rows<<<dim3((unsigned)(z.ns / 32), (unsigned)Moy), 128, 0, s>>>(
       ny, z.ns, Moy, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
   // e^{ikf} / i: f / lambda - 1/4 turns
   const double turns = std::fmod(P.f / P.lambda, 1.0) - 0.25, amp = P.dx2 / (P.lambda * z.dist);
   InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, sym ? 1 : 0,
               make_double2(amp * std::cos(2.0 * M_PI * turns), amp * std::sin(2.0 * M_PI * turns)), accumulate};
-  k_interp_cols<<<dim3((unsigned)((z.Mo + ITX - 1) / ITX), (unsigned)((Moy + ITY - 1) / ITY)), ITX * ITY, 0, s>>>(
+  k_interp_cols<<<dim3((unsigned)((z.Mo + ITX - 1) / ITX), (unsigned)((Moy + ITY - 1) / ITY)), 2 * ITX * ITY, 0, s>>>(
       a, z.d_W, z.d_X, z.d_chirp, reinterpret_cast<double2*>(d_field));
   P.launches += 2;
   FZP_CUDA_TRY(cudaGetLastError());

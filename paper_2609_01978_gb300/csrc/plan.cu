@@ -313,7 +313,9 @@ fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t
   const bool nodes = P.nd.n > 0;
   P.nd.yfull = (P.nd.even || bluestein_even(P)) && up != dn;
   const size_t acc = nodes ? (size_t)(P.nd.yfull ? P.nd.n : P.nd.ns) * P.nd.ns : (size_t)P.M * P.M;
-  FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, acc * sizeof(double2), s));
+  // the dense form on nodes zeroes it in its first launch
+  P.nd.zero_acc = nodes && P.form == FZP_FORM_DENSE && a < b ? (int64_t)acc : 0;
+  if (!P.nd.zero_acc) FZP_CUDA_TRY(cudaMemsetAsync(P.d_Uacc, 0, acc * sizeof(double2), s));
   if (a >= b) return FZP_OK;
   auto run = [&](int64_t j0, int64_t j1, RowKind kind, bool octant) {
     fzp_status st = FZP_OK;
