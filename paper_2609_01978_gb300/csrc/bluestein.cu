@@ -134,6 +134,9 @@ __device__ void dif_inverse(C* x, int logn, const C* __restrict__ tw, int twN) {
   }
 }
 
+// Decimated rows (k_dec): grid points that a column's value is spread over.
+constexpr int DTAPS = 6;
+
 struct RowArgs {
   MaskGeom mg;
   int64_t N, L, L1, L2;
@@ -166,6 +169,11 @@ struct RowArgs {
   PhaseRule ph;      // partitioned convolution: the zone phase of the mask walk
   int half;          // even output grid: columns from the axis on, outputs x and -x added
   int octant;        // columns up to the row's distance from the axis only, the last one halved
+  // decimated rows: chirp turns per squared column and per column (units of
+  // 2^-64), the second difference (2^-32), the sums' weights on the grid points
+  uint64_t Kc, Kl;
+  uint32_t cc2;
+  float T[2][DTAPS][4];
 };
 
 // Aperture transmission of sample (j, i): T e^{i phi}, optional deformation.
@@ -907,8 +915,9 @@ __global__ void __launch_bounds__(STH, 1) k_f2_d16(RowArgs a, int mode) {
   }
 }
 
-// G_s = FFT_P(g_s) for every block s (one CTA per block, grid-strided).
-__global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int64_t col0, int S, int M, double delta, float2* G) {
+// G_s = FFT_P(g_s) for every block s (one CTA per block, grid-strided); blocks
+// every S input columns, W of them long.
+__global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int64_t col0, int S, int W, int M, double delta, float2* G) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* b0 = reinterpret_cast<float2*>(smem_raw);
   float2* b1 = b0 + SBUF;
@@ -926,7 +935,7 @@ __global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int64_t col0, 
       int64_t k = 0;
       bool have = false;
       if (q < M) { k = q - is; have = true; }
-      else if (q > SP - S) { k = (int64_t)q - SP - is; have = true; }
+      else if (q > SP - W) { k = (int64_t)q - SP - is; have = true; }
       if (have) {
         const double kk = (double)k;  // |k| < 2^24: k^2 exact in FP64
         v[r] = cis_turns<float>(0.5 * delta * kk * kk);
@@ -1174,6 +1183,397 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// Decimated rows.  The outputs' band is narrow: between a row's columns the
+// phases of the nodes' exponentials e^{-2 pi i delta (m - m_c) x} differ by at most
+// u = pi delta (n - 1), so over a chunk of D = 16 or 32 columns each of them is a
+// polynomial, and interpolating it from DTAPS = 6 points of a grid of pitch D is
+// off by at most 0.0049 (D u)^6 (the outermost node, a quarter outside the ROI).
+// Transposed: a column's value times the input chirp is spread over the six grid
+// points, and the row goes on as N / D + 5 points through the convolution above:
+// two rows to a 4096-point transform (offsets 0 and 2048: with S + 5 + n < 2050
+// neither meets the other's outputs) instead of N / 3840 transforms a row.
+//
+// A lane takes one chunk of two neighbouring rows, all in registers: the chirp by
+// a 64-bit fixed-point phase walked in 32 bits (as the zone phase), the value, and
+// four running sums (c0 += z, c1 += c0, ...) per 16 columns, which are their
+// binomial moments; the weights T (decimation_weights) take them to the grid
+// points; lanes exchange the overlaps by shuffles.  No table is read per column.
+// What is left is issue-bound on the generators.
+// ---------------------------------------------------------------------------
+constexpr int DROW = SP / 2;                    // offset of the second row
+constexpr int DGRP = DROW / 32;                 // warp groups of chunks a row
+constexpr size_t DEC_SMEM = sizeof(float2) * (2 * SBUF + 15 * 256 + 256 + 2 * DGRP * (DTAPS - 1));
+
+struct DecRow {
+  int64_t dj;
+  int32_t lo, hi;  // the row's chord (lo > hi: empty)
+};
+
+__device__ __forceinline__ float2 cis_rad(float x) { return make_float2(__cosf(x), __sinf(x)); }
+
+// Bits of the 16 columns from x that lie in the row's chord.
+__device__ __forceinline__ uint32_t chord_bits(const DecRow& r, int32_t x) {
+  const int a = max(r.lo - x, 0), b = min(r.hi - x, 15);
+  return a <= b ? (0xFFFFu >> (15 - b + a)) << a : 0u;
+}
+
+__device__ __forceinline__ uint32_t open_bits(const RowArgs& a, const DecRow& r, int32_t x) {
+  const uint32_t in = chord_bits(r, x);
+  uint32_t w = 0u;
+  if (in != 0u && !walk_bits16(walk16((int64_t)x - a.mg.c, r.dj * r.dj, a.ph), a.ph, w)) w = chunk_bits(x, r.dj * r.dj, a.mg);
+  return w & in;
+}
+
+// The running sums of 16 columns; add(z): the next column's value joins c[0] first.
+__device__ __forceinline__ void sums_step(float2 (&c)[4]) {
+#pragma unroll
+  for (int q = 1; q < 4; ++q) c[q] = cadd(c[q], c[q - 1]);
+}
+
+// c += w times the sums of a single value z at column k of the 16.
+__device__ __forceinline__ void sums_at(float2 (&c)[4], int k, float2 z, float w) {
+  const float m = (float)(16 - k);
+  const float b[4] = {w, w * m, w * m * (m + 1.0f) * 0.5f, w * m * (m + 1.0f) * (m + 2.0f) * (1.0f / 6.0f)};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c[q].x = fmaf(b[q], z.x, c[q].x);
+    c[q].y = fmaf(b[q], z.y, c[q].y);
+  }
+}
+
+__device__ __forceinline__ void sums_out(const RowArgs& a, int sub, const float2 (&c)[4], float2 (&tap)[DTAPS]) {
+#pragma unroll
+  for (int q = 0; q < DTAPS; ++q)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      tap[q].x = fmaf(a.T[sub][q][e], c[e].x, tap[q].x);
+      tap[q].y = fmaf(a.T[sub][q][e], c[e].y, tap[q].y);
+    }
+}
+
+// The chirp's 32-bit phase and its first difference at column di0.
+struct Chirp16 {
+  uint32_t f, d;
+};
+__device__ __forceinline__ Chirp16 chirp16(const RowArgs& a, int64_t di0) {
+  Chirp16 p;
+  p.f = (uint32_t)((a.Kc * (uint64_t)(di0 * di0) + a.Kl * (uint64_t)di0) >> 32);
+  p.d = (uint32_t)((a.Kc * (uint64_t)(2 * di0 + 1) + a.Kl + 0x80000000ull) >> 32);
+  return p;
+}
+
+// Folded plates: half weight of the axis column and of the diagonal's columns, as
+// a correction of the sums.  value(k): the chunk's column k.
+template <typename F>
+__device__ __forceinline__ void fold_weights(const RowArgs& a, const DecRow& r, int32_t x, float2 (&c)[4], F value) {
+  const int32_t dj = (int32_t)r.dj, cc = (int32_t)a.mg.c;
+  const int ka = a.half ? cc - x : -1, kd = a.octant ? cc + dj - x : -1, ke = a.octant && !a.half && dj > 0 ? cc - dj - x : -1;
+  if ((unsigned)ka < 16u) sums_at(c, ka, value(ka), -0.5f);
+  if ((unsigned)kd < 16u) sums_at(c, kd, value(kd), ka == kd ? -0.25f : -0.5f);
+  if ((unsigned)ke < 16u) sums_at(c, ke, value(ke), -0.5f);
+}
+
+constexpr float RAD32 = 6.28318530717958648f / 4294967296.0f;  // 2^-32 turns in radians
+
+// Binary plate: both rows share the chirp's sine and cosine.
+template <int D>
+__device__ __forceinline__ void dec_flat(const RowArgs& a, const DecRow (&row)[2], int32_t x0, float2 (&tap)[2][DTAPS]) {
+#pragma unroll 1
+  for (int sub = 0; sub < D / 16; ++sub) {
+    const int32_t x = x0 + 16 * sub;
+    const Chirp16 p0 = chirp16(a, (int64_t)x - a.mg.c);
+    const uint32_t w0 = open_bits(a, row[0], x), w1 = open_bits(a, row[1], x);
+    float2 c[2][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[0][e] = c[1][e] = make_float2(0.0f, 0.0f);
+    uint32_t f = p0.f, d = p0.d;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float2 z = cis_rad((float)(int32_t)f * RAD32);
+      if ((w0 >> k) & 1u) c[0][0] = cadd(c[0][0], z);
+      if ((w1 >> k) & 1u) c[1][0] = cadd(c[1][0], z);
+      sums_step(c[0]);
+      sums_step(c[1]);
+      f += d;
+      d += a.cc2;
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const uint32_t w = e ? w1 : w0;
+      fold_weights(a, row[e], x, c[e], [&](int k) {
+        const float2 z = cis_rad((float)(int32_t)(p0.f + (uint32_t)k * p0.d + (uint32_t)(k * (k - 1) / 2) * a.cc2) * RAD32);
+        return ((w >> k) & 1u) ? z : make_float2(0.0f, 0.0f);
+      });
+      sums_out(a, sub, c[e], tap[e]);
+    }
+  }
+}
+
+// Phase plate: the level's turns taken off the chirp's.
+template <int D>
+__device__ __forceinline__ void dec_levels(const RowArgs& a, const DecRow& row, int32_t x0, float2 (&tap)[DTAPS]) {
+  const uint32_t turn = (uint32_t)((0x100000000ull + (uint32_t)a.mg.levels / 2) / (uint32_t)a.mg.levels);
+#pragma unroll 1
+  for (int sub = 0; sub < D / 16; ++sub) {
+    const int32_t x = x0 + 16 * sub;
+    const uint32_t in = chord_bits(row, x);
+    if (in == 0u) continue;
+    uint32_t lv[4];
+    chunk_levels((int64_t)x - a.mg.c, row.dj * row.dj, a.mg, a.ph, lv);
+    const Chirp16 p0 = chirp16(a, (int64_t)x - a.mg.c);
+    float2 c[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] = make_float2(0.0f, 0.0f);
+    uint32_t f = p0.f, d = p0.d;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const uint32_t q = (lv[k >> 2] >> (8 * (k & 3))) & 0xFFu;
+      const float2 z = cis_rad((float)(int32_t)(f - q * turn) * RAD32);
+      if ((in >> k) & 1u) c[0] = cadd(c[0], z);
+      sums_step(c);
+      f += d;
+      d += a.cc2;
+    }
+    fold_weights(a, row, x, c, [&](int k) {
+      const uint32_t w = k < 8 ? (k < 4 ? lv[0] : lv[1]) : (k < 12 ? lv[2] : lv[3]);
+      const uint32_t q = (w >> (8 * (k & 3))) & 0xFFu;
+      const float2 z = cis_rad((float)(int32_t)(p0.f + (uint32_t)k * p0.d + (uint32_t)(k * (k - 1) / 2) * a.cc2 - q * turn) * RAD32);
+      return ((in >> k) & 1u) ? z : make_float2(0.0f, 0.0f);
+    });
+    sums_out(a, sub, c, tap);
+  }
+}
+
+// Deformed binary plate: the membrane's phase walked along the chunk, one
+// hardware sine and cosine of its sum with the chirp's reduced to [-1/2, 1/2]
+// turns (absolute error below 4e-7 each).
+template <int D, int NR>
+__device__ __forceinline__ void dec_membrane_n(const RowArgs& a, const DecRow& row, const CxRow& cx, int32_t x0, float2 (&tap)[DTAPS]) {
+  MembraneWalk<NR> walk(a.df, cx, (int32_t)(x0 - a.mg.c));
+#pragma unroll 1
+  for (int sub = 0; sub < D / 16; ++sub) {
+    const int32_t x = x0 + 16 * sub;
+    const uint32_t w = open_bits(a, row, x);
+    const Chirp16 p0 = chirp16(a, (int64_t)x - a.mg.c);
+    float2 c[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] = make_float2(0.0f, 0.0f);
+    uint32_t f = p0.f, d = p0.d;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      constexpr float TWO_PI = 6.28318530717958648f, RINT = 12582912.0f;  // 1.5 2^23
+      float t = fmaf((float)(int32_t)f, 1.0f / 4294967296.0f, walk.next());
+      t = __fsub_rn(t, __fsub_rn(__fadd_rn(t, RINT), RINT));
+      const float2 z = cis_rad(TWO_PI * t);
+      if ((w >> k) & 1u) c[0] = cadd(c[0], z);
+      sums_step(c);
+      f += d;
+      d += a.cc2;
+    }
+    sums_out(a, sub, c, tap);
+  }
+}
+template <int D>
+__device__ __forceinline__ void dec_membrane(const RowArgs& a, const DecRow& row, const CxRow& cx, int32_t x0, float2 (&tap)[DTAPS]) {
+  switch (a.df.n) {
+    case 0: dec_membrane_n<D, 0>(a, row, cx, x0, tap); break;
+    case 1: dec_membrane_n<D, 1>(a, row, cx, x0, tap); break;
+    case 2: dec_membrane_n<D, 2>(a, row, cx, x0, tap); break;
+    default: dec_membrane_n<D, 3>(a, row, cx, x0, tap); break;
+  }
+}
+
+// Row pass: rows j0 + 2 p and j0 + 2 p + 1, p = blockIdx.x, blockIdx.x + gridDim.x,
+// ...; warps take groups of 32 chunks.  Output as k_seg.
+template <int MODE, int D>
+__global__ void __launch_bounds__(STH, 2) k_dec(RowArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* b0 = reinterpret_cast<float2*>(smem_raw);
+  float2* b1 = b0 + SBUF;
+  float2* twA = b1 + SBUF;
+  float2* twB = twA + 15 * 256;
+  float2* over = twB + 256;  // [row][group][5]: a group's share of the next group's points
+  seg_twiddles(twA, twB);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const float2* pre = reinterpret_cast<const float2*>(a.pre);
+  const float2* Gs = reinterpret_cast<const float2*>(a.H);
+  const float2* post = reinterpret_cast<const float2*>(a.post);
+  float* C1 = reinterpret_cast<float*>(a.C1);
+  const int S = a.S, W = S + DTAPS - 1;
+  const int32_t base = (int32_t)a.col0;
+  for (int64_t p = blockIdx.x; 2 * p < a.rows; p += gridDim.x) {
+    DecRow row[2];
+    CxRow cx[2];
+    int32_t lo = INT32_MAX, hi = -1;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      row[e].dj = a.j0 + 2 * p + e - a.mg.c;
+      row[e].lo = 0;
+      row[e].hi = -1;
+      const int64_t rem = a.mg.sR - row[e].dj * row[e].dj;
+      if (rem >= 0 && 2 * p + e < a.rows) {
+        int64_t bmax = isqrt_row(rem);
+        if (MODE != SEG_MEMBRANE && a.octant) bmax = min(bmax, row[e].dj);
+        // the row's disc chord, within the grid (a given N may cut the disc)
+        row[e].lo = (int32_t)(MODE != SEG_MEMBRANE && a.half ? a.mg.c : max(a.mg.c - bmax, (int64_t)0));
+        row[e].hi = (int32_t)min(a.mg.c + bmax, a.N - 1);
+        lo = min(lo, row[e].lo);
+        hi = max(hi, row[e].hi);
+      }
+      if (MODE == SEG_MEMBRANE) cx_row_init(a.df, row[e].dj, cx[e]);
+    }
+    float2 acc[16];
+#pragma unroll
+    for (int d = 0; d < 16; ++d) acc[d] = make_float2(0.0f, 0.0f);
+    if (hi >= lo) {
+      const int ch0 = (lo - base) / D, ch1 = (hi - base) / D;
+      const int s0 = ch0 / S, s1 = ch1 / S;
+      for (int s = s0; s <= s1; ++s) {
+        const int g0 = max(ch0 - s * S, 0) >> 5, g1 = min(ch1 - s * S, S - 1) >> 5;
+        for (int g = g0 + warp; g <= g1; g += STH / 32) {
+          const int32_t x0 = base + D * (s * S + 32 * g + lane);
+          float2 tap[2][DTAPS];
+#pragma unroll
+          for (int q = 0; q < DTAPS; ++q) tap[0][q] = tap[1][q] = make_float2(0.0f, 0.0f);
+          if (MODE == SEG_FLAT) {
+            dec_flat<D>(a, row, x0, tap);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              if (MODE == SEG_LEVELS) dec_levels<D>(a, row[e], x0, tap[e]);
+              else dec_membrane<D>(a, row[e], cx[e], x0, tap[e]);
+            }
+          }
+          __syncwarp();
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            // chunk ch's tap q belongs to point ch + q
+            float2 in = tap[e][0], out = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int q = 1; q < DTAPS; ++q) {
+              const int src = (lane - q) & 31;
+              const float2 v = make_float2(__shfl_sync(0xFFFFFFFFu, tap[e][q].x, src), __shfl_sync(0xFFFFFFFFu, tap[e][q].y, src));
+              if (lane >= q) in = cadd(in, v);
+              else out = cadd(out, v);
+            }
+            b0[e * DROW + 32 * g + lane] = in;
+            if (lane < DTAPS - 1) over[(e * DGRP + g) * (DTAPS - 1) + lane] = out;
+          }
+        }
+        __syncthreads();
+        float2 v[16];
+        {
+          const float2* pb = pre + (int64_t)s * S;
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const int e = t + 256 * r, g = e >> 5;
+            const float2 y = __ldg(pb + min(e, W - 1));
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+              float2 x = make_float2(0.0f, 0.0f);
+              if (g >= g0 && g <= g1) x = b0[z * DROW + e];
+              if (lane < DTAPS - 1 && g > g0 && g <= g1 + 1) x = cadd(x, over[(z * DGRP + g - 1) * (DTAPS - 1) + lane]);
+              v[r + 8 * z] = cmul(x, y);
+            }
+          }
+        }
+        // the spectrum sum waits in the second buffer while the columns are made
+#pragma unroll
+        for (int d = 0; d < 16; ++d) acc[d] = s > s0 ? b1[t + 256 * d] : make_float2(0.0f, 0.0f);
+        __syncthreads();  // pass A writes the points' buffer
+        dft16(v);
+#pragma unroll
+        for (int k0 = 1; k0 < 16; ++k0) v[k0] = cmul(v[k0], twA[(k0 - 1) * 256 + t]);
+#pragma unroll
+        for (int k0 = 0; k0 < 16; ++k0) b0[t * 17 + k0] = v[k0];
+        __syncthreads();
+        {
+          const int aa = t & 15, k0 = t >> 4;
+#pragma unroll
+          for (int b = 0; b < 16; ++b) v[b] = b0[(aa + 16 * b) * 17 + k0];
+          dft16(v);
+#pragma unroll
+          for (int c = 1; c < 16; ++c) v[c] = cmul(v[c], twB[c * 16 + aa]);
+#pragma unroll
+          for (int c = 0; c < 16; ++c) b1[k0 * 273 + c * 17 + aa] = v[c];
+        }
+        __syncthreads();
+        float2 g[16];
+        const float2* G = Gs + (int64_t)s * SP + t;
+#pragma unroll
+        for (int d = 0; d < 16; ++d) g[d] = __ldg(G + 256 * d);
+        {
+          const int k0 = t & 15, c = t >> 4;
+#pragma unroll
+          for (int aa = 0; aa < 16; ++aa) v[aa] = b1[k0 * 273 + c * 17 + aa];
+          dft16(v);
+        }
+#pragma unroll
+        for (int d = 0; d < 16; ++d) {
+          acc[d].x = fmaf(v[d].x, g[d].x, fmaf(-v[d].y, g[d].y, acc[d].x));
+          acc[d].y = fmaf(v[d].x, g[d].y, fmaf(v[d].y, g[d].x, acc[d].y));
+        }
+        if (s < s1) {
+          __syncthreads();
+#pragma unroll
+          for (int d = 0; d < 16; ++d) b1[t + 256 * d] = acc[d];
+        }
+      }
+    }
+    // inverse transform as conj(FFT(conj(.))): outputs m = t of the first row at
+    // point t, of the second at DROW + t (n <= 256)
+#pragma unroll
+    for (int d = 0; d < 16; ++d) acc[d].y = -acc[d].y;
+    fft_p(acc, b0, b1, twA, twB);
+    const int64_t jl = a.j0 + 2 * p - a.c1_j0;
+    float2 y[2];
+    if (t < a.M) {
+      const float2 w = post[t];
+      y[0] = cmul(make_float2(acc[0].x, -acc[0].y), w);
+      y[1] = cmul(make_float2(acc[DROW / 256].x, -acc[DROW / 256].y), w);
+    }
+    if (MODE != SEG_MEMBRANE && a.half) {
+      // outputs x and -x meet in the transpose buffer that the transform's last pass does not read
+      if (t < a.M) {
+        b0[t] = y[0];
+        b0[256 + t] = y[1];
+      }
+      __syncthreads();
+      const int hm = a.M / 2;
+      if (t < hm) {
+        y[0] = cadd(b0[hm + t], b0[hm - 1 - t]);
+        y[1] = cadd(b0[256 + hm + t], b0[256 + hm - 1 - t]);
+      }
+    }
+    if (t < (MODE != SEG_MEMBRANE && a.half ? a.M / 2 : a.M)) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        if (2 * p + e < a.rows) {
+          C1[(int64_t)c1_row_re(t) * a.c1_stride + jl + e] = y[e].x;
+          C1[(int64_t)c1_row_im(t) * a.c1_stride + jl + e] = y[e].y;
+        }
+    }
+    __syncthreads();
+  }
+}
+
+// Its tables: the convolution's input chirp on the grid points i, at D (i - i0)
+// columns from the axis, and the outputs' (times 1 / 4096).
+__global__ void k_dec_tables(int64_t npts, int n, double delta, double mc, double i0, float2* pre, float2* post) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < max(npts, (int64_t)n); t += stride) {
+    const double x = (double)t;
+    if (t < npts) pre[t] = cis_turns<float>(x * (delta * mc - 0.5 * delta * x));
+    if (t < n) {
+      float2 z = cis_turns<float>(delta * ((x - mc) * i0 - 0.5 * x * x));
+      z.x *= 1.0f / SP;
+      z.y *= 1.0f / SP;
+      post[t] = z;
+    }
+  }
+}
+
 // Tables: pre(i), post(m)/L, convolution chirp v (length L), twiddles.
 template <typename R>
 __global__ void k_tables(int64_t N, int M, double msh, int64_t L, int64_t c, double kappa, double delta, int turns, void* pre,
@@ -1243,11 +1643,66 @@ DeformCoef deform_coef(const Plan& P) {
     c.q[k] = (float)(P.dx * P.dx / (2.0 * sg * sg));
     c.h2[k] = (float)(d.ridge_h[k] * k2);
     c.rho[k] = (float)std::exp(-2.0 * (P.dx * P.dx / (2.0 * sg * sg)) * nx * nx);
+    c.eta[k] = (float)-std::expm1(-2.0 * (P.dx * P.dx / (2.0 * sg * sg)) * nx * nx);
   }
   return c;
 }
 
 namespace {
+
+// The weights that take 16 columns' running sums to the grid points: the
+// Lagrange polynomials of the six points on the columns of the chunk's part
+// `sub`, fitted by least squares in the sums' own weights 1, m, m (m + 1) / 2,
+// m (m + 1) (m + 2) / 6, m = 16 - k (a cubic follows a node's exponential over
+// half of 16 columns to below 1e-8).
+static void decimation_weights(int D, float (*T)[DTAPS][4]) {
+  double B[16][4], Q[16][4], R[4][4] = {};
+  for (int k = 0; k < 16; ++k) {
+    const double m = 16 - k;
+    B[k][0] = 1; B[k][1] = m; B[k][2] = m * (m + 1) / 2; B[k][3] = m * (m + 1) * (m + 2) / 6;
+  }
+  for (int e = 0; e < 4; ++e) {  // modified Gram-Schmidt
+    for (int k = 0; k < 16; ++k) Q[k][e] = B[k][e];
+    for (int f = 0; f < e; ++f) {
+      for (int k = 0; k < 16; ++k) R[f][e] += Q[k][f] * Q[k][e];
+      for (int k = 0; k < 16; ++k) Q[k][e] -= R[f][e] * Q[k][f];
+    }
+    for (int k = 0; k < 16; ++k) R[e][e] += Q[k][e] * Q[k][e];
+    R[e][e] = std::sqrt(R[e][e]);
+    for (int k = 0; k < 16; ++k) Q[k][e] /= R[e][e];
+  }
+  for (int sub = 0; sub < D / 16; ++sub)
+    for (int q = 0; q < DTAPS; ++q) {
+      double y[4] = {};
+      for (int k = 0; k < 16; ++k) {
+        const double xi = (16 * sub + k + 0.5) / D;  // from the point half a column before the chunk
+        double w = 1;
+        for (int p = 0; p < DTAPS; ++p)
+          if (p != q) w *= (xi - (p - 2)) / (q - p);
+        for (int e = 0; e < 4; ++e) y[e] += Q[k][e] * w;
+      }
+      for (int e = 3; e >= 0; --e) {
+        for (int f = e + 1; f < 4; ++f) y[e] -= R[e][f] * y[f];
+        y[e] /= R[e][e];
+        T[sub][q][e] = (float)y[e];
+      }
+    }
+}
+
+// x turns in units of 2^-64, mod 1
+static uint64_t turns64(double x) {
+  x -= std::floor(x);
+  const double t = std::ldexp(x, 64);
+  return t >= 18446744073709551616.0 ? 0 : (uint64_t)t;
+}
+
+static void (*dec_kernel(int mode, int D))(RowArgs) {
+  switch (mode) {
+    case SEG_FLAT: return D == 32 ? k_dec<SEG_FLAT, 32> : k_dec<SEG_FLAT, 16>;
+    case SEG_LEVELS: return D == 32 ? k_dec<SEG_LEVELS, 32> : k_dec<SEG_LEVELS, 16>;
+    default: return D == 32 ? k_dec<SEG_MEMBRANE, 32> : k_dec<SEG_MEMBRANE, 16>;
+  }
+}
 
 static RowArgs make_args(const Plan& P) {
   const Bluestein& b = P.bs;
@@ -1279,7 +1734,23 @@ static RowArgs make_args(const Plan& P) {
   a.half = b.half ? 1 : 0;
   if (P.nd.n > 0) a.M = P.nd.n;
   else if (b.half) a.M = P.M + 1;
+  if (b.dec) {
+    const double mc = 0.5 * (P.nd.n - 1);
+    a.Kc = turns64(0.5 * P.kappa);
+    a.Kl = turns64(-P.nd.delta * (mc - P.nd.msh - (P.nd.even ? P.nd.n / 2 : 0)));
+    a.cc2 = (uint32_t)((2 * a.Kc + 0x80000000ull) >> 32);
+    decimation_weights(b.dec, a.T);
+  }
   return a;
+}
+
+// Columns to a grid point of the decimated rows, 0: none.  D u <= 0.17 keeps the
+// interpolation's error below 1.2e-7 (3e-8 at the ROI's edge); a deformed phase
+// plate has its general per-sample transmission.
+static int decimation(const Plan& P) {
+  if (P.nd.n == 0 || (P.has_deform && P.levels >= 2)) return 0;
+  const double u = M_PI * P.nd.delta * (P.nd.n - 1);
+  return 32 * u <= 0.17 ? 32 : 16 * u <= 0.17 ? 16 : 0;
 }
 
 template <typename R>
@@ -1307,6 +1778,13 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
     const int M = P.nd.n > 0 ? P.nd.n : P.M;  // outputs per row: the nodes, or the ROI samples
     b.S = 256 * std::min(15, (4097 - M) / 256);
     b.nseg = (P.N - b.col0 + b.S - 1) / b.S;
+    b.dec = decimation(P);
+    if (b.dec) {
+      // two rows to a transform: S + 5 + n < 2050, S a multiple of 32
+      const int64_t chunks = (P.N - b.col0 + b.dec - 1) / b.dec, most = (DROW - M - DTAPS + 1) / 32 * 32;
+      b.nseg = (chunks + most - 1) / most;
+      b.S = (int)(((chunks + b.nseg - 1) / b.nseg + 31) / 32 * 32);
+    }
     b.rows = P.chunk_rows;
     out->pre = sizeof(C) * P.N;
     out->H = sizeof(C) * (size_t)SP * (size_t)b.nseg;
@@ -1318,6 +1796,8 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
     const void* kern[4] = {(const void*)k_seg<SEG_FLAT>, (const void*)k_seg<SEG_LEVELS>,
                            (const void*)k_seg<SEG_MEMBRANE>, (const void*)k_seg<SEG_GENERAL>};
     for (int q = 0; q < 4; ++q) FZP_CUDA_TRY(smem_attr_once(kern[q], (int)SEG_SMEM, attr_seg[q]));
+    static std::atomic<uint64_t> attr_dec[6];
+    for (int q = 0; q < 6; ++q) FZP_CUDA_TRY(smem_attr_once((const void*)dec_kernel(q / 2, q % 2 ? 32 : 16), (int)DEC_SMEM, attr_dec[q]));
     FZP_CUDA_TRY(smem_attr_once((const void*)k_seg_tables, (int)SEG_SMEM, attr_segt));
     return FZP_OK;
   }
@@ -1354,12 +1834,23 @@ fzp_status fill_tables_t(Plan& P, cudaStream_t s) {
   const double delta = nodes ? P.nd.delta : P.delta;
   const double msh = nodes ? P.nd.msh + (P.nd.even ? P.nd.n / 2 : 0) : P.msh;
   b.d_twL = reinterpret_cast<C*>(b.d_post) + M;
+  if (b.dec) {
+    const double mc = 0.5 * (M - 1), i0 = 2.0 + (0.5 + (double)(P.c - b.col0)) / b.dec, dd = delta * b.dec;
+    k_dec_tables<<<64, 256, 0, s>>>(b.nseg * b.S + DTAPS - 1, M, dd, mc, i0, reinterpret_cast<float2*>(b.d_pre),
+                                    reinterpret_cast<float2*>(b.d_post));
+    FZP_CUDA_TRY(cudaGetLastError());
+    const unsigned g = (unsigned)std::min<int64_t>(b.nseg, 1024);
+    k_seg_tables<<<g, STH, SEG_SMEM, s>>>(b.nseg, 0, b.S, b.S + DTAPS - 1, M, dd, reinterpret_cast<float2*>(b.d_H));
+    FZP_CUDA_TRY(cudaGetLastError());
+    P.launches += 2;
+    return FZP_OK;
+  }
   k_tables<R><<<1024, 256, 0, s>>>(half ? P.c + 1 : P.N, M, msh, b.L, half ? 0 : P.c, P.kappa, delta, b.seg && P.has_deform && P.levels < 2 ? 1 : 0, b.d_pre, b.d_post, b.d_tab, b.d_tw, twN,
                                    b.d_twL);
   FZP_CUDA_TRY(cudaGetLastError());
   if (b.seg) {
     const unsigned g = (unsigned)std::min<int64_t>(b.nseg, 1024);
-    k_seg_tables<<<g, STH, SEG_SMEM, s>>>(b.nseg, b.col0, b.S, M, delta, reinterpret_cast<float2*>(b.d_H));
+    k_seg_tables<<<g, STH, SEG_SMEM, s>>>(b.nseg, b.col0, b.S, b.S, M, delta, reinterpret_cast<float2*>(b.d_H));
     FZP_CUDA_TRY(cudaGetLastError());
     P.launches += 2;
     return FZP_OK;
@@ -1417,13 +1908,15 @@ fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s
                             : mode == SEG_LEVELS   ? k_seg<SEG_LEVELS>
                             : mode == SEG_MEMBRANE ? k_seg<SEG_MEMBRANE>
                                                    : k_seg<SEG_GENERAL>;
-    FZP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, kern, STH, SEG_SMEM));
+    const size_t smem = b.dec ? DEC_SMEM : SEG_SMEM;
+    if (b.dec) kern = dec_kernel(mode, b.dec);
+    FZP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, kern, STH, smem));
     if (ctas_per_sm < 1) ctas_per_sm = 1;
     a.j0 = j0;
     a.rows = rows;
-    const int64_t grid = std::min<int64_t>(rows, (int64_t)ctas_per_sm * sms);
+    const int64_t grid = std::min<int64_t>(b.dec ? (rows + 1) / 2 : rows, (int64_t)ctas_per_sm * sms);
     prof_begin(P, s);
-    kern<<<(unsigned)grid, STH, SEG_SMEM, s>>>(a);
+    kern<<<(unsigned)grid, STH, smem, s>>>(a);
     prof_end(P, s);
     P.launches += 1;
     FZP_CUDA_TRY(cudaGetLastError());

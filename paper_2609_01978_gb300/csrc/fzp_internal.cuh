@@ -105,7 +105,7 @@ struct DeformCoef {
   // steps along a row (di -> di + 1) for generators that walk columns:
   // the wrinkle phasor turns by e^{2 pi i kx}; a ridge's ratio g(di+1)/g(di)
   // is multiplied by rho_k = exp(-2 q_k nx_k^2)
-  float zc, zs, rho[3];
+  float zc, zs, rho[3], eta[3];  // eta = 1 - rho
   float z4;  // 4 sin^2(pi kx): the wrinkle's second difference per column
 };
 
@@ -193,6 +193,7 @@ struct Bluestein {
   int seg = 0;
   int S = 0;
   int64_t nseg = 0;
+  int dec = 0;            // decimated rows: columns to a grid point (then S counts those); 0: none
   int64_t col0 = 0;       // first input column (the axis when `half`)
   bool half = false;      // columns from the axis on, outputs x and -x added
   int64_t L_full = 0;     // power of two >= N + M - 1 (what the plan reports)

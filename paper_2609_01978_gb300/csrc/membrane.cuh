@@ -14,7 +14,7 @@ namespace fzp {
 // FP32, walked along the row from the first column: the wrinkle's phasor
 // e^{2 pi i t} (t = di kx + dj ky, integer turns dropped exactly) turns by
 // e^{2 pi i kx} per column, a ridge's g = exp(-q d^2) by its ratio r, which
-// itself scales by rho = exp(-2 q nx^2); the sum is reduced to [-1/2, 1/2]
+// itself scales by rho = exp(-2 q nx^2) = 1 - eta; the sum is reduced to [-1/2, 1/2]
 // turns before one hardware sine or cosine (absolute error below 4e-7; the
 // walk adds ~1e-6 relative over 32 columns).  A ridge below 1e-30 at the
 // first column stays below 1e-29 in the block (its width is hundreds of
@@ -45,12 +45,14 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 // the scaled wrinkle amp sin by its second difference, s' = s + e, e' = e - 4
 // sin^2(pi kx) s (one product instead of a rotation's four, and no growth of the
 // rounding at the small angles of a wrinkle), the taper by its constant second
-// difference, a ridge by its ratio.  Started exactly every 16 (k_seg) or 32
-// columns (k_nodes).  NR ridges.
+// difference, a ridge by its ratio, kept as the ratio less one: g += g r1, r1 <-
+// r1 rho - (1 - rho) (a ratio near one rounded to FP32 is off by 3e-8 and more
+// each, 2e-5 of g over 32 columns).  Started exactly every 16 (k_seg) or 32
+// columns (k_dec, k_nodes).  NR ridges.
 template <int NR>
 struct MembraneWalk {
   float s, e, tap, dt, ddt, z4;
-  float g[NR > 0 ? NR : 1], rr[NR > 0 ? NR : 1], rho[NR > 0 ? NR : 1];
+  float g[NR > 0 ? NR : 1], r1[NR > 0 ? NR : 1], rho[NR > 0 ? NR : 1], eta[NR > 0 ? NR : 1];
 
   __device__ __forceinline__ MembraneWalk(const DeformCoef& d, const CxRow& r, int32_t di0) {
     constexpr float TWO_PI = 6.28318530717958648f;
@@ -69,13 +71,17 @@ struct MembraneWalk {
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
       g[k] = 0.0f;
-      rr[k] = 1.0f;
+      r1[k] = 0.0f;
       rho[k] = d.rho[k];
+      eta[k] = d.eta[k];
       const float d0 = fmaf(fi, d.nx[k], r.cr[k]);
       const float ex = d.q[k] * d0 * d0;
       if (ex < 69.0f) {
         g[k] = d.h2[k] * __expf(-ex);
-        rr[k] = __expf(-d.q[k] * d.nx[k] * fmaf(2.0f, d0, d.nx[k]));
+        // e^-x - 1: its series while |x| is small (ridges are hundreds of columns wide)
+        const float x = d.q[k] * d.nx[k] * fmaf(2.0f, d0, d.nx[k]);
+        const float p = fmaf(x, fmaf(x, fmaf(x, fmaf(x, -1.0f / 120.0f, 1.0f / 24.0f), -1.0f / 6.0f), 0.5f), -1.0f);
+        r1[k] = fabsf(x) < 0.125f ? x * p : __expf(-x) - 1.0f;
       }
     }
   }
@@ -89,8 +95,8 @@ struct MembraneWalk {
 #pragma unroll
     for (int v = 0; v < NR; ++v) {
       wz += g[v];
-      g[v] *= rr[v];
-      rr[v] *= rho[v];
+      g[v] = fmaf(g[v], r1[v], g[v]);
+      r1[v] = fmaf(r1[v], rho[v], -eta[v]);
     }
     return wz;
   }
