@@ -173,7 +173,7 @@ struct RowArgs {
   // 2^-64), the second difference (2^-32), the sums' weights on the grid points
   uint64_t Kc, Kl;
   uint32_t cc2;
-  float T[2][DTAPS][4];
+  float2 T[2][DTAPS][4];  // (each weight twice)
 };
 
 // Aperture transmission of sample (j, i): T e^{i phi}, optional deformation.
@@ -1246,10 +1246,7 @@ __device__ __forceinline__ void sums_out(const RowArgs& a, int sub, const float2
 #pragma unroll
   for (int q = 0; q < DTAPS; ++q)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      tap[q].x = fmaf(a.T[sub][q][e], c[e].x, tap[q].x);
-      tap[q].y = fmaf(a.T[sub][q][e], c[e].y, tap[q].y);
-    }
+    for (int e = 0; e < 4; ++e) tap[q] = fma2(a.T[sub][q][e], c[e], tap[q]);
 }
 
 // The chirp's 32-bit phase and its first difference at column di0.
@@ -1345,37 +1342,40 @@ __device__ __forceinline__ void dec_levels(const RowArgs& a, const DecRow& row, 
   }
 }
 
-// Deformed binary plate: the membrane's phase walked along the chunk, one
-// hardware sine and cosine of its sum with the chirp's reduced to [-1/2, 1/2]
-// turns (absolute error below 4e-7 each).
+// Deformed binary plate: both rows' membrane phases walked along the chunk in
+// pairs, one hardware sine and cosine of the sum with the chirp's reduced to
+// [-1/2, 1/2] turns (absolute error below 4e-7 each).
 template <int D, int NR>
-__device__ __forceinline__ void dec_membrane_n(const RowArgs& a, const DecRow& row, const CxRow& cx, int32_t x0, float2 (&tap)[DTAPS]) {
-  MembraneWalk<NR> walk(a.df, cx, (int32_t)(x0 - a.mg.c));
+__device__ __forceinline__ void dec_membrane_n(const RowArgs& a, const DecRow (&row)[2], const CxRow (&cx)[2], int32_t x0,
+                                               float2 (&tap)[2][DTAPS]) {
+  const int32_t di0 = (int32_t)(x0 - a.mg.c);
+  MembraneWalk2<NR> walk(MembraneWalk<NR>(a.df, cx[0], di0), MembraneWalk<NR>(a.df, cx[1], di0));
 #pragma unroll 1
   for (int sub = 0; sub < D / 16; ++sub) {
     const int32_t x = x0 + 16 * sub;
-    const uint32_t w = open_bits(a, row, x);
+    const uint32_t w0 = open_bits(a, row[0], x), w1 = open_bits(a, row[1], x);
     const Chirp16 p0 = chirp16(a, (int64_t)x - a.mg.c);
-    float2 c[4];
+    float2 c[2][4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) c[e] = make_float2(0.0f, 0.0f);
+    for (int e = 0; e < 4; ++e) c[0][e] = c[1][e] = make_float2(0.0f, 0.0f);
     uint32_t f = p0.f, d = p0.d;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      constexpr float TWO_PI = 6.28318530717958648f, RINT = 12582912.0f;  // 1.5 2^23
-      float t = fmaf((float)(int32_t)f, 1.0f / 4294967296.0f, walk.next());
-      t = __fsub_rn(t, __fsub_rn(__fadd_rn(t, RINT), RINT));
-      const float2 z = cis_rad(TWO_PI * t);
-      if ((w >> k) & 1u) c[0] = cadd(c[0], z);
-      sums_step(c);
+      const float2 t = reduced_rad(fma2(pair2((float)(int32_t)f), pair2(1.0f / 4294967296.0f), walk.next()));
+      if ((w0 >> k) & 1u) c[0][0] = cadd(c[0][0], cis_rad(t.x));
+      if ((w1 >> k) & 1u) c[1][0] = cadd(c[1][0], cis_rad(t.y));
+      sums_step(c[0]);
+      sums_step(c[1]);
       f += d;
       d += a.cc2;
     }
-    sums_out(a, sub, c, tap);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) sums_out(a, sub, c[e], tap[e]);
   }
 }
 template <int D>
-__device__ __forceinline__ void dec_membrane(const RowArgs& a, const DecRow& row, const CxRow& cx, int32_t x0, float2 (&tap)[DTAPS]) {
+__device__ __forceinline__ void dec_membrane(const RowArgs& a, const DecRow (&row)[2], const CxRow (&cx)[2], int32_t x0,
+                                             float2 (&tap)[2][DTAPS]) {
   switch (a.df.n) {
     case 0: dec_membrane_n<D, 0>(a, row, cx, x0, tap); break;
     case 1: dec_membrane_n<D, 1>(a, row, cx, x0, tap); break;
@@ -1438,12 +1438,11 @@ __global__ void __launch_bounds__(STH, 2) k_dec(RowArgs a) {
           for (int q = 0; q < DTAPS; ++q) tap[0][q] = tap[1][q] = make_float2(0.0f, 0.0f);
           if (MODE == SEG_FLAT) {
             dec_flat<D>(a, row, x0, tap);
-          } else {
+          } else if (MODE == SEG_LEVELS) {
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              if (MODE == SEG_LEVELS) dec_levels<D>(a, row[e], x0, tap[e]);
-              else dec_membrane<D>(a, row[e], cx[e], x0, tap[e]);
-            }
+            for (int e = 0; e < 2; ++e) dec_levels<D>(a, row[e], x0, tap[e]);
+          } else {
+            dec_membrane<D>(a, row, cx, x0, tap);
           }
           __syncwarp();
 #pragma unroll
@@ -1655,7 +1654,7 @@ namespace {
 // `sub`, fitted by least squares in the sums' own weights 1, m, m (m + 1) / 2,
 // m (m + 1) (m + 2) / 6, m = 16 - k (a cubic follows a node's exponential over
 // half of 16 columns to below 1e-8).
-static void decimation_weights(int D, float (*T)[DTAPS][4]) {
+static void decimation_weights(int D, float2 (*T)[DTAPS][4]) {
   double B[16][4], Q[16][4], R[4][4] = {};
   for (int k = 0; k < 16; ++k) {
     const double m = 16 - k;
@@ -1684,7 +1683,7 @@ static void decimation_weights(int D, float (*T)[DTAPS][4]) {
       for (int e = 3; e >= 0; --e) {
         for (int f = e + 1; f < 4; ++f) y[e] -= R[e][f] * y[f];
         y[e] /= R[e][e];
-        T[sub][q][e] = (float)y[e];
+        T[sub][q][e] = make_float2((float)y[e], (float)y[e]);
       }
     }
 }

@@ -154,6 +154,23 @@ template <> __device__ __forceinline__ float2 csub(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return r;
 }
+// Pairs of FP32 values, both in one instruction.
+__device__ __forceinline__ float2 pair2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 p, q, s;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n mul.rn.f32x2 s, p, q;\n mov.b64 {%0, %1}, s;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n .reg .b64 p, q, t, s;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n mov.b64 t, {%6, %7};\n"
+      " fma.rn.f32x2 s, p, q, t;\n mov.b64 {%0, %1}, s;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
 
 template <typename R> __device__ __forceinline__ typename Cplx<R>::T cis_turns(double t);
 template <> __device__ __forceinline__ float2 cis_turns<float>(double t) { return cis_turns_f(t); }

@@ -102,37 +102,87 @@ struct MembraneWalk {
   }
 };
 
+// Two of these walks side by side, every step's operations in pairs.
+template <int NR>
+struct MembraneWalk2 {
+  float2 s, e, tap, dt, ddt, mz4;
+  float2 g[NR > 0 ? NR : 1], r1[NR > 0 ? NR : 1], rho[NR > 0 ? NR : 1], meta[NR > 0 ? NR : 1];
+
+  __device__ __forceinline__ MembraneWalk2(const MembraneWalk<NR>& a, const MembraneWalk<NR>& b) {
+    s = make_float2(a.s, b.s);
+    e = make_float2(a.e, b.e);
+    tap = make_float2(a.tap, b.tap);
+    dt = make_float2(a.dt, b.dt);
+    ddt = pair2(a.ddt);
+    mz4 = pair2(-a.z4);
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      g[k] = make_float2(a.g[k], b.g[k]);
+      r1[k] = make_float2(a.r1[k], b.r1[k]);
+      rho[k] = pair2(a.rho[k]);
+      meta[k] = pair2(-a.eta[k]);
+    }
+  }
+  __device__ __forceinline__ float2 next() {
+    float2 wz = mul2(s, tap);
+    e = fma2(mz4, s, e);
+    s = cadd(s, e);
+    tap = cadd(tap, dt);
+    dt = cadd(dt, ddt);
+#pragma unroll
+    for (int v = 0; v < NR; ++v) {
+      wz = cadd(wz, g[v]);
+      g[v] = fma2(g[v], r1[v], g[v]);
+      r1[v] = fma2(r1[v], rho[v], meta[v]);
+    }
+    return wz;
+  }
+};
+
+// The sum with another phase reduced to [-1/2, 1/2] turns, in radians (|x| < 2^22).
+__device__ __forceinline__ float2 reduced_rad(float2 x) {
+  const float2 rint2 = pair2(12582912.0f);  // 1.5 2^23
+  const float2 n = csub(cadd(x, rint2), rint2);
+  return mul2(csub(x, n), pair2(6.28318530717958648f));
+}
+
 // Both masks of a membrane, T cos(phi) and T sin(phi), on the 32 columns from
 // di0 (bit k of `bits`: column k open), as the row's four 16-byte parts in the
-// planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart).  NR ridges.
+// planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart): columns k and
+// k + 16 walk side by side, four at a time to the planes.  NR ridges.
 template <int NR>
 __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits,
                                             uint8_t* base, uint32_t plane, int sw) {
-  constexpr float TWO_PI = 6.28318530717958648f;
-  MembraneWalk<NR> walk(d, r, di0);
+  MembraneWalk2<NR> walk(MembraneWalk<NR>(d, r, di0), MembraneWalk<NR>(d, r, di0 + 16));
 #pragma unroll 1
-  for (int q = 0; q < 4; ++q, bits >>= 8) {
-    uint32_t hc[4], lc[4], hs[4], ls[4];
+  for (int q = 0; q < 4; ++q, bits >>= 4) {
+    uint32_t hc[2][2], lc[2][2], hs[2][2], ls[2][2];
 #pragma unroll
-    for (int k = 0; k < 8; k += 2) {
-      float vc[2], vs[2];
+    for (int k = 0; k < 4; k += 2) {
+      float vc[2][2], vs[2][2];
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        float wz = walk.next();
-        wz -= rintf(wz);
-        const float x = TWO_PI * wz;
-        const uint32_t open = (uint32_t)((int32_t)(bits << (31 - (k + z))) >> 31);
-        vc[z] = __uint_as_float(__float_as_uint(__cosf(x)) & open);
-        vs[z] = __uint_as_float(__float_as_uint(__sinf(x)) & open);
+        const float2 x = reduced_rad(walk.next());
+        const bool oa = (bits >> (k + z)) & 1u, ob = (bits >> (k + z + 16)) & 1u;
+        vc[0][z] = oa ? __cosf(x.x) : 0.0f;
+        vs[0][z] = oa ? __sinf(x.x) : 0.0f;
+        vc[1][z] = ob ? __cosf(x.y) : 0.0f;
+        vs[1][z] = ob ? __sinf(x.y) : 0.0f;
       }
-      split2(vc[0], vc[1], hc[k / 2], lc[k / 2]);
-      split2(vs[0], vs[1], hs[k / 2], ls[k / 2]);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        split2(vc[e][0], vc[e][1], hc[e][k / 2], lc[e][k / 2]);
+        split2(vs[e][0], vs[e][1], hs[e][k / 2], ls[e][k / 2]);
+      }
     }
-    uint8_t* o = base + ((q ^ sw) << 4);
-    *reinterpret_cast<uint4*>(o) = make_uint4(hc[0], hc[1], hc[2], hc[3]);
-    *reinterpret_cast<uint4*>(o + plane) = make_uint4(lc[0], lc[1], lc[2], lc[3]);
-    *reinterpret_cast<uint4*>(o + 2 * plane) = make_uint4(hs[0], hs[1], hs[2], hs[3]);
-    *reinterpret_cast<uint4*>(o + 3 * plane) = make_uint4(ls[0], ls[1], ls[2], ls[3]);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      uint8_t* o = base + ((((q >> 1) + 2 * e) ^ sw) << 4) + 8 * (q & 1);
+      *reinterpret_cast<uint2*>(o) = make_uint2(hc[e][0], hc[e][1]);
+      *reinterpret_cast<uint2*>(o + plane) = make_uint2(lc[e][0], lc[e][1]);
+      *reinterpret_cast<uint2*>(o + 2 * plane) = make_uint2(hs[e][0], hs[e][1]);
+      *reinterpret_cast<uint2*>(o + 3 * plane) = make_uint2(ls[e][0], ls[e][1]);
+    }
   }
 }
 
