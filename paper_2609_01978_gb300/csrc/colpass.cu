@@ -14,11 +14,17 @@
 #include <cmath>
 
 #include "fzp_internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace fzp {
 namespace {
 
 constexpr int TN = 64, TM = 64, TJ = 16, PJ = 128;  // output tiles of 64 (48: NA = 3 outputs per thread and side)
+
+constexpr int CZ = 4;        // blocks of a cluster along the rows
+constexpr int BLOCKS = 288;  // two per SM as far as clusters of four fit into the GPCs
+// whose tile of sums fits in static shared memory
+template <typename R, int NA> constexpr bool col_clusters = sizeof(R) == 4 || NA < 4;
 
 struct ColArgs {
   int64_t c, j0, rows, c1_stride;
@@ -63,6 +69,29 @@ __device__ __forceinline__ double2 kern(const RowPhase<double>& rp, int n) {
   return cis_turns_d(rp.a - (double)n * rp.b);
 }
 
+// FP32, a row and its mirror image: K(dj) + K(-dj) = e^{i pi kappa dj^2} 2 cos(2 pi
+// (n - msh) dj delta), one cosine instead of two sines and cosines.  The first
+// part of a row's phases is the cosine's (msh dj delta, and B split as above),
+// the second the exponential and the factor (the axis row: 1).
+__device__ __forceinline__ void row_pair(const ColArgs& g, double dj, bool second, RowPhase<float>& rp) {
+  if (second) {
+    const float2 e = cis_turns_f(dj * dj * (0.5 * g.kappa));
+    rp.fa = e.x;
+    rp.hi = e.y;
+    rp.lo = dj == 0.0 ? 1.0f : 2.0f;
+    return;
+  }
+  row_phase(g, dj, rp);
+  rp.fa = (float)frac_turns(g.msh * dj * g.delta);
+}
+__device__ __forceinline__ void row_pair(const ColArgs&, double, bool, RowPhase<double>&) {}
+__device__ __forceinline__ float2 kern_pair(const RowPhase<float>& rp, const RowPhase<float>& e, int n) {
+  const float x = (float)n * rp.hi;
+  const float c = e.lo * cospif(2.0f * (rp.fa - (x - floorf(x)) - (float)n * rp.lo));
+  return make_float2(c * e.fa, c * e.hi);
+}
+__device__ __forceinline__ double2 kern_pair(const RowPhase<double>&, const RowPhase<double>&, int) { return make_double2(0.0, 0.0); }
+
 // Factors of a row's kernel values in an output tile from n0: q < 8: e^{-2 pi i
 // (n0 + 8 q) B}; q < 16: e^{-2 pi i (q - 8) B}; 16, 17: e^{2 pi i A} at dj and, of
 // a folded row, at -dj (where B changes sign: the conjugate product).
@@ -74,20 +103,37 @@ __device__ __forceinline__ float2 factor(int, int, const RowPhase<float>&, const
   return make_float2(0.f, 0.f);  // (FP32 evaluates its sines)
 }
 
+__device__ __forceinline__ float2 peer_load(uint32_t addr, float2) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ double2 peer_load(uint32_t addr, double2) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+
 // grid (M/TM, M/TN, ceil(rows/jc)); 256 threads; each thread 4 n x 4 m outputs.
 // TAB: the kernel's columns from a table E [n][estride] instead of their phase.
+// The blocks' sums meet in Uacc: in clusters of CZ along the rows, block k adds up
+// its part of the tile over the cluster through distributed shared memory first.
+// Without that, 304 blocks' FP64 atomics on the same 8,192 values took most of
+// the kernel.
 template <typename R, bool TAB = false, int NA = 4>
 __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
   using C = typename Cplx<R>::T;
   constexpr int TN = 16 * NA, TM = 16 * NA;
-  __shared__ C sK[TJ][TN + 1];
-  __shared__ C sC[TJ][TM + 1];
+  constexpr int TILE = TJ * (TN + 1), POOL = col_clusters<R, NA> && TN * TM > 2 * TILE ? TN * TM : 2 * TILE;
+  __shared__ __align__(16) C pool[POOL];
+  C(*sK)[TN + 1] = reinterpret_cast<C(*)[TN + 1]>(pool);
+  C(*sC)[TM + 1] = reinterpret_cast<C(*)[TM + 1]>(pool + TILE);
   // phases of 128 rows at a time (they are FP64, at two operations per clock and
   // SM): of dj (mirrored rows: -dj) and, folded, of -dj
   __shared__ RowPhase<R> sP[2][PJ];
   // FP64: e^{-2 pi i n B} as products of 8 + 8 phasors per row (an FP64 sine per
   // element took as long as the products), and the rows' e^{2 pi i A}, A at dj and -dj
-  constexpr bool FACT = sizeof(R) == 8 && !TAB;
+  constexpr bool FACT = sizeof(R) == 8 && !TAB, PAIR = sizeof(R) == 4 && !TAB;
   __shared__ C sF[FACT ? TJ : 1][18];
   const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
   const int64_t jb = (int64_t)blockIdx.z * g.jc;
@@ -101,25 +147,17 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
   for (int a = 0; a < NA; ++a)
 #pragma unroll
     for (int b = 0; b < NA; ++b) { acc[a][b].x = 0; acc[a][b].y = 0; }
-  for (int64_t j = jb; j < je; j += TJ) {
-    const int pj = (int)(j - jb) & (PJ - 1);
-    if (!TAB && pj == 0) {
-      const int r = tid & (PJ - 1);
-      if (j + r < je && (tid < PJ || g.kind == ROWS_FOLDED)) {
-        const double dj = (double)(g.j0 + j + r - g.c);
-        RowPhase<R> rp;
-        row_phase(g, (tid >= PJ) != (g.kind == ROWS_MIRRORED) ? -dj : dj, rp);
-        sP[tid / PJ][r] = rp;
-      }
-    }
-    // C tile: TJ rows x TM columns (j contiguous in C1)
-    for (int t = tid; t < TJ * TM; t += 256) {
-      const int jj = t % TJ, mm = t / TJ;
-      const int m = m0 + mm;
+  constexpr int CQ = TJ * TM / 256;
+  C next[CQ];
+  auto load_c = [&](int64_t j) {
+#pragma unroll
+    for (int q = 0; q < CQ; ++q) {
+      const int t = tid + 256 * q, jj = t % TJ, m = m0 + t / TJ;
       C v;
       v.x = 0; v.y = 0;
       if (j + jj < je && m < g.M) {
         const int64_t re = (int64_t)c1_row_re(m) * g.c1_stride + j + jj, im = (int64_t)c1_row_im(m) * g.c1_stride + j + jj;
+#pragma unroll 1
         for (int sl = 0; sl < g.slices; ++sl) {
           const R* S = C1 + sl * g.slice_off;
           v.x += S[re];
@@ -130,7 +168,27 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
           }
         }
       }
-      sC[jj][mm] = v;
+      next[q] = v;
+    }
+  };
+  load_c(jb);
+  for (int64_t j = jb; j < je; j += TJ) {
+    const int pj = (int)(j - jb) & (PJ - 1);
+    if (!TAB && pj == 0) {
+      const int r = tid & (PJ - 1);
+      if (j + r < je && (tid < PJ || g.kind == ROWS_FOLDED)) {
+        const double dj = (double)(g.j0 + j + r - g.c);
+        RowPhase<R> rp;
+        if (PAIR && g.kind == ROWS_FOLDED) row_pair(g, dj, tid >= PJ, rp);
+        else row_phase(g, (tid >= PJ) != (g.kind == ROWS_MIRRORED) ? -dj : dj, rp);
+        sP[tid / PJ][r] = rp;
+      }
+    }
+    // C tile: TJ rows x TM columns (j contiguous in C1), loaded during the last tile's products
+#pragma unroll
+    for (int q = 0; q < CQ; ++q) {
+      const int t = tid + 256 * q;
+      sC[t % TJ][t / TJ] = next[q];
     }
     __syncthreads();
     if (FACT) {
@@ -154,13 +212,15 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
         k = cmul(sF[jj][16], e);
         e.y = -e.y;
         k = cadd(k, cmul(sF[jj][17], e));
+      } else if (PAIR && g.kind == ROWS_FOLDED && j + jj < je) {
+        k = kern_pair(sP[0][pj + jj], sP[1][pj + jj], n0 + nn);
       } else if (j + jj < je) {
         k = kern(sP[0][pj + jj], n0 + nn);
-        if (g.kind == ROWS_FOLDED && g.j0 + j + jj != g.c) k = cadd(k, kern(sP[1][pj + jj], n0 + nn));
       }
       sK[jj][nn] = k;
     }
     __syncthreads();
+    load_c(j + TJ);
     if (na == 0) {
     } else if (na < NA || nb < NA) {  // an edge tile: the outputs it has
 #pragma unroll 1
@@ -192,21 +252,66 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     }
     __syncthreads();
   }
+  auto add = [&](int n, int m, C v) {
+    if (n >= g.ny || m >= g.M) return;
+    double ux = (double)v.x, uy = (double)v.y;
+    if (g.wi != 0.0 || g.wr != 1.0) {
+      const double t = g.wr * ux - g.wi * uy;
+      uy = g.wr * uy + g.wi * ux;
+      ux = t;
+    }
+    atomicAdd(&Uacc[(int64_t)n * g.M + m].x, ux);
+    atomicAdd(&Uacc[(int64_t)n * g.M + m].y, uy);
+  };
+  uint32_t cz = 1, rank = 0;
+  if (col_clusters<R, NA>) asm("mov.u32 %0, %%cluster_nctarank;\n mov.u32 %1, %%cluster_ctarank;" : "=r"(cz), "=r"(rank));
+  if (cz == CZ) {
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+      for (int b = 0; b < NA; ++b) pool[(tn + 16 * a) * TM + tm + 16 * b] = acc[a][b];
+    tc::cluster_sync();
+    uint32_t peer[CZ];
+#pragma unroll
+    for (int q = 0; q < CZ; ++q) peer[q] = tc::mapa(tc::smem_u32(pool), q);
+    constexpr int PART = TN * TM / CZ;
+    for (int e = (int)rank * PART + tid; e < ((int)rank + 1) * PART; e += 256) {
+      C v[CZ];
+#pragma unroll
+      for (int q = 0; q < CZ; ++q) v[q] = peer_load(peer[q] + (uint32_t)(e * sizeof(C)), C{});
+#pragma unroll
+      for (int w = CZ / 2; w > 0; w /= 2)
+#pragma unroll
+        for (int q = 0; q < w; ++q) v[q] = cadd(v[q], v[q + w]);
+      add(n0 + e / TM, m0 + e % TM, v[0]);
+    }
+    tc::cluster_sync();  // the peers may still be reading this block's tile
+    return;
+  }
 #pragma unroll
   for (int a = 0; a < NA; ++a)
 #pragma unroll
-    for (int b = 0; b < NA; ++b) {
-      const int n = n0 + tn + 16 * a, m = m0 + tm + 16 * b;
-      if (n >= g.ny || m >= g.M) continue;
-      double ux = (double)acc[a][b].x, uy = (double)acc[a][b].y;
-      if (g.wi != 0.0 || g.wr != 1.0) {
-        const double t = g.wr * ux - g.wi * uy;
-        uy = g.wr * uy + g.wi * ux;
-        ux = t;
-      }
-      atomicAdd(&Uacc[(int64_t)n * g.M + m].x, ux);
-      atomicAdd(&Uacc[(int64_t)n * g.M + m].y, uy);
-    }
+    for (int b = 0; b < NA; ++b) add(n0 + tn + 16 * a, m0 + tm + 16 * b, acc[a][b]);
+}
+
+template <typename R, bool TAB = false, int NA = 4>
+fzp_status run_colpass(const ColArgs& g, unsigned tx, unsigned ty, const R* C1, double2* Uacc, cudaStream_t s) {
+  unsigned tz = (unsigned)((g.rows + g.jc - 1) / g.jc);
+  const bool clusters = col_clusters<R, NA> && tz >= CZ;
+  if (clusters) tz = (tz + CZ - 1) / CZ * CZ;  // (blocks past the last row add zeros)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tx, ty, tz);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = CZ;
+  cfg.attrs = attr;
+  cfg.numAttrs = clusters ? 1 : 0;
+  FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_colpass<R, TAB, NA>, g, C1, Uacc));
+  return FZP_OK;
 }
 
 __global__ void k_epilogue(int M, double msh, double p, double lf, double f_over_lambda, double amp,
@@ -268,14 +373,11 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   const int T = even ? 48 : TM;
   const int tx = (g.M + T - 1) / T, ty = (g.ny + T - 1) / T;
   const int64_t tiles = (int64_t)tx * ty;
-  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / 304 + TJ - 1) / TJ * TJ));
-  dim3 grid((unsigned)tx, (unsigned)ty, (unsigned)((rows + g.jc - 1) / g.jc));
-  if (even) k_colpass<double, false, 3><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
-  else if (P.precision == FZP_PREC_FP64) k_colpass<double><<<grid, 256, 0, s>>>(g, P.d_C1d, P.d_Uacc);
-  else k_colpass<float><<<grid, 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / BLOCKS + TJ - 1) / TJ * TJ));
   P.launches += 1;
-  FZP_CUDA_TRY(cudaGetLastError());
-  return FZP_OK;
+  return even                              ? run_colpass<double, false, 3>(g, tx, ty, P.d_C1d, P.d_Uacc, s)
+         : P.precision == FZP_PREC_FP64 ? run_colpass<double>(g, tx, ty, P.d_C1d, P.d_Uacc, s)
+                                           : run_colpass<float>(g, tx, ty, P.d_C1, P.d_Uacc, s);
 }
 
 fzp_status column_pass_table(Plan& P, const void* E, int64_t rows, int64_t estride, cudaStream_t s) {
@@ -290,11 +392,9 @@ fzp_status column_pass_table(Plan& P, const void* E, int64_t rows, int64_t estri
   g.estride = estride;
   g.ny = g.M;
   const int t = g.M / TM;
-  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * t * t / 304 + TJ - 1) / TJ * TJ));
-  k_colpass<float, true><<<dim3((unsigned)t, (unsigned)t, (unsigned)((rows + g.jc - 1) / g.jc)), 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * t * t / BLOCKS + TJ - 1) / TJ * TJ));
   P.launches += 1;
-  FZP_CUDA_TRY(cudaGetLastError());
-  return FZP_OK;
+  return run_colpass<float, true>(g, t, t, P.d_C1, P.d_Uacc, s);
 }
 
 fzp_status column_pass_zoom(Plan& P, int64_t rows, double lz, cudaStream_t s) {
@@ -312,11 +412,9 @@ fzp_status column_pass_zoom(Plan& P, int64_t rows, double lz, cudaStream_t s) {
   g.sin_off = 2 * z.ns * P.c1_stride;
   g.ny = z.yfull ? z.n : z.ns;
   const int tx = g.M / TM, ty = g.ny / TN;
-  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tx * ty / 304 + TJ - 1) / TJ * TJ));
-  k_colpass<float><<<dim3((unsigned)tx, (unsigned)ty, (unsigned)((rows + g.jc - 1) / g.jc)), 256, 0, s>>>(g, P.d_C1, P.d_Uacc);
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tx * ty / BLOCKS + TJ - 1) / TJ * TJ));
   P.launches += 1;
-  FZP_CUDA_TRY(cudaGetLastError());
-  return FZP_OK;
+  return run_colpass<float>(g, tx, ty, P.d_C1, P.d_Uacc, s);
 }
 
 fzp_status epilogue(Plan& P, void* d_field, int accumulate, cudaStream_t s) {

@@ -907,9 +907,10 @@ __global__ void __launch_bounds__(512) k_interp_W(const InterpSpec a, const doub
   }
 }
 
-// X[l][o] = sum_k Wy[k][o] V[k][l], k over the ny nodes of the rows' axis: a
-// block per output and 32 nodes, its four warps a quarter of the sum each.
-__global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, const double* __restrict__ Wy,
+// X[l][o] = sum_k Wy[k][o] V[k][l], k over the ny nodes of the rows' axis (sym:
+// of V plus its transpose): a block per output and 32 nodes, its four warps a
+// quarter of the sum each.
+__global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, int sym, const double* __restrict__ Wy,
                                                      const double2* __restrict__ V, double2* __restrict__ X) {
   __shared__ double2 part[4][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, l = blockIdx.x * 32 + lane, o = blockIdx.y;
@@ -920,8 +921,13 @@ __global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, con
   x[0] = x[1] = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = 0; k < n4; k += 2, v += 2 * ns, c += 2 * Mo) {
-    const double2 v0 = v[0], v1 = v[ns];
+    double2 v0 = v[0], v1 = v[ns];
     const double c0 = c[0], c1 = c[Mo];
+    if (sym) {
+      const double2* vt = V + (size_t)l * ns + w * n4 + k;
+      v0 = cadd(v0, vt[0]);
+      v1 = cadd(v1, vt[1]);
+    }
     x[0].x = fma(c0, v0.x, x[0].x);
     x[0].y = fma(c0, v0.y, x[0].y);
     x[1].x = fma(c1, v1.x, x[1].x);
@@ -935,14 +941,13 @@ __global__ void __launch_bounds__(128) k_interp_rows(int ny, int ns, int Mo, con
 struct InterpOut {
   int M, ns;
   int Moy, eveny, Mox, evenx;  // outputs of the two axes (even: M / 2 + 1)
-  int sym;                     // the field is this one plus its transpose
+  int sym;                     // the field is its own transpose
   double2 pre;                 // e^{ikf} dx^2 / (i lambda f)
   int accumulate;
 };
 
-// U[on, om] = sum_l X[l][on] W[l][om] (sym: plus the same with on and om
-// exchanged; only blocks on and below the diagonal run and both are stored),
-// the output chirp and prefactor, and the stores: with an even field output o
+// U[on, om] = sum_l X[l][on] W[l][om] (sym: only blocks on and below the diagonal
+// run and both are stored), the output chirp and prefactor, and the stores: with an even field output o
 // stands for the samples M/2 + o and M/2 - o (o = M/2: sample 0 alone).
 // Block: 8 x 4 outputs (columns x rows), two threads per output with half of
 // the sum each, operands through shared memory.  chirp[i] = e^{i pi x_i^2 /
@@ -954,24 +959,22 @@ __global__ void __launch_bounds__(2 * ITX * ITY) k_interp_cols(const InterpOut a
                                                                double2* __restrict__ out) {
   const int n0 = blockIdx.y * ITY, m0 = blockIdx.x * ITX;
   if (a.sym && m0 >= n0 + ITY) return;
-  __shared__ double2 sXn[64][ITY], sXm[64][ITX];
-  __shared__ double sWm[64][ITX], sWn[64][ITY];
+  __shared__ double2 sXn[64][ITY];
+  __shared__ double sWm[64][ITX];
   __shared__ double2 half[ITX * ITY];
   const int h = a.M / 2, tid = threadIdx.x;
   const int side = tid / (ITX * ITY), q = tid % (ITX * ITY), qn = q / ITX, qm = q % ITX;
   const int on = n0 + qn, om = m0 + qm;
-  double2 u = make_double2(0.0, 0.0), t = u;
+  double2 u = make_double2(0.0, 0.0);
   for (int l0 = 0; l0 < a.ns; l0 += 64) {  // ns is 64 or 128
     if (l0 > 0) __syncthreads();
     for (int e = tid; e < 64 * ITY; e += 2 * ITX * ITY) {
       const int l = e / ITY, c = min(n0 + e % ITY, a.Moy - 1);
       sXn[l][e % ITY] = __ldg(X + (l0 + l) * a.Moy + c);
-      if (a.sym) sWn[l][e % ITY] = __ldg(W + (l0 + l) * a.Mox + c);
     }
     for (int e = tid; e < 64 * ITX; e += 2 * ITX * ITY) {
       const int l = e / ITX, c = min(m0 + e % ITX, a.Mox - 1);
       sWm[l][e % ITX] = __ldg(W + (l0 + l) * a.Mox + c);
-      if (a.sym) sXm[l][e % ITX] = __ldg(X + (l0 + l) * a.Moy + c);
     }
     __syncthreads();
     const int lb = 32 * side;
@@ -981,15 +984,8 @@ __global__ void __launch_bounds__(2 * ITX * ITY) k_interp_cols(const InterpOut a
       const double w = sWm[l][qm];
       u.x = fma(w, x.x, u.x);
       u.y = fma(w, x.y, u.y);
-      if (a.sym) {
-        const double2 y = sXm[l][qm];
-        const double v = sWn[l][qn];
-        t.x = fma(v, y.x, t.x);
-        t.y = fma(v, y.y, t.y);
-      }
     }
   }
-  u = cadd(u, t);
   if (side) half[q] = u;
   __syncthreads();
   if (side) return;
@@ -1356,7 +1352,7 @@ fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cuda
   const bool eveny = z.even && !z.yfull;
   const int ny = z.yfull ? z.n : z.ns, Moy = eveny ? z.Mo : P.M;
   k_interp_rows<<<dim3((unsigned)(z.ns / 32), (unsigned)Moy), 128, 0, s>>>(
-      ny, z.ns, Moy, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
+      ny, z.ns, Moy, sym ? 1 : 0, z.yfull ? z.d_Wy : z.d_W, P.d_Uacc, z.d_X);
   // e^{ikf} / i: f / lambda - 1/4 turns
   const double turns = std::fmod(P.f / P.lambda, 1.0) - 0.25, amp = P.dx2 / (P.lambda * z.dist);
   InterpOut a{P.M, z.ns, Moy, eveny ? 1 : 0, z.Mo, z.even ? 1 : 0, sym ? 1 : 0,
