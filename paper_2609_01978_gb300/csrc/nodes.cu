@@ -302,36 +302,41 @@ __device__ __forceinline__ uint32_t chord_bits(int64_t di0, int64_t bmax) {
   return a & b;
 }
 
-// The exact rule on the block's columns [di0, di0 + 32): bits with value +1 and
-// with value -1 before the chord is applied (MASK_SIGNED: every column +1 or -1).
+// The exact rule on the blocks of the lanes that ask for it (`redo`; whole warp):
+// the warp takes such a row at a time, a column per lane.  Bits with value +1 and
+// with value -1 before the chord is applied (MASK_SIGNED: every column +1 or -1;
+// MASK_QUAD: the level's parity and its upper half).  A plate whose zones end on
+// samples has a tie in every 4 N of them; column after column in one lane each
+// cost 10,000 clocks, a third of a small plate's row pass.
 template <int MASK>
-__device__ __noinline__ void exact_bits(int64_t di0, int64_t dj2, const MaskGeom& g, const PhaseRule& r, uint32_t& pb,
+__device__ __noinline__ void exact_rows(bool redo, int32_t di0, int32_t dj, const MaskGeom& g, const PhaseRule& r, uint32_t& pb,
                                         uint32_t& nb) {
+  const int lane = threadIdx.x & 31;
   pb = nb = 0u;
-  for (int k = 0; k < 32; ++k) {
-    const int64_t d = di0 + k, s = dj2 + d * d;
-    const int64_t z = zone_of(s < g.sR ? s : g.sR, g);
+  for (uint32_t todo = __ballot_sync(0xffffffffu, redo); todo != 0u; todo &= todo - 1u) {
+    const int src = __ffs(todo) - 1;
+    const int64_t d = (int64_t)__shfl_sync(0xffffffffu, di0, src) + lane, j = __shfl_sync(0xffffffffu, dj, src);
+    const int64_t s = j * j + d * d;
+    const uint32_t z = (uint32_t)zone_of(s < g.sR ? s : g.sR, g);  // (zones are below 2^24)
+    bool p, n = false;
     if (MASK == MASK_LEVELS) {
-      const int q = (int)(z % r.lmod);
-      pb |= (uint32_t)((r.pos >> q) & 1ull) << k;
-      nb |= (uint32_t)((r.neg >> q) & 1ull) << k;
+      const uint32_t q = z % (uint32_t)r.lmod;
+      p = (r.pos >> q) & 1ull;
+      n = (r.neg >> q) & 1ull;
     } else if (MASK == MASK_SIGNED) {
-      if (z & 1) nb |= 1u << k;
-      else pb |= 1u << k;
+      n = z & 1u;
+      p = !n;
+    } else if (MASK == MASK_QUAD) {
+      p = z & 1u;
+      n = (z >> 1) & 1u;
     } else {
-      pb |= (uint32_t)((z ^ r.open_even) & 1) << k;
+      p = (z ^ (uint32_t)r.open_even) & 1u;
     }
-  }
-}
-
-// The same for four levels: bits of the level's parity and of its upper half.
-__device__ __noinline__ void exact_quad(int64_t di0, int64_t dj2, const MaskGeom& g, uint32_t& odd, uint32_t& high) {
-  odd = high = 0u;
-  for (int k = 0; k < 32; ++k) {
-    const int64_t d = di0 + k, s = dj2 + d * d;
-    const uint32_t z = (uint32_t)zone_of(s < g.sR ? s : g.sR, g);
-    odd |= (z & 1u) << k;
-    high |= ((z >> 1) & 1u) << k;
+    const uint32_t P = __ballot_sync(0xffffffffu, p), N = __ballot_sync(0xffffffffu, n);
+    if (lane == src) {
+      pb = P;
+      nb = N;
+    }
   }
 }
 
@@ -367,10 +372,12 @@ __device__ __forceinline__ uint32_t chord_up(const RowWalk& w) {
 }
 
 // The block's mask as 16 words of two BF16 values; `one` = +-1 (or +-1/2) in
-// both halves.  Whole warp (the votes), every lane a row.
+// both halves.  Whole warp (the votes), every lane a row.  True: a lane of the
+// warp has `redo` set, its words are exact_rows' (after the stores, when these
+// words' registers are free).
 template <int MASK>
-__device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
-                                            uint32_t chord, uint32_t (&wd)[16]) {
+__device__ __forceinline__ bool block_words(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
+                                            uint32_t chord, uint32_t (&wd)[16], bool& redo) {
   const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);  // upper 32 bits of 2 K
   uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
   uint32_t near = 0xFFFFFFFFu;
@@ -406,22 +413,32 @@ __device__ __forceinline__ void block_words(const RowWalk& w, const MaskGeom& g,
     near = near < 2u * e2 ? 1u : 0u;
   }
   // rare: a phase near a zone boundary, columns beyond the chord
+  redo = false;
   if (__any_sync(0xffffffffu, near != 0u || chord != 0xFFFFFFFFu)) {
-    if (near && chord) {
-      uint32_t pb, nb;
-      exact_bits<MASK>(w.di0, (int64_t)w.dj * w.dj, g, r, pb, nb);
-#pragma unroll
-      for (int q = 0; q < 16; ++q) wd[q] = (pair_mask(pb | nb, q) & one) | (pair_mask(nb, q) & 0x80008000u);
-    }
+    redo = near != 0u && chord != 0u;
 #pragma unroll
     for (int q = 0; q < 16; ++q) wd[q] &= pair_mask(chord, q);
+    return __any_sync(0xffffffffu, redo);
   }
+  return false;
+}
+
+// Word q of a row from the exact rule's bits.
+template <int MASK>
+__device__ __forceinline__ uint32_t exact_word(uint32_t pb, uint32_t nb, uint32_t one, uint32_t chord, int q) {
+  return ((pair_mask(pb | nb, q) & one) | (pair_mask(nb, q) & 0x80008000u)) & pair_mask(chord, q);
+}
+__device__ __forceinline__ void exact_quad_word(uint32_t odd, uint32_t high, uint32_t one, uint32_t chord, int q, uint32_t& re,
+                                                uint32_t& im) {
+  const uint32_t t = pair_mask(odd, q), s = pair_mask(high, q) & 0x80008000u, m = pair_mask(chord, q);
+  re = ~t & (one | s) & m;
+  im = t & (one | (s ^ 0x80008000u)) & m;
 }
 
 // Four levels (T = e^{-2 pi i q / 4} = 1, -i, -1, i, q the phase's top two bits):
 // the block's Re T and Im T, 16 words each.
-__device__ __forceinline__ void block_quad(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
-                                           uint32_t chord, uint32_t (&re)[16], uint32_t (&im)[16]) {
+__device__ __forceinline__ bool block_quad(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t one,
+                                           uint32_t chord, uint32_t (&re)[16], uint32_t (&im)[16], bool& redo) {
   const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);  // upper 32 bits of 2 K
   uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
   uint32_t near = 0xFFFFFFFFu;
@@ -438,28 +455,20 @@ __device__ __forceinline__ void block_quad(const RowWalk& w, const MaskGeom& g, 
     re[q] = ~t & (one | s);
     im[q] = t & (one | (s ^ 0x80008000u));
   }
-  const bool redo = near < 2u * e4 && chord != 0u;
+  redo = near < 2u * e4 && chord != 0u;
   if (__any_sync(0xffffffffu, redo || chord != 0xFFFFFFFFu)) {
-    if (redo) {
-      uint32_t odd = 0u, high = 0u;
-      exact_quad(w.di0, (int64_t)w.dj * w.dj, g, odd, high);
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const uint32_t t = pair_mask(odd, q), s = pair_mask(high, q) & 0x80008000u;
-        re[q] = ~t & (one | s);
-        im[q] = t & (one | (s ^ 0x80008000u));
-      }
-    }
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const uint32_t m = pair_mask(chord, q);
       re[q] &= m;
       im[q] &= m;
     }
+    return __any_sync(0xffffffffu, redo);
   }
+  return false;
 }
 
-// The block's open bits (parity rule, chord applied), for the membrane pass.
+// The block's open bits (parity rule, chord applied), for the membrane pass.  Whole warp.
 __device__ __forceinline__ uint32_t block_open(const RowWalk& w, const MaskGeom& g, const PhaseRule& r) {
   const uint32_t c2 = (uint32_t)(r.K >> 32) * 2u + (uint32_t)((r.K >> 31) & 1u);
   uint32_t f = (uint32_t)(w.phase >> 32), d = (uint32_t)(w.step >> 32);
@@ -473,9 +482,11 @@ __device__ __forceinline__ uint32_t block_open(const RowWalk& w, const MaskGeom&
     d += c2;
   }
   bits = __brev(bits);
-  if (near < 2u * e2 && chord != 0u) {
-    uint32_t nb;
-    exact_bits<MASK_PARITY>(w.di0, (int64_t)w.dj * w.dj, g, r, bits, nb);
+  const bool redo = near < 2u * e2 && chord != 0u;
+  if (__any_sync(0xffffffffu, redo)) {
+    uint32_t pb, nb;
+    exact_rows<MASK_PARITY>(redo, w.di0, w.dj, g, r, pb, nb);
+    if (redo) bits = pb;
   }
   return bits & chord;
 }
@@ -676,7 +687,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
             cx_store2(a.df, cxr, w[0].di0, bits, rp, PLANE, sw);
           } else if constexpr (MASK == MASK_QUAD) {
             uint32_t re[16], im[16];
-            block_quad(w[0], a.mg, a.ph, one, chord_up(w[0]), re, im);
+            bool redo;
+            const bool rare = block_quad(w[0], a.mg, a.ph, one, chord_up(w[0]), re, im, redo);
             if (!stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -685,11 +697,27 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
               *reinterpret_cast<uint4*>(rp + PLANE + ((q ^ sw) << 4)) =
                   make_uint4(im[4 * q], im[4 * q + 1], im[4 * q + 2], im[4 * q + 3]);
             }
+            if (rare) {
+              uint32_t odd, high;
+              exact_rows<MASK>(redo, w[0].di0, w[0].dj, a.mg, a.ph, odd, high);
+              if (redo) {
+                const uint32_t chord = chord_up(w[0]);
+#pragma unroll 1
+                for (int q = 0; q < 16; ++q) {
+                  uint32_t x, y;
+                  exact_quad_word(odd, high, one, chord, q, x, y);
+                  uint8_t* o = rp + (((q >> 2) ^ sw) << 4) + 4 * (q & 3);
+                  *reinterpret_cast<uint32_t*>(o) = x;
+                  *reinterpret_cast<uint32_t*>(o + PLANE) = y;
+                }
+              }
+            }
           } else {
+            bool redo[RPL], rare = false;
 #pragma unroll
             for (int h = 0; h < RPL; ++h) {
               uint32_t wd[16];
-              block_words<MASK>(w[h], a.mg, a.ph, one, chord_up(w[h]), wd);
+              rare |= block_words<MASK>(w[h], a.mg, a.ph, one, chord_up(w[h]), wd, redo[h]);
               if (h == 0 && !stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
 #pragma unroll
               for (int q = 0; q < 4; ++q)
@@ -697,6 +725,22 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
                     make_uint4(wd[4 * q], wd[4 * q + 1], wd[4 * q + 2], wd[4 * q + 3]);
             }
             if (!ok) break;
+            if (rare) {
+#pragma unroll 1
+              for (int h = 0; h < RPL; ++h) {
+                const bool again = h ? redo[RPL - 1] : redo[0];
+                const int32_t di0 = w[0].di0, dj = w[0].dj + 256 * h;
+                const uint32_t chord = h ? chord_up(w[RPL - 1]) : chord_up(w[0]);
+                uint32_t pb, nb;
+                exact_rows<MASK>(again, di0, dj, a.mg, a.ph, pb, nb);
+                if (again) {
+#pragma unroll 1
+                  for (int q = 0; q < 16; ++q)
+                    *reinterpret_cast<uint32_t*>(rp + h * PLANE + (((q >> 2) ^ sw) << 4) + 4 * (q & 3)) =
+                        exact_word<MASK>(pb, nb, one, chord, q);
+                }
+              }
+            }
           }
 #pragma unroll
           for (int h = 0; h < RPL; ++h) row_next<2 * BK>(w[h], a.ph);
@@ -1015,6 +1059,18 @@ __global__ void __launch_bounds__(2 * ITX * ITY) k_interp_cols(const InterpOut a
 }
 
 // ------------------------------------------------------------------ mask export
+template <int MASK>
+__device__ __forceinline__ void mask_words(const RowWalk& w, const MaskGeom& g, const PhaseRule& r, uint32_t disc,
+                                           uint32_t (&wd)[16]) {
+  bool redo;
+  if (!block_words<MASK>(w, g, r, 0x3F803F80u, disc, wd, redo)) return;
+  uint32_t pb, nb;
+  exact_rows<MASK>(redo, w.di0, w.dj, g, r, pb, nb);
+#pragma unroll
+  for (int q = 0; q < 16; ++q)
+    if (redo) wd[q] = exact_word<MASK>(pb, nb, 0x3F803F80u, disc, q);
+}
+
 __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int64_t j0, int64_t rows, uint8_t* out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1032,7 +1088,14 @@ __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int
       uint32_t wd[16];
       if (mask == MASK_QUAD) {
         uint32_t wi[16];
-        block_quad(w, mg, ph, 0x3F803F80u, disc, wd, wi);
+        bool redo;
+        if (block_quad(w, mg, ph, 0x3F803F80u, disc, wd, wi, redo)) {
+          uint32_t odd, high;
+          exact_rows<MASK_QUAD>(redo, w.di0, w.dj, mg, ph, odd, high);
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            if (redo) exact_quad_word(odd, high, 0x3F803F80u, disc, k, wd[k], wi[k]);
+        }
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
           const uint32_t x = (wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu, y = (wi[k / 2] >> (16 * (k & 1))) & 0xFFFFu;
@@ -1043,13 +1106,13 @@ __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int
         one.neg = 0;
         for (int q = 0; q < ph.lmod; ++q) {
           one.pos = 1ull << q;
-          block_words<MASK_LEVELS>(w, mg, one, 0x3F803F80u, disc, wd);
+          mask_words<MASK_LEVELS>(w, mg, one, disc, wd);
 #pragma unroll
           for (int k = 0; k < 32; ++k)
             if ((wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu) v[k] = (uint8_t)(1 + q);
         }
       } else if (mask == MASK_SIGNED) {
-        block_words<MASK_SIGNED>(w, mg, ph, 0x3F803F80u, disc, wd);
+        mask_words<MASK_SIGNED>(w, mg, ph, disc, wd);
 #pragma unroll
         for (int k = 0; k < 32; ++k)
           v[k] = ((disc >> k) & 1u) ? (uint8_t)(1 + ((wd[k / 2] >> (16 * (k & 1) + 15)) & 1u)) : 0;
@@ -1058,7 +1121,7 @@ __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = (uint8_t)((bits >> k) & 1u);
       } else {
-        block_words<MASK_PARITY>(w, mg, ph, 0x3F803F80u, disc, wd);
+        mask_words<MASK_PARITY>(w, mg, ph, disc, wd);
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = ((wd[k / 2] >> (16 * (k & 1))) & 0xFFFFu) ? 1 : 0;
       }
