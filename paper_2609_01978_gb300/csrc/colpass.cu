@@ -39,6 +39,7 @@ struct ColArgs {
   double kappa, delta;
   double msh;     // ROI (or node) shift in pitches: y_n = (n - msh) p
   double wr, wi;  // weight of this pass's field (1, 0 for a single-pass plate)
+  int tri;        // > 0: the field is its own transpose; blockIdx.x counts the tiles m >= n of tri x tri
 };
 
 template <typename R> struct RowPhase;
@@ -135,7 +136,12 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
   // element took as long as the products), and the rows' e^{2 pi i A}, A at dj and -dj
   constexpr bool FACT = sizeof(R) == 8 && !TAB, PAIR = sizeof(R) == 4 && !TAB;
   __shared__ C sF[FACT ? TJ : 1][18];
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
+  int bx = blockIdx.x, by = blockIdx.y;
+  if (g.tri) {
+    for (; bx >= g.tri - by; ++by) bx -= g.tri - by;
+    bx += by;
+  }
+  const int m0 = bx * TM, n0 = by * TN;
   const int64_t jb = (int64_t)blockIdx.z * g.jc;
   const int64_t je = jb + g.jc < g.rows ? jb + g.jc : g.rows;
   const int tid = threadIdx.x;
@@ -315,7 +321,7 @@ fzp_status run_colpass(const ColArgs& g, unsigned tx, unsigned ty, const R* C1, 
 }
 
 __global__ void k_epilogue(int M, double msh, double p, double lf, double f_over_lambda, double amp,
-                           int evenx, int eveny, const double2* __restrict__ Uacc, double2* __restrict__ out,
+                           int evenx, int eveny, int tri, const double2* __restrict__ Uacc, double2* __restrict__ out,
                            int accumulate) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= M * M) return;
@@ -328,7 +334,13 @@ __global__ void k_epilogue(int M, double msh, double p, double lf, double f_over
   w.y *= amp;
   // even: the accumulator holds the samples x >= 0, |m - M/2| of them from the axis
   const int h = M / 2;
-  const double2 u = Uacc[(int64_t)(eveny ? abs(n - h) : n) * (evenx ? h + 1 : M) + (evenx ? abs(m - h) : m)];
+  int un = eveny ? abs(n - h) : n, um = evenx ? abs(m - h) : m;
+  if (tri > 0 && un / tri > um / tri) {  // the accumulator's tiles of `tri` below the diagonal are not filled
+    const int x = un;
+    un = um;
+    um = x;
+  }
+  const double2 u = Uacc[(int64_t)un * (evenx ? h + 1 : M) + um];
   double2 v = make_double2(w.x * u.x - w.y * u.y, w.x * u.y + w.y * u.x);
   if (accumulate) {
     v.x += out[t].x;
@@ -372,12 +384,16 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   // tiles of 64 are four full ones and five slivers that share SMs with them)
   const int T = even ? 48 : TM;
   const int tx = (g.M + T - 1) / T, ty = (g.ny + T - 1) / T;
-  const int64_t tiles = (int64_t)tx * ty;
+  // a symmetric field: the tiles on and above the diagonal (k_epilogue mirrors)
+  const bool tri = P.nd.tri && tx == ty;
+  g.tri = tri ? tx : 0;
+  const int64_t tiles = tri ? (int64_t)tx * (tx + 1) / 2 : (int64_t)tx * ty;
   g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / BLOCKS + TJ - 1) / TJ * TJ));
   P.launches += 1;
-  return even                              ? run_colpass<double, false, 3>(g, tx, ty, P.d_C1d, P.d_Uacc, s)
-         : P.precision == FZP_PREC_FP64 ? run_colpass<double>(g, tx, ty, P.d_C1d, P.d_Uacc, s)
-                                           : run_colpass<float>(g, tx, ty, P.d_C1, P.d_Uacc, s);
+  const unsigned gx = (unsigned)(tri ? tiles : tx), gy = (unsigned)(tri ? 1 : ty);
+  return even                           ? run_colpass<double, false, 3>(g, gx, gy, P.d_C1d, P.d_Uacc, s)
+         : P.precision == FZP_PREC_FP64 ? run_colpass<double>(g, gx, gy, P.d_C1d, P.d_Uacc, s)
+                                        : run_colpass<float>(g, gx, gy, P.d_C1, P.d_Uacc, s);
 }
 
 fzp_status column_pass_table(Plan& P, const void* E, int64_t rows, int64_t estride, cudaStream_t s) {
@@ -422,7 +438,7 @@ fzp_status epilogue(Plan& P, void* d_field, int accumulate, cudaStream_t s) {
   const int count = P.M * P.M;
   const bool even = bluestein_even(P);
   k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lf, P.f / P.lambda, P.dx2 / lf, even ? 1 : 0,
-                                                 even && !P.nd.yfull ? 1 : 0, P.d_Uacc,
+                                                 even && !P.nd.yfull ? 1 : 0, P.nd.tri ? (even ? 48 : TM) : 0, P.d_Uacc,
                                                  reinterpret_cast<double2*>(d_field), accumulate);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
@@ -432,7 +448,7 @@ fzp_status epilogue(Plan& P, void* d_field, int accumulate, cudaStream_t s) {
 fzp_status epilogue_z(Plan& P, void* d_field, int accumulate, double z, cudaStream_t s) {
   const double lz = P.lambda * z;
   const int count = P.M * P.M;
-  k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lz, P.f / P.lambda, P.dx2 / lz, 0, 0, P.d_Uacc,
+  k_epilogue<<<(count + 255) / 256, 256, 0, s>>>(P.M, P.msh, P.p, lz, P.f / P.lambda, P.dx2 / lz, 0, 0, 0, P.d_Uacc,
                                                  reinterpret_cast<double2*>(d_field), accumulate);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());

@@ -258,6 +258,7 @@ struct NodeSet {
   double* d_W = nullptr;   // interpolation [ns][Mo] (owned by the plan, also in a batch)
   double* d_Wy = nullptr;  // [n][M], behind d_W: along y when the rows are not symmetric
   bool yfull = false;      // the call being run takes all n nodes along y
+  bool tri = false;        // its field (not on nodes) is its own transpose: column pass on and above the diagonal
   int64_t zero_acc = 0;    // accumulator elements that the next row pass is to zero first
   int slices = 1;          // images of C1 in the chunk being run, and their distance
   int64_t slice_elems = 0;

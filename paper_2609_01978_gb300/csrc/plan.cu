@@ -307,7 +307,7 @@ static fzp_status chunk_passes(Plan& P, int64_t j0, int64_t rows, RowKind kind, 
 }
 
 fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t s) {
-  *sym = false;
+  *sym = P.nd.tri = false;
   // rows up and down from the axis
   const int64_t c = P.c, up = b - 1 - c, dn = c - a, h = std::min(up, dn);
   const bool nodes = P.nd.n > 0;
@@ -329,8 +329,10 @@ fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t
   fzp_status st = FZP_OK;
   if (h >= 0) {
     // every row that meets the disc: the plate is its own transpose (the row
-    // passes on nodes use that)
-    *sym = nodes && up == dn && (up == P.c || (up + 1) * (up + 1) > P.mg.sR);
+    // passes on nodes use that, otherwise the column pass does)
+    const bool whole = up == dn && (up == P.c || (up + 1) * (up + 1) > P.mg.sR);
+    *sym = nodes && whole;
+    P.nd.tri = !nodes && whole;
     st = run(0, h + 1, ROWS_FOLDED, *sym);
   }
   const int64_t first = std::max<int64_t>(h, std::max(-up, -dn) - 1) + 1;  // one-sided distances
