@@ -55,6 +55,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -265,6 +266,34 @@ def folded_flops(info: dict, nodes: int, j0: int, j1: int) -> float:
     return float(np.sum(blocks)) * (fft + 8.0 * P) + len(d) * fft
 
 
+def decimation(info: dict, lam: float, f: float, M: int, pitch: float, flat: bool = True) -> int:
+    """Columns per grid point of the partitioned row pass with decimated rows
+    (bluestein.cu), 0 where it transforms the columns themselves.  ROI centred."""
+    dof = (M if flat else M - 1) * pitch * 2.0 * info["R"] / (lam * f)
+    n = next((n for n, most in (((128, 80.0), (256, 170.0)) if flat else ((64, 36.0), (128, 80.0))) if dof <= most), 0)
+    if not n:
+        return 0
+    u = math.pi * 1.25 * dof * (n - 1) / n * info["dx"] / (2.0 * info["R"])  # radians per column of the outermost node
+    return 32 if 32 * u <= 0.17 else 16 if 16 * u <= 0.17 else 0
+
+
+def decimated_flops(info: dict, j0: int, j1: int, flat: bool) -> float:
+    """FP32 flops of the decimated row pass for rows [j0, j1): 14 per column left
+    after the folds (four running sums, six grid points' weights per 16 columns)
+    and, for two rows, two 4096-point transforms and the product-sum.  The mask,
+    the membrane's phase and the sines are not counted."""
+    c, n = info["c"], info["N"]
+    inside = disc_samples(n, c, info["s_R"], j0, j1)
+    rows = j1 - j0
+    if flat:
+        h = min(j1 - 1 - c, c - j0)
+        both = disc_samples(n, c, info["s_R"], c - h, c + h + 1) if h >= 0 else 0
+        whole = h >= c or (h + 1) ** 2 > info["s_R"]
+        inside = both / (8.0 if whole else 4.0) + (inside - both) / 2.0
+        rows -= max(0, h)
+    return 14.0 * inside + rows / 2.0 * (2 * 5.0 * 4096 * 12 + 8.0 * 4096)
+
+
 def node_count(info: dict, lam: float, f: float, M: int, pitch: float, deformed: bool = False) -> int:
     """Nodes per axis that the dense form's contraction runs on (nodes.cu), for an
     ROI centred on the focus: the positive half of n nodes for a flat plate,
@@ -293,17 +322,18 @@ def node_flops(info: dict, nodes: int, j0: int, j1: int, deformed: bool = False)
     return 8.0 * nodes * info["passes"] * (both / (8.0 if whole else 4.0) + (inside - both) / 2.0)
 
 
-def membrane_forms_and_roofline(fzp, infos: list, M: int, steps: int, ms: float):
+def membrane_forms_and_roofline(fzp, infos: list, M: int, steps: int, ms: float, decs: list | None = None):
     """Forms chosen over a batch of membranes and the roofline of the step:
     the tensor work of the dense instances (24 M flops per in-disc sample:
     2 membrane passes x 3 split products x 2 real rows x M x 2 flops) when
-    dense instances are at least half the batch, else the FFT work of the
-    partitioned FP32 instances; either over the whole step's time, so a lower
+    dense instances are at least half the batch, else the row transforms' work
+    of the partitioned FP32 instances (decs: the columns per grid point of each
+    instance with decimated rows); either over the whole step's time, so a lower
     bound for a mixed batch."""
     forms = {}
     dense_flops = fft_flops = 0.0
     n_dense = n_fft = 0
-    for inf in infos:
+    for i, inf in enumerate(infos):
         k = ("dense" if inf["form"] == fzp.FORM_DENSE else "bluestein") + "/" + \
             {0: "f64", 1: "f32", 2: "split-bf16", 3: "bf16"}[inf["precision"]]
         forms[k] = forms.get(k, 0) + 1
@@ -311,7 +341,7 @@ def membrane_forms_and_roofline(fzp, infos: list, M: int, steps: int, ms: float)
             dense_flops += 24.0 * M * disc_samples(inf["N"], inf["c"], inf["s_R"], 0, inf["N"])
             n_dense += 1
         elif inf["precision"] == fzp.PREC_FP32 and inf["conv"] == 2:
-            fft_flops += partitioned_flops(inf, 0, inf["N"])
+            fft_flops += decimated_flops(inf, 0, inf["N"], False) if decs and decs[i] else partitioned_flops(inf, 0, inf["N"])
             n_fft += 1
     peaks, peak_kind = _peaks()
     whole = "whole step (graph of every instance's passes)"
@@ -384,7 +414,8 @@ def run_membranes(args, fzp, torch, dev, ws, pg, rank, local):
         ms = float(t.item())
     kernels = b.kernels
     b.close()
-    forms, roof = membrane_forms_and_roofline(fzp, infos, M, args.steps, ms)
+    forms, roof = membrane_forms_and_roofline(fzp, infos, M, args.steps, ms, [
+        decimation(inf, m.lam, fnum * m.D, M, m.lam * fnum / 8, False) for inf, m in zip(infos, mem)])
     # end to end through the public API with host buffers: batch from host
     # parameters (tuned choices cached in-process), propagate, fields to pinned
     # host memory, every instance's metrics, destroy
@@ -847,7 +878,12 @@ def main():
         launches = max(1, prof["dominant_launches"])
         flat = not wl.get("deform")
         nodes = node_count(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], not flat)
-        if info["conv"] == 2:
+        if info["conv"] == 2 and (flat or params.get("levels", 0) < 2) and \
+                decimation(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], flat):
+            flops_launch = decimated_flops(info, j0, j1, flat) * args.steps / launches
+            work = ("14 per column left after the symmetry folds, per two rows 10 P log2 P + 8 P (P = 4096); "
+                    "masks, phases and sines not counted")
+        elif info["conv"] == 2:
             flops_launch = (folded_flops(info, nodes, j0, j1) if flat else partitioned_flops(info, j0, j1)) \
                 * args.steps / launches
             work = ("per block of S columns of a row's chord 5 P log2 P + 8 P, per row 5 P log2 P "

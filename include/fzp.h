@@ -171,8 +171,10 @@ typedef struct fzp_params {
                           inverse 4096-point FFT per row, all on chip (where
                           the ROI samples the field several times finer than
                           its band, the row's outputs are that many
-                          interpolation nodes and M above is their count); FP32
-                          only (FZP_E_UNSUPPORTED with FP64).  Other values
+                          interpolation nodes and M above is their count, and
+                          on grids fine enough the blocks are of points 16 or
+                          32 columns apart that the columns were spread over);
+                          FP32 only (FZP_E_UNSUPPORTED with FP64).  Other values
                           are invalid; the other forms ignore it            */
 } fzp_params;
 

@@ -25,8 +25,9 @@
 // the aperture is never stored.
 //
 // FP32 default (fzp_params.conv): the same convolution partitioned into
-// 4096-point blocks, each row on chip from its mask to its M outputs
-// (k_seg, below); the four-step passes above remain the FP64 path and the
+// 4096-point blocks, each row on chip from its mask to its M outputs (k_seg,
+// below), its columns first spread over a coarse grid where the outputs' band is
+// that narrow (k_dec); the four-step passes above remain the FP64 path and the
 // single-convolution FP32 option.
 #include <algorithm>
 #include <cmath>
@@ -133,9 +134,6 @@ __device__ void dif_inverse(C* x, int logn, const C* __restrict__ tw, int twN) {
     __syncthreads();
   }
 }
-
-// Decimated rows (k_dec): grid points that a column's value is spread over.
-constexpr int DTAPS = 6;
 
 struct RowArgs {
   MaskGeom mg;
@@ -836,8 +834,8 @@ __device__ __forceinline__ void chunk_levels(int64_t di0, int64_t dj2, const Mas
 // stage instead of radix 2's 4, the inverse's last pass forms only the outputs
 // that are kept, and a flat plate's columns from the axis on fit half the
 // length.  4 mm plate (N = 5,057, L 8192 -> 4096), ROI 256^2: 6.2 -> 1.6 ms for
-// the row transforms, 22.2 -> 2.6 ms for a propagation with its metrics (rows
-// folded 8.2).
+// the row transforms (375,000 FP64 operations a row, 2,529 rows: 1.6 ms at 0.58
+// T/s, the pipe's rate), 22.2 -> 2.1 ms for a propagation with its metrics.
 constexpr size_t D16_SMEM = sizeof(double2) * (2 * SBUF + 15 * 256 + 256);
 __global__ void __launch_bounds__(STH, 1) k_f2_d16(RowArgs a, int mode) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -966,8 +964,10 @@ __global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int64_t col0, 
 // diagonal |di| = dj with half weight there (the field is this one plus its
 // transpose).  Half the blocks each, a quarter both, and half the rows; with the
 // outputs on nodes (nodes.cu: 128 instead of 512) the column pass shrinks too.
-// Whole propagation, ROI 512^2: D = 5 cm (N = 63,213) 17.14 -> 2.31 ms, L = 16
-// on N = 50,001 15.75 -> 2.13 ms.
+// Whole propagation, ROI 512^2, with the masks from the walked zone phase: D = 5
+// cm (N = 63,213) 17.1 -> 1.86 ms, L = 16 on N = 50,001 15.7 -> 1.38 ms; such
+// plates now take k_dec, this kernel the grids too small for it, deformed phase
+// plates and ROIs without nodes.
 template <int MODE>
 __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
   constexpr bool FOLD = MODE == SEG_FLAT || MODE == SEG_LEVELS;
@@ -1199,7 +1199,11 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
 // four running sums (c0 += z, c1 += c0, ...) per 16 columns, which are their
 // binomial moments; the weights T (decimation_weights) take them to the grid
 // points; lanes exchange the overlaps by shuffles.  No table is read per column.
-// What is left is issue-bound on the generators.
+// Whole propagations, k_seg -> k_dec: D = 5 cm 1.86 -> 0.80 ms, L = 16 1.38 -> 0.80,
+// four membranes on N <= 34,567 13.2 -> 5.1 ms (9 transforms a row to a half).
+// What bounds it: the issue slots (60 % busy at two CTAs of 128 registers a
+// thread per SM); of a membrane's 45 instructions per column the walk in pairs,
+// the mask's walk and the running sums take two thirds.
 // ---------------------------------------------------------------------------
 constexpr int DROW = SP / 2;                    // offset of the second row
 constexpr int DGRP = DROW / 32;                 // warp groups of chunks a row
@@ -1738,7 +1742,7 @@ static RowArgs make_args(const Plan& P) {
     a.Kc = turns64(0.5 * P.kappa);
     a.Kl = turns64(-P.nd.delta * (mc - P.nd.msh - (P.nd.even ? P.nd.n / 2 : 0)));
     a.cc2 = (uint32_t)((2 * a.Kc + 0x80000000ull) >> 32);
-    decimation_weights(b.dec, a.T);
+    std::copy(&b.T[0][0][0], &b.T[0][0][0] + 2 * DTAPS * 4, &a.T[0][0][0]);
   }
   return a;
 }
@@ -1779,6 +1783,7 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
     b.nseg = (P.N - b.col0 + b.S - 1) / b.S;
     b.dec = decimation(P);
     if (b.dec) {
+      decimation_weights(b.dec, b.T);
       // two rows to a transform: S + 5 + n < 2050, S a multiple of 32
       const int64_t chunks = (P.N - b.col0 + b.dec - 1) / b.dec, most = (DROW - M - DTAPS + 1) / 32 * 32;
       b.nseg = (chunks + most - 1) / most;

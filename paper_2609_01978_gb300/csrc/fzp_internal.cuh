@@ -192,6 +192,9 @@ template <> __device__ __forceinline__ double2 twiddle<double>(int64_t r, int64_
 // --------------------------------------------------------------------------
 // Plan
 // --------------------------------------------------------------------------
+// Decimated rows (k_dec): grid points that a column's value is spread over.
+constexpr int DTAPS = 6;
+
 struct Bluestein {
   int64_t L = 0;     // convolution length, power of two >= N + M - 1
   int64_t L1 = 1;    // four-step split L = L1 * L2 (L1 = 1: single pass)
@@ -211,6 +214,7 @@ struct Bluestein {
   int S = 0;
   int64_t nseg = 0;
   int dec = 0;            // decimated rows: columns to a grid point (then S counts those); 0: none
+  float2 T[2][DTAPS][4];  // their weights (decimation_weights), each twice
   int64_t col0 = 0;       // first input column (the axis when `half`)
   bool half = false;      // columns from the axis on, outputs x and -x added
   int64_t L_full = 0;     // power of two >= N + M - 1 (what the plan reports)

@@ -42,10 +42,17 @@
 // part of s kappa, s = di^2 + dj^2; the 64-bit fixed-point phase s K mod 2^64
 // (its top bit the zone's parity, or its top log2 L bits the level) is carried
 // exactly from block to block, and its upper 32 bits run along a block with
-// two integer additions per sample.  Their error is below E units; a block in
-// which a phase comes within E of a zone boundary (about one in 10^4) takes
-// the exact rule with the threshold table, sample by sample.  Per sample: two
-// additions, three halves for the test, one for the BF16 value.
+// two integer additions per sample.  Their error is below E units; a row of a
+// block in which a phase comes within E of a zone boundary takes the exact rule
+// with the threshold table, a sample per lane (exact_rows; a plate whose zones
+// end on samples has a tie in every 4 N of them).
+// What bounds it: on large flat plates the tensor pipe (1.51 PFLOP/s on N =
+// 120,001, 0.78 of the measured burst); on small ones the length of a unit's
+// chain (8 K blocks, 2,000 clocks each); with membranes the generators.
+// Whole propagations before (every sample against every ROI row, k_dense) and
+// now: 2 mm, ROI 128^2 0.242 -> 0.075 ms; 30 mm off the axis, 256^2 2.36 -> 0.167;
+// 25 cm, 512^2 200 -> 3.32; a rank's eighth of 1 m 422 -> 24.3; four levels on
+// 60,001^2 28.1 -> 0.349; four membranes on N <= 36,363, 128^2 20.0 -> 5.1 ms.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>

@@ -16,22 +16,21 @@
 //      dx_out / (lambda z_F)) as two complex products with the kernel
 //      K[m, u] = e^{i k0 u^2 / (2 z_F) - i k0 x_m u / z_F}: rows, then columns.
 //
-// GB300 mapping: the 2-D transforms are one block per row (the row in shared
-// memory, up to 16384 points = 132 KiB with padding), radix-2 stages fused
-// four at a time in registers, forward transforms left in bit-reversed order
-// for the inverse ones to read back; three row kernels (mask + forward;
-// forward + residual phase + inverse; inverse) and two tiled transposes, so
-// the padded grid crosses HBM five times each way.  The zoom (M P^2 and M^2 P complex
-// multiply-adds) is a dense contraction with the structure of the dense
-// form's: K U1 K^T with the kernel K[m][u] above.  For M a multiple of 128 it
-// runs on the tensor cores through the dense form's kernels: the last inverse
-// transform writes U1 as two real planes, each plane is the loaded B operand
-// of one k_dense row pass (split BF16 hi + lo, three products, FP32 tensor
-// memory, C1 by reduce-add) against split-BF16 images of K, and the tensor
-// column pass adds K C1^T into the FP64 ROI field with weight 1 (real plane)
-// or i (imaginary plane).  Other M take two FP32 complex products on the CUDA
-// cores.  The zoom kernel's phases are reduced in FP64 before the FP32
-// (co)sines; the residual phase of step 2, once per grid sample, without FP64.
+// GB300 mapping.  Whole apertures (k_sa_half, below): the plate is even in x and
+// y and its own transpose, so real half spectra of half the rows, a triangle of
+// the other direction, carry everything, and the zoom runs in the frequency
+// domain on the ROI's interpolation nodes (nodes.cu).  A range of rows: one block
+// per row of the padded grid (the row in shared memory, up to 16384 points = 132
+// KiB with padding), radix-2 stages fused four at a time in registers, forward
+// transforms left in bit-reversed order for the inverse ones to read back; three
+// row kernels (mask + forward; forward + residual phase + inverse; inverse) and
+// two tiled transposes.  The zoom (M P^2 and M^2 P complex multiply-adds) is then
+// a dense contraction K U1 K^T with the kernel K[m][u] above: on nodes, U1 as two
+// real planes that k_nodes loads and splits into BF16 hi + lo; where the ROI's
+// band is too wide for nodes, the planes through k_dense (M a multiple of 128) or
+// two FP32 complex products on the CUDA cores.  The zoom kernel's phases are
+// reduced in FP64 before the FP32 (co)sines; the residual phase of step 2, once
+// per grid sample, without FP64.
 #include <cmath>
 #include <vector>
 
@@ -412,7 +411,7 @@ __global__ void __launch_bounds__(512, 1) k_sa_rows(const SaRowArgs a) {
 // axes, E's columns alike.  Only the lower triangle of H A (by positions, in
 // 256-row tiles) is formed; it is contracted on the tensor cores onto the
 // interpolation nodes (nodes.cu).
-// D = 8 mm (P = 16,384), ROI 512^2: 15.66 -> 1.79 ms a propagation (the row
+// D = 8 mm (P = 16,384), ROI 512^2: 15.66 -> 1.77 ms a propagation (the row
 // transforms 11.1 -> 1.34 ms), error against 64 bits 1.6e-5 -> 1.1e-6.
 struct SaHalfArgs {
   int64_t P;
