@@ -427,6 +427,26 @@ fzp_status metrics(Plan& P, const void* d_field, cudaStream_t stream, fzp_metric
 fzp_status bluestein_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t stream);
 fzp_status dense_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t stream);
 
+// Launch that may overlap the end of the stream's previous kernel (tc_ptx.cuh:
+// the kernel waits for it itself).  The surrogate's chain of nine launches is
+// bound by the gaps between them: gradients of a batch of 256, 130 -> 111 us.
+// (The node form's chain got slower, 78 -> 84 us on the 2 mm plate: its blocks
+// take the place of the running kernel's.)
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // Row index into the C1 layout: kernel row tile t = m / 64 holds the real parts
 // of m = 64t..64t+63 in rows [0,64) and the imaginary parts in rows [64,128).
 __host__ __device__ __forceinline__ int c1_row_re(int m) { return (m >> 6) * 128 + (m & 63); }

@@ -152,6 +152,8 @@ __global__ void __launch_bounds__(GEMM_THREADS) k_gemm(const Gemm g0, const Gemm
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
   const int nk = (p.K + GK - 1) / GK;
   // K step kb into its ring slot: 128 + 64 rows of 128 bytes, swizzled
   auto load = [&](int kb) {
@@ -307,6 +309,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) k_gemm(const Gemm g0, const Gemm
 // The batch's inputs in BF16, row-major (zero padded) and, training, transposed.
 __global__ void k_inputs(int64_t R, int64_t Cn, const float* x, __nv_bfloat16* rows, int64_t ldr, __nv_bfloat16* cols,
                          int64_t ldt) {
+  pdl_trigger();
   const int64_t total = R * Cn;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = t / Cn, c = t % Cn;
@@ -406,8 +409,7 @@ Gemm product(int64_t M, int64_t N, int64_t K, const __nv_bfloat16* A, int64_t ld
 
 fzp_status run_gemm(fzp_surrogate_s& S, const Gemm& a, const Gemm* b, cudaStream_t s) {
   const int na = a.tiles, nb = b ? b->tiles : 0;
-  k_gemm<<<(unsigned)(na + nb), GEMM_THREADS, GEMM_SMEM, s>>>(a, b ? *b : a, na, S.err);
-  FZP_CUDA_TRY(cudaGetLastError());
+  FZP_CUDA_TRY(launch_after(k_gemm, dim3((unsigned)(na + nb)), dim3(GEMM_THREADS), GEMM_SMEM, s, a, b ? *b : a, na, S.err));
   return FZP_OK;
 }
 

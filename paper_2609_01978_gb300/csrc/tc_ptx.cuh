@@ -100,6 +100,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// ---- programmatic dependent launch: a kernel launched with launch_after() may
+// start while its predecessor in the stream runs and does not touch global memory
+// before pdl_wait() (the predecessor complete, its writes visible); pdl_trigger()
+// lets the successor start as soon as every block of this grid is running.  What
+// the predecessor wrote is read with plain loads (a read-only load may be moved
+// over the wait).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- cluster (distributed shared memory) helpers
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
