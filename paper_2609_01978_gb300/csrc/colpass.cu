@@ -22,8 +22,8 @@ namespace {
 constexpr int TN = 64, TM = 64, TJ = 16, PJ = 128;  // output tiles of 64 (48: NA = 3 outputs per thread and side)
 
 constexpr int CZ = 4;        // blocks of a cluster along the rows
-constexpr int BLOCKS = 288;  // two per SM as far as clusters of four fit into the GPCs
-// whose tile of sums fits in static shared memory
+constexpr int BLOCKS = 288;  // two per SM as far as clusters of four fit into the GPCs (of 304 in eights a second wave ran)
+// Clusters: where the tile of sums fits in static shared memory.
 template <typename R, int NA> constexpr bool col_clusters = sizeof(R) == 4 || NA < 4;
 
 struct ColArgs {
@@ -119,8 +119,13 @@ __device__ __forceinline__ double2 peer_load(uint32_t addr, double2) {
 // TAB: the kernel's columns from a table E [n][estride] instead of their phase.
 // The blocks' sums meet in Uacc: in clusters of CZ along the rows, block k adds up
 // its part of the tile over the cluster through distributed shared memory first.
-// Without that, 304 blocks' FP64 atomics on the same 8,192 values took most of
-// the kernel.
+// Without that, 304 blocks put FP64 atomics on the same 8,192 values.  The next
+// tile of C1 loads during the products.  18,965 rows, 64 x 64 nodes: 56 us without
+// clusters and prefetch and with two sine pairs per folded kernel value, 49 with
+// clusters of eight and prefetch, 33 with clusters of four and one cosine (issue
+// slots 28 -> 35 % busy; the waits left are loads and the barriers of 16-row tiles).
+// FP64, 2,529 rows, 129 x 129 outputs, bound by the FP64 pipe: 0.46 ms, with the
+// tiles on and above the diagonal only a propagation takes 0.09 ms less.
 template <typename R, bool TAB = false, int NA = 4>
 __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
   using C = typename Cplx<R>::T;

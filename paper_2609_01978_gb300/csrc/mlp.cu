@@ -7,7 +7,7 @@
 // mean squared error over batch and outputs; optimiser AdamW (decoupled weight
 // decay on weights, not biases).  Weights are kept as FP32 masters; every matrix
 // product takes BF16 operands (weights, layer inputs, back-propagated errors)
-// and accumulates in FP32 in tensor memory (tcgen05.mma kind::f16, M128 N128).
+// and accumulates in FP32 in tensor memory (tcgen05.mma kind::f16, M128 N64).
 //
 // Matrix products, all as C[M x N] = A[M x K] . B[N x K]^T with K contiguous:
 //   forward  z_l   = h_{l-1} . W_l^T          (A = h, B = W)
@@ -21,7 +21,9 @@
 // its epilogue, and a layer's two backward products share a launch.  Every
 // product keeps one accumulation in K order: a split of the longest (dh of the
 // output layer, K = 4160) was no slower to write but moves g in its last FP32
-// bits, and with them the BF16 rounding of 3 % of g's values.
+// bits, and with them the BF16 rounding of 3 % of g's values.  A launch overlaps
+// the end of the one before.  Gradients of that batch: 46 launches, 1,154 us;
+// fused 130; overlapped 111.
 #include <cuda_bf16.h>
 
 #include <algorithm>
