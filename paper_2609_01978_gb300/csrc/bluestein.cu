@@ -600,9 +600,8 @@ enum { SEG_FLAT = 0, SEG_LEVELS = 1, SEG_MEMBRANE = 2, SEG_GENERAL = 3 };
 // A membrane's phase (turns, 2 w / lambda) on the 16 columns from di0, CLOSED
 // where the plate is (bits: open columns), to shared memory at a pitch of one.
 constexpr float CLOSED = 1e30f;
-template <int NR>
-__device__ __forceinline__ void membrane_chunk(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits, float* o) {
-  MembraneWalk<NR> walk(d, r, di0);
+template <typename Walk>
+__device__ __forceinline__ void membrane_chunk(Walk walk, uint32_t bits, float* o) {
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const float w = walk.next();
@@ -1048,11 +1047,15 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
           for (int q = 0; q < 16; ++q) tc[q] = __ldg(pt + min(t + 256 * q, lim));
           if (w != 0u) {
             const int32_t di0 = (int32_t)(is + xo - a.mg.c);
-            switch (a.df.n) {
-              case 0: membrane_chunk<0>(a.df, cxr, di0, w, o); break;
-              case 1: membrane_chunk<1>(a.df, cxr, di0, w, o); break;
-              case 2: membrane_chunk<2>(a.df, cxr, di0, w, o); break;
-              default: membrane_chunk<3>(a.df, cxr, di0, w, o); break;
+            if (a.df.direct) {
+              membrane_chunk(MembraneDirect(a.df, cxr, di0), w, o);
+            } else {
+              switch (a.df.n) {
+                case 0: membrane_chunk(MembraneWalk<0>(a.df, cxr, di0), w, o); break;
+                case 1: membrane_chunk(MembraneWalk<1>(a.df, cxr, di0), w, o); break;
+                case 2: membrane_chunk(MembraneWalk<2>(a.df, cxr, di0), w, o); break;
+                default: membrane_chunk(MembraneWalk<3>(a.df, cxr, di0), w, o); break;
+              }
             }
           } else {
 #pragma unroll
@@ -1349,11 +1352,9 @@ __device__ __forceinline__ void dec_levels(const RowArgs& a, const DecRow& row, 
 // Deformed binary plate: both rows' membrane phases walked along the chunk in
 // pairs, one hardware sine and cosine of the sum with the chirp's reduced to
 // [-1/2, 1/2] turns (absolute error below 4e-7 each).
-template <int D, int NR>
-__device__ __forceinline__ void dec_membrane_n(const RowArgs& a, const DecRow (&row)[2], const CxRow (&cx)[2], int32_t x0,
+template <int D, typename Walk2>
+__device__ __forceinline__ void dec_membrane_n(const RowArgs& a, const DecRow (&row)[2], Walk2 walk, int32_t x0,
                                                float2 (&tap)[2][DTAPS]) {
-  const int32_t di0 = (int32_t)(x0 - a.mg.c);
-  MembraneWalk2<NR> walk(MembraneWalk<NR>(a.df, cx[0], di0), MembraneWalk<NR>(a.df, cx[1], di0));
 #pragma unroll 1
   for (int sub = 0; sub < D / 16; ++sub) {
     const int32_t x = x0 + 16 * sub;
@@ -1377,14 +1378,23 @@ __device__ __forceinline__ void dec_membrane_n(const RowArgs& a, const DecRow (&
     for (int e = 0; e < 2; ++e) sums_out(a, sub, c[e], tap[e]);
   }
 }
+template <int NR>
+__device__ __forceinline__ MembraneWalk2<NR> walk_rows(const DeformCoef& d, const CxRow (&cx)[2], int32_t di0) {
+  return MembraneWalk2<NR>(MembraneWalk<NR>(d, cx[0], di0), MembraneWalk<NR>(d, cx[1], di0));
+}
 template <int D>
 __device__ __forceinline__ void dec_membrane(const RowArgs& a, const DecRow (&row)[2], const CxRow (&cx)[2], int32_t x0,
                                              float2 (&tap)[2][DTAPS]) {
+  const int32_t di0 = (int32_t)(x0 - a.mg.c);
+  if (a.df.direct) {
+    dec_membrane_n<D>(a, row, MembraneDirect2(MembraneDirect(a.df, cx[0], di0), MembraneDirect(a.df, cx[1], di0)), x0, tap);
+    return;
+  }
   switch (a.df.n) {
-    case 0: dec_membrane_n<D, 0>(a, row, cx, x0, tap); break;
-    case 1: dec_membrane_n<D, 1>(a, row, cx, x0, tap); break;
-    case 2: dec_membrane_n<D, 2>(a, row, cx, x0, tap); break;
-    default: dec_membrane_n<D, 3>(a, row, cx, x0, tap); break;
+    case 0: dec_membrane_n<D>(a, row, walk_rows<0>(a.df, cx, di0), x0, tap); break;
+    case 1: dec_membrane_n<D>(a, row, walk_rows<1>(a.df, cx, di0), x0, tap); break;
+    case 2: dec_membrane_n<D>(a, row, walk_rows<2>(a.df, cx, di0), x0, tap); break;
+    default: dec_membrane_n<D>(a, row, walk_rows<3>(a.df, cx, di0), x0, tap); break;
   }
 }
 
@@ -1647,7 +1657,10 @@ DeformCoef deform_coef(const Plan& P) {
     c.h2[k] = (float)(d.ridge_h[k] * k2);
     c.rho[k] = (float)std::exp(-2.0 * (P.dx * P.dx / (2.0 * sg * sg)) * nx * nx);
     c.eta[k] = (float)-std::expm1(-2.0 * (P.dx * P.dx / (2.0 * sg * sg)) * nx * nx);
+    // full width along a row (in columns) below 64
+    if (P.dx * P.dx * nx * nx * 64.0 * 64.0 > d.ridge_width[k] * d.ridge_width[k]) c.direct = 1;
   }
+  if (c.z4 > 3.0f) c.direct = 1;
   return c;
 }
 

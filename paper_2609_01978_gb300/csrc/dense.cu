@@ -532,7 +532,8 @@ __device__ __forceinline__ void expand_signed(uint32_t disc, uint32_t odd, uint3
 }
 
 // Chunks [q0, q0 + nq) of the row (8 columns each); di0 = column of the block
-// start minus c; NR ridges.
+// start minus c; NR ridges, walked along the row; NR < 0: every column by itself
+// (DeformCoef::direct).
 template <int NR>
 __device__ __forceinline__ void cx_store_n(const DeformCoef& d, const CxRow& r, int64_t di0, uint32_t bits,
                                            int sinpart, uint8_t* hi_row, uint8_t* lo_row, int sw, int q0, int nq) {
@@ -565,16 +566,21 @@ __device__ __forceinline__ void cx_store_n(const DeformCoef& d, const CxRow& r, 
       float v[2];
 #pragma unroll
       for (int z = 0; z < 2; ++z) {
-        float wz = d.amp2 * ws * fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f);
+        float wz;
+        if constexpr (NR < 0) {
+          wz = membrane_turns(d, r, fi);
+        } else {
+          wz = d.amp2 * ws * fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f);
 #pragma unroll
-        for (int e = 0; e < NR; ++e) {
-          wz = fmaf(d.h2[e], g[e], wz);
-          g[e] *= rr[e];
-          rr[e] *= d.rho[e];
+          for (int e = 0; e < NR; ++e) {
+            wz = fmaf(d.h2[e], g[e], wz);
+            g[e] *= rr[e];
+            rr[e] *= d.rho[e];
+          }
+          const float nws = fmaf(ws, d.zc, wc * d.zs);
+          wc = fmaf(wc, d.zc, -ws * d.zs);
+          ws = nws;
         }
-        const float nws = fmaf(ws, d.zc, wc * d.zs);
-        wc = fmaf(wc, d.zc, -ws * d.zs);
-        ws = nws;
         fi += 1.0f;
         wz -= rintf(wz);
         const float x = TWO_PI * wz;
@@ -592,7 +598,8 @@ __device__ __forceinline__ void cx_store_n(const DeformCoef& d, const CxRow& r, 
 // (0 to 3, uniform over the launch).
 __device__ __forceinline__ void cx_store(const DeformCoef& d, const CxRow& r, int64_t di0, uint32_t bits, int sinpart,
                                          uint8_t* hi_row, uint8_t* lo_row, int sw, int q0, int nq) {
-  switch (d.n) {
+  switch (d.direct ? -1 : d.n) {
+    case -1: cx_store_n<-1>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
     case 0: cx_store_n<0>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
     case 1: cx_store_n<1>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
     case 2: cx_store_n<2>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;

@@ -8,17 +8,13 @@
 
 namespace fzp {
 
-// Membrane pass: one row's T cos(phi) (or T sin(phi)) on 8-column chunks of a
-// 32-column block given the block's open bits, as BF16 hi and lo planes (the
-// 16-byte chunks of the 64-byte-swizzled row).  phi / 2 pi = 2 w / lambda in
-// FP32, walked along the row from the first column: the wrinkle's phasor
-// e^{2 pi i t} (t = di kx + dj ky, integer turns dropped exactly) turns by
-// e^{2 pi i kx} per column, a ridge's g = exp(-q d^2) by its ratio r, which
-// itself scales by rho = exp(-2 q nx^2) = 1 - eta; the sum is reduced to [-1/2, 1/2]
-// turns before one hardware sine or cosine (absolute error below 4e-7; the
-// walk adds ~1e-6 relative over 32 columns).  A ridge below 1e-30 at the
-// first column stays below 1e-29 in the block (its width is hundreds of
-// columns) and is left out.
+// Membrane generators: T cos(phi) and T sin(phi) of a row's columns given their
+// open bits.  phi / 2 pi = 2 w / lambda in FP32: the wrinkle's turns t = di kx + dj
+// ky (integer turns dropped exactly) through a hardware sine, times the taper,
+// plus a Gaussian per ridge; walked along the row where the deformation is smooth
+// on the columns (MembraneWalk), evaluated column by column where it is not
+// (MembraneDirect).  The sum is reduced to [-1/2, 1/2] turns before one hardware
+// sine or cosine (absolute error below 4e-7).
 struct CxRow {
   float fjkh, fjkl, fj2, cr[3];  // row terms: dj kyh, dj kyl, dj^2, ridge offsets
 };
@@ -47,8 +43,11 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 // rounding at the small angles of a wrinkle), the taper by its constant second
 // difference, a ridge by its ratio, kept as the ratio less one: g += g r1, r1 <-
 // r1 rho - (1 - rho) (a ratio near one rounded to FP32 is off by 3e-8 and more
-// each, 2e-5 of g over 32 columns).  Started exactly every 16 (k_seg) or 32
-// columns (k_dec, k_nodes).  NR ridges.
+// each, 2e-5 of g over 32 columns).  Started exactly every 16 (k_seg, k_nodes) or
+// 32 columns (k_dec).  NR ridges.  A ridge below 1e-30 at the first column is left
+// out of the walk: DeformCoef::direct keeps ridges from here whose walk could
+// rise again (a full width below 64 columns along the row; at that width it is
+// still below 1e-15 after 32 columns).
 template <int NR>
 struct MembraneWalk {
   float s, e, tap, dt, ddt, z4;
@@ -102,7 +101,44 @@ struct MembraneWalk {
   }
 };
 
-// Two of these walks side by side, every step's operations in pairs.
+// The same phase evaluated at the column, for ridges and wrinkles of any width.
+__device__ __forceinline__ float membrane_turns(const DeformCoef& d, const CxRow& r, float fi) {
+  constexpr float TWO_PI = 6.28318530717958648f;
+  const float th = fmaf(fi, d.kxh, r.fjkh);
+  float tt = (th - rintf(th)) + fmaf(fi, d.kxl, r.fjkl);
+  tt -= rintf(tt);
+  float wz = d.amp2 * __sinf(TWO_PI * tt) * fmaf(-d.tq, fmaf(fi, fi, r.fj2), 1.0f);
+#pragma unroll
+  for (int e = 0; e < 3; ++e)
+    if (e < d.n) {
+      const float dd = fmaf(fi, d.nx[e], r.cr[e]);
+      wz = fmaf(d.h2[e], __expf(-d.q[e] * dd * dd), wz);
+    }
+  return wz;
+}
+
+struct MembraneDirect {
+  const DeformCoef& d;
+  const CxRow& r;
+  float fi;
+  __device__ __forceinline__ MembraneDirect(const DeformCoef& d_, const CxRow& r_, int32_t di0) : d(d_), r(r_), fi((float)di0) {}
+  __device__ __forceinline__ float next() {
+    const float wz = membrane_turns(d, r, fi);
+    fi += 1.0f;
+    return wz;
+  }
+};
+
+struct MembraneDirect2 {
+  MembraneDirect a, b;
+  __device__ __forceinline__ MembraneDirect2(const MembraneDirect& a_, const MembraneDirect& b_) : a(a_), b(b_) {}
+  __device__ __forceinline__ float2 next() {
+    const float wa = a.next();
+    return make_float2(wa, b.next());
+  }
+};
+
+// Two walks side by side, every step's operations in pairs.
 template <int NR>
 struct MembraneWalk2 {
   float2 s, e, tap, dt, ddt, mz4;
@@ -149,11 +185,9 @@ __device__ __forceinline__ float2 reduced_rad(float2 x) {
 // Both masks of a membrane, T cos(phi) and T sin(phi), on the 32 columns from
 // di0 (bit k of `bits`: column k open), as the row's four 16-byte parts in the
 // planes cos hi, cos lo, sin hi, sin lo (`plane` bytes apart): columns k and
-// k + 16 walk side by side, four at a time to the planes.  NR ridges.
-template <int NR>
-__device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits,
-                                            uint8_t* base, uint32_t plane, int sw) {
-  MembraneWalk2<NR> walk(MembraneWalk<NR>(d, r, di0), MembraneWalk<NR>(d, r, di0 + 16));
+// k + 16 walk side by side, four at a time to the planes.
+template <typename Walk2>
+__device__ __forceinline__ void cx_store2_n(Walk2 walk, uint32_t bits, uint8_t* base, uint32_t plane, int sw) {
 #pragma unroll 1
   for (int q = 0; q < 4; ++q, bits >>= 4) {
     uint32_t hc[2][2], lc[2][2], hs[2][2], ls[2][2];
@@ -186,13 +220,22 @@ __device__ __forceinline__ void cx_store2_n(const DeformCoef& d, const CxRow& r,
   }
 }
 
+template <int NR>
+__device__ __forceinline__ MembraneWalk2<NR> walk32(const DeformCoef& d, const CxRow& r, int32_t di0) {
+  return MembraneWalk2<NR>(MembraneWalk<NR>(d, r, di0), MembraneWalk<NR>(d, r, di0 + 16));
+}
+
 __device__ __forceinline__ void cx_store2(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits, uint8_t* base,
                                           uint32_t plane, int sw) {
+  if (d.direct) {
+    cx_store2_n(MembraneDirect2(MembraneDirect(d, r, di0), MembraneDirect(d, r, di0 + 16)), bits, base, plane, sw);
+    return;
+  }
   switch (d.n) {
-    case 0: cx_store2_n<0>(d, r, di0, bits, base, plane, sw); break;
-    case 1: cx_store2_n<1>(d, r, di0, bits, base, plane, sw); break;
-    case 2: cx_store2_n<2>(d, r, di0, bits, base, plane, sw); break;
-    default: cx_store2_n<3>(d, r, di0, bits, base, plane, sw); break;
+    case 0: cx_store2_n(walk32<0>(d, r, di0), bits, base, plane, sw); break;
+    case 1: cx_store2_n(walk32<1>(d, r, di0), bits, base, plane, sw); break;
+    case 2: cx_store2_n(walk32<2>(d, r, di0), bits, base, plane, sw); break;
+    default: cx_store2_n(walk32<3>(d, r, di0), bits, base, plane, sw); break;
   }
 }
 
