@@ -1803,7 +1803,9 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
       b.S = (int)(((chunks + b.nseg - 1) / b.nseg + 31) / 32 * 32);
     }
     b.rows = P.chunk_rows;
-    out->pre = sizeof(C) * P.N;
+    // decimated: a value per grid point, which on grids of up to 35 columns are
+    // more than the columns (a block is at least 32 + 5 points)
+    out->pre = sizeof(C) * (size_t)(b.dec ? b.nseg * b.S + DTAPS - 1 : P.N);
     out->H = sizeof(C) * (size_t)SP * (size_t)b.nseg;
     out->tab = sizeof(C) * (b.L + (int)b.L2 + std::max(P.M, M) + 4096);
     out->Z = 0;

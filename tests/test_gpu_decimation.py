@@ -65,3 +65,24 @@ def test_membranes(env, N, ridges):
                                               (126001, 64, 0.0, 4)])
 def test_several_transforms_per_row(env, N, M, shift, levels):
     _compare(*env, N, M, lambda N, c: [(c - 4, c + 5), (c // 2, c // 2 + 7), (3, 40)], shift, levels)
+
+
+@pytest.mark.parametrize("N", [3, 31, 33, 35, 37])
+@pytest.mark.parametrize("shift", [0.0, 7.25])
+def test_smallest_grids(env, N, shift):
+    """Grids of fewer columns than one block has grid points: the centre of a large
+    plate (open there), and a whole small plate under a fine ROI pitch."""
+    fzp, torch = env
+    for D, M, p, opened in [(5e-3, 64, 1e-8, 1), ((N - 0.5) * LAM * 5 / 4, 64, 1e-9, 0)]:
+        geom = dict(D=D, f=5 * D, lam=LAM, M=M, pitch=p, N=N, centre_open=opened)
+        if shift:
+            geom["x0"] = -(M / 2 - shift) * p
+        with fzp.Plan(form=fzp.FORM_BLUESTEIN, precision=fzp.PREC_FP32, **geom) as plan, \
+                fzp.Plan(form=fzp.FORM_BLUESTEIN, precision=fzp.PREC_FP64, **geom) as exact:
+            for a, b in [(0, N), (N // 2, N // 2 + 1), (0, N // 2), (N // 2 - 1, N)]:
+                U, _ = run_plan(fzp, torch, plan, M, a, b)
+                R, _ = run_plan(fzp, torch, exact, M, a, b)
+                if abs(R).max() == 0:
+                    assert abs(U).max() == 0, (a, b)
+                else:
+                    assert rel_l2(U, R) <= TOL, (D, a, b)
