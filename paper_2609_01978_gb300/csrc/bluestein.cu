@@ -593,9 +593,10 @@ constexpr int SBUF = SB1 > SB0 ? SB1 : SB0;
 constexpr int NO_LEVEL = 64;      // level byte of a column outside the disc: phasor 0
 constexpr size_t SEG_SMEM = sizeof(float2) * (2 * SBUF + 15 * 256 + 256 + NO_LEVEL + 2) + SP;
 // row kernels: binary plate (chunk bits), phase plate (chunk zone steps),
-// deformed binary plate (chunk bits and the membrane phasor), general
-// transmission (a deformed phase plate)
-enum { SEG_FLAT = 0, SEG_LEVELS = 1, SEG_MEMBRANE = 2, SEG_GENERAL = 3 };
+// deformed binary plate (chunk bits and the membrane phasor, walked or, with
+// DeformCoef::direct, by column), general transmission (a deformed phase plate)
+enum { SEG_FLAT = 0, SEG_LEVELS = 1, SEG_MEMBRANE = 2, SEG_GENERAL = 3, SEG_DIRECT = 4 };
+constexpr bool seg_membrane(int mode) { return mode == SEG_MEMBRANE || mode == SEG_DIRECT; }
 
 // A membrane's phase (turns, 2 w / lambda) on the 16 columns from di0, CLOSED
 // where the plate is (bits: open columns), to shared memory at a pitch of one.
@@ -1000,7 +1001,7 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
 #pragma unroll
     for (int d = 0; d < 16; ++d) acc[d] = make_float2(0.0f, 0.0f);
     CxRow cxr;
-    if (MODE == SEG_MEMBRANE) cx_row_init(a.df, dj, cxr);
+    if (seg_membrane(MODE)) cx_row_init(a.df, dj, cxr);
     if (rem >= 0) {
       int64_t bmax = isqrt_row(rem);
       if (FOLD && a.octant) bmax = min(bmax, dj);
@@ -1030,7 +1031,7 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
 #pragma unroll
           for (int q = 0; q < 16; ++q)
             if (((mk[16 * q + (t >> 4)] >> (t & 15)) & 1u) == 0) v[q] = make_float2(0.0f, 0.0f);
-        } else if (MODE == SEG_MEMBRANE) {
+        } else if (seg_membrane(MODE)) {
           uint32_t w = 0u;
           if (meets && !walk_bits16(walk16(is + xo - a.mg.c, dj * dj, a.ph), a.ph, w)) w = chunk_bits(is + xo, dj * dj, a.mg);
           w &= inside;
@@ -1047,7 +1048,7 @@ __global__ void __launch_bounds__(STH, 2) k_seg(RowArgs a) {
           for (int q = 0; q < 16; ++q) tc[q] = __ldg(pt + min(t + 256 * q, lim));
           if (w != 0u) {
             const int32_t di0 = (int32_t)(is + xo - a.mg.c);
-            if (a.df.direct) {
+            if (MODE == SEG_DIRECT) {
               membrane_chunk(MembraneDirect(a.df, cxr, di0), w, o);
             } else {
               switch (a.df.n) {
@@ -1382,11 +1383,11 @@ template <int NR>
 __device__ __forceinline__ MembraneWalk2<NR> walk_rows(const DeformCoef& d, const CxRow (&cx)[2], int32_t di0) {
   return MembraneWalk2<NR>(MembraneWalk<NR>(d, cx[0], di0), MembraneWalk<NR>(d, cx[1], di0));
 }
-template <int D>
+template <int D, bool DIRECT>
 __device__ __forceinline__ void dec_membrane(const RowArgs& a, const DecRow (&row)[2], const CxRow (&cx)[2], int32_t x0,
                                              float2 (&tap)[2][DTAPS]) {
   const int32_t di0 = (int32_t)(x0 - a.mg.c);
-  if (a.df.direct) {
+  if (DIRECT) {
     dec_membrane_n<D>(a, row, MembraneDirect2(MembraneDirect(a.df, cx[0], di0), MembraneDirect(a.df, cx[1], di0)), x0, tap);
     return;
   }
@@ -1428,14 +1429,14 @@ __global__ void __launch_bounds__(STH, 2) k_dec(RowArgs a) {
       const int64_t rem = a.mg.sR - row[e].dj * row[e].dj;
       if (rem >= 0 && 2 * p + e < a.rows) {
         int64_t bmax = isqrt_row(rem);
-        if (MODE != SEG_MEMBRANE && a.octant) bmax = min(bmax, row[e].dj);
+        if (!seg_membrane(MODE) && a.octant) bmax = min(bmax, row[e].dj);
         // the row's disc chord, within the grid (a given N may cut the disc)
-        row[e].lo = (int32_t)(MODE != SEG_MEMBRANE && a.half ? a.mg.c : max(a.mg.c - bmax, (int64_t)0));
+        row[e].lo = (int32_t)(!seg_membrane(MODE) && a.half ? a.mg.c : max(a.mg.c - bmax, (int64_t)0));
         row[e].hi = (int32_t)min(a.mg.c + bmax, a.N - 1);
         lo = min(lo, row[e].lo);
         hi = max(hi, row[e].hi);
       }
-      if (MODE == SEG_MEMBRANE) cx_row_init(a.df, row[e].dj, cx[e]);
+      if (seg_membrane(MODE)) cx_row_init(a.df, row[e].dj, cx[e]);
     }
     float2 acc[16];
 #pragma unroll
@@ -1456,7 +1457,7 @@ __global__ void __launch_bounds__(STH, 2) k_dec(RowArgs a) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) dec_levels<D>(a, row[e], x0, tap[e]);
           } else {
-            dec_membrane<D>(a, row, cx, x0, tap);
+            dec_membrane<D, MODE == SEG_DIRECT>(a, row, cx, x0, tap);
           }
           __syncwarp();
 #pragma unroll
@@ -1546,7 +1547,7 @@ __global__ void __launch_bounds__(STH, 2) k_dec(RowArgs a) {
       y[0] = cmul(make_float2(acc[0].x, -acc[0].y), w);
       y[1] = cmul(make_float2(acc[DROW / 256].x, -acc[DROW / 256].y), w);
     }
-    if (MODE != SEG_MEMBRANE && a.half) {
+    if (!seg_membrane(MODE) && a.half) {
       // outputs x and -x meet in the transpose buffer that the transform's last pass does not read
       if (t < a.M) {
         b0[t] = y[0];
@@ -1559,7 +1560,7 @@ __global__ void __launch_bounds__(STH, 2) k_dec(RowArgs a) {
         y[1] = cadd(b0[256 + hm + t], b0[256 + hm - 1 - t]);
       }
     }
-    if (t < (MODE != SEG_MEMBRANE && a.half ? a.M / 2 : a.M)) {
+    if (t < (!seg_membrane(MODE) && a.half ? a.M / 2 : a.M)) {
 #pragma unroll
       for (int e = 0; e < 2; ++e)
         if (2 * p + e < a.rows) {
@@ -1716,6 +1717,7 @@ static void (*dec_kernel(int mode, int D))(RowArgs) {
   switch (mode) {
     case SEG_FLAT: return D == 32 ? k_dec<SEG_FLAT, 32> : k_dec<SEG_FLAT, 16>;
     case SEG_LEVELS: return D == 32 ? k_dec<SEG_LEVELS, 32> : k_dec<SEG_LEVELS, 16>;
+    case SEG_DIRECT: return D == 32 ? k_dec<SEG_DIRECT, 32> : k_dec<SEG_DIRECT, 16>;
     default: return D == 32 ? k_dec<SEG_MEMBRANE, 32> : k_dec<SEG_MEMBRANE, 16>;
   }
 }
@@ -1811,12 +1813,14 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
     out->Z = 0;
     out->G = 0;
     out->X = (size_t)P.nd.ns * P.M * sizeof(double2);
-    static std::atomic<uint64_t> attr_segt{0}, attr_seg[4];
-    const void* kern[4] = {(const void*)k_seg<SEG_FLAT>, (const void*)k_seg<SEG_LEVELS>,
-                           (const void*)k_seg<SEG_MEMBRANE>, (const void*)k_seg<SEG_GENERAL>};
-    for (int q = 0; q < 4; ++q) FZP_CUDA_TRY(smem_attr_once(kern[q], (int)SEG_SMEM, attr_seg[q]));
-    static std::atomic<uint64_t> attr_dec[6];
-    for (int q = 0; q < 6; ++q) FZP_CUDA_TRY(smem_attr_once((const void*)dec_kernel(q / 2, q % 2 ? 32 : 16), (int)DEC_SMEM, attr_dec[q]));
+    static std::atomic<uint64_t> attr_segt{0}, attr_seg[5];
+    const void* kern[5] = {(const void*)k_seg<SEG_FLAT>, (const void*)k_seg<SEG_LEVELS>, (const void*)k_seg<SEG_MEMBRANE>,
+                           (const void*)k_seg<SEG_GENERAL>, (const void*)k_seg<SEG_DIRECT>};
+    for (int q = 0; q < 5; ++q) FZP_CUDA_TRY(smem_attr_once(kern[q], (int)SEG_SMEM, attr_seg[q]));
+    static std::atomic<uint64_t> attr_dec[8];
+    const int modes[4] = {SEG_FLAT, SEG_LEVELS, SEG_MEMBRANE, SEG_DIRECT};
+    for (int q = 0; q < 8; ++q)
+      FZP_CUDA_TRY(smem_attr_once((const void*)dec_kernel(modes[q / 2], q % 2 ? 32 : 16), (int)DEC_SMEM, attr_dec[q]));
     FZP_CUDA_TRY(smem_attr_once((const void*)k_seg_tables, (int)SEG_SMEM, attr_segt));
     return FZP_OK;
   }
@@ -1921,11 +1925,13 @@ fzp_status rows_t(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t s
   if (b.seg) {
     // resident CTAs only: each takes every gridDim.x-th row of the range
     int ctas_per_sm = 0;
-    const int mode = P.has_deform ? (P.levels >= 2 ? SEG_GENERAL : SEG_MEMBRANE) : (P.levels >= 2 ? SEG_LEVELS : SEG_FLAT);
+    const int mode = P.has_deform ? (P.levels >= 2 ? SEG_GENERAL : a.df.direct ? SEG_DIRECT : SEG_MEMBRANE)
+                                  : (P.levels >= 2 ? SEG_LEVELS : SEG_FLAT);
     a.octant = octant ? 1 : 0;
     void (*kern)(RowArgs) = mode == SEG_FLAT       ? k_seg<SEG_FLAT>
                             : mode == SEG_LEVELS   ? k_seg<SEG_LEVELS>
                             : mode == SEG_MEMBRANE ? k_seg<SEG_MEMBRANE>
+                            : mode == SEG_DIRECT   ? k_seg<SEG_DIRECT>
                                                    : k_seg<SEG_GENERAL>;
     const size_t smem = b.dec ? DEC_SMEM : SEG_SMEM;
     if (b.dec) kern = dec_kernel(mode, b.dec);

@@ -36,13 +36,13 @@ def env():
 @pytest.mark.parametrize("width", [1, 2, 5, 8, 12, 40, 63.5, 64.5])
 def test_ridge_widths(env, form, N, cluster, width):
     fzp, torch = env
-    D = (N - 0.5) * DX
+    D, M = (N - 0.5) * DX, 64 if form == "fp32" else 128
     ridges = [(3e-5, -2e-5, math.pi / 2, 6e-8, width * DX), (-4e-5, 1e-5, 0.4, 5e-8, width * DX), (0.0, 6e-5, 0.02, 4e-8, width * DX)]
-    geom = dict(D=D, f=5 * D, lam=LAM, M=128, pitch=LAM * 5 / 8, N=N,
+    geom = dict(D=D, f=5 * D, lam=LAM, M=M, pitch=LAM * 5 / 8, N=N,
                 deform=fzp.make_deform(amp=1.2e-7, period=1.1e-3, theta=0.7, taper=0.4, ridges=ridges))
     how = dict(form=fzp.FORM_BLUESTEIN, precision=fzp.PREC_FP32) if form == "fp32" else \
         dict(form=fzp.FORM_DENSE, precision=fzp.PREC_SPLIT_BF16, cluster=cluster)
     with fzp.Plan(**geom, **how) as plan, fzp.Plan(form=fzp.FORM_BLUESTEIN, precision=fzp.PREC_FP64, **geom) as exact:
-        U, _ = run_plan(fzp, torch, plan, 128, 0, N)
-        R, _ = run_plan(fzp, torch, exact, 128, 0, N)
+        U, _ = run_plan(fzp, torch, plan, M, 0, N)
+        R, _ = run_plan(fzp, torch, exact, M, 0, N)
     assert rel_l2(U, R) <= (1e-5 if form == "fp32" else 3e-5)
