@@ -14,6 +14,7 @@
 #include <cmath>
 
 #include "fzp_internal.cuh"
+#include "sums.cuh"
 #include "tc_ptx.cuh"
 
 namespace fzp {
@@ -118,12 +119,14 @@ __device__ __forceinline__ double2 peer_load(uint32_t addr, double2) {
 // grid (M/TM, M/TN, ceil(rows/jc)); 256 threads; each thread 4 n x 4 m outputs.
 // TAB: the kernel's columns from a table E [n][estride] instead of their phase.
 // The blocks' sums meet in Uacc: in clusters of CZ along the rows, block k adds up
-// its part of the tile over the cluster through distributed shared memory first.
+// its part of the tile over the cluster through distributed shared memory first
+// (sum4: with what the FP32 additions round off, as if in FP64).
 // Without that, 304 blocks put FP64 atomics on the same 8,192 values.  The next
 // tile of C1 loads during the products.  18,965 rows, 64 x 64 nodes: 56 us without
 // clusters and prefetch and with two sine pairs per folded kernel value, 49 with
 // clusters of eight and prefetch, 33 with clusters of four and one cosine (issue
-// slots 28 -> 35 % busy; the waits left are loads and the barriers of 16-row tiles).
+// slots 28 -> 35 % busy; the waits left are loads and the barriers of 16-row tiles),
+// 35 with sum4 in place of FP32 additions.
 // FP64, 2,529 rows, 129 x 129 outputs, bound by the FP64 pipe: 0.46 ms, with the
 // tiles on and above the diagonal only a propagation takes 0.09 ms less.
 template <typename R, bool TAB = false, int NA = 4>
@@ -263,9 +266,8 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     }
     __syncthreads();
   }
-  auto add = [&](int n, int m, C v) {
+  auto add = [&](int n, int m, double ux, double uy) {
     if (n >= g.ny || m >= g.M) return;
-    double ux = (double)v.x, uy = (double)v.y;
     if (g.wi != 0.0 || g.wr != 1.0) {
       const double t = g.wr * ux - g.wi * uy;
       uy = g.wr * uy + g.wi * ux;
@@ -287,14 +289,14 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     for (int q = 0; q < CZ; ++q) peer[q] = tc::mapa(tc::smem_u32(pool), q);
     constexpr int PART = TN * TM / CZ;
     for (int e = (int)rank * PART + tid; e < ((int)rank + 1) * PART; e += 256) {
-      C v[CZ];
+      R x[CZ], y[CZ];
 #pragma unroll
-      for (int q = 0; q < CZ; ++q) v[q] = peer_load(peer[q] + (uint32_t)(e * sizeof(C)), C{});
-#pragma unroll
-      for (int w = CZ / 2; w > 0; w /= 2)
-#pragma unroll
-        for (int q = 0; q < w; ++q) v[q] = cadd(v[q], v[q + w]);
-      add(n0 + e / TM, m0 + e % TM, v[0]);
+      for (int q = 0; q < CZ; ++q) {
+        const C v = peer_load(peer[q] + (uint32_t)(e * sizeof(C)), C{});
+        x[q] = v.x;
+        y[q] = v.y;
+      }
+      add(n0 + e / TM, m0 + e % TM, sum4(x), sum4(y));
     }
     tc::cluster_sync();  // the peers may still be reading this block's tile
     return;
@@ -302,7 +304,7 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
 #pragma unroll
   for (int a = 0; a < NA; ++a)
 #pragma unroll
-    for (int b = 0; b < NA; ++b) add(n0 + tn + 16 * a, m0 + tm + 16 * b, acc[a][b]);
+    for (int b = 0; b < NA; ++b) add(n0 + tn + 16 * a, m0 + tm + 16 * b, (double)acc[a][b].x, (double)acc[a][b].y);
 }
 
 template <typename R, bool TAB = false, int NA = 4>
