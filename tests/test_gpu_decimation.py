@@ -86,3 +86,20 @@ def test_smallest_grids(env, N, shift):
                     assert abs(U).max() == 0, (a, b)
                 else:
                     assert rel_l2(U, R) <= TOL, (D, a, b)
+
+
+def test_chirp_at_the_largest_grids(env):
+    """N = 16,000,241 (its chirp rate has 0.996 of a unit below 2^-64 turns per
+    squared column): three rows about the axis.  Left out, that part would turn the
+    rim by 2e-5 rad and move the row's field by a third of it.  Tolerance: sine and
+    cosine 4e-7, three tables 6e-8 each, interpolation 1.2e-7, 24 butterfly stages
+    of 3e-8 each: 1.4e-6, so 2e-6."""
+    fzp, torch = env
+    N = 16000241
+    D = (N - 0.5) * LAM * 5 / 4
+    geom = dict(D=D, f=5 * D, lam=LAM, M=64, pitch=LAM * 5 / 8, N=N, stripe_rows=256, form=fzp.FORM_BLUESTEIN)
+    c = N // 2
+    with fzp.Plan(precision=fzp.PREC_FP32, **geom) as plan, fzp.Plan(precision=fzp.PREC_FP64, **geom) as exact:
+        U, _ = run_plan(fzp, torch, plan, 64, c - 1, c + 2)
+        R, _ = run_plan(fzp, torch, exact, 64, c - 1, c + 2)
+    assert rel_l2(U, R) <= 2e-6
