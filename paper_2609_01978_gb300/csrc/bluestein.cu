@@ -1794,9 +1794,11 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
   b.L2 = b.L < Traits<R>::L2MAX ? b.L : Traits<R>::L2MAX;
   b.L1 = b.L / b.L2;
   if (P.M > b.L2) return set_error(FZP_E_UNSUPPORTED, "M larger than the inner FFT length");
-  // the F1 twiddles are read from the L2-entry table with stride L2 / L1
-  if (b.L1 > b.L2) return set_error(FZP_E_UNSUPPORTED, "FFT length %lld above %lld", (long long)b.L,
-                                    (long long)b.L2 * b.L2);
+  // the F1 twiddles are read from the L2-entry table with stride L2 / L1 (a plan
+  // that runs half the length is held to the same limit as fzp_plan_query)
+  const int64_t L2_full = std::min<int64_t>(b.L_full, Traits<R>::L2MAX);
+  if (b.L1 > b.L2 || b.L_full > L2_full * L2_full)
+    return set_error(FZP_E_UNSUPPORTED, "FFT length %lld above %lld", (long long)b.L_full, (long long)L2_full * L2_full);
   if (b.seg) {
     // partitioned convolution: S + M - 1 <= 4096, S a multiple of 256 (at most 15 x 256)
     const int M = P.nd.n > 0 ? P.nd.n : P.M;  // outputs per row: the nodes, or the ROI samples
