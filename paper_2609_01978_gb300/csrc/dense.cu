@@ -1158,24 +1158,35 @@ fzp_status c1_tensor_map(const Plan& P, CUtensorMap* tm) {
 
 namespace {
 
-// Layout of the dense form's tables for a kernel matrix of `ncols` columns.
+// What every dense plan has: the ROI's tiles, the cluster size (CTAs sharing each
+// stripe's mask; default: the largest of 4, 2, 1 that divides the tile pairs),
+// the promotion and the GPU's SMs, a CTA each.  Returns the tile pairs holding
+// ROI rows.
+fzp_status layout_common(Plan& P, int* used) {
+  Dense& d = P.dn;
+  d.ntiles = 2 * P.M / BM;
+  *used = (d.ntiles + TILES - 1) / TILES;
+  d.cluster = P.cluster_req > 0 ? P.cluster_req : (*used % 4 == 0 ? 4 : *used % 2 == 0 ? 2 : 1);
+  d.promote_kblocks = P.promote_req > 0 ? P.promote_req : 128;  // 4096 samples per TMEM chunk
+  int dev = 0;
+  FZP_CUDA_TRY(cudaGetDevice(&dev));
+  FZP_CUDA_TRY(cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev));
+  d.max_ctas = d.num_sms;
+  return FZP_OK;
+}
+
+// Layout of k_dense's tables for a kernel matrix of `ncols` columns.
 fzp_status layout_cols(Plan& P, int64_t ncols, FormSizes* out) {
   Dense& d = P.dn;
+  int used = 0;
+  const fzp_status st = layout_common(P, &used);
+  if (st != FZP_OK) return st;
   d.kblocks = (ncols + BK - 1) / BK;
-  d.ntiles = 2 * P.M / BM;
-  const int used = (d.ntiles + TILES - 1) / TILES;  // tile pairs holding ROI rows
-  // cluster: CTAs sharing each stripe's mask (default: the largest of 4, 2, 1
-  // that divides the pairs); pairs padded with zero tiles to a multiple of it
-  d.cluster = P.cluster_req > 0 ? P.cluster_req : (used % 4 == 0 ? 4 : used % 2 == 0 ? 2 : 1);
-  d.npairs = (used + d.cluster - 1) / d.cluster * d.cluster;
-  d.promote_kblocks = P.promote_req > 0 ? P.promote_req : 128;  // 4096 samples per TMEM chunk
+  d.npairs = (used + d.cluster - 1) / d.cluster * d.cluster;  // padded with zero tiles
   // one promotion per unit: units of several promotions of one stripe
   // (measured with 4) kept C1's DRAM writes the same and, the clusters of a
   // wave drifting apart along K, read the kernel matrix 2.7 times as often
   d.group_kblocks = d.promote_kblocks;
-  int dev = 0;
-  FZP_CUDA_TRY(cudaGetDevice(&dev));
-  FZP_CUDA_TRY(cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev));
   out->A = (size_t)d.npairs * (size_t)d.kblocks * A_BYTES;
   out->sched = sizeof(int) * (size_t)(3 * ((d.kblocks + d.group_kblocks - 1) / d.group_kblocks) + 1);
   static std::atomic<uint64_t> attr1{0}, attr2{0}, attr4{0}, attr1c{0}, attr2c{0}, attr4c{0}, attr1l{0},
@@ -1191,7 +1202,6 @@ fzp_status layout_cols(Plan& P, int64_t ncols, FormSizes* out) {
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<4, true, true>, (int)dense_smem_bytes(), attr4l));
   // The kernel is persistent: launch only CTAs that are resident at once.  A
   // cluster must fit in one GPC, so with clusters fewer than all SMs may hold one.
-  d.max_ctas = d.num_sms;
   if (d.cluster > 1) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(d.num_sms / d.cluster * d.cluster));
@@ -1354,8 +1364,11 @@ fzp_status run_dense(Plan& P, DenseArgs& a, int mode, const char* name, cudaStre
 }  // namespace
 
 fzp_status dense_layout(Plan& P, FormSizes* out) {
-  const fzp_status st = layout_cols(P, P.N, out);
-  return st == FZP_OK && P.nd.n > 0 ? nodes_layout(P, out) : st;
+  if (P.nd.n == 0) return layout_cols(P, P.N, out);
+  // k_nodes: single CTAs on every SM, none of k_dense's attributes or clusters
+  int used = 0;
+  const fzp_status st = layout_common(P, &used);
+  return st == FZP_OK ? nodes_layout(P, out) : st;
 }
 
 fzp_status dense_fill_tables(Plan& P, cudaStream_t s) {
