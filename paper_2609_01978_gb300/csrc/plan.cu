@@ -437,7 +437,7 @@ fzp_status fzp_plan(const fzp_params* params, fzp_plan_t* out) {
     if (e == cudaSuccess) e = cudaMalloc(&P->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&P->d_metrics, 8192 * sizeof(double) + (size_t)P->M * P->M * sizeof(double2));
     if (e == cudaSuccess) e = cudaMemset(P->d_err, 0, sizeof(int));
-    P->device_bytes += (size_t)P->M * P->M * sizeof(double2) * 2 + 8192 * sizeof(double) + sizeof(int);
+    P->device_bytes += (nacc + (size_t)P->M * P->M) * sizeof(double2) + 8192 * sizeof(double) + sizeof(int);
     if (e != cudaSuccess) {
       st = set_error(e == cudaErrorMemoryAllocation ? FZP_E_OOM : FZP_E_CUDA, "workspace allocation: %s",
                      cudaGetErrorString(e));
