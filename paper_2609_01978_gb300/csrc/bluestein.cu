@@ -2015,7 +2015,9 @@ fzp_status bluestein_fill_tables(Plan& P, cudaStream_t s) {
 
 fzp_status bluestein_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream_t stream) {
   P.dominant = P.precision == FZP_PREC_FP64 ? "bluestein_f2<double>"
-                                             : (P.bs.seg ? "k_seg (partitioned convolution)" : "bluestein_f2<float>");
+               : P.bs.dec                       ? "k_dec (partitioned convolution, decimated rows)"
+               : P.bs.seg                       ? "k_seg (partitioned convolution)"
+                                                : "bluestein_f2<float>";
   return P.precision == FZP_PREC_FP64 ? rows_t<double>(P, j0, rows, false, stream) : rows_t<float>(P, j0, rows, octant, stream);
 }
 

@@ -1,5 +1,5 @@
-"""What a plan reports about itself is what it runs: CTAs, device memory, the name
-of the dominant kernel."""
+"""What a plan reports about itself is what it runs: CTAs and the name of the
+dominant kernel."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -30,3 +30,13 @@ def test_ctas(env, M, scale, nodes):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     with fzp.Plan(form=fzp.FORM_DENSE, precision=fzp.PREC_SPLIT_BF16, **_geom(1501, M, scale)) as plan:
         assert plan.info["ctas"] == sms if nodes else plan.info["ctas"] % 4 == 0
+
+
+@pytest.mark.parametrize("N,kw,name", [(1501, {}, "k_seg"), (5831, {}, "k_dec"), (5831, dict(conv=1), "bluestein_f2<float>")])
+def test_dominant_kernel_of_the_fp32_form(env, N, kw, name):
+    fzp, torch = env
+    with fzp.Plan(form=fzp.FORM_BLUESTEIN, precision=fzp.PREC_FP32, **_geom(N, 64), **kw) as plan:
+        plan.profile(True)
+        plan.propagate_roi(0, 8, torch.empty((64, 64), dtype=torch.complex128, device="cuda"))
+        plan.propagate_roi(N // 2, N // 2 + 2, torch.empty((64, 64), dtype=torch.complex128, device="cuda"))
+        assert plan.profile_read()["dominant_name"].startswith(name)
