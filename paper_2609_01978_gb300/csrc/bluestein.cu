@@ -1915,8 +1915,9 @@ fzp_status build_tables_t(Plan& P) {
   if (P.nd.n > 0) {
     FZP_CUDA_TRY(cudaMalloc(&P.nd.d_X, z.X));
     P.device_bytes += z.X;
-    st = nodes_upload(P);
-    if (st != FZP_OK) return st;
+    // the tables are built while the host factors the interpolation
+    st = fill_tables_t<R>(P, 0);
+    return st == FZP_OK ? nodes_upload(P) : st;
   }
   return fill_tables_t<R>(P, 0);
 }

@@ -1418,8 +1418,9 @@ fzp_status dense_build_tables(Plan& P) {
   if (P.nd.n > 0) {
     FZP_CUDA_TRY(cudaMalloc(&P.nd.d_X, z.X));
     P.device_bytes += z.X;
-    st = nodes_upload(P);
-    if (st != FZP_OK) return st;
+    // the kernel images are built while the host factors the interpolation
+    st = dense_fill_tables(P, 0);
+    return st == FZP_OK ? nodes_upload(P) : st;
   } else if (P.dn.extra_ctas > 0) {
     FZP_CUDA_TRY(cudaMalloc(&P.dn.d_sched2, z.sched));
     FZP_CUDA_TRY(cudaStreamCreateWithFlags(&P.dn.s2, cudaStreamNonBlocking));

@@ -59,6 +59,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <memory>
+#include <new>
 #include <vector>
 
 #include "fzp_internal.cuh"
@@ -900,60 +902,109 @@ __global__ void k_nodes_table(int nt, int64_t ncols, int64_t kblocks, const floa
 // into small blocks over the whole GPU and the chirp is applied per axis.
 __device__ __forceinline__ double sinc_d(double z) { return fabs(z) < 1e-9 ? 1.0 : sin(z) / z; }
 
-// W from the Cholesky factors of the node matrix (host): a block per four
-// outputs, a thread per (output, node), both triangular solves with the
-// unknowns in registers.  F: per parity the factor by columns, then by rows
-// (ns x ns each), reciprocals on the diagonal.
+// W from the Cholesky factors of the node matrix (host): a block per output, a
+// warp per parity, both triangular solves with U = ns / 32 unknowns per lane in
+// registers and the pivots by shuffles, the factor's columns loaded eight steps
+// ahead.  A chain of 2 ns steps bounds it: 26 us for 64 nodes (70 with a block of
+// four outputs, a barrier per step and one parity after the other; the 2 mm plan
+// 309 -> 233 us with that, a faster factorisation and the tables built meanwhile).  F: per parity the factor by columns, then by rows (ns x ns each),
+// reciprocals on the diagonal.
 struct InterpSpec {
   int n, ns, M, Mo, even;
   double h, c, half;  // node pitch and band (radians) per ROI half width; half width in pitches
   double msh, chirp;  // ROI shift; p^2 / (2 lambda f)
 };
 
-__global__ void __launch_bounds__(512) k_interp_W(const InterpSpec a, const double* __restrict__ F, double* __restrict__ W,
-                                                  double* __restrict__ Wy, double2* __restrict__ chirp) {
+template <int U>
+__global__ void __launch_bounds__(64) k_interp_W(const InterpSpec a, const double* __restrict__ F, double* __restrict__ W,
+                                                 double* __restrict__ Wy, double2* __restrict__ chirp) {
+  constexpr int ns = 32 * U;
+  __shared__ double w[2][ns];
+  const int lane = threadIdx.x & 31, side = threadIdx.x >> 5, o = blockIdx.x;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.M; i += gridDim.x * blockDim.x) {
     const double t = (double)i - a.msh;
     chirp[i] = cis_turns_d(t * t * a.chirp);
   }
-  __shared__ double pivot[2][4];
-  const int ns = a.ns, r = threadIdx.x % ns, q = threadIdx.x / ns, o = blockIdx.x * 4 + q;
   const double xo = (a.even ? (double)o : (double)o - 0.5 * (a.M - 1)) / a.half;
-  const double x = ((double)(a.even ? r + ns : r) - 0.5 * (a.n - 1)) * a.h;
-  const double sm = sinc_d(a.c * (xo - x)), sp = a.even ? sinc_d(a.c * (xo + x)) : 0.0;
-  double w[2] = {0.0, 0.0};
-  for (int side = 0; side < (a.even && Wy ? 2 : 1); ++side) {
-    const double* C = F + (size_t)side * 2 * ns * ns;  // by columns, behind it by rows
-    const double* R = C + (size_t)ns * ns;
-    const double inv = C[r * ns + r];
-    double v = side ? sm - sp : sm + sp;
-    for (int k = 0; k < ns; ++k) {
-      if (r == k) pivot[k & 1][q] = v = v * inv;
-      __syncthreads();
-      if (r > k) v = fma(-C[k * ns + r], pivot[k & 1][q], v);
-    }
-    __syncthreads();
-    for (int k = ns - 1; k >= 0; --k) {
-      if (r == k) pivot[k & 1][q] = v = v * inv;
-      __syncthreads();
-      if (r < k) v = fma(-R[k * ns + r], pivot[k & 1][q], v);
-    }
-    __syncthreads();
-    w[side] = v;
+  const double* C = F + (size_t)side * 2 * ns * ns;  // by columns, behind it by rows
+  const double* R = C + (size_t)ns * ns;
+  double v[U], inv[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int r = lane + 32 * u;
+    const double x = ((double)(a.even ? r + ns : r) - 0.5 * (a.n - 1)) * a.h;
+    const double sm = sinc_d(a.c * (xo - x)), sp = a.even ? sinc_d(a.c * (xo + x)) : 0.0;
+    v[u] = side ? sm - sp : sm + sp;
+    inv[u] = C[r * ns + r];
   }
-  if (o >= a.Mo) return;
-  W[(size_t)r * a.Mo + o] = w[0];
-  if (a.even && Wy) {
-    // the matrix of all nodes: w(+-x_k) = (even +- odd) / 2, at x_o and mirrored at -x_o
-    const int hm = a.M / 2, kp = ns + r, km = ns - 1 - r;
-    const double same = 0.5 * (w[0] + w[1]), other = 0.5 * (w[0] - w[1]);
-    if (o < hm) {
-      Wy[(size_t)kp * a.M + hm + o] = same;
-      Wy[(size_t)km * a.M + hm + o] = other;
+  // columns of the factor eight steps ahead of the pivots
+  constexpr int G = 8;
+  double next[G][U];
+  auto load = [&](const double* T, int k0, int dir) {
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int u = 0; u < U; ++u) next[g][u] = T[(k0 + dir * g) * ns + lane + 32 * u];
+  };
+  load(C, 0, 1);
+#pragma unroll
+  for (int kb = 0; kb < U; ++kb)
+#pragma unroll 1
+    for (int k0 = 0; k0 < 32; k0 += G) {
+      double c[G][U];
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int u = 0; u < U; ++u) c[g][u] = next[g][u];
+      const int k1 = 32 * kb + k0 + G;
+      if (k1 < ns) load(C, k1, 1);
+      else load(R, ns - 1, -1);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const double pivot = __shfl_sync(0xffffffffu, v[kb] * inv[kb], k0 + g);
+        if (lane == k0 + g) v[kb] = pivot;
+        if (lane > k0 + g) v[kb] = fma(-c[g][kb], pivot, v[kb]);
+#pragma unroll
+        for (int u = kb + 1; u < U; ++u) v[u] = fma(-c[g][u], pivot, v[u]);
+      }
     }
-    if (o > 0) {
-      Wy[(size_t)kp * a.M + hm - o] = other;
-      Wy[(size_t)km * a.M + hm - o] = same;
+#pragma unroll
+  for (int kb = U - 1; kb >= 0; --kb)
+#pragma unroll 1
+    for (int k0 = 31; k0 >= 0; k0 -= G) {
+      double c[G][U];
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int u = 0; u < U; ++u) c[g][u] = next[g][u];
+      const int k1 = 32 * kb + k0 - G;
+      if (k1 >= 0) load(R, k1, -1);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const double pivot = __shfl_sync(0xffffffffu, v[kb] * inv[kb], k0 - g);
+        if (lane == k0 - g) v[kb] = pivot;
+        if (lane < k0 - g) v[kb] = fma(-c[g][kb], pivot, v[kb]);
+#pragma unroll
+        for (int u = 0; u < kb; ++u) v[u] = fma(-c[g][u], pivot, v[u]);
+      }
+    }
+#pragma unroll
+  for (int u = 0; u < U; ++u) w[side][lane + 32 * u] = v[u];
+  __syncthreads();
+  for (int r = threadIdx.x; r < ns; r += blockDim.x) {
+    W[(size_t)r * a.Mo + o] = w[0][r];
+    if (a.even && Wy) {
+      // the matrix of all nodes: w(+-x_k) = (even +- odd) / 2, at x_o and mirrored at -x_o
+      const int hm = a.M / 2, kp = ns + r, km = ns - 1 - r;
+      const double same = 0.5 * (w[0][r] + w[1][r]), other = 0.5 * (w[0][r] - w[1][r]);
+      if (o < hm) {
+        Wy[(size_t)kp * a.M + hm + o] = same;
+        Wy[(size_t)km * a.M + hm + o] = other;
+      }
+      if (o > 0) {
+        Wy[(size_t)kp * a.M + hm - o] = other;
+        Wy[(size_t)km * a.M + hm - o] = same;
+      }
     }
   }
 }
@@ -1169,7 +1220,7 @@ int mask_kind(const Plan& P) {
 // (radians): the normal equations of the least-squares interpolation.
 // parity +1 / -1: of even / odd functions, over the nodes x > 0.
 void node_factor(int n, int ns, int parity, double h, double c, double* T) {
-  std::vector<double> dist(n);
+  double dist[256];  // n <= 256
   for (int q = 0; q < n; ++q) {
     const double z = c * q * h;
     dist[q] = q ? std::sin(z) / z : 1.0;
@@ -1177,16 +1228,23 @@ void node_factor(int n, int ns, int parity, double h, double c, double* T) {
   for (int l = 0; l < ns; ++l)
     for (int k = l; k < ns; ++k)  // x_k + x_l = (k + l + 1) h on the half grid
       T[(size_t)l * ns + k] = dist[k - l] + (parity ? parity * dist[k + l + 1] : 0.0) + (k == l ? 1e-13 : 0.0);
-  for (int l = 0; l < ns; ++l) {
-    double* __restrict__ cl = &T[(size_t)l * ns];
-    const double r = 1.0 / std::sqrt(std::max(cl[l], 1e-15));
-    for (int k = l + 1; k < ns; ++k) cl[k] *= r;
-    for (int q = l + 1; q < ns; ++q) {
-      double* __restrict__ cq = &T[(size_t)q * ns];
-      const double f = cl[q];
-      for (int k = q; k < ns; ++k) cq[k] -= f * cl[k];
+  // column by column from those before it, four at a time (one store per four products)
+  for (int q = 0; q < ns; ++q) {
+    double* __restrict__ cq = &T[(size_t)q * ns];
+    int l = 0;
+    for (; l + 4 <= q; l += 4) {
+      const double *c0 = &T[(size_t)l * ns], *c1 = c0 + ns, *c2 = c1 + ns, *c3 = c2 + ns;
+      const double f0 = c0[q], f1 = c1[q], f2 = c2[q], f3 = c3[q];
+      for (int k = q; k < ns; ++k) cq[k] = (((cq[k] - f0 * c0[k]) - f1 * c1[k]) - f2 * c2[k]) - f3 * c3[k];
     }
-    cl[l] = r;
+    for (; l < q; ++l) {
+      const double* c0 = &T[(size_t)l * ns];
+      const double f0 = c0[q];
+      for (int k = q; k < ns; ++k) cq[k] -= f0 * c0[k];
+    }
+    const double r = 1.0 / std::sqrt(std::max(cq[q], 1e-15));
+    for (int k = q + 1; k < ns; ++k) cq[k] *= r;
+    cq[q] = r;
   }
   double* L = T + (size_t)ns * ns;
   for (int k = 0; k < ns; ++k)
@@ -1321,12 +1379,15 @@ fzp_status nodes_upload(Plan& P) {
   z.d_Wy = full ? z.d_W + nw : z.d_W;
   double* dL = z.d_W + (total - nf);
   z.d_chirp = reinterpret_cast<double2*>(dL - 2 * (size_t)P.M);  // 16-byte aligned: even counts throughout
-  std::vector<double> L(nf);
+  std::unique_ptr<double[]> L(new (std::nothrow) double[nf]);
+  if (!L) return set_error(FZP_E_OOM, "host allocation failed");
   InterpSpec a{z.n, z.ns, P.M, z.Mo, z.even ? 1 : 0, z.h / z.half, M_PI * z.band * z.half, z.half, P.msh, P.p * P.p / (2.0 * P.lambda * z.dist)};
-  node_factor(z.n, z.ns, z.even ? 1 : 0, a.h, a.c, L.data());
-  if (full) node_factor(z.n, z.ns, -1, a.h, a.c, L.data() + (size_t)2 * z.ns * z.ns);
-  FZP_CUDA_TRY(cudaMemcpy(dL, L.data(), nf * sizeof(double), cudaMemcpyHostToDevice));
-  k_interp_W<<<(unsigned)((z.Mo + 3) / 4), 4 * z.ns>>>(a, dL, z.d_W, full ? z.d_Wy : nullptr, z.d_chirp);
+  node_factor(z.n, z.ns, z.even ? 1 : 0, a.h, a.c, L.get());
+  if (full) node_factor(z.n, z.ns, -1, a.h, a.c, L.get() + (size_t)2 * z.ns * z.ns);
+  FZP_CUDA_TRY(cudaMemcpy(dL, L.get(), nf * sizeof(double), cudaMemcpyHostToDevice));
+  double* Wy = full ? z.d_Wy : nullptr;
+  if (z.ns == 64) k_interp_W<2><<<(unsigned)z.Mo, full ? 64 : 32>>>(a, dL, z.d_W, Wy, z.d_chirp);
+  else k_interp_W<4><<<(unsigned)z.Mo, full ? 64 : 32>>>(a, dL, z.d_W, Wy, z.d_chirp);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
