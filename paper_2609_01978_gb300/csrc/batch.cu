@@ -9,7 +9,9 @@
 // transmission) are dense candidates as binary amplitude plates (two membrane
 // passes); odd-level phase plates and deformed phase plates have the
 // Bluestein form only.  Results are cached
-// per (N, M, deformed, levels, centre configuration, requested convolution)
+// per (N, M, deformed, levels, centre configuration, requested convolution, and
+// the routes that the ROI's pitch and place and the membrane open: the two forms'
+// nodes, an even field, decimated rows, columns evaluated one by one)
 // for the process and, when FZP_TUNE_CACHE names a file, in that file (one
 // "key value..." line per problem).
 //
@@ -52,11 +54,17 @@ std::map<std::string, Choice> g_tune;
 bool g_tune_loaded = false;
 
 // The request's Bluestein convolution is part of the key: a choice measured
-// with the partitioned convolution does not hold for the single one.
-std::string tune_key(int64_t N, int M, bool deformed, int levels, int centre_open, int conv) {
-  char buf[112];
-  snprintf(buf, sizeof(buf), "N=%lld,M=%d,deformed=%d,levels=%d,centre_open=%d,conv=%d", (long long)N, M,
-           deformed ? 1 : 0, levels, centre_open, conv);
+// with the partitioned convolution does not hold for the single one.  So are the
+// routes that decide what the candidates cost: ROIs of one size that differ in
+// pitch or place do not share a choice (nor do entries of a cache file written
+// before the routes were in it).  geo: the request as an FP32 plan; dense_nodes: the
+// nodes of its dense plan.
+std::string tune_key(const Plan& geo, int dense_nodes, int conv) {
+  char buf[160];
+  snprintf(buf, sizeof(buf), "N=%lld,M=%d,deformed=%d,levels=%d,centre_open=%d,conv=%d,nodes=%d/%d,even=%d,dec=%d,direct=%d",
+           (long long)geo.N, geo.M, geo.has_deform ? 1 : 0, geo.levels, geo.mg.centre_open, conv, dense_nodes, geo.nd.n,
+           geo.msh == (double)(geo.M / 2) ? 1 : 0, bluestein_decimation(geo),
+           geo.has_deform ? deform_coef(geo).direct : 0);
   return buf;
 }
 
@@ -67,9 +75,9 @@ void tune_load() {
   if (!path) return;
   FILE* fh = fopen(path, "r");
   if (!fh) return;
-  char key[96];
+  char key[160];
   Choice c;
-  while (fscanf(fh, "%95s %d %d %d %d %d %lf", key, &c.form, &c.precision, &c.promote, &c.row_batch, &c.cluster,
+  while (fscanf(fh, "%159s %d %d %d %d %d %lf", key, &c.form, &c.precision, &c.promote, &c.row_batch, &c.cluster,
                 &c.ms_probe) == 7)
     g_tune[key] = c;
   fclose(fh);
@@ -106,13 +114,14 @@ static fzp_plan_t probe_candidate(const fzp_params& base, const Choice& c, doubl
   fzp_plan_info_get(plan, &info);
   // probe stripe: enough rows for two full waves of dense work items (one item =
   // 256 rows x one pair of 128-row kernel tiles) so that neither form is timed
-  // on an under-filled GPU; centred rows carry the most zone boundaries
+  // on an under-filled GPU; centred rows carry the most zone boundaries, and as
+  // many on either side of the axis so that flat plates fold them
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t pairs = std::max<int64_t>(1, (2 * (int64_t)p.M / 128 + 1) / 2);
   const int64_t half = 128 * ((2 * sms + pairs - 1) / pairs);
-  const int64_t j0 = std::max<int64_t>(0, info.c - half), j1 = std::min<int64_t>(info.N, info.c + half);
+  const int64_t j0 = std::max<int64_t>(0, info.c - half), j1 = std::min<int64_t>(info.N, info.c + half + 1);
   float t = 0;
   if (ok) ok = fzp_propagate_roi(plan, j0, j1, field, 0, nullptr) == FZP_OK;  // warm
   if (ok) {
@@ -143,7 +152,16 @@ fzp_status autotune(const fzp_params* in, fzp_params* chosen, fzp_plan_t* keep) 
   fzp_status st = validate_and_derive(&probe, geo);
   if (st != FZP_OK) return st;
   const bool deformed = in->deform != nullptr;
-  const std::string key = tune_key(geo.N, geo.M, deformed, geo.levels, geo.mg.centre_open, in->conv);
+  int dense_nodes = 0;
+  {
+    Plan d;
+    fzp_params p = *in;
+    p.form = FZP_FORM_DENSE;
+    p.precision = FZP_PREC_SPLIT_BF16;
+    p.cluster = 0;
+    if (validate_and_derive(&p, d) == FZP_OK) dense_nodes = d.nd.n;
+  }
+  const std::string key = tune_key(geo, dense_nodes, in->conv);
   *chosen = *in;
   std::lock_guard<std::mutex> lock(g_tune_mu);
   tune_load();
@@ -162,9 +180,10 @@ fzp_status autotune(const fzp_params* in, fzp_params* chosen, fzp_plan_t* keep) 
   // amplitude plates (membrane passes with split mask values)
   if (!deformed && geo.levels % 2 == 0) {
     // cluster 0: the plan's own choice (4 CTAs for M = 512); 1: single-CTA kernel
+    // (on nodes both are the same single CTAs)
     cands.push_back({FZP_FORM_DENSE, FZP_PREC_SPLIT_BF16, 128, 0, 0, 0});
     cands.push_back({FZP_FORM_DENSE, FZP_PREC_SPLIT_BF16, 256, 0, 0, 0});
-    cands.push_back({FZP_FORM_DENSE, FZP_PREC_SPLIT_BF16, 128, 0, 1, 0});
+    if (dense_nodes == 0) cands.push_back({FZP_FORM_DENSE, FZP_PREC_SPLIT_BF16, 128, 0, 1, 0});
   } else if (deformed && geo.levels == 0) {
     // membrane passes are limited by their generators: single CTAs and 2- and
     // 4-CTA clusters (small ROIs padded) trade generator share per CTA against

@@ -1636,6 +1636,14 @@ static size_t f1_smem(const RowArgs& a) {
 
 }  // namespace
 
+// D u <= 0.17 keeps the interpolation's error below 1.2e-7 (3e-8 at the ROI's
+// edge); a deformed phase plate has its general per-sample transmission.
+int bluestein_decimation(const Plan& P) {
+  if (P.nd.n == 0 || (P.has_deform && P.levels >= 2)) return 0;
+  const double u = M_PI * P.nd.delta * (P.nd.n - 1);
+  return 32 * u <= 0.17 ? 32 : 16 * u <= 0.17 ? 16 : 0;
+}
+
 DeformCoef deform_coef(const Plan& P) {
   DeformCoef c{};
   const fzp_deform& d = P.deform;
@@ -1768,15 +1776,6 @@ static RowArgs make_args(const Plan& P) {
   return a;
 }
 
-// Columns to a grid point of the decimated rows, 0: none.  D u <= 0.17 keeps the
-// interpolation's error below 1.2e-7 (3e-8 at the ROI's edge); a deformed phase
-// plate has its general per-sample transmission.
-static int decimation(const Plan& P) {
-  if (P.nd.n == 0 || (P.has_deform && P.levels >= 2)) return 0;
-  const double u = M_PI * P.nd.delta * (P.nd.n - 1);
-  return 32 * u <= 0.17 ? 32 : 16 * u <= 0.17 ? 16 : 0;
-}
-
 template <typename R>
 fzp_status layout_t(Plan& P, FormSizes* out) {
   using C = typename Cplx<R>::T;
@@ -1804,7 +1803,7 @@ fzp_status layout_t(Plan& P, FormSizes* out) {
     const int M = P.nd.n > 0 ? P.nd.n : P.M;  // outputs per row: the nodes, or the ROI samples
     b.S = 256 * std::min(15, (4097 - M) / 256);
     b.nseg = (P.N - b.col0 + b.S - 1) / b.S;
-    b.dec = decimation(P);
+    b.dec = bluestein_decimation(P);
     if (b.dec) {
       decimation_weights(b.dec, b.T);
       // two rows to a transform: S + 5 + n < 2050, S a multiple of 32

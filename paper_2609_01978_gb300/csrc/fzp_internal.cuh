@@ -356,6 +356,9 @@ inline size_t c1_elems(const Plan& P) {
   return all;
 }
 
+// Columns to a grid point of the FP32 form's decimated rows (host), 0: none.
+int bluestein_decimation(const Plan& P);
+
 // FP32 deformation coefficients of a plan with a deformation (host).
 DeformCoef deform_coef(const Plan& P);
 

@@ -99,3 +99,20 @@ def test_autotune_picks_partitioned_fp32_for_sixteen_levels(env):
         j0 = g.c + int(g.R / g.dx / 3)
         _, I = run_plan(fzp, torch, plan, 256, j0, j0 + 64)
     assert rel_l2(I, np.abs(O.field_czt(g, j0, j0 + 64)) ** 2) <= 1e-4
+
+
+def test_tuned_choices_follow_the_pitch(env, tmp_path, monkeypatch):
+    """Two ROIs of one plate, M and conv whose pitches take different routes (nodes or
+    none; decimated rows or none) are tuned one by one; the same pitch is not."""
+    fzp, torch, O = env
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("FZP_TUNE_CACHE", str(cache))
+    lam, N = 632.8e-9, 6007
+    D = (N - 0.5) * lam * 5 / 4
+    kw = dict(D=D, f=5 * D, lam=lam, M=512, N=N, precision=fzp.PREC_AUTO_1E4)
+    keys = []
+    for pitch in (lam * 5 / 8, lam * 5 / 8, 4 * lam * 5 / 8):
+        fzp.Plan(pitch=pitch, **kw).close()
+        keys.append([line.split()[0] for line in cache.read_text().splitlines()])
+    assert len(keys[0]) == 1 and keys[1] == keys[0]
+    assert len(keys[2]) == 2 and keys[2][0] != keys[2][1]
