@@ -1992,10 +1992,39 @@ __global__ void k_mask(MaskGeom mg, int64_t N, int64_t j0, int64_t rows, uint8_t
   }
 }
 
+// The same through the walked zone phase and its exact rule, as the partitioned row
+// pass makes its masks: a thread per 16 columns from col0, mirrored to the columns
+// left of the axis where the row pass runs the others only.
+__global__ void k_mask_walk(MaskGeom mg, PhaseRule ph, int64_t N, int64_t j0, int64_t rows, int64_t col0, uint8_t* out) {
+  const int64_t chunks = (N - col0 + 15) / 16, total = rows * chunks;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = t / chunks, x = col0 + 16 * (t % chunks), dj = j0 + r - mg.c, dj2 = dj * dj, di0 = x - mg.c;
+    uint32_t lv[4] = {0u, 0u, 0u, 0u}, w = 0u;
+    // (a chunk that misses the disc is closed, as in the row pass)
+    const int64_t near = di0 > 0 ? di0 : di0 + 15 < 0 ? di0 + 15 : 0;
+    const bool meets = dj2 + near * near <= mg.sR;
+    if (meets) {
+      if (mg.levels >= 2) chunk_levels(di0, dj2, mg, ph, lv);
+      else if (!walk_bits16(walk16(di0, dj2, ph), ph, w)) w = chunk_bits(x, dj2, mg);
+    }
+    for (int k = 0; k < 16 && x + k < N; ++k) {
+      const int64_t di = di0 + k;
+      uint8_t v = 0;
+      if (meets && dj2 + di * di <= mg.sR) v = mg.levels >= 2 ? (uint8_t)(1 + ((lv[k >> 2] >> (8 * (k & 3))) & 0xFFu)) : (uint8_t)((w >> k) & 1u);
+      out[r * N + x + k] = v;
+      if (col0 > 0 && mg.c - di >= 0) out[r * N + mg.c - di] = v;
+    }
+  }
+}
+
 }  // namespace
 
 fzp_status bluestein_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t s) {
-  k_mask<<<1024, 256, 0, s>>>(P.mg, P.N, j0, rows, out);
+  // a deformed phase plate's row pass takes the zone rule per sample
+  if (P.bs.seg && !(P.has_deform && P.levels >= 2))
+    k_mask_walk<<<1024, 256, 0, s>>>(P.mg, phase_rule(P, nullptr), P.N, j0, rows, P.bs.col0, out);
+  else
+    k_mask<<<1024, 256, 0, s>>>(P.mg, P.N, j0, rows, out);
   P.launches += 1;
   FZP_CUDA_TRY(cudaGetLastError());
   return FZP_OK;
