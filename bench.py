@@ -33,11 +33,10 @@ config); --form bluestein times the plain FP32 form itself, with --conv its
 row convolution (partitioned into 4096-point blocks, the default, or the
 paper's single L-point convolution).  Beside the dense form the line carries
 the plain FP32 form with both convolutions ("plain_fp32": partitioned,
-"plain_fp32_single"), each timed on the whole aperture up to D = 0.25 m and
-on 16 stripes spread evenly over the aperture above (--plain-rows R rows in
-all; the partitioned convolution's cost per row follows the row's disc
-chord, so a central sample would understate it); --e2e-steps 0 leaves out
-the end-to-end leg; --ref-rows sets the oracle's rows per step in the
+"plain_fp32_single"), timed on the whole aperture (the single convolution
+above D = 0.25 m on 16,385 rows about the axis: its rows all cost the same, and
+mirror images fold as in the whole; --plain-rows R central rows in either);
+--e2e-steps 0 leaves out the end-to-end leg; --ref-rows sets the oracle's rows per step in the
 reference arm.
 
 The cpu_baseline leg also checks parity: the oracle's FP64 field of its timed
@@ -107,8 +106,8 @@ SACZT_SAMPLE_D = 2e-3
 # launches), from a one-pass ncu capture of this workload; reported only while
 # the kernel's sources hash to what was captured (null otherwise).
 KERNEL_SOURCES = {
-    "dense": ["nodes.cu", "dense.cu", "membrane.cuh", "tc_ptx.cuh", "fzp_internal.cuh"],
-    "bluestein": ["bluestein.cu", "fzp_internal.cuh"],
+    "dense": ["nodes.cu", "dense.cu", "membrane.cuh", "zone_phase.cuh", "tc_ptx.cuh", "fzp_internal.cuh"],
+    "bluestein": ["bluestein.cu", "membrane.cuh", "zone_phase.cuh", "fzp_internal.cuh"],
 }
 TRAFFIC = {
     # both launches of a row pass (the cluster launch and the single-CTA band
@@ -292,6 +291,16 @@ def decimated_flops(info: dict, j0: int, j1: int, flat: bool) -> float:
         inside = both / (8.0 if whole else 4.0) + (inside - both) / 2.0
         rows -= max(0, h)
     return 14.0 * inside + rows / 2.0 * (2 * 5.0 * 4096 * 12 + 8.0 * 4096)
+
+
+def plain_range(N: int, plain_rows: int, conv: str) -> tuple:
+    """Rows [a, b) on which the plain FP32 form is timed: all of them, or about
+    `plain_rows` central ones, as many on either side of the axis (-1: all, but
+    16,385 for the single convolution of more than 316,057 rows)."""
+    want = plain_rows if plain_rows >= 0 else (0 if conv == "partitioned" or N <= 316057 else 16384)
+    c = (N - 1) // 2
+    h = c if want <= 0 else min(c, max(1, want // 2))
+    return c - h, c + h + 1
 
 
 def node_count(info: dict, lam: float, f: float, M: int, pitch: float, deformed: bool = False) -> int:
@@ -711,7 +720,8 @@ def main():
     ap.add_argument("--e2e-steps", type=int, default=3)
     ap.add_argument("--no-plain", action="store_true", help="skip timing the plain FP32 Bluestein form")
     ap.add_argument("--plain-rows", type=int, default=-1,
-                    help="rows of the plain form's timed sample (0: all; -1: all up to N = 316,057, else 16,384)")
+                    help="rows of the plain form's timed sample (0: all; -1: all, with the single convolution "
+                         "16,385 above N = 316,057)")
     ap.add_argument("--replicas", action="store_true",
                     help="N > 1: every rank propagates the whole aperture (weak scaling) instead of its rows")
     ap.add_argument("--instances", type=int, default=256, help="membranes workload: instances per batch")
@@ -968,23 +978,18 @@ def main():
     # the split-BF16 dense form with it), both of its row convolutions:
     # partitioned (the library's FP32 default) and single (one L-point
     # convolution per row, the paper's structure); one warm and one timed
-    # step each, on the whole aperture or on 16 stripes spread evenly over it
+    # step each.  The partitioned form runs the whole aperture, as the dense form
+    # does (a part of the rows would not take the same symmetry folds); the
+    # single convolution, whose rows all cost the same, a central sample of
+    # large apertures with as many rows on either side of the axis
     plain = {}
     if args.form == "dense" and not args.no_plain:
-        prow = args.plain_rows if args.plain_rows >= 0 else (0 if N <= 316057 else 16384)
-        rows = N if prow <= 0 else min(N, prow)
-        if rows == N:
-            ranges = [(0, N)]
-        else:
-            ns, h = 16, max(1, rows // 16)
-            ranges = [(max(0, int((k + 0.5) * N / ns) - h // 2), max(0, int((k + 0.5) * N / ns) - h // 2) + h)
-                      for k in range(ns)]
-            rows = ns * h
         for conv, key in ((fzp.CONV_PARTITIONED, "partitioned"), (fzp.CONV_SINGLE, "single")):
+            pa, pb_ = plain_range(N, args.plain_rows, key)
+            rows = pb_ - pa
             with fzp.Plan(**dict(params, form=fzp.FORM_BLUESTEIN, precision=fzp.PREC_FP32, conv=conv)) as pb:
                 def run_rows():
-                    for k, (a, b) in enumerate(ranges):
-                        pb.propagate_roi(a, b, U, accumulate=k > 0, stream=stream)
+                    pb.propagate_roi(pa, pb_, U, stream=stream)
                 run_rows()
                 torch.cuda.synchronize(dev)
                 e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -995,12 +1000,12 @@ def main():
                 torch.cuda.synchronize(dev)
                 pms = e0.elapsed_time(e1)
                 if parity is not None:
-                    pa, pb_ = parity["rows"]
+                    ra, rb = parity["rows"]
                     parity[f"rel_l2_I_bluestein_fp32_{key}"] = _rel_l2(
-                        _rows_intensity(fzp, torch, pb, M, pa, pb_, stream, dev), Iref)
+                        _rows_intensity(fzp, torch, pb, M, ra, rb, stream, dev), Iref)
             rec = {"form": "bluestein", "conv": key, "dtype": "f32", "value": rows * N / (pms / 1e3) / 1e9,
                    "unit": UNIT, "ms_per_step": pms, "rows": rows,
-                   "row_sample": "whole aperture" if rows == N else f"16 stripes of {rows // 16} rows spread over N"}
+                   "row_sample": "whole aperture" if rows == N else f"{rows} rows about the axis"}
             if rows == N:
                 rec.update(fwhm_x=mb["fwhm_x"], de_lobe=mb["de_lobe"])
             plain[key] = rec

@@ -169,3 +169,16 @@ def test_membrane_batch_roofline_follows_the_majority_form():
     inside = bench.disc_samples(base["N"], base["c"], base["s_R"], 0, base["N"])
     assert roof["bound"] == "tensor" and abs(roof["achieved"] - 2 * 24.0 * 256 * inside / 1e12) < 1e-9
     assert bench.membrane_forms_and_roofline(fzp, [], 256, 1, ms) == ({}, None)
+
+
+def test_plain_comparator_takes_the_same_folds():
+    """The FP32 form that the dense form is compared with runs rows that are their
+    own mirror image: the whole aperture, or a sample centred on the axis."""
+    import bench
+    for N in (2529, 316057, 316059, 1264223):
+        assert bench.plain_range(N, -1, "partitioned") == (0, N)
+        for rows, conv in ((-1, "single"), (0, "single"), (1024, "partitioned"), (10 * N, "single")):
+            a, b = bench.plain_range(N, rows, conv)
+            assert 0 <= a and b <= N and a + b - 1 == N - 1
+    assert bench.plain_range(1264223, -1, "single") == (632111 - 8192, 632111 + 8193)
+    assert bench.plain_range(316057, -1, "single") == (0, 316057)
