@@ -328,6 +328,7 @@ struct Plan {
   float* d_C1 = nullptr;       // row intermediate [2M][chunk_rows] (FP32 forms)
   double* d_C1d = nullptr;     // row intermediate [2M][chunk_rows] (FP64 form)
   int64_t chunk_rows = 0;
+  bool c1_images = true;        // false: no memory for more than one image of C1
   int64_t c1_rows = 0;          // rows of C1: 2M rounded up to 512
   double2* d_Uacc = nullptr;   // FP64 ROI accumulator M*M
   int* d_err = nullptr;        // device error word (bounded waits)
@@ -349,10 +350,12 @@ struct Plan {
 };
 
 // Elements of a plan's row intermediate: C1 of one chunk; a small membrane on
-// nodes takes eight images of its two masks' rows.
+// nodes takes eight images of its two masks' rows where the memory is there (they
+// make its sums reproducible; c1_images).
 inline size_t c1_elems(const Plan& P) {
   const size_t all = (size_t)((2 * (int64_t)P.M + 511) / 512 * 512) * (size_t)P.chunk_rows;
-  if (P.nd.n > 0 && P.has_deform && P.N <= 8192) return all > 2048u * (size_t)P.chunk_rows ? all : 2048u * (size_t)P.chunk_rows;
+  if (P.c1_images && P.form == FZP_FORM_DENSE && P.nd.n > 0 && P.has_deform && P.N <= 8192)
+    return all > 2048u * (size_t)P.chunk_rows ? all : 2048u * (size_t)P.chunk_rows;
   return all;
 }
 

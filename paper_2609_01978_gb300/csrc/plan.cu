@@ -411,7 +411,8 @@ fzp_status fzp_plan(const fzp_params* params, fzp_plan_t* out) {
     const int64_t M2 = (2 * (int64_t)P->M + 511) / 512 * 512;
     P->chunk_rows = chunk_rows_for(*P);
     P->c1_rows = M2;
-    // The row intermediate of one chunk.  When it cannot be allocated the
+    // The row intermediate of one chunk.  When it cannot be allocated its
+    // further images (c1_elems) are given up, then the
     // chunk is halved (down to 256 rows) and the allocation retried, as the
     // paper's engine halves its row batch on a GPU out-of-memory error
     // (Fig. 18 Stage 2); only then is FZP_E_OOM returned.
@@ -427,7 +428,15 @@ fzp_status fzp_plan(const fzp_params* params, fzp_plan_t* out) {
         P->device_bytes += bytes;
         break;
       }
-      if (e != cudaErrorMemoryAllocation || P->chunk_rows <= 256) break;
+      if (e != cudaErrorMemoryAllocation) break;
+      if (P->c1_images) {
+        P->c1_images = false;
+        if (c1_elems(*P) * esz < bytes) {
+          cudaGetLastError();
+          continue;
+        }
+      }
+      if (P->chunk_rows <= 256) break;
       cudaGetLastError();
       P->chunk_rows = std::max<int64_t>(256, (P->chunk_rows / 2 + 255) / 256 * 256);
     }
