@@ -1129,16 +1129,21 @@ __device__ __forceinline__ void mask_words(const RowWalk& w, const MaskGeom& g, 
     if (redo) wd[q] = exact_word<MASK>(pb, nb, 0x3F803F80u, disc, q);
 }
 
+// A warp takes 32 rows by MASK_COLS columns (a walk starts at any column; one warp per
+// 32 whole rows took 742 us for 512 rows of 5,057 columns, the row walker that
+// exported these masks before the nodes 670; now 49).
+constexpr int MASK_COLS = 256;
 __global__ void k_mask_nodes(MaskGeom mg, PhaseRule ph, int mask, int64_t N, int64_t j0, int64_t rows, uint8_t* out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r0 = warp * 32; r0 < rows; r0 += nwarps * 32) {
-    const int64_t r = r0 + lane;
+  const int64_t parts = (N + MASK_COLS - 1) / MASK_COLS;
+  for (int64_t item = warp; item < (rows + 31) / 32 * parts; item += nwarps) {
+    const int64_t r = item / parts * 32 + lane, ib = item % parts * MASK_COLS, ie = ib + MASK_COLS < N ? ib + MASK_COLS : N;
     const int64_t dj = j0 + r - mg.c;
     RowWalk w;
-    row_start(w, dj, -mg.c, r < rows, mg, ph);
-    for (int64_t i0 = 0; i0 < N; i0 += 32) {
+    row_start(w, dj, ib - mg.c, r < rows, mg, ph);
+    for (int64_t i0 = ib; i0 < ie; i0 += 32) {
       const uint32_t disc = chord_bits(w.di0, w.bmax);
       uint8_t v[32];
 #pragma unroll
@@ -1496,7 +1501,7 @@ fzp_status nodes_epilogue(Plan& P, void* d_field, int accumulate, bool sym, cuda
 }
 
 fzp_status nodes_mask(Plan& P, int64_t j0, int64_t rows, uint8_t* out, cudaStream_t s) {
-  const int64_t warps = (rows + 31) / 32;
+  const int64_t warps = (rows + 31) / 32 * ((P.N + MASK_COLS - 1) / MASK_COLS);
   const unsigned grid = (unsigned)std::min<int64_t>((warps + 3) / 4, 65535);
   k_mask_nodes<<<grid, 128, 0, s>>>(P.mg, phase_rule(P, nullptr), mask_kind(P), P.N, j0, rows, out);
   P.launches += 1;
