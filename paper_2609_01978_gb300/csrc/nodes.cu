@@ -1336,21 +1336,56 @@ static void place_nodes(Plan& P, bool even, double band, int hi) {
   z.msh = -first / z.h;
 }
 
+// Do the nodes pay?  The interpolation runs in FP64 at two multiply-adds per clock
+// and SM (0.63 million a microsecond), so on small grids with a large ROI, where it
+// cannot fold (off the axis, membranes), it takes longer than all that the nodes
+// save.  Microseconds of both sides, fitted to whole propagations of N = 41 to 5,401
+// with either route (general / nodes):
+//   FP32, membrane, 512^2, 128 nodes: N = 401 120 / 202, 801 161 / 213, 1,601 258 / 233
+//   FP32, off the axis, 1024^2, 128 nodes: 801 245 / 415, 1,601 295 / 423
+//   FP32, on the axis, 512^2: 41 73 / 68, 1,601 117 / 82; 64^2: 41 48 / 55
+//   dense, off the axis, 1024^2, 128 nodes: 801 260 / 423, 2,401 355 / 434, 3,601 538 / 436
+//   dense, membrane, 1024^2, 64 nodes: 201 310 / 340, 401 372 / 343
+//   SA-CZT, off the axis, 1024^2, 128 nodes: 401 431 / 479, 801 719 / 485
+// FP32 grids of 2,000 and more columns keep the nodes, whose error is the smaller one
+// (N = 2,401, 512^2: 1.6e-7 of the field against 3.5e-7) and whose rows are decimated
+// from about 3,000 on.
+static bool nodes_pay(const Plan& P) {
+  const NodeSet& z = P.nd;
+  const double ns = z.ns, Mo = z.Mo, M2 = (double)P.M * P.M, N = (double)P.N;
+  const bool sym = !P.has_deform;  // the field of a whole flat plate is its own transpose
+  const double interp = 1.15 * (2.0 * ns * Mo * ns * (sym ? 2.0 : 1.0) + 2.0 * ns * Mo * Mo * (sym ? 0.5 : 1.0)) / 630e3;
+  const double epilogue = 1e-4 * M2;  // the general one: an FP64 sine pair per sample
+  if (P.form == FZP_FORM_SACZT)
+    return 88.0 + interp < (P.M % 128 ? 30.0 + 0.9 * N : 148.0 + 0.45 * N) + epilogue;
+  if (P.form == FZP_FORM_DENSE) {
+    const double passes = P.passes.empty() ? 1.0 : (double)P.passes.size();
+    const double row = P.has_deform ? 0.14 : P.M > 512 ? 0.075 : 0.045;
+    return interp < (P.M > 64 ? 25.0 : 5.0) + epilogue + 70.0 * (passes - 1.0) + row * N * passes;
+  }
+  const double side = P.M / 1024.0, row = sym ? 0.079 * side * side : 0.284 * std::pow(side, 1.6);
+  return N >= 2000.0 || interp + 7.0 < epilogue + row * N;
+}
+
 void nodes_choose(Plan& P) {
   P.nd = NodeSet{};
   const bool centred = P.msh == (double)(P.M / 2);
   if (P.form == FZP_FORM_SACZT) {
     // the propagated plane fills the padded grid, P dx wide, at the distance z_F
     if (saczt_layout(P) == FZP_OK) place_nodes(P, centred, (double)P.sa.P * P.dx * P.p / (P.lambda * P.sa.zF), 128);
-    P.nd.dist = P.sa.zF;
+    const double dist = P.sa.zF;
+    if (P.nd.n > 0 && !nodes_pay(P)) P.nd = NodeSet{};
+    P.nd.dist = dist;
     return;
   }
-  P.nd.dist = P.f;
   const bool dense = P.form == FZP_FORM_DENSE && P.precision == FZP_PREC_SPLIT_BF16 && P.cluster_req <= 1 && P.levels <= 4;
   const bool seg = P.form == FZP_FORM_BLUESTEIN && P.precision == FZP_PREC_FP32 && P.conv_req != 1;
+  P.nd.dist = P.f;
   if (!dense && !seg) return;
   const bool flat = !P.has_deform;
   place_nodes(P, flat && centred, 2.0 * P.R / (P.lambda * P.f) * P.p, dense && !flat ? 64 : 128);
+  if (P.nd.n > 0 && !nodes_pay(P)) P.nd = NodeSet{};
+  P.nd.dist = P.f;
 }
 
 bool nodes_two_masks(const Plan& P) {
