@@ -124,7 +124,8 @@ typedef struct fzp_params {
                           Split-BF16 plans whose ROI samples the field several
                           times finer than its band contract onto that many
                           interpolation nodes instead, in single CTAs (0 and 1;
-                          nodes.cu); 2 and 4 keep the clusters                    */
+                          nodes.cu), unless the grid is too small for the
+                          interpolation to pay; 2 and 4 keep the clusters         */
   int32_t levels;      /* 0 or 1: binary amplitude FZP (Fig. 2: open where the
                           paraxial zone index is odd).  L >= 2: L-level phase FZP
                           (Fig. 18 Stage 3): transmission e^{-2 pi i q/L} inside
@@ -197,19 +198,25 @@ typedef struct fzp_plan_info {
   int32_t form;          /* resolved fzp_form                                      */
   int32_t precision;     /* fzp_precision                                          */
   int32_t stripe_rows;   /* resolved stripe height                                 */
-  int64_t fft_length;    /* Bluestein length L = 2^ceil(log2(N + M - 1)) (Sec. 2.6) */
+  int64_t fft_length;    /* Bluestein length L = 2^ceil(log2(N + M - 1)) (Sec. 2.6);
+                            FP64 with a flat plate and the ROI on the axis runs
+                            the columns from the axis on, about half of it       */
   size_t device_bytes;   /* device memory owned by the plan (batch: by the batch)  */
   int32_t promote;       /* dense: K blocks per tensor-memory accumulation chunk   */
   int32_t row_batch;     /* Bluestein: aperture rows per FFT pass launch           */
   int64_t chunk_rows;    /* aperture rows per row-pass chunk                       */
-  int32_t cluster;       /* dense: CTAs per cluster sharing each mask tile         */
+  int32_t cluster;       /* dense: CTAs per cluster sharing each mask tile (what the
+                            request resolves to; plans on nodes run single CTAs)  */
   int32_t fft_inner;     /* Bluestein: inner FFT length L2 of the four-step split
                             L = L1 L2 (L itself when L <= the inner limit)        */
   int32_t ctas;          /* dense: CTAs of the persistent row-pass launch (whole
-                            clusters that are resident at once)                   */
+                            clusters that are resident at once; on nodes one on
+                            every SM)                                             */
   int32_t levels;        /* phase levels L (0: binary amplitude FZP)               */
   int32_t passes;        /* dense form: signed-mask passes per row chunk (1, or L/2
-                            for a phase plate with L >= 4)                         */
+                            for a phase plate with L >= 4, 2 for a membrane; on 64
+                            nodes a membrane's two, and those of four levels, run
+                            as one)                                               */
   int32_t centre_open;   /* 1: positive-centred binary plate (even zones open)     */
   int32_t conv;          /* Bluestein: 1 single L-point convolution per row, 2
                             partitioned into 4096-point blocks; 0 other forms      */

@@ -950,11 +950,12 @@ __global__ void __launch_bounds__(STH) k_seg_tables(int64_t nseg, int64_t col0, 
 // Row pass of the partitioned convolution: rows j0 + r, r = blockIdx.x,
 // blockIdx.x + gridDim.x, ... (interleaved, so every CTA gets rows from the
 // whole range of chord lengths); writes C1 like k_f3.  The transmission of a
-// block's samples: SEG_FLAT, binary amplitude plate without deformation, open
-// bits per chunk of 16 columns (chunk_bits); SEG_LEVELS, phase plate without
-// deformation, zone steps per chunk (chunk_zones) and the level's phasor from
-// a table; SEG_GENERAL, the transmission function per sample (membrane
-// phase).  A block's input chirp loads are issued together before the
+// block's samples, by chunks of 16 columns whose zone phase is walked (the exact
+// rule where it comes near a zone's end): SEG_FLAT, binary amplitude plate, open
+// bits; SEG_LEVELS, phase plate, a level byte per column and the level's phasor
+// from a table; SEG_MEMBRANE and SEG_DIRECT, deformed binary plate, open bits and
+// the membrane's phase; SEG_GENERAL, deformed phase plate, the transmission
+// function per sample.  A block's input chirp loads are issued together before the
 // transmission is evaluated, and the spectra G_s before the last FFT pass,
 // so each waits one memory latency.
 //
