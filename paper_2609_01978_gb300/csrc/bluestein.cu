@@ -1671,10 +1671,11 @@ DeformCoef deform_coef(const Plan& P) {
     c.h2[k] = (float)(d.ridge_h[k] * k2);
     c.rho[k] = (float)std::exp(-2.0 * (P.dx * P.dx / (2.0 * sg * sg)) * nx * nx);
     c.eta[k] = (float)-std::expm1(-2.0 * (P.dx * P.dx / (2.0 * sg * sg)) * nx * nx);
-    // full width along a row (in columns) below 64
-    if (P.dx * P.dx * nx * nx * 64.0 * 64.0 > d.ridge_width[k] * d.ridge_width[k]) c.direct = 1;
+    const double across = std::fabs(nx) * P.dx;  // the full width along a row is width / across columns
+    if (12.0 * across > d.ridge_width[k]) c.direct = 2;
+    else if (64.0 * across > d.ridge_width[k]) c.direct = std::max(c.direct, 1);
   }
-  if (c.z4 > 3.0f) c.direct = 1;
+  if (c.z4 > 3.0f) c.direct = 2;
   return c;
 }
 

@@ -595,11 +595,16 @@ __device__ __forceinline__ void cx_store_n(const DeformCoef& d, const CxRow& r, 
 }
 
 // The membrane values of a block's row parts, specialised on the ridge count
-// (0 to 3, uniform over the launch).
+// (0 to 3, uniform over the launch).  DIRECT: by column (kernels of their own: beside
+// the walks it made them 1.7 % slower).
+template <bool DIRECT>
 __device__ __forceinline__ void cx_store(const DeformCoef& d, const CxRow& r, int64_t di0, uint32_t bits, int sinpart,
                                          uint8_t* hi_row, uint8_t* lo_row, int sw, int q0, int nq) {
-  switch (d.direct ? -1 : d.n) {
-    case -1: cx_store_n<-1>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
+  if (DIRECT) {
+    cx_store_n<-1>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq);
+    return;
+  }
+  switch (d.n) {
     case 0: cx_store_n<0>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
     case 1: cx_store_n<1>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
     case 2: cx_store_n<2>(d, r, di0, bits, sinpart, hi_row, lo_row, sw, q0, nq); break;
@@ -637,7 +642,7 @@ __device__ __forceinline__ void ld_store(const float* src, uint8_t* hi_row, uint
 // generator warps form CL phases of 8 / CL warps; phase p generates the stages of
 // the CTA's global K blocks G with G % CL == p, so CL stages are in flight at once
 // and each warp has CL stage times for its rows.
-template <int CL, bool CX, bool LD = false>
+template <int CL, bool CX, bool LD = false, bool DIRECT = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_dense(const DenseArgs a, const __grid_constant__ CUtensorMap tmC1) {
   // CX: membrane pass (B planes hi and lo per stage, 3 stages); else 4 stages of one B plane.
   // LD (with CX): the B planes come from a loaded FP32 matrix (a.ld_src) instead of the generator.
@@ -885,7 +890,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_dense(const DenseArgs a, con
         // membrane pass: T cos(phi) or T sin(phi), hi and lo planes
         uint32_t bits = CL == 1 ? walker_bits(w, kb * BK, state, a.mg.thr) : block_finish(w, kb * BK, a.mg, cur);
         if (a.mg.centre_open) bits = disc_bits(w, kb * BK) & ~bits;
-        cx_store(a.df, cxr, kb * BK - a.mg.c, bits, a.cx_sin, rowp, rowp + B_BYTES, sw, cp * (4 / NCP), 4 / NCP);
+        cx_store<DIRECT>(a.df, cxr, kb * BK - a.mg.c, bits, a.cx_sin, rowp, rowp + B_BYTES, sw, cp * (4 / NCP), 4 / NCP);
       } else if (a.level_mode) {
         // phase-plate pass: +1 / -1 on the pass's level sets
         uint32_t pb, nb;
@@ -1190,13 +1195,16 @@ fzp_status layout_cols(Plan& P, int64_t ncols, FormSizes* out) {
   out->A = (size_t)d.npairs * (size_t)d.kblocks * A_BYTES;
   out->sched = sizeof(int) * (size_t)(3 * ((d.kblocks + d.group_kblocks - 1) / d.group_kblocks) + 1);
   static std::atomic<uint64_t> attr1{0}, attr2{0}, attr4{0}, attr1c{0}, attr2c{0}, attr4c{0}, attr1l{0},
-      attr2l{0}, attr4l{0};
+      attr2l{0}, attr4l{0}, attr1d{0}, attr2d{0}, attr4d{0};
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<1, false>, (int)dense_smem_bytes(), attr1));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<2, false>, (int)dense_smem_bytes(), attr2));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<4, false>, (int)dense_smem_bytes(), attr4));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<1, true>, (int)dense_smem_bytes(), attr1c));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<2, true>, (int)dense_smem_bytes(), attr2c));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<4, true>, (int)dense_smem_bytes(), attr4c));
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<1, true, false, true>, (int)dense_smem_bytes(), attr1d));
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<2, true, false, true>, (int)dense_smem_bytes(), attr2d));
+  FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<4, true, false, true>, (int)dense_smem_bytes(), attr4d));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<1, true, true>, (int)dense_smem_bytes(), attr1l));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<2, true, true>, (int)dense_smem_bytes(), attr2l));
   FZP_CUDA_TRY(smem_attr_once((const void*)k_dense<4, true, true>, (int)dense_smem_bytes(), attr4l));
@@ -1332,6 +1340,9 @@ fzp_status run_dense(Plan& P, DenseArgs& a, int mode, const char* name, cudaStre
     if (mode == 2) {
       if (CL == 2) FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_dense<2, true, true>, a, tm));
       else FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_dense<4, true, true>, a, tm));
+    } else if (mode == 1 && a.df.direct > 1) {
+      if (CL == 2) FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_dense<2, true, false, true>, a, tm));
+      else FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_dense<4, true, false, true>, a, tm));
     } else if (mode == 1) {
       if (CL == 2) FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_dense<2, true>, a, tm));
       else FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_dense<4, true>, a, tm));
@@ -1341,6 +1352,8 @@ fzp_status run_dense(Plan& P, DenseArgs& a, int mode, const char* name, cudaStre
     }
   } else if (mode == 2) {
     k_dense<1, true, true><<<grid, NUM_THREADS, dense_smem_bytes(), s>>>(a, tm);
+  } else if (mode == 1 && a.df.direct > 1) {
+    k_dense<1, true, false, true><<<grid, NUM_THREADS, dense_smem_bytes(), s>>>(a, tm);
   } else if (mode == 1) {
     k_dense<1, true><<<grid, NUM_THREADS, dense_smem_bytes(), s>>>(a, tm);
   } else {

@@ -107,12 +107,14 @@ struct DeformCoef {
   // is multiplied by rho_k = exp(-2 q_k nx_k^2)
   float zc, zs, rho[3], eta[3];  // eta = 1 - rho
   float z4;  // 4 sin^2(pi kx): the wrinkle's second difference per column
-  // 1: the generators evaluate every column instead of walking.  In FP32 a walk of
-  // 32 columns holds a ridge to 8e-7 of its height down to a full width of 64
-  // columns along the row, to 6e-6 at 16, and loses it at 8 (0.03) and below; 16
-  // columns: 5e-6 at 6, lost at 4 and below; a column by itself: 1.5e-7 at any.  The
-  // wrinkle's second difference is ill-conditioned below a period of 3 columns
-  // (3e-7 at 3, 5e-6 at 2.1).
+  // Columns evaluated one by one instead of walked: 1 by the FP32 rows, 2 by the dense
+  // generators, too.  In FP32 a walk of 32 columns holds a ridge to 8e-7 of its height
+  // down to a full width of 64 columns along the row, to 6e-6 at 16, and loses it
+  // at 8 (0.03) and below; 16 columns: 2e-6 at 12, lost at 4 and below; a column by
+  // itself: 1.5e-7 at any.  The wrinkle's second difference is ill-conditioned below
+  // a period of 3 columns (3e-7 at 3, 5e-6 at 2.1).  The FP32 rows evaluate from 64
+  // columns down (they did at any width before they walked), the dense forms,
+  // whose values are kept to 2^-17, from 12.
   int direct;
 };
 

@@ -45,9 +45,8 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 // r1 rho - (1 - rho) (a ratio near one rounded to FP32 is off by 3e-8 and more
 // each, 2e-5 of g over 32 columns).  Started exactly every 16 (k_seg, k_nodes) or
 // 32 columns (k_dec).  NR ridges.  A ridge below 1e-30 at the first column is left
-// out of the walk: DeformCoef::direct keeps ridges from here whose walk could
-// rise again (a full width below 64 columns along the row; at that width it is
-// still below 1e-15 after 32 columns).
+// out of the walk: DeformCoef::direct keeps ridges from here that could rise again
+// within it.
 template <int NR>
 struct MembraneWalk {
   float s, e, tap, dt, ddt, z4;
@@ -225,9 +224,11 @@ __device__ __forceinline__ MembraneWalk2<NR> walk32(const DeformCoef& d, const C
   return MembraneWalk2<NR>(MembraneWalk<NR>(d, r, di0), MembraneWalk<NR>(d, r, di0 + 16));
 }
 
+// DIRECT: by column (kernels of their own: beside the walks it made them 4 % slower).
+template <bool DIRECT>
 __device__ __forceinline__ void cx_store2(const DeformCoef& d, const CxRow& r, int32_t di0, uint32_t bits, uint8_t* base,
                                           uint32_t plane, int sw) {
-  if (d.direct) {
+  if (DIRECT) {
     cx_store2_n(MembraneDirect2(MembraneDirect(d, r, di0), MembraneDirect(d, r, di0 + 16)), bits, base, plane, sw);
     return;
   }

@@ -83,7 +83,7 @@ constexpr int EPI_BOX = 32;
 constexpr int EPI_BYTES = EPI_WARPS * 2 * EPI_BOX * EPI_BOX * 4;  // two boxes per warp
 constexpr int ERR_BASE = 300;
 
-enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4, MASK_LOADED = 5 };
+enum { MASK_PARITY = 0, MASK_SIGNED = 1, MASK_LEVELS = 2, MASK_MEMBRANE = 3, MASK_QUAD = 4, MASK_LOADED = 5, MASK_DIRECT = 6 };  // (membranes: walked, by column)
 
 struct NodeArgs {
   MaskGeom mg;              // c = 0 for a folded (flat) plate
@@ -105,7 +105,7 @@ struct NodeArgs {
 
 template <int NT, int MASK>
 struct Shape {
-  static constexpr bool CX = MASK == MASK_MEMBRANE;
+  static constexpr bool CX = MASK == MASK_MEMBRANE || MASK == MASK_DIRECT;
   static constexpr bool LD = MASK == MASK_LOADED;                 // a real FP32 matrix in place of the masks
   static constexpr bool TWO = CX || MASK == MASK_QUAD;            // two masks: one accumulator each
   static constexpr int BN = (NT == 1 && !TWO && !LD) ? 512 : 256; // rows per unit
@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_nodes(const NodeArgs a, cons
           } else if constexpr (CX) {
             const uint32_t bits = block_open(w[0], a.mg, a.ph);
             if (!stage_wait(&empty[stage], phase ^ 1, abort_flag, a.err, ERR_BASE + 5)) { ok = false; break; }
-            cx_store2(a.df, cxr, w[0].di0, bits, rp, PLANE, sw);
+            cx_store2<MASK == MASK_DIRECT>(a.df, cxr, w[0].di0, bits, rp, PLANE, sw);
           } else if constexpr (MASK == MASK_QUAD) {
             uint32_t re[16], im[16];
             bool redo;
@@ -1471,7 +1471,7 @@ fzp_status nodes_rows(Plan& P, int64_t j0, int64_t rows, bool octant, cudaStream
   const int mask = mask_kind(P);
   if (mask == MASK_MEMBRANE) {
     a.df = deform_coef(P);
-    return launch<1, MASK_MEMBRANE>(P, a, s);
+    return a.df.direct > 1 ? launch<1, MASK_DIRECT>(P, a, s) : launch<1, MASK_MEMBRANE>(P, a, s);
   }
   if (mask == MASK_QUAD) return launch<1, MASK_QUAD>(P, a, s);
   if (z.ns == 64) return mask == MASK_PARITY ? launch<1, MASK_PARITY>(P, a, s) : launch<1, MASK_SIGNED>(P, a, s);

@@ -1,8 +1,8 @@
 """Membranes whose ridges are a few columns wide, in every form that takes a
 membrane: rows of the FP32 form without decimation, with 16 and with 32 columns
 to a grid point, the dense form on nodes and in clusters.  Widths on both sides
-of the generators' rule (64 columns along the row: below it every column is
-evaluated, above it the phase is walked); a ridge across the rows, one at an
+of the generators' rule (every column evaluated below 64 columns along the row,
+in the dense form below 12; walked above); a ridge across the rows, one at an
 angle, one nearly along them.
 
 Fields are compared with the FP64 form's.  Tolerance as for smooth membranes: FP32
@@ -33,7 +33,7 @@ def env():
 
 @pytest.mark.parametrize("form,N,cluster", [("fp32", 1501, 0), ("fp32", 2921, 0), ("fp32", 5831, 0), ("dense", 1501, 0),
                                             ("dense", 1501, 1), ("dense", 1501, 2)])
-@pytest.mark.parametrize("width", [1, 2, 5, 8, 12, 40, 63.5, 64.5])
+@pytest.mark.parametrize("width", [1, 2, 5, 8, 11.5, 12, 40, 63.5, 64.5])
 def test_ridge_widths(env, form, N, cluster, width):
     fzp, torch = env
     D, M = (N - 0.5) * DX, 64 if form == "fp32" else 128
