@@ -303,16 +303,24 @@ def plain_range(N: int, plain_rows: int, conv: str) -> tuple:
     return c - h, c + h + 1
 
 
-def node_count(info: dict, lam: float, f: float, M: int, pitch: float, deformed: bool = False) -> int:
-    """Nodes per axis that the dense form's contraction runs on (nodes.cu), for an
-    ROI centred on the focus: the positive half of n nodes for a flat plate,
-    all of them for a membrane; 0 where the ROI's band takes the general kernel."""
+def node_count(info: dict, lam: float, f: float, M: int, pitch: float, deformed: bool = False, dense: bool = True) -> int:
+    """Nodes per axis that the dense form's contraction (or the FP32 form's rows)
+    run on (nodes.cu), for an ROI centred on the focus: the positive half of n
+    nodes for a flat plate, all of them for a membrane; 0 where the ROI's band
+    takes the general kernel."""
     dof = (M - (1 if deformed else 0)) * pitch * 2.0 * info["R"] / (lam * f)
     for n, most in ((64, 36.0), (128, 80.0), (256, 170.0)):
         ns = n if deformed else n // 2
-        if ns in (64, 128) and not (deformed and ns > 64) and dof <= most:
+        if ns in (64, 128) and not (deformed and dense and ns > 64) and dof <= most:
             return ns
     return 0
+
+
+def upload_bytes(info: dict, nodes: int, parities: int) -> int:
+    """Bytes that a plan copies to the device: the zone-threshold table and, on nodes,
+    the factor of each parity's node matrix, by columns and by rows (a centred flat
+    plate has two parities, other plates and the instances of a batch one)."""
+    return 8 * (info["n_thresholds"] + 2 * parities * nodes * nodes)
 
 
 def node_flops(info: dict, nodes: int, j0: int, j1: int, deformed: bool = False) -> float:
@@ -437,7 +445,8 @@ def run_membranes(args, fzp, torch, dev, ws, pg, rank, local):
         h2d = 0
         for _ in range(n_e2e):
             b2 = fzp.Batch(probs)
-            h2d = sum(8 * b2.info(i)["n_thresholds"] for i in range(len(probs)))
+            h2d = sum(upload_bytes(inf, node_count(inf, m.lam, fnum * m.D, M, m.lam * fnum / 8, True, inf["conv"] == 0), 1)
+                      for inf, m in zip(infos, mem))
             b2.propagate(fields, stream=stream)
             for i in range(len(probs)):
                 hosts[i].copy_(fields[i], non_blocking=True)
@@ -849,6 +858,7 @@ def main():
     # roofline of the dominant kernel, from CUDA events on its own stream
     peaks, peak_kind = _peaks()
     avg_ms = prof["dominant_ms"] / max(1, prof["dominant_launches"])
+    nodes = 0  # (the SA-CZT's are not modelled here)
     if args.form == "dense":
         # algorithmic work of the contraction: 2 real rows (Re, Im) x M outputs x
         # 2 flops x 2 split terms per aperture sample inside the disc = 8 M
@@ -887,7 +897,8 @@ def main():
     else:
         launches = max(1, prof["dominant_launches"])
         flat = not wl.get("deform")
-        nodes = node_count(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], not flat)
+        if info["conv"] == 2:
+            nodes = node_count(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], not flat, False)
         if info["conv"] == 2 and (flat or params.get("levels", 0) < 2) and \
                 decimation(info, wl["lam"], wl["fnum"] * wl["D"], M, params["pitch"], flat):
             flops_launch = decimated_flops(info, j0, j1, flat) * args.steps / launches
@@ -922,7 +933,7 @@ def main():
         h2d = 0
         for _ in range(args.e2e_steps):
             with fzp.Plan(**params) as p2:
-                h2d = 8 * p2.info["n_thresholds"]  # the zone-threshold table, the plan's one upload
+                h2d = upload_bytes(p2.info, nodes, 1 if wl.get("deform") else 2)
                 p2.propagate_roi(j0, j1, U, stream=stream)
                 if sharded:
                     pg.all_reduce(U)

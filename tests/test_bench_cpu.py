@@ -182,3 +182,17 @@ def test_plain_comparator_takes_the_same_folds():
             assert 0 <= a and b <= N and a + b - 1 == N - 1
     assert bench.plain_range(1264223, -1, "single") == (632111 - 8192, 632111 + 8193)
     assert bench.plain_range(316057, -1, "single") == (0, 316057)
+
+
+def test_uploaded_bytes_count_the_node_factors():
+    """What a plan copies to the device: its zone thresholds and the factors of its
+    node matrices (64 nodes: 4,096 values by columns and as many by rows)."""
+    import bench
+    info = {"n_thresholds": 1000, "R": 0.5}
+    assert bench.upload_bytes(info, 0, 2) == 8000
+    assert bench.upload_bytes(info, 64, 2) == 8000 + 8 * 4 * 4096
+    assert bench.upload_bytes(info, 64, 1) == 8000 + 8 * 2 * 4096
+    lam, f = 550e-9, 5.0
+    flat = lambda M, **k: bench.node_count(info, lam, f, M, lam * 5 / 8, **k)
+    assert flat(512) == 64 and flat(1024) == 128 and flat(128, deformed=True) == 64
+    assert flat(512, deformed=True) == 0 and flat(512, deformed=True, dense=False) == 128
