@@ -129,8 +129,10 @@ __device__ __forceinline__ double2 peer_load(uint32_t addr, double2) {
 // 35 with sum4 in place of FP32 additions.
 // FP64, 2,529 rows, 129 x 129 outputs, bound by the FP64 pipe: 0.46 ms, with the
 // tiles on and above the diagonal only a propagation takes 0.09 ms less.
-template <typename R, bool TAB = false, int NA = 4>
-__global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
+// Large grids (FP32 outputs that are ROI samples) run it at 80 registers, three blocks
+// to an SM (MINB) instead of two of 111.
+template <typename R, bool TAB = false, int NA = 4, int MINB = 1>
+__global__ void __launch_bounds__(256, MINB) k_colpass(ColArgs g, const R* __restrict__ C1, double2* __restrict__ Uacc) {
   using C = typename Cplx<R>::T;
   constexpr int TN = 16 * NA, TM = 16 * NA;
   constexpr int TILE = TJ * (TN + 1), POOL = col_clusters<R, NA> && TN * TM > 2 * TILE ? TN * TM : 2 * TILE;
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(256) k_colpass(ColArgs g, const R* __restrict_
     for (int b = 0; b < NA; ++b) add(n0 + tn + 16 * a, m0 + tm + 16 * b, (double)acc[a][b].x, (double)acc[a][b].y);
 }
 
-template <typename R, bool TAB = false, int NA = 4>
+template <typename R, bool TAB = false, int NA = 4, int MINB = 1>
 fzp_status run_colpass(const ColArgs& g, unsigned tx, unsigned ty, const R* C1, double2* Uacc, cudaStream_t s) {
   unsigned tz = (unsigned)((g.rows + g.jc - 1) / g.jc);
   const bool clusters = col_clusters<R, NA> && tz >= CZ;
@@ -323,7 +325,7 @@ fzp_status run_colpass(const ColArgs& g, unsigned tx, unsigned ty, const R* C1, 
   attr[0].val.clusterDim.z = CZ;
   cfg.attrs = attr;
   cfg.numAttrs = clusters ? 1 : 0;
-  FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_colpass<R, TAB, NA>, g, C1, Uacc));
+  FZP_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_colpass<R, TAB, NA, MINB>, g, C1, Uacc));
   return FZP_OK;
 }
 
@@ -395,11 +397,33 @@ fzp_status column_pass(Plan& P, int64_t j0, int64_t rows, RowKind kind, cudaStre
   const bool tri = P.nd.tri && tx == ty;
   g.tri = tri ? tx : 0;
   const int64_t tiles = tri ? (int64_t)tx * (tx + 1) / 2 : (int64_t)tx * ty;
-  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (rows * tiles / BLOCKS + TJ - 1) / TJ * TJ));
+  // As many blocks a tile as are resident at once (8 x 8 tiles: four; with the quotient
+  // not rounded down five, which clusters made eight: 8,001 rows in BF16 877 -> 1,045 us).
+  // More tiles than half of the blocks: unevenly long blocks, unless the second of a tile
+  // had too few rows to be worth its sums (101 rows of 16 x 16 tiles: 50 us in one block
+  // a tile, 63 in two).
+  const int64_t fit = BLOCKS / tiles, share = fit > 1 ? (rows + fit - 1) / fit : rows * tiles / BLOCKS;
+  g.jc = std::min<int64_t>(2048, std::max<int64_t>(2 * TJ, (share + TJ - 1) / TJ * TJ));
+  if (fit <= 1 && rows > g.jc && rows < g.jc + 64 && rows <= 2048) g.jc = rows;
+  // several waves: three blocks to an SM, as many a tile as leave the last wave fullest
+  const int64_t least = (rows + 2047) / 2048;
+  const bool many = !nodes && P.precision != FZP_PREC_FP64 && tiles * least > BLOCKS;
+  if (many) {
+    int64_t best = INT64_MAX;
+    for (int64_t z = least; z <= least + 8; ++z) {
+      const int64_t jc = ((rows + z - 1) / z + TJ - 1) / TJ * TJ, run = z < CZ ? z : (z + CZ - 1) / CZ * CZ;
+      const int64_t t = (tiles * run + BLOCKS * 3 / 2 - 1) / (BLOCKS * 3 / 2) * jc;
+      if (t < best) {
+        best = t;
+        g.jc = jc;
+      }
+    }
+  }
   P.launches += 1;
   const unsigned gx = (unsigned)(tri ? tiles : tx), gy = (unsigned)(tri ? 1 : ty);
   return even                           ? run_colpass<double, false, 3>(g, gx, gy, P.d_C1d, P.d_Uacc, s)
          : P.precision == FZP_PREC_FP64 ? run_colpass<double>(g, gx, gy, P.d_C1d, P.d_Uacc, s)
+         : many                         ? run_colpass<float, false, 4, 3>(g, gx, gy, P.d_C1, P.d_Uacc, s)
                                         : run_colpass<float>(g, gx, gy, P.d_C1, P.d_Uacc, s);
 }
 
