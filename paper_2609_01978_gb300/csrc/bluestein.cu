@@ -1645,6 +1645,12 @@ int bluestein_decimation(const Plan& P) {
   return 32 * u <= 0.17 ? 32 : 16 * u <= 0.17 ? 16 : 0;
 }
 
+int64_t bluestein_wave(const Plan& P) {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) cudaGetLastError();
+  return (P.bs.dec ? 4 : 2) * (int64_t)sms;  // two CTAs to an SM, two decimated rows to a transform
+}
+
 DeformCoef deform_coef(const Plan& P) {
   DeformCoef c{};
   const fzp_deform& d = P.deform;

@@ -364,6 +364,9 @@ inline size_t c1_elems(const Plan& P) {
 // Columns to a grid point of the FP32 form's decimated rows (host), 0: none.
 int bluestein_decimation(const Plan& P);
 
+// Rows of the partitioned row pass that are in flight at once.
+int64_t bluestein_wave(const Plan& P);
+
 // FP32 deformation coefficients of a plan with a deformation (host).
 DeformCoef deform_coef(const Plan& P);
 

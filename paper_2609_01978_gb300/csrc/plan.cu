@@ -324,6 +324,14 @@ fzp_status propagate_rows(Plan& P, int64_t a, int64_t b, bool* sym, cudaStream_t
     return st;
   };
   if (!P.fold) return run(a, b, ROWS_PLAIN, false);
+  // A range about the axis that is not its own mirror image has two parts, folded and
+  // one-sided, each with its launches: where they take as many waves of CTAs as the
+  // rows one by one, those run (32 rows of 2,001, FP32, 256^2: 87 -> 63 us).
+  if (h >= 0 && up != dn && P.form == FZP_FORM_BLUESTEIN && P.bs.seg) {
+    const int64_t wave = bluestein_wave(P);
+    auto waves = [&](int64_t n) { return (n + wave - 1) / wave; };
+    if (waves(up + dn + 1) <= waves(h + 1) + waves(std::abs(up - dn))) return run(-dn, up + 1, ROWS_PLAIN, false);
+  }
   // a flat plate: the rows at distance d on either side of the axis have one
   // row transform; h: the distances present on both sides
   fzp_status st = FZP_OK;
