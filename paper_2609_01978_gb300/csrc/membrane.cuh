@@ -76,7 +76,7 @@ struct MembraneWalk {
       const float ex = d.q[k] * d0 * d0;
       if (ex < 69.0f) {
         g[k] = d.h2[k] * __expf(-ex);
-        // e^-x - 1: its series while |x| is small (ridges are hundreds of columns wide)
+        // e^-x - 1: its series while |x| is small (wide ridges)
         const float x = d.q[k] * d.nx[k] * fmaf(2.0f, d0, d.nx[k]);
         const float p = fmaf(x, fmaf(x, fmaf(x, fmaf(x, -1.0f / 120.0f, 1.0f / 24.0f), -1.0f / 6.0f), 0.5f), -1.0f);
         r1[k] = fabsf(x) < 0.125f ? x * p : __expf(-x) - 1.0f;
